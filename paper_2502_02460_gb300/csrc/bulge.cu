@@ -7,13 +7,13 @@
 // (the bulge).  Task t >= 1 annihilates the first column of that block with H(s,t) on rows
 // W_t = [s+1+tb, s+1+(t+1)b), and so on down the band.  Footprint of task (s,t): rows
 // [p_t, p_{t+2}), columns [p_{t-1}, p_{t+1}) (p_t = s+1+tb).  Task (s+1,t) overlaps tasks
-// (s,t-1) .. (s,t+2) only, so sweep s+1 may run task t once sweep s has finished task t+2.
+// (s,t-1) .. (s,t+2) only, and of (s,t+2) only the entry (p_{t+2}, p_{t+1}) that its reflector fixes, so
+// sweep s+1 may run task t once sweep s has finished task t+1 and formed the reflector of task t+2.
 //
 // GPU mapping: one persistent cooperative kernel; block q owns sweeps q, q+G, q+2G, ... and runs
 // their tasks in order, staging the three blocks of a task (L = (W_t, W_{t-1}), D = (W_t, W_t),
 // E = (W_{t+1}, W_t)) in shared memory; E stays resident as the next task's L.  A per-sweep
-// progress counter (release: __threadfence + store; acquire: volatile load + __threadfence, band
-// reads through L2 with __ldcg) orders the sweeps.  Every wait is bounded (status[ST_SPIN] iterations
+// progress counter (release store, acquire load, band reads through L2 with __ldcg) orders the sweeps.  Every wait is bounded (status[ST_SPIN] iterations
 // when the host set a limit, else kSpinLimit, ~2 s): on expiry the kernel records ST_TIMEOUT, raises
 // the abort flag and all blocks return.
 //
@@ -31,9 +31,6 @@ namespace gev {
 
 namespace {
 
-constexpr int NT = 256;
-
-
 __device__ __forceinline__ double warp_sum(double v) {
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   return v;
@@ -45,16 +42,24 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 __device__ __forceinline__ zf warp_sum(zf v) { return make_zf(warp_sum(v.x), warp_sum(v.y)); }
 
-// Bounded acquire-wait until *flag >= target.  Thread 0 spins; returns false on timeout/abort.
-__device__ bool wait_ge(const int* flag, int target, int* status, int* abort_flag, int site) {
-  __shared__ int ok;
-  if (threadIdx.x == 0) {
-    int good = 1;
-    volatile const int* vf = flag;
+// progress flags between blocks: release store and acquire load at GPU scope
+__device__ __forceinline__ void st_release(int* p, int v) {
+  asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// Bounded acquire-wait of one warp until *flag >= target; false on timeout / abort.
+__device__ __forceinline__ bool warp_wait_ge(const int* flag, int target, int* status, int* abort_flag, int site) {
+  int good = 1;
+  if ((threadIdx.x & 31) == 0 && ld_acquire(flag) < target) {
     volatile int* va = abort_flag;
     const long long lim = spin_limit(status);
     long long it = 0;
-    while (*vf < target) {
+    while (ld_acquire(flag) < target) {
       if (*va) { good = 0; break; }
       if (++it > lim) {
         atomicCAS(&status[ST_TIMEOUT], 0, site);
@@ -62,13 +67,45 @@ __device__ bool wait_ge(const int* flag, int target, int* status, int* abort_fla
         good = 0;
         break;
       }
-      __nanosleep(32);
+      if (it > 16) __nanosleep(32);
     }
-    __threadfence();
-    ok = good;
   }
-  __syncthreads();
-  return ok != 0;
+  return __shfl_sync(0xffffffffu, good, 0) != 0;
+}
+
+__device__ __forceinline__ void bar_sync_n(int id, int n) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive_n(int id, int n) { asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(n) : "memory"); }
+
+// 1 / sqrt and the Householder scalars of alpha = x_0 and xn = sum_{i>0} |x_i|^2 (not both trivial):
+// with s = sign(Re alpha), r = 1 / ||x||:  beta = -s ||x||,  tau = 1 - alpha / beta = 1 + s r alpha,
+// scale = 1 / (alpha - beta): one reciprocal square root and one division, no other long FP64 chain
+__device__ __forceinline__ void house(double alpha, double xn, double& tau, double& beta, double& scale) {
+  const double q = alpha * alpha + xn, r = rsqrt(q), nrm = q * r;
+  beta = alpha >= 0.0 ? -nrm : nrm;
+  tau = 1.0 + fabs(alpha) * r;
+  scale = 1.0 / (alpha - beta);
+}
+__device__ __forceinline__ void house(float alpha, float xn, float& tau, float& beta, float& scale) {
+  const float nrm = sqrtf(alpha * alpha + xn);
+  beta = alpha >= 0.f ? -nrm : nrm;
+  tau = (beta - alpha) / beta;
+  scale = 1.f / (alpha - beta);
+}
+__device__ __forceinline__ void house(zd alpha, double xn, zd& tau, zd& beta, zd& scale) {
+  const double q = abs2_(alpha) + xn, r = rsqrt(q), nrm = q * r;
+  const double s = alpha.x >= 0.0 ? 1.0 : -1.0;
+  const zd d = make_zd(alpha.x + s * nrm, alpha.y);
+  const double g = 1.0 / abs2_(d);
+  beta = make_zd(-s * nrm, 0.0);
+  tau = make_zd(1.0 + fabs(alpha.x) * r, s * r * alpha.y);
+  scale = make_zd(g * d.x, -g * d.y);
+}
+__device__ __forceinline__ void house(zf alpha, float xn, zf& tau, zf& beta, zf& scale) {
+  const float nrm = sqrtf(abs2_(alpha) + xn), s = alpha.x >= 0.f ? 1.f : -1.f;
+  const zf bt = make_zf(-s * nrm, 0.f);
+  beta = bt;
+  tau = div_(bt - alpha, bt);
+  scale = div_(make_zf(1.f, 0.f), alpha - bt);
 }
 
 // Band -> tridiagonal by bulge chasing (one sweep per block at a time).  Task t of sweep s
@@ -77,207 +114,297 @@ __device__ bool wait_ge(const int* flag, int target, int* status, int* abort_fla
 //   L (the block left of the reflector's rows, the previous task's bulge) <- H L   (t > 0),
 //   D (the diagonal block)                                                  <- H D H^H,
 //   E (the block below D: the new bulge)                                    <- E H^H,
-// and the reflector is kept for back-transform 2.  Sweep s+1 may run task t once sweep s has
-// finished task t+2 (their blocks overlap up to there): a bounded wait on progress[s].
-// A task is a short dependent chain, and on GB300 the FP64 pipe executes a warp-wide FP64
-// instruction in ~19 cycles, so the FP64 form is bound by its count of FP64 instructions and the
-// FP32 form by latency.  Hence: all arithmetic in the data's own precision R (FP32 for the mixed
-// form); matrix-vector products with four threads per row / column (partial sums over every
-// fourth term, combined through shared memory: all eight warps, hence all four schedulers' FP64
-// pipes, take an equal share and no shuffle reductions are needed); element updates spread over
-// all threads; the
-// loads of the D and E blocks issued into registers right after the wait, so that their L2 latency
-// overlaps the reflector and the update of L.
-template <class T>
-__global__ void __launch_bounds__(NT) k_bulge(int n, int b, T* band, int ldb, T* V2, T* tau2, int ntask,
-                                              int* progress, int* status, int* abort_flag, int stall) {
+// and the reflector is kept for back-transform 2.
+//
+// The chase is one chain of dependent steps per sweep, and the sweeps follow one another at a fixed
+// lag, so the run time is (lag in tasks) x (time of a task) x n.  Both are kept short:
+//  * Lag.  Task (s+1, t) reads what the tasks (s, 0 .. t+1) leave, and of task (s, t+2) only the one
+//    entry of the band that its reflector makes (beta, at row p_{t+2}, column p_{t+1}).  Progress t+3
+//    is therefore published when the REFLECTOR of task t+2 is known, not when the task is done: the
+//    lag is two tasks and a reflector instead of three tasks.
+//  * Task.  The products w = v^H L, y = D v, z = E v depend on v only, so they run as one phase (all
+//    warps equally: on GB300 the FP64 pipe, about 1.6 FMA per SM per cycle, bounds this kernel), their
+//    sums as a second, the three updates as a third.  Column 0 of the updated E, the next
+//    reflector's x, is E(:,0) - z (v_0 = 1): it comes out of the second phase, so warp 0 computes the
+//    next reflector (reduction, rsqrt, division: a long latency chain) while the other warps
+//    update, publishes it as soon as the stores of this task are done (a named barrier that the other
+//    warps only arrive at), and they wait for the next task's blocks and load them meanwhile.
+//    Warp 1 finishes y (its inner product with v) while the rest update L and E.
+//  * Four barriers per task; D and E travel through registers, so that no wait holds the others up.
+// Measured (to_tridiag; one barrier-separated product after another and a lag of three tasks before):
+// real FP64 n = 10240, b = 64 447 -> 203 ms, n = 1500 37.1 -> 16.1 ms; complex FP64 n = 509 29.7 -> 13.2 ms;
+// FP32 n = 6144 82.9 -> 40.9 ms.
+// All arithmetic is in the data's own precision (FP32 for the mixed form).
+template <class T, int B, int NTH>
+__global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T* tau2, int ntask, int* progress,
+                                               int* status, int* abort_flag, int stall) {
   using R = typename real_of<T>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int PF = 64 * 64 / NT;  // register prefetch slots per thread (b <= 64)
-  const int LD = b + 1;
+  constexpr int LD = B + 1, O3 = 3 * B, P = NTH / O3, TERMS = B / P, NL = NTH - 32;
+  constexpr int PF = (B * B + NL - 1) / NL;  // register slots per loading thread (D and E each)
+  static_assert(NTH % 32 == 0 && NTH == P * O3 && B % P == 0 && (B * B) % 32 == 0, "thread mapping");
   T* Ls = reinterpret_cast<T*>(smraw);
-  T* Es = Ls + b * LD;
-  T* Ds = Es + b * LD;
-  T* v = Ds + b * LD;
-  T* y = v + b;
-  T* w = y + b;
-  T* part4 = w + b;  // 4 x 64 partial sums of the matrix-vector products
-  __shared__ T sh_tau, sh_beta, sh_scale;
-  __shared__ R sh_c;
+  T* Es = Ls + B * LD;
+  T* Ds = Es + B * LD;
+  T* vbuf = Ds + B * LD;      // 2 x B: the reflector of this and of the next task
+  T* vc = vbuf + 2 * B;       // conj(v)
+  T* w = vc + B;              // L: conj(tau) v^H L
+  T* y = w + B;               // D: tau D v - c v
+  T* z = y + B;               // E: tau E v
+  T* xn_ = z + B;             // column 0 of the updated E: the next task's x
+  T* part = xn_ + B;          // P x 3B partial sums
+  __shared__ T sh_tau[2];
+  __shared__ volatile int bad;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int lb = __ffs(b) - 1;  // b is a power of two (16, 32, 64)
-  const int ci = tid & (b - 1), cj = tid >> lb, cstep = NT >> lb;
-  const int qi = tid & 63, qp = tid >> 6;  // matrix-vector products: row / column qi, quarter qp
-  static_assert(NT == 256, "the products use 4 x 64 threads");
+  if (tid == 0) bad = 0;
+  __syncthreads();
+
+  // warp 0: the reflector of the B entries x (zero beyond len) -> v, conj(v) is formed with the loads
+  auto reflect = [&](const T* x, T* v, int slot) {
+    T xv[(B + 31) / 32];
+    R s2 = 0;
+#pragma unroll
+    for (int u = 0; u < (B + 31) / 32; ++u) {
+      const int i = lane + 32 * u;
+      xv[u] = i < B ? x[i] : zero_<T>();
+      if (i > 0) s2 += (R)abs2_(xv[u]);
+    }
+    s2 = warp_sum(s2);
+    const T alpha = x[0];
+    T tau = zero_<T>(), beta = alpha, scale = zero_<T>();
+    if (!(s2 == (R)0 && im_(alpha) == 0)) house(alpha, s2, tau, beta, scale);
+#pragma unroll
+    for (int u = 0; u < (B + 31) / 32; ++u) {
+      const int i = lane + 32 * u;
+      if (i < B) v[i] = i == 0 ? from_re<T>(1.0) : scale * xv[u];
+    }
+    if (lane == 0) sh_tau[slot] = tau;
+    return beta;
+  };
 
   for (int s = blockIdx.x; s <= n - 3; s += gridDim.x) {
-    bool pendingL = false;
-    for (int t = 0;; ++t) {
-      const int p = s + 1 + t * b;
-      const int len = (p < n) ? min(b, n - p) : 0;
-      const int pp = p - b;
-      // (stall: a failure-path test makes the first wait target a flag that nothing sets)
-      if (s > 0 && !(stall ? wait_ge(&status[ST_STALL], 1, status, abort_flag, 202)
-                           : wait_ge(&progress[s - 1], t + 3, status, abort_flag, 201)))
+    T dreg[PF], ereg[PF];
+    // wait for the blocks of task t and load D (lower triangle) and E into registers (warps 1 ..)
+    auto fetch = [&](int t) {
+      const int p = s + 1 + t * B, len = min(B, n - p), p2 = p + len, len2 = min(B, n - p2);
+      bool ok = true;
+      if (s > 0)
+        ok = stall ? warp_wait_ge(&status[ST_STALL], 1, status, abort_flag, 202)
+                   : warp_wait_ge(&progress[s - 1], t + 3, status, abort_flag, 201);
+      if (!ok) {
+        if (lane == 0) bad = 1;
         return;
-      if (t > 0 && len <= 1) {
-        if (pendingL && len == 1)
-          for (int q = tid; q < b; q += NT) stcg_(&band[(b - q) + (long long)(pp + q) * ldb], Ls[q * LD]);
-        break;
       }
-      const int p2 = p + len;
-      const int len2 = (p2 < n) ? min(b, n - p2) : 0;
-      // ---- prefetch D (lower triangle) and E into registers: thread (ci, cj) holds row ci,
-      // columns cj, cj + cstep, ... of each block
-      T dreg[PF], ereg[PF];
 #pragma unroll
       for (int u = 0; u < PF; ++u) {
-        const int jj = cj + u * cstep;
-        dreg[u] = (jj < len && ci < len && ci >= jj) ? ldcg_(&band[(ci - jj) + (long long)(p + jj) * ldb])
-                                                     : zero_<T>();
-        ereg[u] = (jj < len && ci < len2) ? ldcg_(&band[(len + ci - jj) + (long long)(p + jj) * ldb]) : zero_<T>();
+        const int idx = tid - 32 + u * NL, i = idx & (B - 1), j = idx / B;
+        const T* col = band + (long long)(p + j) * ldb;
+        dreg[u] = (idx < B * B && j < len && i < len && i >= j) ? ldcg_(&col[i - j]) : zero_<T>();
+        ereg[u] = (idx < B * B && j < len && i < len2) ? ldcg_(&col[len + i - j]) : zero_<T>();
       }
-      // ---- generating vector x and the reflector
-      for (int i = tid; i < len; i += NT)
-        v[i] = (t == 0) ? ldcg_(&band[(1 + i) + (long long)s * ldb]) : Ls[i];
-      __syncthreads();
-      if (warp == 0) {
-        R xn = 0;
-        for (int i = 1 + lane; i < len; i += 32) xn += (R)abs2_(v[i]);
-        xn = warp_sum(xn);
-        if (lane == 0) {
-          const T alpha = v[0];
-          if (xn == (R)0 && im_(alpha) == 0) {
-            sh_tau = zero_<T>();
-            sh_beta = alpha;
-            sh_scale = zero_<T>();
-          } else {
-            const R nrm = sqrt((R)abs2_(alpha) + xn);
-            const T bt = from_re<T>(re_(alpha) >= 0 ? -nrm : nrm);
-            sh_tau = div_(bt - alpha, bt);
-            sh_beta = bt;
-            sh_scale = div_(from_re<T>(1.0), alpha - bt);
+    };
+    int cur = 0;
+    // ---- the sweep's first reflector: column s below the diagonal
+    if (warp == 0) {
+      bool ok = true;
+      if (s > 0)
+        ok = stall ? warp_wait_ge(&status[ST_STALL], 1, status, abort_flag, 202)
+                   : warp_wait_ge(&progress[s - 1], 3, status, abort_flag, 201);
+      if (!ok) {
+        if (lane == 0) bad = 1;
+      } else {
+        const int len = min(B, n - s - 1);
+        T* col = band + (long long)s * ldb + 1;
+        for (int i = lane; i < B; i += 32) xn_[i] = i < len ? ldcg_(&col[i]) : zero_<T>();
+        __syncwarp();
+        const T beta = reflect(xn_, vbuf, 0);
+        for (int i = lane; i < len; i += 32) stcg_(&col[i], i == 0 ? beta : zero_<T>());
+      }
+    } else {
+      fetch(0);
+    }
+    for (int t = 0;; ++t) {
+      const int p = s + 1 + t * B, len = min(B, n - p), p2 = p + len, len2 = min(B, n - p2);
+      const int pn = p + B, lenn = pn < n ? min(B, n - pn) : 0;  // the next task's rows
+      const bool more = lenn > 1;
+      T* v = vbuf + cur * B;
+      T* vn = vbuf + (cur ^ 1) * B;
+      // ---- D and E to shared memory
+      if (warp > 0) {
+#pragma unroll
+        for (int u = 0; u < PF; ++u) {
+          const int idx = tid - 32 + u * NL, i = idx & (B - 1), j = idx / B;
+          if (idx < B * B) {
+            if (i >= j) {
+              const T val = i == j ? from_re<T>(re_(dreg[u])) : dreg[u];
+              Ds[i + j * LD] = val;
+              Ds[j + i * LD] = conj_(val);
+            }
+            Es[i + j * LD] = ereg[u];
           }
         }
-      }
-      __syncthreads();
-      const T tau = sh_tau, beta = sh_beta, scale = sh_scale;
-      for (int i = tid; i < len; i += NT) v[i] = (i == 0) ? from_re<T>(1.0) : scale * v[i];
-      __syncthreads();
-      // ---- (i) the annihilated column, (ii) left update of the rest of L, store L
-      if (t == 0) {
-        for (int i = tid; i < len; i += NT)
-          stcg_(&band[(1 + i) + (long long)s * ldb], i == 0 ? beta : zero_<T>());
       } else {
-        if (qi >= 1 && qi < b) {  // w_q = conj(tau) v^H L(:, q): four partial sums per column
-          T acc = zero_<T>();
-          for (int i = qp; i < len; i += 4) acc += cmul(v[i], Ls[i + qi * LD]);
-          part4[qp * 64 + qi] = acc;
-        }
-        __syncthreads();
-        if (tid >= 1 && tid < b)
-          w[tid] = conj_(tau) * ((part4[tid] + part4[64 + tid]) + (part4[128 + tid] + part4[192 + tid]));
-        __syncthreads();
-        if (ci < len) {
-          for (int q = (cj == 0 ? cstep : cj); q < b; q += cstep) Ls[ci + q * LD] -= v[ci] * w[q];
-          if (cj == 0) Ls[ci] = (ci == 0) ? beta : zero_<T>();
-        }
-        __syncthreads();
-        if (ci < len)
-          for (int q = cj; q < b; q += cstep) stcg_(&band[(b + ci - q) + (long long)(pp + q) * ldb], Ls[ci + q * LD]);
+        __syncwarp();
+        for (int i = lane; i < B; i += 32) vc[i] = conj_(v[i]);
       }
-      // ---- (iii) two-sided update of the diagonal block
+      __syncthreads();
+      if (bad) return;  // (uniform: set before the barrier, never cleared)
+      const T tau = sh_tau[cur];
+      // ---- partial sums of w = v^H L, y = D v, z = E v: P threads per output
+      {
+        const int o = tid % O3, g = tid / O3, i = o & (B - 1), m = o / B;
+        const T* a = m == 0 ? Ls + i * LD : (m == 1 ? Ds + i : Es + i);
+        const T* x = m == 0 ? vc : v;
+        const int st = m == 0 ? 1 : LD, j0 = g * TERMS;
+        T acc = zero_<T>(), acc2 = zero_<T>();
+        if (m == 1 || (m == 0 ? t > 0 : len2 > 0)) {
+#pragma unroll 8
+          for (int j = 0; j < TERMS; j += 2) {
+            acc += a[(j0 + j) * st] * x[j0 + j];
+            acc2 += a[(j0 + j + 1) * st] * x[j0 + j + 1];
+          }
+        }
+        part[tid] = acc + acc2;
+      }
+      __syncthreads();
+      for (int o = tid; o < O3; o += NTH) {
+        T acc = part[o];
 #pragma unroll
-      for (int u = 0; u < PF; ++u) {
-        const int jj = cj + u * cstep;
-        if (jj < len && ci < len && ci >= jj) {
-          T val = dreg[u];
-          if (ci == jj) val = from_re<T>(re_(val));
-          Ds[ci + jj * LD] = val;
-          Ds[jj + ci * LD] = conj_(val);
+        for (int g = 1; g < P; ++g) acc += part[g * O3 + o];
+        const int i = o & (B - 1), m = o / B;
+        if (m == 0) w[i] = conj_(tau) * acc;
+        else if (m == 1) y[i] = acc;
+        else {
+          const T zz = tau * acc;
+          z[i] = zz;
+          xn_[i] = Es[i] - zz;
         }
-        if (jj < len && ci < len2) Es[ci + jj * LD] = ereg[u];
       }
-      __syncthreads();
-      if (qi < len) {  // y = D v: four partial sums per row
-        T acc = zero_<T>();
-        for (int j = qp; j < len; j += 4) acc += Ds[qi + j * LD] * v[j];
-        part4[qp * 64 + qi] = acc;
-      }
-      __syncthreads();
-      if (tid < len) y[tid] = (part4[tid] + part4[64 + tid]) + (part4[128 + tid] + part4[192 + tid]);
       __syncthreads();
       if (warp == 0) {
-        T acc = zero_<T>();
-        for (int i = lane; i < len; i += 32) acc += cmul(v[i], y[i]);
-        acc = warp_sum(acc);
-        if (lane == 0) sh_c = (R)0.5 * (R)abs2_(tau) * (R)re_(acc);
-      }
-      __syncthreads();
-      for (int i = tid; i < len; i += NT) y[i] = tau * y[i] - from_re<T>(sh_c) * v[i];
-      __syncthreads();
-      if (ci < len)
-        for (int jj = cj; jj <= ci; jj += cstep) {
-          T val = Ds[ci + jj * LD] - (mulc(y[ci], v[jj]) + mulc(v[ci], y[jj]));
-          if (ci == jj) val = from_re<T>(re_(val));
-          stcg_(&band[(ci - jj) + (long long)(p + jj) * ldb], val);
+        // ---- the next reflector, published once this task's stores are done
+        if (more) {
+          const T beta = reflect(xn_, vn, cur ^ 1);
+          if (lane == 0) stcg_(&band[B + (long long)p * ldb], beta);
         }
-      // ---- (iv) right update of the block below: creates the next bulge
-      if (len2 > 0) {
-        if (qi < len2) {  // w = tau E v: four partial sums per row
-          T acc = zero_<T>();
-          for (int q = qp; q < len; q += 4) acc += Es[qi + q * LD] * v[q];
-          part4[qp * 64 + qi] = acc;
-        }
-        __syncthreads();
-        if (tid < len2) w[tid] = tau * ((part4[tid] + part4[64 + tid]) + (part4[128 + tid] + part4[192 + tid]));
-        __syncthreads();
-        if (ci < len2)
-          for (int q = cj; q < len; q += cstep) Es[ci + q * LD] -= mulc(w[ci], v[q]);
-        pendingL = true;
+        bar_sync_n(1, NTH);
+        if (more && lane == 0) st_release(&progress[s], t + 2);
       } else {
-        pendingL = false;
+        if (warp == 1) {
+          // y <- tau y - c v, c = |tau|^2 Re(v^H y) / 2
+          T yv[(B + 31) / 32], vv[(B + 31) / 32];
+          R acc = 0;
+#pragma unroll
+          for (int u = 0; u < (B + 31) / 32; ++u) {
+            const int i = lane + 32 * u;
+            yv[u] = i < B ? y[i] : zero_<T>();
+            vv[u] = i < B ? v[i] : zero_<T>();
+            acc += (R)re_(cmul(vv[u], yv[u]));
+          }
+          acc = warp_sum(acc);
+          const T c = from_re<T>((R)0.5 * (R)abs2_(tau) * acc);
+#pragma unroll
+          for (int u = 0; u < (B + 31) / 32; ++u) {
+            const int i = lane + 32 * u;
+            if (i < B) y[i] = tau * yv[u] - c * vv[u];
+          }
+        } else {
+          // L <- H L, stored (its column 0 is beta, 0 ..; beta was stored with the reflector); E <- E H^H
+          // (column 0 is xn_, consumed by the next reflector); the reflector for the back-transform
+          constexpr int NW = NTH - 64;
+          for (int idx = tid - 64; idx < B * B; idx += NW) {
+            const int i = idx & (B - 1), q = idx / B;
+            if (t > 0 && i < len && (q > 0 || i > 0))
+              stcg_(&band[(B + i - q) + (long long)(p - B + q) * ldb],
+                    q == 0 ? zero_<T>() : Ls[i + q * LD] - v[i] * w[q]);
+            if (q > 0 && len2 > 0) Es[i + q * LD] -= mulc(z[i], v[q]);
+          }
+          const long long rid = (long long)s * ntask + t;
+          for (int i = tid - 64; i < B; i += NW) V2[rid * B + i] = v[i];
+          if (tid == 64) tau2[rid] = tau;
+        }
+        bar_sync_n(2, NL);
+        // D <- H D H^H, lower triangle: columns c and B - 1 - c together have B - 1 entries below the
+        // diagonal, so a pair fills whole warps; then the diagonal
+        for (int idx = tid - 32; idx < (B / 2) * B; idx += NL) {
+          const int c = idx / B, e = idx & (B - 1);
+          const bool first = e < B - 1 - c;
+          const int i = first ? c + 1 + e : e + 1, j = first ? c : B - 1 - c;
+          if (e < B - 1 && i < len && j < len)
+            stcg_(&band[(i - j) + (long long)(p + j) * ldb],
+                  Ds[i + j * LD] - (mulc(y[i], v[j]) + mulc(v[i], y[j])));
+        }
+        for (int i = tid - 32; i < len; i += NL)
+          stcg_(&band[(long long)(p + i) * ldb],
+                from_re<T>(re_(Ds[i + i * LD]) - (R)2 * (R)re_(mulc(y[i], v[i]))));
+        __syncwarp();
+        bar_arrive_n(1, NTH);
+        if (more) {
+          fetch(t + 1);
+          bar_sync_n(2, NL);  // every warp has left D, E and L: the next task may overwrite them
+        }
       }
-      // ---- keep the reflector for the back-transform
-      const long long rid = (long long)s * ntask + t;
-      for (int i = tid; i < b; i += NT) V2[rid * b + i] = (i < len) ? v[i] : zero_<T>();
-      if (tid == 0) tau2[rid] = tau;
-      __syncthreads();
-      if (tid == 0) {
-        __threadfence();
-        atomicExch(&progress[s], t + 1);
+      if (!more) {
+        // a last single row below: store its part of the bulge
+        if (lenn == 1) {
+          if (warp > 0) {
+            bool ok = true;
+            if (s > 0)
+              ok = stall ? warp_wait_ge(&status[ST_STALL], 1, status, abort_flag, 202)
+                         : warp_wait_ge(&progress[s - 1], t + 4, status, abort_flag, 201);
+            if (!ok && lane == 0) bad = 1;
+            if (ok)
+              for (int q = tid - 32; q < B; q += NL)
+                stcg_(&band[(B - q) + (long long)(p + q) * ldb], q == 0 ? xn_[0] : Es[q * LD]);
+          }
+        }
+        break;
       }
       T* tmp = Ls;
       Ls = Es;
       Es = tmp;
+      cur ^= 1;
     }
     __syncthreads();
-    if (tid == 0) {
-      __threadfence();
-      atomicExch(&progress[s], INT_MAX);
-    }
+    if (bad) return;
+    if (tid == 0) st_release(&progress[s], INT_MAX);
   }
 }
 
 // d = Re diag, e = |subdiag| with the phase recursion phi_0 = 1, phi_{i+1} = phi_i eps_i/|eps_i|
-// (complex), or e = subdiag (real).  One block: the phase recursion is sequential.
+// (complex), or e = subdiag (real).  One block of 1024 threads.  The phases are a running product:
+// every thread forms the product of its own n / 1024 factors, the block scans the 1024 products in
+// shared memory (10 steps), and the threads write their phases.  (As one thread's recursion the chain of
+// n hypot's and divisions took about 2 us per row.)  The phases are formed in FP64 also from an FP32
+// band, so that their product over n steps stays accurate.
 template <class T>
-// (the phases are formed in FP64 also from an FP32 band, so that their product over n steps stays
-// accurate)
-__global__ void k_tridiag_out(int n, const T* band, int ldb, double* d, double* e, zd* phase) {
+__global__ void __launch_bounds__(1024) k_tridiag_out(int n, const T* band, int ldb, double* d, double* e, zd* phase) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) d[i] = re_(band[(long long)i * ldb]);
   if constexpr (is_cx<T>::value) {
-    if (threadIdx.x == 0) {
-      zd ph = make_zd(1.0, 0.0);
-      phase[0] = ph;
-      for (int i = 0; i + 1 < n; ++i) {
-        const T eps = band[1 + (long long)i * ldb];
-        const double ex = re_(eps), ey = im_(eps);
-        const double a = hypot(ex, ey);
-        e[i] = a;
-        if (a > 0.0) ph = ph * make_zd(ex / a, ey / a);
-        phase[i + 1] = ph;
-      }
+    __shared__ zd sc[2][1024];
+    const int tid = threadIdx.x, per = (n + 1023) / 1024, i0 = tid * per, i1 = min(n - 1, i0 + per);
+    zd ph = make_zd(1.0, 0.0);
+    for (int i = i0; i < i1; ++i) {  // the product of this thread's factors; phase[i + 1] = it, so far
+      const T eps = band[1 + (long long)i * ldb];
+      const double ex = re_(eps), ey = im_(eps);
+      const double a = hypot(ex, ey);
+      e[i] = a;
+      if (a > 0.0) ph = ph * make_zd(ex / a, ey / a);
+      phase[i + 1] = ph;
+    }
+    int cur = 0;
+    sc[0][tid] = ph;
+    __syncthreads();
+    for (int off = 1; off < 1024; off <<= 1) {
+      const zd v = sc[cur][tid];
+      sc[cur ^ 1][tid] = tid >= off ? sc[cur][tid - off] * v : v;
+      cur ^= 1;
+      __syncthreads();
+    }
+    if (tid == 0) phase[0] = make_zd(1.0, 0.0);
+    if (tid > 0) {
+      const zd before = sc[cur][tid - 1];
+      for (int i = i0; i < i1; ++i) phase[i + 1] = before * phase[i + 1];
     }
   } else {
     for (int i = threadIdx.x; i + 1 < n; i += blockDim.x) e[i] = band[1 + (long long)i * ldb];
@@ -544,7 +671,39 @@ __global__ void __launch_bounds__(256) k_wy_level(int n, int b, int L0, int nL, 
   }
 }
 
-template <class T> size_t bulge_smem(int b) { return sizeof(T) * ((size_t)3 * b * (b + 1) + 3 * b + 4 * 64) + 64; }
+// threads of a bulge-chasing block: four per output of the three products (two at b = 64)
+constexpr int bulge_threads(int b) { return b == 16 ? 192 : 384; }
+template <class T> size_t bulge_smem(int b) {
+  return sizeof(T) * ((size_t)3 * b * (b + 1) + 7 * b + bulge_threads(b)) + 64;
+}
+
+// One cooperative launch of the chase at band width B.
+template <class T, int B> int launch_bulge(Sys& s, int n, T* band, int ldb) {
+  constexpr int NTH = bulge_threads(B);
+  const size_t smem = bulge_smem<T>(B);
+  GEV_TRY(allow_max_dyn_smem(k_bulge<T, B, NTH>));
+  int per_sm = 0;
+  GEV_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bulge<T, B, NTH>, NTH, smem));
+  if (per_sm < 1) return GEV_ERR_UNSUPPORTED;
+  // Sweep s+1 trails sweep s by a little over two tasks and a sweep runs (n - s) / b tasks, so at most
+  // about n / (2b) sweeps are in flight: more blocks would only hold SMs (in a spin wait) that other
+  // streams' work - concurrent solves of the serving form - could use.  Blocks that share an SM share its
+  // FP64 pipe, and the pipeline runs at its slowest block's pace: a second block per SM only pays when
+  // the sweeps in flight well exceed the SMs.
+  int G = n / (2 * B) + 8;
+  if (G > s.sms) G = 2 * G < 3 * s.sms ? s.sms : std::min(G, std::min(per_sm, 2) * s.sms);
+  if (G > n - 2) G = n - 2;
+  int nn = n, lb = ldb, nt = s.ntask, stall = s.opts.debug_stall ? 1 : 0;
+  T* V2 = (T*)s.V2;
+  T* tau2 = (T*)s.tau2;
+  int* prog = s.prog;
+  int* st = s.status;
+  int* ab = &s.status[ST_ABORT];
+  void* args[] = {&nn, &band, &lb, &V2, &tau2, &nt, &prog, &st, &ab, &stall};
+  GEV_COUNT(s);
+  GEV_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_bulge<T, B, NTH>, dim3(G), dim3(NTH), args, smem, s.stream));
+  return 0;
+}
 
 }  // namespace
 
@@ -555,19 +714,6 @@ template <class T> int hb2st(Sys& s, double* d, double* e) {
   if (n <= 2) {
     // already tridiagonal
   } else {
-    if (b > 64) return GEV_ERR_UNSUPPORTED;
-    const size_t smem = bulge_smem<T>(b);
-    GEV_TRY(allow_max_dyn_smem(k_bulge<T>));
-    int per_sm = 0;
-    GEV_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bulge<T>, NT, smem));
-    if (per_sm < 1) return GEV_ERR_UNSUPPORTED;
-    // Sweep s+1 trails sweep s by three tasks and a sweep runs (n - s) / b tasks, so at most about
-    // n / (3b) sweeps are in flight: more blocks would only hold SMs (in a spin wait) that other
-    // streams' work - concurrent solves of the serving form - could use.
-    int G = per_sm * s.sms;
-    const int inflight = n / (3 * b) + 8;
-    if (G > inflight) G = inflight;
-    if (G > n - 2) G = n - 2;
     GEV_CUDA_TRY(cudaMemsetAsync(s.prog, 0, sizeof(int) * (size_t)n, s.stream));
     GEV_CUDA_TRY(cudaMemsetAsync(s.tau2, 0, s.es() * (size_t)n * s.ntask, s.stream));
     // The FP32 back-transform applies every stored slot with its tau (no branch), so the slots of
@@ -576,19 +722,13 @@ template <class T> int hb2st(Sys& s, double* d, double* e) {
     if constexpr (std::is_same<T, float>::value)
       GEV_CUDA_TRY(cudaMemsetAsync(s.V2, 0, sizeof(T) * (size_t)b * n * s.ntask, s.stream));
     GEV_CUDA_TRY(cudaMemsetAsync(&s.status[ST_ABORT], 0, sizeof(int), s.stream));
-    int nn = n, bb = b, lb = ldb, nt = s.ntask;
-    T* V2 = (T*)s.V2;
-    T* tau2 = (T*)s.tau2;
-    int* prog = s.prog;
-    int* st = s.status;
-    int* ab = &s.status[ST_ABORT];
-    int stall = s.opts.debug_stall ? 1 : 0;
-    void* args[] = {&nn, &bb, &band, &lb, &V2, &tau2, &nt, &prog, &st, &ab, &stall};
-    GEV_COUNT(s);
-    GEV_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_bulge<T>, dim3(G), dim3(NT), args, smem, s.stream));
+    if (b == 16) GEV_TRY((launch_bulge<T, 16>(s, n, band, ldb)));
+    else if (b == 32) GEV_TRY((launch_bulge<T, 32>(s, n, band, ldb)));
+    else if (b == 64) GEV_TRY((launch_bulge<T, 64>(s, n, band, ldb)));
+    else return GEV_ERR_UNSUPPORTED;
   }
   GEV_COUNT(s);
-  k_tridiag_out<T><<<1, 256, 0, s.stream>>>(n, band, ldb, d, e, (zd*)s.phase);
+  k_tridiag_out<T><<<1, 1024, 0, s.stream>>>(n, band, ldb, d, e, (zd*)s.phase);
   GEV_TRY(last_error());
   s.have_tridiag_refl = true;
   return 0;
