@@ -21,11 +21,14 @@
 // Data flow: a split pass writes the 8 digit planes of op(A) and op(B) to global memory in the
 // order the MMAs consume them (one 16-deep k-slice of a 128-row A tile = 8 planes x 4 KB,
 // contiguous; of a 64-column B tile = 8 x 2 KB), so the GEMM kernel moves them with plain bulk
-// asynchronous copies into a 4-stage shared-memory ring.  Warp roles: warp 8 issues the copies,
-// warp 9 issues the 36 MMAs per slice (tcgen05, accumulators in TMEM: 6 exact diagonals + 1
-// shared, 64 columns each), warps 0-7 (one TMEM lane per output row, half of its 64 columns
-// each) drain the exact accumulators at every chunk end and write C.  Every mbarrier wait is bounded; on expiry the kernel records
-// ST_TIMEOUT, waits (bounded) for its copies and MMAs in flight, frees TMEM and returns.
+// asynchronous copies into a 4-stage shared-memory ring.  Warp roles: warp 16 issues the copies,
+// warp 17 issues the 36 MMAs per slice (tcgen05, accumulators in TMEM: 6 exact diagonals + 1
+// shared, 64 columns each), warps 0-15 (one TMEM lane per output row, a quarter of its 64 columns
+// each) drain the exact accumulators at every chunk end and write C.  The kernel is persistent for
+// short K, and its epilogue uses integer arithmetic only (see to_fp64): together they took the
+// 8192 x 8192 x 128 update from 1.97 to 0.90 ms, back-transform 2 at n = 10240, k = 2560 from 365 to
+// 167 ms.  Every mbarrier wait is bounded; on expiry the kernel records ST_TIMEOUT, waits (bounded) for
+// its copies and MMAs in flight, frees TMEM and returns.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -49,9 +52,9 @@ constexpr int A_STAGE = NSLICE * A_TILE;   // 32 KB
 constexpr int B_STAGE = NSLICE * B_TILE;   // 16 KB
 constexpr int STAGE = A_STAGE + B_STAGE;   // 48 KB
 constexpr int SMEM_OZ = NSTAGE * STAGE + 1024;
-constexpr int NEPI_W = 8;                  // epilogue warps: TMEM lanes 32 (w % 4), columns 32 (w / 4)
-constexpr int HC = ON / 2;                  // output columns per epilogue thread
-constexpr int NTH = 32 * (NEPI_W + 2);      // + copy warp 8 + MMA warp 9
+constexpr int NEPI_W = 16;                 // epilogue warps: TMEM lanes 32 (w % 4), columns 16 (w / 4)
+constexpr int HC = ON / 4;                  // output columns per epilogue thread
+constexpr int NTH = 32 * (NEPI_W + 2);      // + copy warp 16 + MMA warp 17
 constexpr int TMEM_COLS_OZ = 512;
 constexpr int SHARED_SLOT = DEXACT - 1;    // TMEM slot of d = 8, 9; exact d at slot d - 2
 constexpr int GROUP_M = 16;                // raster: 16 row tiles share their B slices in L2
@@ -97,32 +100,66 @@ __device__ __forceinline__ double opnd_at(const Opnd& o, long long r, long long 
   return (a == b) ? z.x : (a == 0 ? -y : y);
 }
 
-// E[r] = max exponent over the kept entries of vector r (R vectors of K elements).  E holds a very
-// negative value on entry (atomicMax).  Block 32 x 8; grid.y covers K in slices of 1024.
-// fast_r: consecutive vectors are adjacent in memory (threads run across vectors); otherwise a
-// warp reads along one vector.
-__global__ void k_vec_exp(int R, int K, Opnd o, int fast_r, int* E) {
-  const int k_lo = blockIdx.y * 1024, k_hi = min(K, k_lo + 1024);
-  if (fast_r) {
-    const int r = blockIdx.x * 32 + threadIdx.x;
-    if (r >= R) return;
+// The two operands of one product, for the passes that handle both in one launch.
+struct Opnd2 {
+  Opnd o[2];
+  int R[2];     // vectors: rows of op(A), columns of op(B)
+  int fast[2];  // 1: consecutive vectors are adjacent in memory
+  int* E[2];    // their exponents
+  int TR[2];    // rows of a plane tile (OM, ON)
+  int RT[2];    // row tiles
+  unsigned char* out[2];
+  int nblk0;    // grid blocks of operand 0 (the rest: operand 1)
+};
+
+// E[r] = max exponent over the kept entries of vector r, both operands in one launch; grid.y covers K
+// in slabs.  Blocks of 256 threads take 32 vectors: a warp reads across 32 vectors (fast) or along one.
+// One slab: E is written; several: atomicMax into a very negative initial value.
+__global__ void __launch_bounds__(256) k_vec_exp(Opnd2 q, int K, int slab, int slabs) {
+  const int w = blockIdx.x < q.nblk0 ? 0 : 1, blk = blockIdx.x - (w ? q.nblk0 : 0);
+  const Opnd o = q.o[w];
+  const int R = q.R[w], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int k_lo = blockIdx.y * slab, k_hi = min(K, k_lo + slab);
+  int* E = q.E[w];
+  if (q.fast[w]) {
+    __shared__ int red[8][32];
+    const int r = blk * 32 + lane;
     int e = EXP_ZERO;
-    for (int k = k_lo + threadIdx.y; k < k_hi; k += 8) e = max(e, exp_above(opnd_at(o, r, k)));
-    if (e != EXP_ZERO) atomicMax(&E[r], e);
+    if (r < R) {
+#pragma unroll 8
+      for (int k = k_lo + warp; k < k_hi; k += 8) e = max(e, exp_above(opnd_at(o, r, k)));
+    }
+    red[warp][lane] = e;
+    __syncthreads();
+    if (warp == 0 && r < R) {
+#pragma unroll
+      for (int u = 1; u < 8; ++u) e = max(e, red[u][lane]);
+      if (slabs == 1) E[r] = e;
+      else if (e != EXP_ZERO) atomicMax(&E[r], e);
+    }
   } else {
-    const int r = blockIdx.x * 8 + threadIdx.y;
-    if (r >= R) return;  // uniform across the warp
-    int e = EXP_ZERO;
-    for (int k = k_lo + threadIdx.x; k < k_hi; k += 32) e = max(e, exp_above(opnd_at(o, r, k)));
-    e = __reduce_max_sync(0xffffffffu, e);
-    if (threadIdx.x == 0 && e != EXP_ZERO) atomicMax(&E[r], e);
+#pragma unroll 1
+    for (int u = 0; u < 4; ++u) {
+      const int r = blk * 32 + warp * 4 + u;
+      if (r >= R) return;  // uniform across the warp
+      int e = EXP_ZERO;
+#pragma unroll 8
+      for (int k = k_lo + lane; k < k_hi; k += 32) e = max(e, exp_above(opnd_at(o, r, k)));
+      e = __reduce_max_sync(0xffffffffu, e);
+      if (lane == 0) {
+        if (slabs == 1) E[r] = e;
+        else if (e != EXP_ZERO) atomicMax(&E[r], e);
+      }
+    }
   }
 }
 
 __device__ __forceinline__ int clamp_exp(int e) { return e < -1100 ? EXP_ZERO : e; }
 
-// the balanced radix-2^7 digits of x 2^(55-E) (|x| < 2^E), as BF16 bit patterns of a_p 2^-7p
-__device__ __forceinline__ void digits(double x, int E, uint16_t out[NSLICE]) {
+// the balanced radix-2^7 digits of x 2^(55-E) (|x| < 2^E), as floats a_p 2^-7p.  X + sum_p 2^6 2^(56-7p)
+// has the digits a_p + 64 in its plain 7-bit fields (the top one may reach 128), so a digit is a shift, a
+// mask that also sets the exponent of 1.5 2^23, and one exact FMA: no carries and no integer conversion.
+__device__ __forceinline__ void digits(double x, int E, float out[NSLICE]) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const int be = (int)((bits >> 52) & 0x7FF);
   long long X = 0;
@@ -136,48 +173,89 @@ __device__ __forceinline__ void digits(double x, int E, uint16_t out[NSLICE]) {
     else if (s > -64) u = m >> (-s);  // bits below 2^-55 of the scale are dropped
     X = (bits >> 63) ? -(long long)u : (long long)u;
   }
+  constexpr unsigned long long BIAS = (64ull << 49) | (64ull << 42) | (64ull << 35) | (64ull << 28) | (64ull << 21) |
+                                      (64ull << 14) | (64ull << 7) | 64ull;
+  const unsigned long long Y = (unsigned long long)(X + (long long)BIAS);  // >= 0
 #pragma unroll
   for (int p = 1; p <= NSLICE; ++p) {
-    const int sh = 56 - 7 * p;
-    long long a;
-    if (sh > 0) a = (X + (1ll << (sh - 1))) >> sh;  // nearest integer to X 2^-sh: |a| <= 64
-    else a = X;
-    X -= a * (1ll << sh);
-    const float v = (float)a * __int_as_float((127 - 7 * p) << 23);  // a 2^-7p, exact
-    out[p - 1] = __bfloat16_as_ushort(__float2bfloat16_rn(v));         // exact: |a| <= 64
+    const uint32_t f = (uint32_t)(Y >> (56 - 7 * p)) & (p == 1 ? 0xFFu : 0x7Fu);
+    const float sc = __int_as_float((127 - 7 * p) << 23);  // 2^-7p
+    out[p - 1] = fmaf(__int_as_float(0x4B400000 | f), sc, -(12582912.0f + 64.0f) * sc);  // exact
   }
 }
 
-// Digit planes of one operand: vector r (a row of op(A) or a column of op(B)), element k, rows
-// padded to RT tiles of TR, k to KT slices of 16.  One thread per (r, 8 consecutive k): it writes
-// 16 bytes to each of the 8 planes of tile (r / TR, k / 16).
-__global__ void k_split(int R, int K, Opnd o, int fast_r, const int* E, int TR, int RT, int KT, unsigned char* out) {
-  const long long Rp = (long long)RT * TR, G = 2LL * KT;
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= Rp * G) return;
-  long long r, g;
-  if (fast_r) { r = t % Rp; g = t / Rp; } else { g = t % G; r = t / G; }
-  const int Er = (r < R) ? clamp_exp(E[r]) : EXP_ZERO;
-  uint16_t dg[8][NSLICE];
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);  // exact: |a_p| <= 64
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// the digits of two neighbouring elements into the 8 planes (4 bytes each)
+__device__ __forceinline__ void store_pair(double x0, double x1, int E, unsigned char* dst, int tile_bytes) {
+  float a[NSLICE], b[NSLICE];
+  digits(x0, E, a);
+  digits(x1, E, b);
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const long long k = g * 8 + q;
-    const double v = (r < R && k < K) ? opnd_at(o, r, k) : 0.0;
-    digits(v, Er, dg[q]);
+  for (int p = 0; p < NSLICE; ++p)
+    *reinterpret_cast<uint32_t*>(dst + (long long)p * tile_bytes) = pack_bf16(a[p], b[p]);
+}
+
+// Digit planes of both operands in one launch.  A warp takes 8 vectors x 16 elements (one slice of one
+// 8-row group): lane = 4 (row) + pair, so that every plane receives two contiguous 128-byte rows of core
+// matrices and global memory is read in 64-byte runs whichever index is contiguous.
+__global__ void __launch_bounds__(256) k_split(Opnd2 q, int K, int KT) {
+  const int w = blockIdx.x < q.nblk0 ? 0 : 1;
+  const long long blk = blockIdx.x - (w ? q.nblk0 : 0);
+  const Opnd o = q.o[w];
+  const int R = q.R[w], TR = q.TR[w], lane = threadIdx.x & 31;
+  const long long RG = (long long)q.RT[w] * (TR / 8), u = blk * 8 + (threadIdx.x >> 5);
+  if (u >= RG * KT) return;
+  long long rg, kt;
+  if (q.fast[w]) { rg = u % RG; kt = u / RG; } else { kt = u % KT; rg = u / KT; }
+  const long long r = rg * 8 + (lane >> 2);
+  const int Er = (r < R) ? clamp_exp(q.E[w][r]) : EXP_ZERO;
+  double x[4];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const long long k = kt * 16 + (h >> 1) * 8 + (lane & 3) * 2 + (h & 1);
+    x[h] = (r < R && k < K) ? opnd_at(o, r, k) : 0.0;
   }
-  const long long rt = r / TR, kt = g >> 1;
   const int tile_bytes = TR * KS * 2;
-  unsigned char* base =
-      out + ((rt * KT + kt) * NSLICE) * (long long)tile_bytes + toff16((int)(r % TR), (int)(g & 1) * 8);
+  unsigned char* base = q.out[w] + (((r / TR) * KT + kt) * NSLICE) * (long long)tile_bytes;
 #pragma unroll
-  for (int p = 0; p < NSLICE; ++p) {
-    uint4 v;
-    v.x = (uint32_t)dg[0][p] | ((uint32_t)dg[1][p] << 16);
-    v.y = (uint32_t)dg[2][p] | ((uint32_t)dg[3][p] << 16);
-    v.z = (uint32_t)dg[4][p] | ((uint32_t)dg[5][p] << 16);
-    v.w = (uint32_t)dg[6][p] | ((uint32_t)dg[7][p] << 16);
-    *reinterpret_cast<uint4*>(base + (long long)p * tile_bytes) = v;
+  for (int h = 0; h < 2; ++h)
+    store_pair(x[2 * h], x[2 * h + 1], Er, base + toff16((int)(r % TR), h * 8 + (lane & 3) * 2), tile_bytes);
+}
+
+// The same for K <= 16 NS in one pass: the warp holds its 8 vectors entirely, so the exponents come out
+// of the registers and no separate exponent pass (nor an initialised E) is needed.
+template <int NS>
+__global__ void __launch_bounds__(128) k_split_short(Opnd2 q, int K, int KT) {
+  const int w = blockIdx.x < q.nblk0 ? 0 : 1;
+  const long long blk = blockIdx.x - (w ? q.nblk0 : 0);
+  const Opnd o = q.o[w];
+  const int R = q.R[w], TR = q.TR[w], lane = threadIdx.x & 31;
+  const long long rg = blk * 4 + (threadIdx.x >> 5);
+  if (rg >= (long long)q.RT[w] * (TR / 8)) return;
+  const long long r = rg * 8 + (lane >> 2);
+  double x[NS * 4];
+  int e = EXP_ZERO;
+#pragma unroll
+  for (int h = 0; h < NS * 4; ++h) {
+    const long long k = (h >> 1) * 8 + (lane & 3) * 2 + (h & 1);
+    x[h] = (r < R && k < K) ? opnd_at(o, r, k) : 0.0;
   }
+#pragma unroll
+  for (int h = 0; h < NS * 4; ++h) e = max(e, exp_above(x[h]));
+  e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+  e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+  if ((lane & 3) == 0 && r < R) q.E[w][r] = e;
+  const int Er = clamp_exp(e);
+  const int tile_bytes = TR * KS * 2;
+  unsigned char* base = q.out[w] + ((r / TR) * KT * NSLICE) * (long long)tile_bytes + toff16((int)(r % TR), (lane & 3) * 2);
+#pragma unroll
+  for (int h = 0; h < 2 * NS; ++h)
+    if ((h >> 1) < KT)
+      store_pair(x[2 * h], x[2 * h + 1], Er, base + (long long)(h >> 1) * NSLICE * tile_bytes + (h & 1) * 128, tile_bytes);
 }
 
 // K slices of a row tile of a block-diagonal op(A): the first slice of the tile's K range and the
@@ -253,19 +331,16 @@ __global__ void k_split_bd(int M, BdOp o, int bm, int bk, int MT, int* E, unsign
   if (lane == 0) E[i] = e;
   if (!act) return;
   const int Er = clamp_exp(e);
-  uint16_t dg[8][NSLICE];
+  float dg[8][NSLICE];
 #pragma unroll
   for (int q = 0; q < 8; ++q) digits(v[q], Er, dg[q]);
   const int tile_bytes = OM * KS * 2;
   unsigned char* base = out + (((long long)mt * c + (lane >> 1)) * NSLICE) * tile_bytes + toff16((int)(i % OM), (lane & 1) * 8);
 #pragma unroll
   for (int p = 0; p < NSLICE; ++p) {
-    uint4 w;
-    w.x = (uint32_t)dg[0][p] | ((uint32_t)dg[1][p] << 16);
-    w.y = (uint32_t)dg[2][p] | ((uint32_t)dg[3][p] << 16);
-    w.z = (uint32_t)dg[4][p] | ((uint32_t)dg[5][p] << 16);
-    w.w = (uint32_t)dg[6][p] | ((uint32_t)dg[7][p] << 16);
-    *reinterpret_cast<uint4*>(base + (long long)p * tile_bytes) = w;
+    *reinterpret_cast<uint4*>(base + (long long)p * tile_bytes) =
+        make_uint4(pack_bf16(dg[0][p], dg[1][p]), pack_bf16(dg[2][p], dg[3][p]), pack_bf16(dg[4][p], dg[5][p]),
+                   pack_bf16(dg[6][p], dg[7][p]));
   }
 }
 
@@ -284,71 +359,118 @@ struct OzP {
   // block-diagonal op(A) (0: off): block j has rows [j bd_bm, (j+1) bd_bm) and its non-zero columns
   // [j bd_bk, (j+1) bd_bk); the A planes then hold, per row tile, only that tile's K range (compact)
   int bd_bm, bd_bk;
+  // alpha: 0 general, 1, -1; beta: 0, 1, 2 general (a comparison of doubles is an FP64 instruction)
+  int amode, bmode;
 };
 
+int alpha_mode(double a) { return a == 1.0 ? 1 : (a == -1.0 ? -1 : 0); }
+int beta_mode(double b) { return b == 0.0 ? 0 : (b == 1.0 ? 1 : 2); }
 
-// an exact FP32 chunk sum (a multiple of 2^-49 below 2^8 in magnitude) in units of 2^-49
-__device__ __forceinline__ long long units49(uint32_t b) {
-  const uint32_t e = (b >> 23) & 0xFF;
-  const unsigned long long m = (unsigned long long)((b & 0x7FFFFFu) | 0x800000u) << 40;
-  unsigned long long t;
-  asm("shr.b64 %0, %1, %2;" : "=l"(t) : "l"(m), "r"(141u - e));  // m 2^(e - 101); 0 for e = 0
-  return (b >> 31) ? -(long long)t : (long long)t;
-}
-
-// x 2^e without a library call (two exact power-of-two factors cover |e| <= 2046)
-__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
-__device__ __forceinline__ double scale2(double x, int e) {
-  if (e >= -1022 && e <= 1023) return x * pow2(e);
-  e = max(-2044, min(2046, e));
-  const int h = e / 2;
-  return (x * pow2(h)) * pow2(e - h);
-}
-
-
-// (a 10-warp CTA puts 3 warps on one SM sub-partition of 16K registers: at most 168 registers per thread)
-__global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
-  extern __shared__ __align__(1024) unsigned char smem[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+// One work item of the product kernel: an output tile (a share of its k-slices when K is split).
+struct OzItem {
+  int m0, n0, z, s_lo, nst, nt;
+  long long a_tile;  // A-plane slice kt of the tile is slice a_tile + kt
+  bool skip;         // nothing of the tile is wanted (c_lower)
+};
+__device__ __forceinline__ OzItem oz_item(const OzP& p, int it) {
+  OzItem w;
+  const int tiles = p.MT * p.NT;
+  w.z = it / tiles;
+  const int t = it % tiles;
   // grouped raster: GROUP_M row tiles sweep the column tiles together
   const int per_group = GROUP_M * p.NT;
-  const int first = (blockIdx.x / per_group) * GROUP_M;
+  const int first = (t / per_group) * GROUP_M;
   const int gm = min(p.MT - first, GROUP_M);
-  const int within = blockIdx.x % per_group;
-  const int mt = first + within % gm, nt = within / gm;
-  const int m0 = mt * OM, n0 = nt * ON;
+  const int within = t % per_group;
+  const int mt = first + within % gm;
+  w.nt = within / gm;
+  w.m0 = mt * OM;
+  w.n0 = w.nt * ON;
   // complex products: rows 2i, 2i + 1 and elements 2l, 2l + 1 belong to complex row i / element l
   const int rs = p.cx ? 1 : 0;
-  const long long mr0 = m0 >> rs, mrn = OM >> rs;
-  if (p.c_lower && n0 > mr0 + mrn - 1) return;
+  const long long mr0 = w.m0 >> rs, mrn = OM >> rs;
+  w.skip = p.c_lower && w.n0 > mr0 + mrn - 1;
   // k-slices holding non-zero products for this tile (absolute k = local k + koff)
   long long kb = 0, ke = p.K >> rs;
   if (p.tri_a == 1) ke = std::min<long long>(ke, mr0 + mrn - p.koff);
   else if (p.tri_a == 2) kb = std::max<long long>(kb, mr0 - p.koff);
-  if (p.tri_b == 1) kb = std::max<long long>(kb, (long long)n0 - p.koff);
-  else if (p.tri_b == 2) ke = std::min<long long>(ke, (long long)n0 + ON - p.koff);
+  if (p.tri_b == 1) kb = std::max<long long>(kb, (long long)w.n0 - p.koff);
+  else if (p.tri_b == 2) ke = std::min<long long>(ke, (long long)w.n0 + ON - p.koff);
   kb <<= rs;
   ke <<= rs;
   int s_lo = (int)(kb / KS), s_hi = (int)(ke > 0 ? (ke + KS - 1) / KS : 0);
   if (s_hi < s_lo) s_hi = s_lo;
-  // A-plane slices: a_kt per row tile, slice kt read at kt - a_off
-  int a_kt = p.KT, a_off = 0;
+  w.a_tile = (long long)mt * p.KT;
   if (p.bd_bm) {
     int f = 0, c = 0;
     bd_range(p.bd_bm, p.bd_bk, mt, &f, &c);
     s_lo = min(f, p.KT);
     s_hi = min(f + c, p.KT);
-    a_kt = c;
-    a_off = f;
+    w.a_tile = (long long)mt * c - f;
   }
-  if (p.ksplit > 1) {  // this CTA's share of the slices
-    const int tot = s_hi - s_lo, z = blockIdx.y;
-    const int a = s_lo + (int)((long long)tot * z / p.ksplit);
-    const int b = s_lo + (int)((long long)tot * (z + 1) / p.ksplit);
+  if (p.ksplit > 1) {  // this item's share of the slices
+    const int tot = s_hi - s_lo;
+    const int a = s_lo + (int)((long long)tot * w.z / p.ksplit);
+    const int b = s_lo + (int)((long long)tot * (w.z + 1) / p.ksplit);
     s_lo = a;
     s_hi = b;
   }
-  const int nst = s_hi - s_lo, nchunk = (nst + CHUNK - 1) / CHUNK;
+  w.s_lo = s_lo;
+  w.nst = s_hi - s_lo;
+  return w;
+}
+
+
+// (acc 2^-49 + sh) 2^e rounded once to FP64, in integer arithmetic: GB300 runs about 1.7 FP64 operations
+// (conversions included) per SM per cycle, and at eight of them per output the epilogue of a 128 x 64
+// tile took about 19 us.  sh (|sh| < 2^-18) joins acc in units of 2^-81 (acc:lo, 96 bits); the magnitude is
+// normalised with a count of leading zeros and rounded to nearest even.
+__device__ __forceinline__ double to_fp64(long long acc, float sh, int e) {
+  const uint32_t sb = __float_as_uint(sh);
+  const int se = (int)((sb >> 23) & 0xFF);
+  const unsigned long long sm = (sb & 0x7FFFFFu) | 0x800000u;
+  const int sft = se - 150 + 81;  // sh 2^81 = sm 2^sft (a zero or denormal sh has sft < -24)
+  long long si = sft >= 0 ? (long long)(sm << sft) : (sft > -25 ? (long long)(sm >> -sft) : 0);
+  if (sb >> 31) si = -si;
+  acc += si >> 32;
+  uint32_t lo = (uint32_t)si;
+  const bool neg = acc < 0;
+  unsigned long long m = (unsigned long long)acc;
+  if (neg) {  // two's complement of the 96 bits
+    lo = 0u - lo;
+    m = ~m + (lo == 0 ? 1ull : 0ull);
+  }
+  int ex = 63 - 49 + e;  // exponent of bit 63 of m
+  if ((m >> 32) == 0) {
+    m = (m << 32) | lo;
+    lo = 0;
+    ex -= 32;
+  }
+  if (m == 0) return 0.0;
+  const int lz = __clzll((long long)m);
+  const unsigned long long low = ((unsigned long long)lo) << lz;  // lz < 32 whenever lo != 0
+  m = (m << lz) | (low >> 32);
+  ex -= lz;
+  const uint32_t rem = ((uint32_t)m & 0x7FFu) | ((uint32_t)low != 0u ? 1u : 0u);
+  unsigned long long mant = m >> 11;  // 2^52 <= mant < 2^53
+  mant += (rem > 0x400u || (rem == 0x400u && (mant & 1))) ? 1ull : 0ull;
+  // (a carry to 2^53 moves the exponent up by itself: the fields add, up to infinity)
+  unsigned long long b = mant + ((unsigned long long)(ex + 1022) << 52);
+  if (ex > 1023) b = 0x7FF0000000000000ull;
+  else if (ex < -1022) b = ex < -1076 ? 0ull : (mant + (1ull << (-1023 - ex))) >> (-1022 - ex);  // subnormal
+  return __longlong_as_double((long long)(b | (neg ? 1ull << 63 : 0ull)));
+}
+
+// Persistent: a CTA per SM walks over the work items.  The copy warp runs ahead into the next item's
+// slices while the epilogue works, and the epilogue first drains all sums of an item into registers and
+// releases the tensor memory, so the conversion to FP64, the loads of C and the stores overlap the next
+// item's MMAs: an item costs max(MMAs + drain, epilogue) instead of their sum plus a launch and the first
+// copies.  Sixteen epilogue warps of 16 columns: the conversion is a chain of integer instructions and
+// needs warps in flight more than it needs registers (18 warps: at most 112 registers per thread).
+__global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int items = p.MT * p.NT * p.ksplit, rs = p.cx ? 1 : 0;
 
   unsigned char* ctrl = smem + NSTAGE * STAGE;
   uint64_t* full = reinterpret_cast<uint64_t*>(ctrl);  // [NSTAGE]: slice landed
@@ -362,174 +484,180 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
   int* consumed = reinterpret_cast<int*>(ctrl + 448);
   if (tid == 0) {
     for (int s = 0; s < NSTAGE; ++s) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(&full[s])));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(&empty[s])));
+      mbar_init(su32(&full[s]), 1);
+      mbar_init(su32(&empty[s]), 1);
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(cfull)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(su32(cempty)), "r"(NEPI_W));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(su32(done)));
+    mbar_init(su32(cfull), 1);
+    mbar_init(su32(cempty), NEPI_W);
+    mbar_init(su32(done), 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     *err = 0;
     *issued = 0;
     *consumed = 0;
   }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(su32(tslot)),
-                 "r"(TMEM_COLS_OZ));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  if (warp == 0) tmem_alloc(su32(tslot), TMEM_COLS_OZ);
+  fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  fence_after();
   const uint32_t tmem = *tslot;
 
   if (warp == NEPI_W) {
     // ---- copy warp: digit-plane slices into the stage ring
     if (lane == 0) {
-      const unsigned char* a_src = p.Ap + ((long long)mt * a_kt - a_off) * A_STAGE;
-      const unsigned char* b_src = p.Bp + (long long)nt * p.KT * B_STAGE;
-      for (int s = 0; s < nst; ++s) {
-        const int slot = s % NSTAGE;
-        if (s >= NSTAGE && !bar_wait(su32(&empty[slot]), ((s / NSTAGE) - 1) & 1, err)) {
-          if (!*err) *err = 411;
-          break;
+      int sg = 0;  // slices issued, over all items
+      for (int it = blockIdx.x; it < items && !*err; it += gridDim.x) {
+        const OzItem w = oz_item(p, it);
+        if (w.skip) continue;
+        const unsigned char* a_src = p.Ap + (w.a_tile + w.s_lo) * A_STAGE;
+        const unsigned char* b_src = p.Bp + ((long long)w.nt * p.KT + w.s_lo) * B_STAGE;
+        for (int s = 0; s < w.nst; ++s, ++sg) {
+          const int slot = sg % NSTAGE;
+          if (sg >= NSTAGE && !bar_wait(su32(&empty[slot]), ((sg / NSTAGE) - 1) & 1, err)) {
+            if (!*err) *err = 411;
+            break;
+          }
+          const uint32_t fb = su32(&full[slot]);
+          mbar_expect_tx(fb, STAGE);
+          const uint32_t dst = su32(smem + slot * STAGE);
+          bulk_g2s(dst, a_src + (long long)s * A_STAGE, A_STAGE, fb);
+          bulk_g2s(dst + A_STAGE, b_src + (long long)s * B_STAGE, B_STAGE, fb);
+          *issued = sg + 1;
         }
-        const uint32_t fb = su32(&full[slot]);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(STAGE) : "memory");
-        const uint32_t dst = su32(smem + slot * STAGE);
-        const long long kt = s_lo + s;
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
-            "l"(a_src + kt * A_STAGE), "r"(A_STAGE), "r"(fb)
-            : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                dst + A_STAGE),
-            "l"(b_src + kt * B_STAGE), "r"(B_STAGE), "r"(fb)
-            : "memory");
-        *issued = s + 1;
       }
     }
   } else if (warp == NEPI_W + 1) {
     // ---- MMA warp: 36 digit-pair products per 16-deep slice
     if (lane == 0) {
       const uint32_t id = idesc_bf16(OM, ON);
-      for (int s = 0; s < nst; ++s) {
-        const int slot = s % NSTAGE, c = s / CHUNK;
-        const bool chunk_start = (s % CHUNK) == 0;
-        if (chunk_start && c > 0 && !bar_wait(su32(cempty), (c - 1) & 1, err)) {
-          if (!*err) *err = 412;
-          break;
-        }
-        if (!bar_wait(su32(&full[slot]), (s / NSTAGE) & 1, err)) {
-          if (!*err) *err = 413;
-          break;
-        }
-        *consumed = s + 1;
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        const uint32_t a0 = su32(smem + slot * STAGE), b0 = a0 + A_STAGE;
+      int sg = 0, cg = 0;  // slices and chunks, over all items
+      for (int it = blockIdx.x; it < items && !*err; it += gridDim.x) {
+        const OzItem w = oz_item(p, it);
+        if (w.skip) continue;
+        for (int s = 0; s < w.nst; ++s, ++sg) {
+          const int slot = sg % NSTAGE;
+          const bool chunk_start = (s % CHUNK) == 0;
+          if (chunk_start && cg > 0 && !bar_wait(su32(cempty), (cg - 1) & 1, err)) {
+            if (!*err) *err = 412;
+            break;
+          }
+          if (!bar_wait(su32(&full[slot]), (sg / NSTAGE) & 1, err)) {
+            if (!*err) *err = 413;
+            break;
+          }
+          *consumed = sg + 1;
+          fence_after();
+          const uint32_t a0 = su32(smem + slot * STAGE), b0 = a0 + A_STAGE;
 #pragma unroll
-        for (int pa = 1; pa <= NSLICE; ++pa) {
+          for (int pa = 1; pa <= NSLICE; ++pa) {
 #pragma unroll
-          for (int qb = 1; qb + pa <= DMAX; ++qb) {
-            const int d = pa + qb;
-            int col, en;
-            if (d <= DEXACT) {  // the first pair of diagonal d (pa = 1) restarts it at a chunk start
-              col = (d - 2) * ON;
-              en = (chunk_start && pa == 1) ? 0 : 1;
-            } else {  // the shared slot starts with the first MMA of d = 8 (pa = 1, qb = 7)
-              col = SHARED_SLOT * ON;
-              en = (s == 0 && pa == 1 && qb == DEXACT) ? 0 : 1;
+            for (int qb = 1; qb + pa <= DMAX; ++qb) {
+              const int d = pa + qb;
+              int col, en;
+              if (d <= DEXACT) {  // the first pair of diagonal d (pa = 1) restarts it at a chunk start
+                col = (d - 2) * ON;
+                en = (chunk_start && pa == 1) ? 0 : 1;
+              } else {  // the shared slot starts with the item's first MMA of d = 8 (pa = 1, qb = 7)
+                col = SHARED_SLOT * ON;
+                en = (s == 0 && pa == 1 && qb == DEXACT) ? 0 : 1;
+              }
+              mma_bf16(tmem + col, sdesc16(a0 + (pa - 1) * A_TILE), sdesc16(b0 + (qb - 1) * B_TILE), id, en);
             }
-            mma_bf16(tmem + col, sdesc16(a0 + (pa - 1) * A_TILE), sdesc16(b0 + (qb - 1) * B_TILE), id, en);
+          }
+          commit(su32(&empty[slot]));
+          if ((s % CHUNK) == CHUNK - 1 || s == w.nst - 1) {
+            commit(su32(cfull));
+            ++cg;
           }
         }
-        commit(su32(&empty[slot]));
-        if ((s % CHUNK) == CHUNK - 1 || s == nst - 1) commit(su32(cfull));
       }
       commit(su32(done));
       if (!bar_wait_plain(su32(done), 0) && !*err) *err = 414;
     }
   } else {
-    // ---- epilogue warps: drain the exact diagonals per chunk, then write C
+    // ---- epilogue warps: drain the sums per chunk, then convert and write C
     const int quarter = warp & 3, col0 = (warp >> 2) * HC;
-    const int row = quarter * 32 + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
-    long long acc[HC];
+    const bool read_c = p.ksplit == 1 && p.bmode != 0;
+    int cg = 0;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+      const OzItem w = oz_item(p, it);
+      if (w.skip) continue;
+      long long acc[HC];
+      float sh[HC];
 #pragma unroll
-    for (int c = 0; c < HC; ++c) acc[c] = 0;
-    bool good = true;
-    for (int c = 0; c < nchunk; ++c) {
-      if (!bar_wait(su32(cfull), c & 1, err)) {
-        if (!*err) *err = 415;
-        good = false;
-        break;
+      for (int c = 0; c < HC; ++c) {
+        acc[c] = 0;
+        sh[c] = 0.f;
       }
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-#pragma unroll
-      for (int d = 2; d <= DEXACT; ++d) {
-        uint32_t r0[16], r1[16];
-        tmem_ld16(lane_base + (uint32_t)((d - 2) * ON), r0);
-        tmem_ld16(lane_base + (uint32_t)((d - 2) * ON + 16), r1);
-        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          acc[q] += units49(r0[q]);
-          acc[16 + q] += units49(r1[q]);
+      const int nchunk = (w.nst + CHUNK - 1) / CHUNK;
+      bool good = true;
+      for (int c = 0; c < nchunk; ++c, ++cg) {
+        if (!bar_wait(su32(cfull), cg & 1, err)) {
+          if (!*err) *err = 415;
+          good = false;
+          break;
         }
+        fence_after();
+        if (c == nchunk - 1) {
+          uint32_t r[16];
+          tmem_ld16(lane_base + (uint32_t)(SHARED_SLOT * ON), r);
+          tmem_wait_ld();
+#pragma unroll
+          for (int q = 0; q < HC; ++q) sh[q] = __uint_as_float(r[q]);
+        }
+#pragma unroll
+        for (int d = 2; d <= DEXACT; ++d) {
+          // the sums are integers times 2^-7d below 2^24: exact as 32-bit integers, one wide
+          // multiply-add each into units of 2^-49
+          uint32_t r[16];
+          tmem_ld16(lane_base + (uint32_t)((d - 2) * ON), r);
+          tmem_wait_ld();
+          const float up = __int_as_float((127 + 7 * d) << 23);  // 2^7d
+          const int f = 1 << (d == 2 ? 30 : 49 - 7 * d);
+#pragma unroll
+          for (int q = 0; q < HC; ++q) {
+            const long long t = (long long)__float2int_rn(__uint_as_float(r[q]) * up) * f;
+            acc[q] += d == 2 ? t << 5 : t;
+          }
+        }
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(su32(cempty));
       }
-      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(cempty)) : "memory");
-    }
-    const bool any = good && nchunk > 0;
-    const int gi = m0 + row;
-    const int Ei = (any && gi < p.M) ? p.E[gi] : EXP_ZERO;
+      if (!good) break;
+      const int gi = w.m0 + quarter * 32 + lane;
+      const bool any = nchunk > 0, row_ok = gi < p.M;
+      const int Ei = (any && row_ok) ? p.E[gi] : EXP_ZERO;
+      const int cmax = p.c_lower ? min(p.N, (gi >> rs) + 1) : p.N;  // columns [0, cmax) of this row are wanted
+      double* crow = p.ksplit > 1 ? p.ws + (long long)w.z * p.M * p.N + gi : p.C + gi;
+      const long long ld = p.ksplit > 1 ? p.M : p.ldc;
+      if (row_ok) {
 #pragma unroll
-    for (int cb = 0; cb < HC; cb += 16) {
-      uint32_t r[16];
-      if (any) {
-        tmem_ld16(lane_base + (uint32_t)(SHARED_SLOT * ON + cb), r);
-        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-      } else {
+        for (int h = 0; h < HC; h += 4) {
+          // the loads of 4 outputs (column exponents, C) first, so that they overlap
+          double cin[4];
+          int fj[4];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) r[q] = 0u;
-      }
-      if (gi < p.M) {
-#pragma unroll
-        for (int h = 0; h < 16; h += 8) {
-          // the loads of 8 outputs (column exponents, C) first, so that they overlap
-          const bool read_c = p.ksplit == 1 && p.beta != 0.0;
-          double cin[8];
-          int fj[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int gj = n0 + col0 + cb + h + u;
-            const bool ok = gj < p.N && !(p.c_lower && (gi >> rs) < gj);
-            fj[u] = (ok && any) ? p.F[gj] : EXP_ZERO;
-            cin[u] = (ok && read_c) ? p.C[gi + gj * p.ldc] : 0.0;
+          for (int u = 0; u < 4; ++u) {
+            const int gj = w.n0 + col0 + h + u;
+            fj[u] = (any && gj < cmax) ? p.F[gj] : EXP_ZERO;
+            cin[u] = (read_c && gj < cmax) ? crow[gj * ld] : 0.0;
           }
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int q = h + u;
-            const int gj = n0 + col0 + cb + q;
-            if (gj >= p.N || (p.c_lower && (gi >> rs) < gj)) continue;
+          for (int u = 0; u < 4; ++u) {
+            const int gj = w.n0 + col0 + h + u;
+            if (gj >= cmax) continue;
             double v = 0.0;
-            if (any) {
-              const int Fj = fj[u];
-              if (Ei >= EXP_BAD || Fj >= EXP_BAD) {
-                v = __longlong_as_double(0x7FF8000000000000ll);  // an Inf / NaN entry reached this output
-              } else if (Ei >= -1100 && Fj >= -1100) {
-                const double sum = (double)acc[cb + q] * 0x1p-49 + (double)__uint_as_float(r[q]);
-                v = scale2(sum, Ei + Fj + 2);
-              }
+            if (Ei >= -1100 && fj[u] >= -1100) v = to_fp64(acc[h + u], sh[h + u], Ei + fj[u] + 2);
+            // an Inf / NaN entry reached this output
+            if (any && (Ei >= EXP_BAD || fj[u] >= EXP_BAD)) v = __longlong_as_double(0x7FF8000000000000ll);
+            if (p.ksplit == 1) {
+              if (p.amode == -1) v = -v;
+              else if (p.amode == 0) v = p.alpha * v;
+              if (p.bmode == 1) v += cin[u];
+              else if (p.bmode == 2) v = fma(p.beta, cin[u], v);
             }
-            if (p.ksplit > 1) {
-              p.ws[(long long)blockIdx.y * p.M * p.N + gi + (long long)gj * p.M] = v;
-            } else {
-              const double o = p.alpha * v;
-              p.C[gi + gj * p.ldc] = read_c ? o + p.beta * cin[u] : o;
-            }
+            crow[gj * ld] = v;
           }
         }
       }
@@ -541,10 +669,9 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
     for (int s = *consumed; s < *issued; ++s) bar_wait_plain(su32(&full[s % NSTAGE]), (s / NSTAGE) & 1);
     atomicCAS(&p.status[ST_TIMEOUT], 0, *err);
   }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  fence_before();
   __syncthreads();
-  if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TMEM_COLS_OZ));
+  if (warp == 0) tmem_dealloc(tmem, TMEM_COLS_OZ);
 }
 
 // C = alpha sum_z ws[z] + beta C in a fixed order (deterministic)
@@ -588,6 +715,40 @@ size_t gemm_f64_emulated_scratch(int M, int N, int K) { return oz_layout(M, N, K
 
 namespace {
 
+// Exponents and digit planes of both operands.  K <= 128 (the thin products of the panels): one launch
+// that holds whole vectors in registers; else an exponent pass and a split pass, each over both operands.
+// (For a 1500 x 32 x 32 product the former two exponent and two split launches with their two memsets
+// took about 36 us.)
+void split_both(Sys& s, int M, int N, int K, const Opnd& a, const Opnd& b, int fast_a, int fast_b, int* E, int* F,
+                unsigned char* Ap, unsigned char* Bp, int MT, int NT, int KT) {
+  Opnd2 q{};
+  q.o[0] = a; q.o[1] = b;
+  q.R[0] = M; q.R[1] = N;
+  q.fast[0] = fast_a; q.fast[1] = fast_b;
+  q.E[0] = E; q.E[1] = F;
+  q.TR[0] = OM; q.TR[1] = ON;
+  q.RT[0] = MT; q.RT[1] = NT;
+  q.out[0] = Ap; q.out[1] = Bp;
+  const long long ga = (long long)MT * (OM / 8), gb = (long long)NT * (ON / 8);  // 8-row groups
+  if (K <= 128) {
+    q.nblk0 = (int)cdiv(ga, 4);
+    const unsigned nb = q.nblk0 + cdiv(gb, 4);
+    GEV_COUNT(s);
+    if (K <= 64) k_split_short<4><<<nb, 128, 0, s.stream>>>(q, K, KT);
+    else k_split_short<8><<<nb, 128, 0, s.stream>>>(q, K, KT);
+    return;
+  }
+  constexpr int SLAB = 512;
+  const int slabs = K <= 2 * SLAB ? 1 : (int)cdiv(K, SLAB);
+  if (slabs > 1) cudaMemsetAsync(E, 0x80, (size_t)((unsigned char*)(F + NT * ON) - (unsigned char*)E), s.stream);
+  q.nblk0 = (int)cdiv(M, 32);
+  GEV_COUNT(s);
+  k_vec_exp<<<dim3(q.nblk0 + cdiv(N, 32), slabs), 256, 0, s.stream>>>(q, K, slabs == 1 ? K : SLAB, slabs);
+  q.nblk0 = (int)cdiv(ga * KT, 8);
+  GEV_COUNT(s);
+  k_split<<<q.nblk0 + cdiv(gb * KT, 8), 256, 0, s.stream>>>(q, K, KT);
+}
+
 // C (M x N, real, ldc) = alpha op(A) op(B) + beta C with op(A) = the M x K operand a and op(B) the
 // N x K operand b (vectors = columns of op(B)), K in the operands' element units (embedded for
 // complex data); ka / kb: bytes of one underlying element step along K of a / b, to offset the
@@ -622,38 +783,33 @@ void emulate(Sys& s, int M, int N, int K, Opnd a, size_t a_kstep, Opnd b, size_t
     ap.X = static_cast<const unsigned char*>(a.X) + (size_t)ku * a_kstep;
     bp.X = static_cast<const unsigned char*>(b.X) + (size_t)ku * b_kstep;
     ap.koff = bp.koff = ku;
-    if (Kc > 0) {
-      cudaMemsetAsync(E, 0x80, L.Mp * sizeof(int), s.stream);
-      cudaMemsetAsync(F, 0x80, L.Np * sizeof(int), s.stream);
-      const dim3 eb(32, 8);
-      GEV_COUNT(s);
-      k_vec_exp<<<dim3(fast_a ? cdiv(M, 32) : cdiv(M, 8), cdiv(Kc, 1024)), eb, 0, s.stream>>>(M, Kc, ap, fast_a, E);
-      GEV_COUNT(s);
-      k_vec_exp<<<dim3(fast_b ? cdiv(N, 32) : cdiv(N, 8), cdiv(Kc, 1024)), eb, 0, s.stream>>>(N, Kc, bp, fast_b, F);
-      GEV_COUNT(s);
-      k_split<<<cdiv((long long)MT * OM * 2 * KT, 256), 256, 0, s.stream>>>(M, Kc, ap, fast_a, E, OM, MT, KT, Ap);
-      GEV_COUNT(s);
-      k_split<<<cdiv((long long)NT * ON * 2 * KT, 256), 256, 0, s.stream>>>(N, Kc, bp, fast_b, F, ON, NT, KT, Bp);
-    }
+    if (Kc > 0) split_both(s, M, N, Kc, ap, bp, fast_a, fast_b, E, F, Ap, Bp, MT, NT, KT);
     OzP p{};
     p.M = M; p.N = N; p.K = Kc; p.koff = ku; p.c_lower = c_lower;
     p.tri_a = tri_a; p.tri_b = tri_b; p.cx = rs;
     p.MT = MT; p.NT = NT; p.KT = KT;
     p.alpha = alpha; p.beta = (k0 == 0) ? beta : 1.0;
     p.C = C; p.ldc = ldc; p.Ap = Ap; p.Bp = Bp; p.E = E; p.F = F; p.status = s.status;
-    // split K when the output has too few tiles to fill the GPU and K is long
+    // split K when the output has too few tiles to fill the GPU; a share is at least 8 slices (about 7 us
+    // of MMAs, of the order of the launch that sums the shares)
     long long tiles = (long long)MT * NT;
     if (c_lower) tiles = (tiles + MT) / 2;
     int ks = 1;
-    if (tiles < s.sms && KT >= 2 * CHUNK) {
-      ks = (int)std::min<long long>((2LL * s.sms + tiles - 1) / tiles, KT / CHUNK);
-      ks = std::min(ks, 16);
+    if (2 * tiles <= s.sms && KT >= 16) {
+      ks = (int)std::min<long long>(s.sms / tiles, KT / 8);
+      ks = std::min(ks, 64);
       while (ks > 1 && (size_t)ks * M * N * sizeof(double) > s.splitws_bytes) --ks;
     }
     p.ksplit = ks;
     p.ws = ks > 1 ? static_cast<double*>(s.splitws) : nullptr;
+    p.amode = alpha_mode(p.alpha);
+    p.bmode = beta_mode(p.beta);
+    // long items: one CTA each, scheduled by the hardware as SMs come free (triangular tiles differ in
+    // length, and the epilogue is a small part); short ones: persistent CTAs (8192^3 and the triangular
+    // products of n = 10240 ran 8 - 15 % slower persistent, 8192 x 8192 x 128 1.9 times faster)
+    const long long work = (long long)MT * NT * ks;
     GEV_COUNT(s);
-    ozaki_kernel<<<dim3(MT * NT, ks), NTH, SMEM_OZ, s.stream>>>(p);
+    ozaki_kernel<<<KT >= 48 * ks ? work : std::min<long long>(work, s.sms), NTH, SMEM_OZ, s.stream>>>(p);
     if (ks > 1) {
       const long long total = (long long)M * N;
       unsigned blocks = cdiv(total, 256);
@@ -750,19 +906,27 @@ bool gemm_f64_bdiag(Sys& s, int M, int N, int K, const BdOp& a, int bm, int bk, 
   const Opnd b{B, ldb, 1, 0, a.cx ? 2 : 0, 0, 0};
   GEV_COUNT(s);
   k_split_bd<<<cdiv((long long)L.MT * OM * 32, 256), 256, 0, s.stream>>>(Me, a, bme, bke, L.MT, E, Ap);
+  Opnd2 q{};
+  q.o[0] = b;
+  q.R[0] = N;
+  q.E[0] = F;
+  q.TR[0] = ON;
+  q.RT[0] = L.NT;
+  q.out[0] = Bp;
   if (b_below_two) {  // every entry of B below 2 in magnitude: the column exponents are 1, no pass over B
     GEV_COUNT(s);
     k_fill_exp<<<cdiv(L.Np, 256), 256, 0, s.stream>>>((int)L.Np, 1, F);
-  } else {
-    cudaMemsetAsync(F, 0x80, L.Np * sizeof(int), s.stream);
+  } else if (Ke > 0) {
+    const int slabs = (int)cdiv(Ke, 512);
+    if (slabs > 1) cudaMemsetAsync(F, 0x80, L.Np * sizeof(int), s.stream);
+    q.nblk0 = (int)cdiv(N, 32);
+    GEV_COUNT(s);
+    k_vec_exp<<<dim3(q.nblk0, slabs), 256, 0, s.stream>>>(q, Ke, slabs == 1 ? Ke : 512, slabs);
   }
   if (Ke > 0) {
-    if (!b_below_two) {
-      GEV_COUNT(s);
-      k_vec_exp<<<dim3(cdiv(N, 8), cdiv(Ke, 1024)), dim3(32, 8), 0, s.stream>>>(N, Ke, b, 0, F);
-    }
+    q.nblk0 = (int)cdiv((long long)L.NT * (ON / 8) * L.KT, 8);
     GEV_COUNT(s);
-    k_split<<<cdiv((long long)L.NT * ON * 2 * L.KT, 256), 256, 0, s.stream>>>(N, Ke, b, 0, F, ON, L.NT, L.KT, Bp);
+    k_split<<<q.nblk0, 256, 0, s.stream>>>(q, Ke, L.KT);
   }
   OzP p{};
   p.M = Me; p.N = N; p.K = Ke; p.koff = 0; p.c_lower = 0;
@@ -775,8 +939,10 @@ bool gemm_f64_bdiag(Sys& s, int M, int N, int K, const BdOp& a, int bm, int bk, 
   p.Ap = Ap; p.Bp = Bp; p.E = E; p.F = F; p.status = s.status;
   p.bd_bm = bme;
   p.bd_bk = bke;
+  p.amode = alpha_mode(alpha);
+  p.bmode = beta_mode(beta);
   GEV_COUNT(s);
-  ozaki_kernel<<<dim3(L.MT * L.NT, 1), NTH, SMEM_OZ, s.stream>>>(p);
+  ozaki_kernel<<<std::min<long long>((long long)L.MT * L.NT, s.sms), NTH, SMEM_OZ, s.stream>>>(p);
   return true;
 }
 
