@@ -19,6 +19,7 @@
 //    smallest eigenvalue of the node starting at a.  At the top merge only the k lowest
 //    eigenvectors are formed.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <vector>
 
@@ -71,129 +72,207 @@ struct DcArrays {
 };
 
 // ------------------------------------------------------------------------------------ tearing --
+// dw = d with |e[m-1]| taken off both sides of every leaf boundary m = floor(q n / nleaf)
 __global__ void k_tear(int n, int nleaf, const double* d, const double* e, double* dw) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dw[i] = d[i];
-  __syncthreads();
-}
-__global__ void k_tear2(int n, int nleaf, const double* e, double* dw) {
-  // boundary of leaf q (q = 1 .. nleaf-1) at row floor(q n / nleaf)
-  for (int q = 1 + blockIdx.x * blockDim.x + threadIdx.x; q < nleaf; q += gridDim.x * blockDim.x) {
-    const int m = (int)(((long long)q * n) / nleaf);
-    const double rho = fabs(e[m - 1]);
-    dw[m - 1] -= rho;
-    dw[m] -= rho;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    double v = d[i];
+    const int q0 = (int)(((long long)i * nleaf) / n);
+    for (int q = max(1, q0 - 1); q <= min(nleaf - 1, q0 + 2); ++q) {
+      const int m = (int)(((long long)q * n) / nleaf);
+      if (m == i || m == i + 1) v -= fabs(e[m - 1]);
+    }
+    dw[i] = v;
   }
 }
 
 // ------------------------------------------------------------------------------------- leaves --
-// Implicit QL on the leaf (rows [a, a+sz)), eigenvectors accumulated in shared memory; thread 0
-// runs the scalar recurrence and records each sweep's rotations, all threads apply them.
+// 1 / sqrt of q = f^2 + g^2 when q is comfortably inside the range (an integer test of the exponent: an
+// FP64 comparison costs as much as a multiplication here); else false and the caller takes hypot
+__device__ __forceinline__ bool rsqrt_safe(double q, double& ri) {
+  const int e = (__double2hiint(q) >> 20) & 0x7FF;
+  if (e < 1023 - 900 || e > 1023 + 900) return false;
+  ri = rsqrt(q);
+  return true;
+}
+
+// Implicit QL on the leaf (rows [a, a+sz)), eigenvectors accumulated in shared memory.  Warp 0 runs the
+// scalar recurrence (lane 0; the split search is one ballot) and records each sweep's rotations, warp 1
+// (a lane per row) applies the previous sweep's meanwhile: one barrier per sweep.  The recurrence is one
+// dependent FP64 chain of about 900 rotations for 32 rows: a rotation is one rsqrt and multiplications
+// (hypot and two divisions before, and one thread's split search: 2.4 ms for any matrix of leaves of 32;
+// 0.65 ms now).
 __global__ void __launch_bounds__(64) k_leaf(int n, int nleaf, const double* dw, const double* e,
                                              double* w, double* Q, long long ldq, int* colmap,
                                              int* status) {
   __shared__ double Z[LEAF][LEAF + 1];
   __shared__ double dd[LEAF], ee[LEAF];
-  __shared__ double rc[LEAF], rs[LEAF];
-  __shared__ int ri[LEAF];
-  __shared__ int nrot, done, fail;
+  __shared__ double rc[2][LEAF], rs[2][LEAF];
+  __shared__ int s_hi[2], s_nrot[2];  // a sweep's rotations act on columns hi - t, hi - t + 1, t < nrot
+  __shared__ int done[2], fail;  // done: by sweep parity, like the rotations
   __shared__ int perm[LEAF];
   const int q = blockIdx.x;
   const int a = (int)(((long long)q * n) / nleaf);
   const int c = (int)(((long long)(q + 1) * n) / nleaf);
   const int sz = c - a;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
   for (int i = tid; i < sz; i += blockDim.x) {
     dd[i] = dw[a + i];
     ee[i] = (i + 1 < sz) ? e[a + i] : 0.0;
     for (int j = 0; j < sz; ++j) Z[i][j] = (i == j) ? 1.0 : 0.0;
   }
-  if (tid == 0) { done = 0; fail = 0; }
+  if (tid < LEAF) perm[tid] = tid;
+  if (tid == 0) { done[0] = done[1] = 0; fail = 0; s_nrot[0] = s_nrot[1] = 0; }
   __syncthreads();
-  // thread-0 state of the QL iteration
-  int l = 0, iter = 0, total = 0;
+  int l = 0, total = 0, par = 0;  // warp 0's state of the iteration (uniform over the warp)
   while (true) {
-    if (tid == 0) {
-      nrot = 0;
-      // advance to the next sweep to perform (or finish)
-      while (true) {
-        if (l >= sz) { done = 1; break; }
-        int m = l;
-        while (m + 1 < sz) {
-          const double dsum = fabs(dd[m]) + fabs(dd[m + 1]);
-          if (fabs(ee[m]) <= EPS * dsum) break;
-          ++m;
-        }
-        if (m == l) { ++l; iter = 0; continue; }
-        if (++total > 30 * sz) { fail = 1; done = 1; break; }
-        ++iter;
+    if (tid < 32) {
+      int nrot = 0, m = l;
+      // the next sweep to perform: the first l with a coupling below it, and the end m of its block
+      const bool small = lane + 1 >= sz || fabs(ee[lane]) <= EPS * (fabs(dd[lane]) + fabs(dd[lane + 1 < sz ? lane + 1 : lane]));
+      const unsigned cut = __ballot_sync(0xffffffffu, small);
+      while (l < sz) {
+        m = l + __ffs(cut >> l) - 1;  // (bit sz - 1 is set)
+        if (m > l) break;
+        ++l;
+      }
+      bool stop = l >= sz;
+      if (!stop && ++total > 30 * sz) {
+        stop = true;
+        if (lane == 0) fail = 1;
+      }
+      if (stop) {
+        if (lane == 0) done[par] = 1;
+      } else if (lane == 0) {
         double g = (dd[l + 1] - dd[l]) / (2.0 * ee[l]);
         double r = hypot(g, 1.0);
         g = dd[m] - dd[l] + ee[l] / (g + copysign(r, g));
-        double s = 1.0, cc = 1.0, p = 0.0;
+        double sn = 1.0, cc = 1.0, p = 0.0;
         bool early = false;
+        double ei = ee[m - 1], di = dd[m - 1], dn = dd[m];  // e_i, d_i, d_{i+1}
         for (int i = m - 1; i >= l; --i) {
-          const double f = s * ee[i], b = cc * ee[i];
-          r = hypot(f, g);
-          ee[i + 1] = r;
-          if (r == 0.0) { dd[i + 1] -= p; ee[m] = 0.0; early = true; break; }
-          s = f / r;
-          cc = g / r;
-          g = dd[i + 1] - p;
-          r = (dd[i] - g) * s + 2.0 * cc * b;
-          p = s * r;
+          const double f = sn * ei, b = cc * ei;
+          const double en = i > l ? ee[i - 1] : 0.0, dm = i > l ? dd[i - 1] : 0.0;  // the next step's
+          const double qq = fma(f, f, g * g);
+          double ri;
+          if (rsqrt_safe(qq, ri)) {
+            r = qq * ri;
+            sn = f * ri;
+            cc = g * ri;
+          } else {
+            r = hypot(f, g);
+            if (r == 0.0) { ee[i + 1] = r; dd[i + 1] = dn - p; ee[m] = 0.0; early = true; break; }
+            sn = f / r;
+            cc = g / r;
+          }
+          if (i + 1 < m) ee[i + 1] = r;  // (ee[m] is zeroed below)
+          g = dn - p;
+          const double rr = fma(di - g, sn, 2.0 * cc * b);
+          p = sn * rr;
           dd[i + 1] = g + p;
-          g = cc * r - b;
-          ri[nrot] = i; rc[nrot] = cc; rs[nrot] = s; ++nrot;
+          g = fma(cc, rr, -b);
+          rc[par][nrot] = cc;
+          rs[par][nrot] = sn;
+          ++nrot;
+          dn = di;
+          di = dm;
+          ei = en;
         }
         if (!early) { dd[l] -= p; ee[l] = g; ee[m] = 0.0; }
-        break;  // one sweep recorded
+        s_hi[par] = m - 1;
+        s_nrot[par] = nrot;
+      }
+      __syncwarp();
+      if (stop && lane == 0) s_nrot[par] = 0;
+    } else if (lane < sz) {
+      const int pv = par ^ 1, nr = s_nrot[pv], hi = s_hi[pv];
+      if (nr > 0) {
+        double z1 = Z[lane][hi + 1];
+        for (int t = 0; t < nr; ++t) {
+          const int i = hi - t;
+          const double zi = Z[lane][i], cs = rc[pv][t], sn = rs[pv][t];
+          Z[lane][i + 1] = sn * zi + cs * z1;
+          z1 = cs * zi - sn * z1;
+        }
+        Z[lane][hi - nr + 1] = z1;
       }
     }
     __syncthreads();
-    const int nr = nrot;
-    for (int row = tid; row < sz; row += blockDim.x) {
-      for (int t = 0; t < nr; ++t) {
-        const int i = ri[t];
-        const double zi = Z[row][i], zi1 = Z[row][i + 1];
-        Z[row][i + 1] = rs[t] * zi + rc[t] * zi1;
-        Z[row][i] = rc[t] * zi - rs[t] * zi1;
-      }
-    }
-    __syncthreads();
-    if (done) break;
+    if (done[par]) break;  // (warp 1 has applied the last sweep: done is set in a round without rotations)
+    par ^= 1;
   }
-  if (tid == 0) {
-    if (fail) atomicCAS(&status[ST_NOCONV], 0, 301);
-    for (int i = 0; i < sz; ++i) perm[i] = i;
-    for (int i = 1; i < sz; ++i) {  // stable insertion sort of eigenvalue indices
-      int pi = perm[i];
-      int j = i - 1;
-      while (j >= 0 && dd[perm[j]] > dd[pi]) { perm[j + 1] = perm[j]; --j; }
-      perm[j + 1] = pi;
+  if (tid < 32) {
+    if (lane == 0 && fail) atomicCAS(&status[ST_NOCONV], 0, 301);
+    if (lane < sz) {  // stable rank of the eigenvalue
+      const double v = dd[lane];
+      int pos = 0;
+      for (int j = 0; j < sz; ++j) {
+        const double u = dd[j];
+        pos += (u < v || (u == v && j < lane)) ? 1 : 0;
+      }
+      perm[pos < LEAF ? pos : LEAF - 1] = lane;
     }
   }
   __syncthreads();
   for (int i = tid; i < sz; i += blockDim.x) {
     w[a + i] = dd[perm[i]];
     colmap[a + i] = a + i;
-    for (int j = 0; j < sz; ++j) Q[(a + j) + (long long)(a + i) * ldq] = Z[j][perm[i]];
+  }
+  for (int t = tid; t < sz * sz; t += blockDim.x) {
+    const int i = t / sz, j = t % sz;
+    Q[(a + j) + (long long)(a + i) * ldq] = Z[j][perm[i]];
   }
 }
 
 // ------------------------------------------------------------------------------ merge: prepare --
-// One block per node: z, rank merge of the two sorted pole lists, deflation scan (thread 0),
-// rotations applied to the physical columns, sort of the deflated list, gather order by type.
-__global__ void __launch_bounds__(1024) k_merge_prep(int n, Node* nodes, const double* e,
-                                                      const double* w, double* Q, long long ldq,
-                                                      DcArrays A) {
+// exclusive block scan of one 64-bit value per thread (several packed counters); tot: the sum
+template <int NTH>
+__device__ __forceinline__ unsigned long long block_excl_scan(unsigned long long v, unsigned long long* sm,
+                                                               unsigned long long& tot) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned long long x = v;
+  for (int off = 1; off < 32; off <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, off);
+    if (lane >= off) x += y;
+  }
+  __syncthreads();  // sm may still be read by the previous scan
+  if (lane == 31) sm[wid] = x;
+  __syncthreads();
+  unsigned long long before = 0, t = 0;
+#pragma unroll
+  for (int q = 0; q < NTH / 32; ++q) {
+    if (q < wid) before += sm[q];
+    t += sm[q];
+  }
+  tot = t;
+  return before + x - v;
+}
+
+// One block per node: z, rank merge of the two sorted pole lists, deflation, rotations applied to the
+// physical columns, sort of the deflated list, gather order by type.
+// Deflation looks at one entry after another: an entry with r |z_i| <= tol deflates; else it is tested
+// against the last one kept, and where a rotation of the two leaves an off-diagonal <= tol the earlier
+// one deflates and the later one, changed, is tested against its successor.  All tests on unchanged
+// entries are independent, so they run in parallel and only the entries that follow a rotation are
+// tested again, one by one; the lists come from prefix sums.  (As one thread's scan over global memory
+// the kernel took 14.8 ms for the top merge at n = 10240 and 2.1 ms at n = 1500: 0.05 ms now at 1500.)
+constexpr int PREP_NTH = 512;
+__global__ void __launch_bounds__(PREP_NTH) k_merge_prep(int n, int nleaf, int span, Node* nodes, const double* e,
+                                                         const double* w, double* Q, long long ldq,
+                                                         DcArrays A) {
   Node& nd = nodes[blockIdx.x];
-  const int a = nd.a, m = nd.m, c = nd.c;
+  const int a = (int)(((long long)blockIdx.x * span * n) / nleaf);
+  const int m = (int)(((long long)(blockIdx.x * span + span / 2) * n) / nleaf);
+  const int c = (int)(((long long)(blockIdx.x + 1) * span * n) / nleaf);
   const int n1 = m - a, nn = c - a;
-  const int tid = threadIdx.x, NTH = blockDim.x;
+  const int tid = threadIdx.x;
+  constexpr int NTH = PREP_NTH;
   const double rho = e[m - 1];
   const double sg = rho < 0 ? -1.0 : 1.0;
   const double r = 2.0 * fabs(rho);
   const double isq2 = 0.70710678118654752440;
+  __shared__ unsigned long long scan_sm[NTH / 32];
+  __shared__ double zred[NTH / 32];
+  __shared__ int sR, s_next, s_swap;
   // rank merge: child 1 = w[a .. m), child 2 = w[m .. c), both ascending
   for (int i = tid; i < nn; i += NTH) {
     double di;
@@ -224,101 +303,179 @@ __global__ void __launch_bounds__(1024) k_merge_prep(int n, Node* nodes, const d
     A.csrc[a + pos] = col;
     A.tb[a + pos] = tbits;
   }
+  if (tid == 0) { sR = 0; s_next = INT_MAX; }
   __syncthreads();
-  __shared__ int sK, sD, sR;
-  if (tid == 0) {
-    const double dmax = fmax(fabs(A.dsort[a]), fabs(A.dsort[c - 1]));
-    const double tol = 8.0 * EPS * fmax(dmax, r);
-    int K = 0, D = 0, R = 0;
-    int prev = -1;  // sorted index of the pending non-deflated candidate
-    double zn2 = 0.0;
-    for (int i = 0; i < nn; ++i) {
-      const int ii = a + i;
-      const double zi = A.zs[ii];
-      if (r * fabs(zi) <= tol) {  // negligible coupling: eigenpair kept as is
-        A.df_d[a + D] = A.dsort[ii];
-        A.df_col[a + D] = A.csrc[ii];
-        ++D;
-        continue;
-      }
-      if (prev >= 0) {
-        const int pj = a + prev;
-        const double zp = A.zs[pj];
+  const double tol = 8.0 * EPS * fmax(fmax(fabs(A.dsort[a]), fabs(A.dsort[c - 1])), r);
+  const int per = (nn + NTH - 1) / NTH, i0 = min(nn, tid * per), i1 = min(nn, i0 + per);
+  // the entries that couple (r |z| > tol), in order: index list in A.pos_r; flag 4 in A.tb
+  int cnt = 0;
+  for (int i = i0; i < i1; ++i) {
+    const bool big = !(r * fabs(A.zs[a + i]) <= tol);
+    if (big) ++cnt;
+    A.pos_d[a + i] = big ? 1 : 0;
+  }
+  unsigned long long tot;
+  int at = (int)block_excl_scan<NTH>((unsigned long long)cnt, scan_sm, tot);
+  const int nbig = (int)tot;
+  for (int i = i0; i < i1; ++i)
+    if (A.pos_d[a + i]) A.pos_r[a + at++] = i;
+  __syncthreads();
+  // tests of neighbouring kept entries on their original values; rflag (A.org): the pair (q - 1, q) rotates
+  for (int q = tid; q < nbig; q += NTH) {
+    int fl = 0;
+    if (q > 0) {
+      const int pj = a + A.pos_r[a + q - 1], ii = a + A.pos_r[a + q];
+      const double zp = A.zs[pj], zi = A.zs[ii];
+      const double tau = hypot(zp, zi);
+      const double cs = zi / tau, sn = zp / tau;
+      fl = fabs((A.dsort[ii] - A.dsort[pj]) * cs * sn) <= tol ? 1 : 0;
+    }
+    A.org[a + q] = fl;
+  }
+  __syncthreads();
+  // the rotations: runs of flagged pairs, by one thread; A.org[q] = 1 in the end: entry q - 1 deflated
+  for (int q0 = 1;;) {
+    if (tid == 0) s_next = INT_MAX;
+    __syncthreads();
+    int f = INT_MAX;
+    for (int q = q0 + tid; q < nbig; q += NTH)
+      if (A.org[a + q]) { f = q; break; }
+    if (f != INT_MAX) atomicMin(&s_next, f);
+    __syncthreads();
+    const int first = s_next;
+    __syncthreads();
+    if (first == INT_MAX) break;
+    if (tid == 0) {
+      int q = first, R = sR;
+      while (true) {
+        const int pj = a + A.pos_r[a + q - 1], ii = a + A.pos_r[a + q];
+        const double zp = A.zs[pj], zi = A.zs[ii];
         const double tau = hypot(zp, zi);
         const double cs = zi / tau, sn = zp / tau;
         const double dp = A.dsort[pj], di = A.dsort[ii];
-        if (fabs((di - dp) * cs * sn) <= tol) {
-          // rotate the pair so z_prev = 0: prev deflates
-          A.zs[ii] = tau;
-          A.zs[pj] = 0.0;
-          A.dsort[pj] = cs * cs * dp + sn * sn * di;
-          A.dsort[ii] = sn * sn * dp + cs * cs * di;
-          const int cp = A.csrc[pj], ci = A.csrc[ii];
-          A.rot_p[a + R] = cp;
-          A.rot_i[a + R] = ci;
-          A.rot_c[a + R] = cs;
-          A.rot_s[a + R] = sn;
-          ++R;
-          const int u = A.tb[pj] | A.tb[ii];
-          A.tb[pj] = u;
-          A.tb[ii] = u;
-          A.df_d[a + D] = A.dsort[pj];
-          A.df_col[a + D] = cp;
-          ++D;
-          prev = i;
-          continue;
+        if (q > first && !(fabs((di - dp) * cs * sn) <= tol)) {
+          A.org[a + q] = 0;
+          ++q;
+          break;
         }
-        // prev is final
-        A.nd_d[a + K] = dp;
-        A.nd_z[a + K] = zp;
-        A.nd_col[a + K] = A.csrc[pj];
-        A.nd_g[a + K] = A.tb[pj];  // temporarily the type bits
-        zn2 += zp * zp;
-        ++K;
+        // rotate the pair so z_prev = 0: prev deflates
+        A.org[a + q] = 1;
+        A.zs[ii] = tau;
+        A.zs[pj] = 0.0;
+        A.dsort[pj] = cs * cs * dp + sn * sn * di;
+        A.dsort[ii] = sn * sn * dp + cs * cs * di;
+        A.rot_p[a + R] = A.csrc[pj];
+        A.rot_i[a + R] = A.csrc[ii];
+        A.rot_c[a + R] = cs;
+        A.rot_s[a + R] = sn;
+        ++R;
+        const int u = A.tb[pj] | A.tb[ii];
+        A.tb[pj] = u;
+        A.tb[ii] = u;
+        if (++q >= nbig) break;
       }
-      prev = i;
+      sR = R;
+      s_next = q;
     }
-    if (prev >= 0) {
-      const int pj = a + prev;
-      A.nd_d[a + K] = A.dsort[pj];
-      A.nd_z[a + K] = A.zs[pj];
-      A.nd_col[a + K] = A.csrc[pj];
-      A.nd_g[a + K] = A.tb[pj];
-      zn2 += A.zs[pj] * A.zs[pj];
-      ++K;
-    }
-    // stable insertion sort of the deflated list (rotations perturb its order only locally)
-    for (int i = 1; i < D; ++i) {
-      const double dv = A.df_d[a + i];
-      const int cv = A.df_col[a + i];
-      int j = i - 1;
-      while (j >= 0 && A.df_d[a + j] > dv) {
-        A.df_d[a + j + 1] = A.df_d[a + j];
-        A.df_col[a + j + 1] = A.df_col[a + j];
-        --j;
+    __syncthreads();
+    q0 = s_next;
+    __syncthreads();
+  }
+  const int R = sR;
+  // marks per sorted entry i (A.pos_d): bit 0 couples, bit 1 deflated by a rotation, bit 2 partner of one
+  if (R > 0) {
+    for (int q = 1 + tid; q < nbig; q += NTH)
+      if (A.org[a + q]) {
+        atomicOr(&A.pos_d[a + A.pos_r[a + q - 1]], 2);
+        atomicOr(&A.pos_d[a + A.pos_r[a + q]], 4);
       }
-      A.df_d[a + j + 1] = dv;
-      A.df_col[a + j + 1] = cv;
+    __syncthreads();
+  }
+  // kept entries in order; deflated ones in the order in which the scan meets them (a rotated one when
+  // it meets its partner)
+  unsigned long long kd = 0;
+  double zz = 0.0;
+  for (int i = i0; i < i1; ++i) {
+    const int f = A.pos_d[a + i];
+    if ((f & 3) == 1) kd += 1;
+    if (!(f & 1) || (f & 4)) kd += 1ull << 32;
+  }
+  unsigned long long pre = block_excl_scan<NTH>(kd, scan_sm, tot);
+  const int K = (int)(tot & 0xffffffffu), D = (int)(tot >> 32);
+  {
+    int kp = (int)(pre & 0xffffffffu), dpos = (int)(pre >> 32);
+    for (int i = i0; i < i1; ++i) {
+      const int f = A.pos_d[a + i];
+      if ((f & 3) == 1) {
+        const double z = A.zs[a + i];
+        A.nd_d[a + kp] = A.dsort[a + i];
+        A.nd_z[a + kp] = z;
+        A.nd_col[a + kp] = A.csrc[a + i];
+        A.nd_g[a + kp] = A.tb[a + i];  // the type bits, replaced by the gather slot below
+        zz += z * z;
+        ++kp;
+      }
+      int src = -1;
+      if (!(f & 1)) src = i;
+      else if (f & 4) {  // the deflated entry is the kept-list predecessor of i
+        src = i - 1;
+        while (!(A.pos_d[a + src] & 1)) --src;
+      }
+      if (src >= 0) {
+        A.df_d[a + dpos] = A.dsort[a + src];
+        A.df_col[a + dpos] = A.csrc[a + src];
+        ++dpos;
+      }
     }
-    // gather order: top-only, mixed, bottom-only
-    int K1 = 0, K2 = 0, K3 = 0;
-    for (int i = 0; i < K; ++i) {
+  }
+  for (int off = 16; off > 0; off >>= 1) zz += __shfl_down_sync(0xffffffffu, zz, off);
+  if ((tid & 31) == 0) zred[tid >> 5] = zz;
+  __syncthreads();
+  // stable sort of the deflated list: rotations perturb its order only locally, so transpositions of
+  // neighbours, odd and even pairs in turn, end after a few passes
+  for (int idle = 0, ph = 0; R > 0 && idle < 2; ph ^= 1) {
+    if (tid == 0) s_swap = 0;
+    __syncthreads();
+    for (int j = ph + 2 * tid; j + 1 < D; j += 2 * NTH) {
+      const double d0 = A.df_d[a + j], d1 = A.df_d[a + j + 1];
+      if (d0 > d1) {
+        const int c0 = A.df_col[a + j];
+        A.df_d[a + j] = d1;
+        A.df_d[a + j + 1] = d0;
+        A.df_col[a + j] = A.df_col[a + j + 1];
+        A.df_col[a + j + 1] = c0;
+        s_swap = 1;
+      }
+    }
+    __syncthreads();
+    idle = s_swap ? 0 : idle + 1;
+    __syncthreads();
+  }
+  // gather order: top-only, mixed, bottom-only (counters packed, 21 bits each)
+  {
+    const int pk = (K + NTH - 1) / NTH, k0 = min(K, tid * pk), k1 = min(K, k0 + pk);
+    unsigned long long t3 = 0;
+    for (int i = k0; i < k1; ++i) {
       const int t = A.nd_g[a + i];
-      if (t == 1) ++K1; else if (t == 3) ++K2; else ++K3;
+      t3 += t == 1 ? 1ull : (t == 3 ? 1ull << 21 : 1ull << 42);
     }
-    int c1 = 0, c2 = K1, c3 = K1 + K2;
-    for (int i = 0; i < K; ++i) {
+    const unsigned long long p3 = block_excl_scan<NTH>(t3, scan_sm, tot);
+    const int K1 = (int)(tot & 0x1fffff), K2 = (int)((tot >> 21) & 0x1fffff), K3 = (int)(tot >> 42);
+    int c1 = (int)(p3 & 0x1fffff), c2 = K1 + (int)((p3 >> 21) & 0x1fffff), c3 = K1 + K2 + (int)(p3 >> 42);
+    for (int i = k0; i < k1; ++i) {
       const int t = A.nd_g[a + i];
       A.nd_g[a + i] = (t == 1) ? c1++ : (t == 3 ? c2++ : c3++);
     }
-    nd.K = K; nd.K1 = K1; nd.K2 = K2; nd.K3 = K3; nd.ndefl = D; nd.nrot = R;
-    nd.r = r; nd.zn2 = zn2;
-    nd.Kout = K; nd.Dout = D;
-    sK = K; sD = D; sR = R;
+    if (tid == 0) {
+      double zn2 = 0.0;
+      for (int q = 0; q < NTH / 32; ++q) zn2 += zred[q];
+      nd.a = a; nd.m = m; nd.c = c;
+      nd.K = K; nd.K1 = K1; nd.K2 = K2; nd.K3 = K3; nd.ndefl = D; nd.nrot = R;
+      nd.r = r; nd.zn2 = zn2;
+      nd.Kout = K; nd.Dout = D;
+    }
   }
-  __syncthreads();
   // apply the rotations, in order, to the physical columns (rows a .. c-1)
-  const int R = sR;
   for (int t = 0; t < R; ++t) {
     const int cp = A.rot_p[a + t], ci = A.rot_i[a + t];
     const double cs = A.rot_c[a + t], sn = A.rot_s[a + t];
@@ -327,7 +484,6 @@ __global__ void __launch_bounds__(1024) k_merge_prep(int n, Node* nodes, const d
       Q[row + (long long)cp * ldq] = cs * qp - sn * qi;
       Q[row + (long long)ci * ldq] = sn * qp + cs * qi;
     }
-    __syncthreads();
   }
 }
 
@@ -439,22 +595,39 @@ __global__ void __launch_bounds__(256) k_secular(Node* nodes, DcArrays A, int* s
 }
 
 // Gu-Eisenstat: z'_i^2 = prod_j (lambda_j - delta_i) / (r prod_{j != i} (delta_j - delta_i)).
-__global__ void k_zprime(Node* nodes, DcArrays A) {
+// One warp per entry: the lanes take the factors j = lane, lane + 32, ..., two factors to a division (an
+// FP64 division costs about ten multiplications), and their products are multiplied in a fixed order.
+// By interlacing every factor is in (0, 1), so no partial product is smaller than the whole; the products
+// of two differences stay in range while the poles' spread does (pair, else one division per factor).
+// (One thread per entry before, a chain of divisions: 9.3 ms for all levels at n = 10240, 2.7 ms now.)
+__global__ void __launch_bounds__(256) k_zprime(Node* nodes, DcArrays A) {
   const Node nd = nodes[blockIdx.y];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int K = nd.K;
-  if (i >= K) return;
+  if (i >= K) return;  // uniform per warp
   const int a = nd.a;
   const double* delta = A.nd_d + a;
   const double* mu = A.mu + a;
   const int* org = A.org + a;
   const double di = delta[i];
   auto lam_minus = [&](int j) { return (delta[org[j]] - di) + mu[j]; };
-  double prod = lam_minus(K - 1) / nd.r;
-  for (int j = 0; j < i; ++j) prod *= lam_minus(j) / (delta[j] - di);
-  for (int j = i; j < K - 1; ++j) prod *= lam_minus(j) / (delta[j + 1] - di);
-  const double zi = A.nd_z[a + i];
-  A.zp[a + i] = copysign(sqrt(fabs(prod)), zi);
+  auto den = [&](int j) { return delta[j < i ? j : j + 1] - di; };
+  const double spread = fmax(delta[K - 1] - delta[0], nd.r * nd.zn2);
+  const bool pair = spread > 1e-100 && spread < 1e100;
+  double prod = 1.0;
+  int j = lane;
+  if (pair) {
+    for (; j + 32 < K - 1; j += 64) {
+      const double num = lam_minus(j) * lam_minus(j + 32), dd = den(j) * den(j + 32);
+      prod *= num / dd;
+    }
+  }
+  for (; j < K - 1; j += 32) prod *= lam_minus(j) / den(j);
+  for (int off = 16; off > 0; off >>= 1) prod *= __shfl_down_sync(0xffffffffu, prod, off);
+  if (lane == 0) {
+    prod *= lam_minus(K - 1) / nd.r;
+    A.zp[a + i] = copysign(sqrt(fabs(prod)), A.nd_z[a + i]);
+  }
 }
 
 // Final positions of roots and deflated entries within each node; eigenvalues in sorted order.
@@ -481,16 +654,24 @@ __global__ void k_positions(Node* nodes, DcArrays A, int kcut, int* status) {
   }
 }
 
-// Count the roots / deflated entries whose position is below kcut (prefixes: positions increase).
-__global__ void k_count_out(Node* nodes, DcArrays A, int kcut) {
-  Node& nd = nodes[blockIdx.x];
-  if (threadIdx.x != 0) return;
-  const int a = nd.a;
-  int ko = 0, dout = 0;
-  for (int t = 0; t < nd.K; ++t) if (A.pos_r[a + t] < kcut) ++ko;
-  for (int u = 0; u < nd.ndefl; ++u) if (A.pos_d[a + u] < kcut) ++dout;
-  nd.Kout = ko;
-  nd.Dout = dout;
+// The roots / deflated entries of the top merge whose position is below kcut are prefixes of their lists
+// (positions increase): Kout and Dout, by bisection.  The deflation count goes to the status words.
+__global__ void k_count_out(Node* nodes, DcArrays A, int kcut, int* status) {
+  Node& nd = nodes[0];
+  if (threadIdx.x > 1) return;
+  const int* pos = (threadIdx.x ? A.pos_d : A.pos_r) + nd.a;
+  int lo = 0, hi = threadIdx.x ? nd.ndefl : nd.K;
+  while (lo < hi) {
+    const int md = (lo + hi) >> 1;
+    if (pos[md] < kcut) lo = md + 1;
+    else hi = md;
+  }
+  if (threadIdx.x) {
+    nd.Dout = lo;
+    status[ST_DEFLATED] = nd.ndefl;
+  } else {
+    nd.Kout = lo;
+  }
 }
 
 // U (gather order rows x Kout, ld ldu) column j: u_i = z'_i/(delta_i - lambda_j), normalised.
@@ -562,8 +743,44 @@ __global__ void k_finalize(Node* nodes, DcArrays A, double* w) {
   }
 }
 
-__global__ void k_copy_int(int n, const int* src, int* dst) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
+// The eigenvector products of all nodes of a level in one launch, for levels of short nodes: top rows
+// Qb(a.., :) = Qg(a.., top-only and mixed) U(0 .., :), bottom rows Qb(m.., :) = Qg(m.., mixed and
+// bottom-only) U(K1 .., :).  blockIdx.z = 2 node + half, 16 x 16 outputs per block, one per thread; R: the
+// type of the products and sums (FP32 in the mixed form).  On the FP64 pipe (1.7 multiply-adds per SM
+// per cycle) a level of nodes of s rows takes about n s^2 / 2 of them, spread over all SMs, where the
+// tensor-core engine takes a split and a product launch (about 35 us) for each half of each node.  The whole
+// divide and conquer (with the scans above): n = 256 4.2 -> 1.6 ms, n = 1500 12.8 -> 3.5, n = 10240 113.7 -> 53.0.
+constexpr int MT = 16, MK = 32;
+template <class R>
+__global__ void __launch_bounds__(MT * MT) k_merge_products(const Node* nodes, const double* Qg, const double* U,
+                                                            long long ldq, double* Qb) {
+  const Node& nd = nodes[blockIdx.z >> 1];
+  const int half = blockIdx.z & 1;
+  const int a = nd.a, r0 = half ? nd.m : a, nrow = half ? nd.c - nd.m : nd.m - a, Kout = nd.Kout;
+  const int i0 = blockIdx.x * MT, j0 = blockIdx.y * MT;
+  if (i0 >= nrow || j0 >= Kout) return;
+  const int k0 = half ? nd.K1 : 0, KK = half ? nd.K2 + nd.K3 : nd.K1 + nd.K2;
+  __shared__ R As[MK][MT + 1], Bs[MT][MK + 1];
+  const int tid = threadIdx.x, ti = tid % MT, tj = tid / MT;
+  const double* Aq = Qg + r0 + (long long)(a + k0) * ldq;
+  const double* Bq = U + (long long)a * ldq + k0;
+  R acc0 = 0, acc1 = 0;
+  for (int kb = 0; kb < KK; kb += MK) {
+    for (int t = tid; t < MT * MK; t += MT * MT) {
+      const int i = t % MT, k = t / MT;
+      As[k][i] = (i0 + i < nrow && kb + k < KK) ? (R)Aq[i0 + i + (long long)(kb + k) * ldq] : (R)0;
+      const int kk = t % MK, j = t / MK;
+      Bs[j][kk] = (j0 + j < Kout && kb + kk < KK) ? (R)Bq[kb + kk + (long long)(j0 + j) * ldq] : (R)0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < MK; k += 2) {
+      acc0 += As[k][ti] * Bs[tj][k];
+      acc1 += As[k + 1][ti] * Bs[tj][k + 1];
+    }
+    __syncthreads();
+  }
+  if (i0 + ti < nrow && j0 + tj < Kout) Qb[r0 + i0 + ti + (long long)(a + j0 + tj) * ldq] = (double)(acc0 + acc1);
 }
 
 // Z[:, p] = Q[:, colmap[p]] for p < k (rows 0 .. n-1).
@@ -612,69 +829,59 @@ int stedc(Sys& s, const double* d, const double* e, int k, double* w, double* Z,
   int nleaf = 1;
   while ((n + nleaf - 1) / nleaf > LEAF) nleaf *= 2;
   const unsigned eb = cdiv(n, 256) < 1024u ? cdiv(n, 256) : 1024u;
+  GEV_CUDA_TRY(cudaMemsetAsync(&s.status[ST_DEFLATED], 0, sizeof(int), st));
   GEV_COUNT(s);
   k_tear<<<eb, 256, 0, st>>>(n, nleaf, d, e, A.dwork);
-  if (nleaf > 1) {
-    GEV_COUNT(s);
-    k_tear2<<<cdiv(nleaf, 256), 256, 0, st>>>(n, nleaf, e, A.dwork);
-  }
   GEV_COUNT(s);
   k_leaf<<<nleaf, 64, 0, st>>>(n, nleaf, A.dwork, e, w, Qa, ldq, A.colmap, s.status);
   GEV_TRY(last_error());
 
+  // Levels whose nodes have at most kBatch rows run their products in one launch with everything read
+  // from the node descriptors on the device, so the host does not wait for them: n s^2 / 2 multiply-adds on the
+  // FP64 pipe (4.5e11 per second over the chip) against 2 n / s products of about 35 us: equal at s about 390
+  // for any n.
+  constexpr int kBatch = 384;
   std::vector<Node> hn;
-  int top_deflated = 0;
   for (int span = 2; span <= nleaf; span *= 2) {
     const int nnodes = nleaf / span;
     const bool top = (span == nleaf);
-    hn.assign(nnodes, Node{});
-    for (int q = 0; q < nnodes; ++q) {
-      hn[q].a = (int)(((long long)q * span * n) / nleaf);
-      hn[q].m = (int)(((long long)(q * span + span / 2) * n) / nleaf);
-      hn[q].c = (int)(((long long)(q + 1) * span * n) / nleaf);
-    }
-    GEV_CUDA_TRY(cudaMemcpyAsync(A.nodes, hn.data(), sizeof(Node) * nnodes, cudaMemcpyHostToDevice, st));
+    const int smax = (int)std::min<long long>(n, ((long long)span * n) / nleaf + 1);  // rows of a node, at most
+    const bool batch = smax <= kBatch;
     GEV_COUNT(s);
-    k_merge_prep<<<nnodes, 1024, 0, st>>>(n, A.nodes, e, w, Qa, ldq, A);
+    k_merge_prep<<<nnodes, PREP_NTH, 0, st>>>(n, nleaf, span, A.nodes, e, w, Qa, ldq, A);
     GEV_TRY(last_error());
-    GEV_CUDA_TRY(cudaMemcpyAsync(hn.data(), A.nodes, sizeof(Node) * nnodes, cudaMemcpyDeviceToHost, st));
-    GEV_CUDA_TRY(cudaStreamSynchronize(st));
-    int Kmax = 0, Tmax = 0;
-    for (auto& x : hn) {
-      Kmax = std::max(Kmax, x.K);
-      Tmax = std::max(Tmax, x.K + x.ndefl);
-    }
-    if (Kmax > 0) {
-      GEV_COUNT(s);
-      k_secular<<<dim3(cdiv(Kmax, 8), nnodes), 256, 0, st>>>(A.nodes, A, s.status);
-      GEV_COUNT(s);
-      k_zprime<<<dim3(cdiv(Kmax, 128), nnodes), 128, 0, st>>>(A.nodes, A);
-    }
+    GEV_COUNT(s);
+    k_secular<<<dim3(cdiv(smax, 8), nnodes), 256, 0, st>>>(A.nodes, A, s.status);
+    GEV_COUNT(s);
+    k_zprime<<<dim3(cdiv(smax, 8), nnodes), 256, 0, st>>>(A.nodes, A);
     const int kcut = top ? k : 0x7fffffff;
     GEV_COUNT(s);
-    k_positions<<<dim3(cdiv(Tmax, 256), nnodes), 256, 0, st>>>(A.nodes, A, kcut, s.status);
-    GEV_TRY(last_error());
+    k_positions<<<dim3(cdiv(smax, 256), nnodes), 256, 0, st>>>(A.nodes, A, kcut, s.status);
     if (top) {
       GEV_COUNT(s);
-      k_count_out<<<nnodes, 32, 0, st>>>(A.nodes, A, kcut);
-      GEV_CUDA_TRY(cudaMemcpyAsync(hn.data(), A.nodes, sizeof(Node) * nnodes, cudaMemcpyDeviceToHost, st));
-      GEV_CUDA_TRY(cudaStreamSynchronize(st));
-      top_deflated = hn[0].ndefl;
+      k_count_out<<<1, 32, 0, st>>>(A.nodes, A, kcut, s.status);
     }
-    int Koutmax = 0;
-    for (auto& x : hn) Koutmax = std::max(Koutmax, x.Kout);
-    if (Koutmax > 0) {
-      GEV_COUNT(s);
-      k_vectors<<<dim3(Koutmax, nnodes), 256, 0, st>>>(A.nodes, A, U, ldq);
-    }
-    if (Tmax > 0) {
-      GEV_COUNT(s);
-      k_gather<<<dim3(Tmax, nnodes), 256, 0, st>>>(A.nodes, A, Qa, ldq, Qg, Qb);
-    }
+    GEV_TRY(last_error());
+    GEV_COUNT(s);
+    k_vectors<<<dim3(smax, nnodes), 256, 0, st>>>(A.nodes, A, U, ldq);
+    GEV_COUNT(s);
+    k_gather<<<dim3(smax, nnodes), 256, 0, st>>>(A.nodes, A, Qa, ldq, Qg, Qb);
     GEV_TRY(last_error());
     // eigenvector update: top rows use the top-only and mixed columns, bottom rows the mixed and
     // bottom-only ones
-    for (auto& x : hn) {
+    if (batch) {
+      const dim3 grid(cdiv((smax + 1) / 2 + 1, MT), cdiv(smax, MT), 2 * nnodes);
+      GEV_COUNT(s);
+      if (s.dc_lowp) k_merge_products<float><<<grid, MT * MT, 0, st>>>(A.nodes, Qg, U, ldq, Qb);
+      else k_merge_products<double><<<grid, MT * MT, 0, st>>>(A.nodes, Qg, U, ldq, Qb);
+      GEV_TRY(last_error());
+    } else {
+      hn.resize(nnodes);
+      GEV_CUDA_TRY(cudaMemcpyAsync(hn.data(), A.nodes, sizeof(Node) * nnodes, cudaMemcpyDeviceToHost, st));
+      GEV_CUDA_TRY(cudaStreamSynchronize(st));
+    }
+    for (int q = 0; !batch && q < nnodes; ++q) {
+      const Node& x = hn[q];
       if (x.Kout == 0) continue;
       const int n1 = x.m - x.a, n2 = x.c - x.m;
       const double* Ub = U + (long long)x.a * ldq;  // column a, rows 0 .. K-1 (gather order)
@@ -698,20 +905,19 @@ int stedc(Sys& s, const double* d, const double* e, int k, double* w, double* Z,
         GEV_CUDA_TRY(cudaMemset2DAsync(Qb + x.m + (long long)x.a * ldq, ldq * 8, 0, n2 * 8, x.Kout, st));
     }
     GEV_COUNT(s);
-    k_finalize<<<dim3(cdiv(Tmax, 256), nnodes), 256, 0, st>>>(A.nodes, A, w);
+    k_finalize<<<dim3(cdiv(smax, 256), nnodes), 256, 0, st>>>(A.nodes, A, w);
     GEV_TRY(last_error());
-    GEV_COUNT(s);
-    k_copy_int<<<eb, 256, 0, st>>>(n, A.colmap2, A.colmap);
+    std::swap(A.colmap, A.colmap2);
     std::swap(Qa, Qb);
   }
   // the k lowest eigenvectors
   GEV_COUNT(s);
   k_output<<<k, 256, 0, st>>>(n, k, Qa, ldq, A.colmap, Z, ldz);
   GEV_TRY(last_error());
-  GEV_CUDA_TRY(cudaMemsetAsync(&s.status[ST_DEFLATED], 0, sizeof(int), st));
-  GEV_CUDA_TRY(cudaMemcpyAsync(&s.status[ST_DEFLATED], &top_deflated, sizeof(int), cudaMemcpyHostToDevice, st));
-  GEV_CUDA_TRY(cudaStreamSynchronize(st));
-  if (deflated) *deflated = top_deflated;
+  if (deflated) {
+    GEV_CUDA_TRY(cudaMemcpyAsync(deflated, &s.status[ST_DEFLATED], sizeof(int), cudaMemcpyDeviceToHost, st));
+    GEV_CUDA_TRY(cudaStreamSynchronize(st));
+  }
   return 0;
 }
 
