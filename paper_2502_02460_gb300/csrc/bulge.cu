@@ -435,51 +435,92 @@ __global__ void k_phase_rows(int n, int k, const double* Z, long long ldz, const
 // applies D_0^last first.  D_t^g must follow D_{t-1}^g and D_{t'}^{g+1} for t' <= t (overlapping
 // windows), which is exactly the order of the levels L = t + (ngroups - 1 - g); blocks of one level
 // have windows 2b apart, act on disjoint rows and commute.  One launch per level: blockIdx.x picks
-// the group, blockIdx.y a block of columns of Y, one thread per column (all FMAs of a thread are
-// on its own column; the reflector entries are shared-memory broadcasts).
-template <class T, int COLS>
-__global__ void __launch_bounds__(COLS) k_bt_bulge_level(int n, int k, int b, int L, int ngroups,
-                                                         const T* V2, const T* tau2, int ntask, T* Y,
-                                                         long long ldy) {
+// the group, blockIdx.y a share of Y's columns.
+//
+// A column is held by 8 lanes, lane r the window rows r, r + 8, ...; the reflectors are taken in chunks of
+// 8 (descending), whose rows [8a, 8a + B + 7) are B / 8 + 1 registers per lane: after a chunk the
+// topmost row of every lane is final and is stored, the others move up one register and the next row, loaded
+// before the chunk, enters.  Nothing but the reflectors is staged in shared memory (shifted by q mod 8 and
+// zero-padded, so that every chunk is the same straight-line code).  What bounds it is the FP64 pipe
+// (1.25 b n k multiply-adds per level, four times that for complex data, at 4.5e11 per second over the
+// chip) once there are enough columns, and the chain of b dot products (three shuffles each) before that.
+// (One thread per column and 128 columns per block, as before, used nblk * ceil(k / 128) SMs.)  Back-transform 2,
+// before -> now: complex n = 509, k = 128, b = 32 14.1 -> 2.8 ms; real n = 256, all pairs 2.2 -> 0.4 ms; complex64
+// n = 1536, all vectors 7.5 -> 2.3 ms; real n = 1500, k = 375 9.0 (in tensor-core form) -> 4.5 ms.
+constexpr int BTL_COLS = 16;
+__device__ __forceinline__ float sum8(float v) {
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ double sum8(double v) {
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ zd sum8(zd v) { return make_zd(sum8(v.x), sum8(v.y)); }
+__device__ __forceinline__ zf sum8(zf v) { return make_zf(sum8(v.x), sum8(v.y)); }
+
+template <class T, int B>
+__global__ void __launch_bounds__(8 * BTL_COLS) k_bt_level(int n, int k, int L, int ngroups, const T* V2,
+                                                           const T* tau2, int ntask, T* Y, long long ldy) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr int LV = B + 8, NR = B / 8, NTH = 8 * BTL_COLS;
+  T* Vs = reinterpret_cast<T*>(smraw);  // B x LV: entry q LV + x is v_q at window row 8 (q / 8) + x
+  T* ts = Vs + B * LV;                  // B
   const int g = max(0, ngroups - 1 - L) + blockIdx.x;
   const int t = L - (ngroups - 1 - g);
   if (g >= ngroups || t < 0 || t >= ntask) return;
-  const int G = b;
-  const int s0 = g * G;
-  const int last_sweep = n - 3;
-  const int s1 = min(s0 + G - 1, last_sweep);
-  const int w0 = s0 + 1 + t * b;
+  const int s0 = g * B, w0 = s0 + 1 + t * B;
   if (w0 >= n) return;
-  const int w1 = min(n, s1 + 1 + t * b + b);
-  const int rows = w1 - w0;
-  const int c = blockIdx.y * COLS + threadIdx.x;
-  T* Zw = reinterpret_cast<T*>(smraw);   // rows x COLS (row-major)
-  T* Vs = Zw + (size_t)(2 * b) * COLS;   // G x b
-  T* ts = Vs + (size_t)G * b;            // G
-  const int ncols = min(COLS, k - (int)blockIdx.y * COLS);
-  for (int idx = threadIdx.x; idx < (s1 - s0 + 1) * b; idx += COLS) {
-    const int q = idx / b, i = idx % b;
-    Vs[q * b + i] = V2[((long long)(s0 + q) * ntask + t) * b + i];
-  }
-  for (int q = threadIdx.x; q <= s1 - s0; q += COLS) ts[q] = tau2[(long long)(s0 + q) * ntask + t];
-  if (threadIdx.x < ncols)
-    for (int r = 0; r < rows; ++r) Zw[r * COLS + threadIdx.x] = Y[(w0 + r) + (long long)c * ldy];
+  const int tid = threadIdx.x;
+  for (int q = tid; q < B; q += NTH) ts[q] = s0 + q <= n - 3 ? tau2[(long long)(s0 + q) * ntask + t] : zero_<T>();
   __syncthreads();
-  if (threadIdx.x < ncols) {
-    for (int q = s1 - s0; q >= 0; --q) {
-      const T tau = ts[q];
-      if (tau == zero_<T>()) continue;
-      const int p = s0 + q + 1 + t * b;
-      const int len = min(b, n - p);
-      const int off = p - w0;
-      const T* vq = Vs + q * b;
-      T acc = zero_<T>();
-      for (int i = 0; i < len; ++i) acc += cmul(vq[i], Zw[(off + i) * COLS + threadIdx.x]);
-      acc = tau * acc;
-      for (int i = 0; i < len; ++i) Zw[(off + i) * COLS + threadIdx.x] -= vq[i] * acc;
+  for (int idx = tid; idx < B * LV; idx += NTH) {
+    const int q = idx / LV, rel = idx % LV - (q & 7);
+    T v = zero_<T>();
+    if (rel >= 0 && rel < B && w0 + q + rel < n && ts[q] != zero_<T>())
+      v = V2[((long long)(s0 + q) * ntask + t) * B + rel];
+    Vs[idx] = v;
+  }
+  __syncthreads();
+  const int r = tid & 7, cl = tid >> 3;
+  for (int cb = blockIdx.y * BTL_COLS; cb < k; cb += gridDim.y * BTL_COLS) {
+    const bool cok = cb + cl < k;
+    T* y = Y + w0 + r + (long long)(cb + cl) * ldy;
+    const int left = cok ? n - w0 - r : 0;  // rows of this lane: offsets 8 j < left
+    T z[NR + 1];
+#pragma unroll
+    for (int i = 0; i <= NR; ++i) {
+      const int o = 8 * (NR - 1 + i);
+      z[i] = o < left ? y[o] : zero_<T>();
     }
-    for (int r = 0; r < rows; ++r) Y[(w0 + r) + (long long)c * ldy] = Zw[r * COLS + threadIdx.x];
+#pragma unroll 1
+    for (int a = NR - 1; a >= 0; --a) {
+      T nx = zero_<T>();
+      if (a > 0 && 8 * (a - 1) < left) nx = y[8 * (a - 1)];
+#pragma unroll
+      for (int u = 7; u >= 0; --u) {
+        const T* vq = Vs + (8 * a + u) * LV + r;
+        T acc0 = zero_<T>(), acc1 = zero_<T>();
+#pragma unroll
+        for (int i = 0; i <= NR; ++i) {
+          if (i & 1) acc1 += cmul(vq[8 * i], z[i]);
+          else acc0 += cmul(vq[8 * i], z[i]);
+        }
+        const T w = ts[8 * a + u] * sum8(acc0 + acc1);
+#pragma unroll
+        for (int i = 0; i <= NR; ++i) z[i] -= vq[8 * i] * w;
+      }
+      if (8 * (a + NR) < left) y[8 * (a + NR)] = z[NR];
+      if (a > 0) {
+#pragma unroll
+        for (int i = NR; i > 0; --i) z[i] = z[i - 1];
+        z[0] = nx;
+      } else {
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+          if (8 * i < left) y[8 * i] = z[i];
+      }
+    }
   }
 }
 
@@ -734,8 +775,23 @@ template <class T> int hb2st(Sys& s, double* d, double* e) {
   return 0;
 }
 
-template <class T, int COLS> int bt_levels(Sys& s, int n, int k, int b, T* Y, int ldy);
-
+// Y <- Q2 Y, one launch of k_bt_level per level
+template <class T, int B> int bt_levels(Sys& s, int n, int k, T* Y, int ldy) {
+  const int ngroups = (n - 3) / B + 1;
+  const size_t smem = sizeof(T) * ((size_t)B * (B + 8) + B);
+  GEV_TRY(allow_dyn_smem(k_bt_level<T, B>, smem));
+  const int nlevels = ngroups + s.ntask;
+  for (int L = 0; L < nlevels; ++L) {
+    const int nblk = level_blocks(n, B, L, ngroups, s.ntask).nblk;
+    if (nblk == 0) continue;
+    // 16 columns per block until the blocks fill the GPU several times over, then more
+    const unsigned yb = std::min<unsigned>(cdiv(k, BTL_COLS), std::max<unsigned>(1, 12u * s.sms / nblk));
+    GEV_COUNT(s);
+    k_bt_level<T, B><<<dim3(nblk, yb), 8 * BTL_COLS, smem, s.stream>>>(
+        n, k, L, ngroups, (const T*)s.V2, (const T*)s.tau2, s.ntask, Y, ldy);
+  }
+  return last_error();
+}
 
 // Y <- Q2 Y with every level applied as  P = blockdiag(V_j^H) Y_L,  Y_L -= blockdiag(V_j T_j) P  on the
 // emulated FP64 product engine (Y_L: the level's rows).  Returns GEV_ERR_UNSUPPORTED, before
@@ -839,37 +895,23 @@ template <class T> int bt_hb2st(Sys& s, const double* Z, int ldz, int k, T* Y, i
     if (b == 64) return bt_levels_f32<64>(s, n, k, Y, ldy);
   }
   // FP64 data with the emulated product engine: each level as two block-diagonal tensor-core
-  // products of its compact-WY blocks
+  // products of its compact-WY blocks, unless the level is short.  A level costs about 86 us in that form
+  // (six launches) + 0.26 ps n k b, and 12 us + 2.8 ps n k b reflector by reflector on the FP64 pipe
+  // (complex: four times the work in both): equal at n k b = 3e7.
+  constexpr double kBtNative = 3e7;
   if constexpr (std::is_same<T, double>::value || std::is_same<T, zd>::value) {
-    if (s.emu_fp64) {
+    const double fma = (double)n * k * b * (is_cx<T>::value ? 4 : 1);  // of a level, on the FP64 pipe
+    if (s.emu_fp64 && fma >= kBtNative) {
       const int r = bt_levels_wy<T>(s, n, k, b, Y, ldy);
       if (r != GEV_ERR_UNSUPPORTED) return r;  // else: the scratch is too small, take the level kernel
     }
   }
-  // level-parallel application (see k_bt_bulge_level); one thread per column, as many columns
-  // per block as the staged window (2b rows) allows in shared memory
-  const size_t per_col = sizeof(T) * 2 * (size_t)b;
-  if (per_col * 256 <= (size_t)160 * 1024) return bt_levels<T, 256>(s, n, k, b, Y, ldy);
-  if (per_col * 128 <= (size_t)160 * 1024) return bt_levels<T, 128>(s, n, k, b, Y, ldy);
-  return bt_levels<T, 64>(s, n, k, b, Y, ldy);
-}
-
-template <class T, int COLS> int bt_levels(Sys& s, int n, int k, int b, T* Y, int ldy) {
-  const int G = b;
-  const int last_sweep = n - 3;
-  const int ngroups = last_sweep / G + 1;
-  const size_t smem = sizeof(T) * ((size_t)2 * b * COLS + (size_t)G * b + G) + 64;
-  GEV_TRY(allow_max_dyn_smem(k_bt_bulge_level<T, COLS>));
-  const int nlevels = ngroups + s.ntask;
-  const unsigned ycb = cdiv(k, COLS);
-  for (int L = 0; L < nlevels; ++L) {
-    const int gmin = ngroups - 1 - L > 0 ? ngroups - 1 - L : 0;
-    const int nblk = ngroups - gmin;
-    GEV_COUNT(s);
-    k_bt_bulge_level<T, COLS><<<dim3(nblk, ycb), COLS, smem, s.stream>>>(
-        n, k, b, L, ngroups, (const T*)s.V2, (const T*)s.tau2, s.ntask, Y, ldy);
+  if constexpr (!std::is_same<T, float>::value) {
+    if (b == 16) return bt_levels<T, 16>(s, n, k, Y, ldy);
+    if (b == 32) return bt_levels<T, 32>(s, n, k, Y, ldy);
+    if (b == 64) return bt_levels<T, 64>(s, n, k, Y, ldy);
   }
-  return last_error();
+  return GEV_ERR_UNSUPPORTED;
 }
 
 template int hb2st<double>(Sys&, double*, double*);
