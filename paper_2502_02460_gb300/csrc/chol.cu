@@ -73,91 +73,190 @@ __device__ void inv_lower_blocked(int jb, const T* L, T* X, T* tmp) {
   }
 }
 
-// Factor the jb x jb diagonal block in place (lower) and write its inverse to Dinv, blocked by SB:
-// for each SB-column sub-panel, one warp factors the SB x SB diagonal block in registers (lane i holds
-// row i; the pivot column travels by shuffles), all threads solve the rows below against it and update
-// the trailing block.  A non-positive pivot records its index (first one, atomicCAS) and stops.
+// 1 / d for a positive d: the hardware's 20-bit reciprocal and two Newton-Raphson steps (y += y (1 - d y)),
+// within an ulp of the quotient; outside the exponents where the steps are safe, the division
+__device__ __forceinline__ double recip(double d) {
+  const int e = (__double2hiint(d) >> 20) & 0x7FF;
+  if (e < 24 || e > 2020) return 1.0 / d;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(d));
+  y = fma(y, fma(-d, y, 1.0), y);
+  return fma(y, fma(-d, y, 1.0), y);
+}
+
+// Factor the jb x jb diagonal block (lower) and invert the factor, blocked by SB, on 16 warps.  Step kb:
+//   1. warps 0 - 7 factor and invert the SB x SB diagonal block, one entry (i, j), j <= i, per thread:
+//      before pivot j the thread holds a_ij of the trailing matrix, after it x_ij of the inverse of the
+//      unit lower factor (a = L^ D L^^H, no square root in the chain of pivots).  Pivot p costs a thread one
+//      scaled row factor l_ip = a_ip / d_p and one multiply-add, a barrier and, in the one warp that owns
+//      the next pivot, its reciprocal; column p of a and row p of x travel through shared memory.  Meanwhile
+//      warps 8 - 15 finish the trailing update of the step before (beyond this diagonal block) and form
+//      S = L(kb.., 0:kb) X(0:kb, 0:kb) for this block row of the inverse;
+//   2. all: L21 = A21 X11^H with the inverted diagonal block, and X(kb.., 0:kb) = -X11 S;
+//   3. all: the next diagonal block takes its trailing update.
+// FP64 bounds it: 2 jb^3 / 6 multiply-adds at 1.7 per cycle on one SM are 28 us for 64 real rows (113 us
+// complex).  One warp gets a quarter of that rate at most (a warp instruction occupies its scheduler's FP64
+// unit for about 75 cycles), so a pivot chain in one warp's registers took 36 us for each 16 rows: 150 us for the
+// block, 70 us now.
+// L goes to A (when wanted) and X = L^{-1} to Xout, both with zeros above the diagonal.  A non-positive
+// pivot records its index (first one, atomicCAS) and stops; nothing is written then.
+constexpr int PD_NT = 512, PD_G = 256;  // threads in all, threads of the diagonal block's group
 template <class T>
-__global__ void k_potrf_diag(int jb, T* A, long long lda, T* Dinv, long long ldd, int* status, int j0) {
+__global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long lda, int want_l, T* Xout, long long ldx,
+                                                      int* status, int j0) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* L = reinterpret_cast<T*>(smraw);
   T* X = L + NBMAX * LDS;
-  T* tmp = X + NBMAX * LDS;
+  T* S = X + NBMAX * LDS;  // SB x kb
   __shared__ int fail;
+  __shared__ T s_col[2][SB], s_row[2][SB];
+  __shared__ double s_rinv[2], s_d[SB], s_rs[SB];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) fail = 0;
-  for (int t = tid; t < jb * jb; t += blockDim.x) {
+  for (int t = tid; t < jb * jb; t += PD_NT) {
     int i = t % jb, j = t / jb;
     L[i + j * LDS] = (i >= j) ? A[i + j * lda] : zero_<T>();
+    X[i + j * LDS] = zero_<T>();
   }
   __syncthreads();
   for (int kb = 0; kb < jb; kb += SB) {
-    const int bs = min(SB, jb - kb);
-    // (a) the diagonal block, by warp 0
-    if (warp == 0) {
-      T r[SB];
-      const int i = lane;
-#pragma unroll
-      for (int j = 0; j < SB; ++j) r[j] = (i < bs && j <= i) ? L[(kb + i) + (kb + j) * LDS] : zero_<T>();
-      int bad = -1;
-#pragma unroll
-      for (int p = 0; p < SB; ++p) {
-        if (p < bs && bad < 0) {  // uniform over the warp
-          const double dpp = re_(shfl_(r[p], p));
-          if (!(dpp > 0.0)) {
-            bad = p;
-          } else {
-            const double piv = sqrt(dpp);
-            if (i == p) r[p] = from_re<T>(piv);
-            else if (i > p) r[p] = (1.0 / piv) * r[p];
-#pragma unroll
-            for (int j = p + 1; j < SB; ++j) {
-              const T ljp = shfl_(r[p], j);
-              if (j < bs && i >= j && i < bs) r[j] -= mulc(r[p], ljp);
-            }
+    const int bs = min(SB, jb - kb), r0 = kb + bs, nr = jb - r0;
+    if (tid < PD_G) {
+      const int i = tid % SB, j = tid / SB;  // warp w: columns 2w, 2w + 1
+      const bool live = i < bs && j <= i;
+      T a = live ? L[(kb + i) + (kb + j) * LDS] : zero_<T>();
+      T x = from_re<T>(i == j ? 1.0 : 0.0);
+      // what pivot q needs: column q of a, row q of x, 1 / d_q
+      auto publish = [&](int q) {
+        if (j == q && i >= q) s_col[q & 1][i] = a;
+        if (i == q && j <= q) s_row[q & 1][j] = x;
+        if (warp == q / 2) {  // (uniform) the warp that holds (q, q)
+          const double dq = re_(shfl_(a, (q & 1) * SB + q));
+          const double ri = dq > 0.0 ? recip(dq) : 0.0;
+          if (lane == 0) {
+            s_rinv[q & 1] = ri;
+            s_d[q] = dq;
           }
         }
-      }
-      if (bad >= 0) {
-        if (lane == 0) {
-          fail = 1;
-          atomicCAS(&status[ST_NOT_SPD], 0, j0 + kb + bad + 1);
+      };
+      publish(0);
+      for (int p = 0; p < bs; ++p) {
+        asm volatile("bar.sync 1, %0;\n" ::"n"(PD_G) : "memory");
+        if (!(s_d[p] > 0.0)) {
+          if (tid == 0) {
+            fail = 1;
+            atomicCAS(&status[ST_NOT_SPD], 0, j0 + kb + p + 1);
+          }
+          break;  // uniform over the group
         }
-      } else {
+        if (live && i > p) {
+          const T li = s_rinv[p & 1] * s_col[p & 1][i];
+          const bool fac = j > p;
+          const T m = fac ? conj_(s_col[p & 1][j]) : s_row[p & 1][j];
+          const T cur = (fac ? a : x) - li * m;
+          if (fac) a = cur;
+          else x = cur;
+        }
+        if (p + 1 < bs) publish(p + 1);
+      }
+      asm volatile("bar.sync 1, %0;\n" ::"n"(PD_G) : "memory");
+      if (tid < bs) s_rs[tid] = s_d[tid] > 0.0 ? rsqrt(s_d[tid]) : 0.0;
+      asm volatile("bar.sync 1, %0;\n" ::"n"(PD_G) : "memory");
+      if (live) {  // L = L^ D^{1/2} with l^_ij = a_ij / d_j, X = D^{-1/2} x
+        L[(kb + i) + (kb + j) * LDS] = i == j ? from_re<T>(sqrt(s_d[i])) : s_rs[j] * a;
+        X[(kb + i) + (kb + j) * LDS] = s_rs[i] * x;
+      }
+    } else if (kb > 0) {
+      // trailing update of the previous step: rows >= r0, columns kb .. row
+      const int pc = kb - SB, rect = nr * bs, all = rect + nr * (nr + 1) / 2;
+      for (int t = tid - PD_G; t < all; t += PD_NT - PD_G) {
+        int i, j;
+        if (t < rect) {
+          i = t % nr;
+          j = t / nr - bs;
+        } else {
+          const int u = t - rect;
+          i = (int)((__fsqrt_rn(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
+          while (i * (i + 1) / 2 > u) --i;
+          while ((i + 1) * (i + 2) / 2 <= u) ++i;
+          j = u - i * (i + 1) / 2;
+        }
+        i += r0;
+        j += r0;
+        T acc = zero_<T>(), acc1 = zero_<T>();
 #pragma unroll
-        for (int j = 0; j < SB; ++j)
-          if (i < bs && j <= i) L[(kb + i) + (kb + j) * LDS] = r[j];
+        for (int p = 0; p < SB; p += 2) {
+          acc += mulc(L[i + (pc + p) * LDS], L[j + (pc + p) * LDS]);
+          acc1 += mulc(L[i + (pc + p + 1) * LDS], L[j + (pc + p + 1) * LDS]);
+        }
+        L[i + j * LDS] -= acc + acc1;
+      }
+      // S = L(kb .. r0 - 1, 0:kb) X(0:kb, 0:kb)
+      for (int t = tid - PD_G; t < SB * kb; t += PD_NT - PD_G) {
+        const int q = t % SB, c = t / SB;
+        if (q < bs) {
+          T acc = zero_<T>(), acc1 = zero_<T>();
+          int k = c;
+          for (; k + 1 < kb; k += 2) {
+            acc += L[(kb + q) + k * LDS] * X[k + c * LDS];
+            acc1 += L[(kb + q) + (k + 1) * LDS] * X[(k + 1) + c * LDS];
+          }
+          if (k < kb) acc += L[(kb + q) + k * LDS] * X[k + c * LDS];
+          S[t] = acc + acc1;
+        }
       }
     }
     __syncthreads();
     if (fail) return;
-    const int r0 = kb + bs, nr = jb - r0;
-    if (nr <= 0) break;
-    // (b) rows below: L21 = A21 L11^{-H}, one thread per row
-    for (int i = r0 + tid; i < jb; i += blockDim.x) {
-      for (int p = 0; p < bs; ++p) {
-        T x = L[i + (kb + p) * LDS];
-        for (int q = 0; q < p; ++q) x -= mulc(L[i + (kb + q) * LDS], L[(kb + p) + (kb + q) * LDS]);
-        L[i + (kb + p) * LDS] = (1.0 / re_(L[(kb + p) + (kb + p) * LDS])) * x;
+    // L21 = A21 X11^H into registers, X(kb.., 0:kb) = -X11 S
+    constexpr int NO = ((NBMAX - SB) * SB + PD_NT - 1) / PD_NT;
+    T o[NO];
+#pragma unroll
+    for (int u = 0; u < NO; ++u) {
+      const int t = tid + u * PD_NT;
+      o[u] = zero_<T>();
+      if (t < nr * SB) {
+        const int i = r0 + t % nr, p = t / nr;
+        for (int q = 0; q <= p; ++q) o[u] += mulc(L[i + (kb + q) * LDS], X[(kb + p) + (kb + q) * LDS]);
       }
     }
-    __syncthreads();
-    // (c) trailing update A22 -= L21 L21^H (lower triangle)
-    for (int t = tid; t < nr * nr; t += blockDim.x) {
-      const int i = r0 + t % nr, j = r0 + t / nr;
-      if (j <= i) {
+    for (int t = tid; t < SB * kb; t += PD_NT) {
+      const int q = t % SB, c = t / SB;
+      if (q < bs) {
         T acc = zero_<T>();
-        for (int p = 0; p < bs; ++p) acc += mulc(L[i + (kb + p) * LDS], L[j + (kb + p) * LDS]);
-        L[i + j * LDS] -= acc;
+        for (int l = 0; l <= q; ++l) acc += X[(kb + q) + (kb + l) * LDS] * S[l + c * SB];
+        X[(kb + q) + c * LDS] = -acc;
+      }
+    }
+    if (nr <= 0) break;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < NO; ++u) {
+      const int t = tid + u * PD_NT;
+      if (t < nr * SB) L[(r0 + t % nr) + (kb + t / nr) * LDS] = o[u];
+    }
+    __syncthreads();
+    // the next diagonal block
+    const int bn = min(SB, nr);
+    if (tid < SB * SB) {
+      const int i = tid % SB, j = tid / SB;
+      if (i < bn && j <= i) {
+        T acc = zero_<T>(), acc1 = zero_<T>();
+#pragma unroll
+        for (int p = 0; p < SB; p += 2) {
+          acc += mulc(L[(r0 + i) + (kb + p) * LDS], L[(r0 + j) + (kb + p) * LDS]);
+          acc1 += mulc(L[(r0 + i) + (kb + p + 1) * LDS], L[(r0 + j) + (kb + p + 1) * LDS]);
+        }
+        L[(r0 + i) + (r0 + j) * LDS] -= acc + acc1;
       }
     }
     __syncthreads();
   }
-  inv_lower_blocked(jb, L, X, tmp);
-  for (int t = tid; t < jb * jb; t += blockDim.x) {
+  __syncthreads();
+  for (int t = tid; t < jb * jb; t += PD_NT) {
     int i = t % jb, j = t / jb;
-    A[i + j * lda] = (i >= j) ? L[i + j * LDS] : zero_<T>();
-    Dinv[i + j * ldd] = X[i + j * LDS];
+    if (want_l) A[i + j * lda] = L[i + j * LDS];
+    Xout[i + j * ldx] = X[i + j * LDS];
   }
 }
 
@@ -201,7 +300,7 @@ template <class T> int potrf(Sys& s, T* A, int lda) {
     const int jb = nb < n - j ? nb : n - j;
     T* Ajj = A + j + (long long)j * lda;
     GEV_COUNT(s);
-    k_potrf_diag<T><<<1, 256, diag_smem<T>(), s.stream>>>(jb, Ajj, lda, Dinv, nb, s.status, j);
+    k_potrf_diag<T><<<1, PD_NT, diag_smem<T>(), s.stream>>>(jb, Ajj, lda, 1, Dinv, nb, s.status, j);
     GEV_TRY(last_error());
     const int m = n - j - jb;
     if (m <= 0) break;
@@ -272,8 +371,7 @@ template <class T> void potrf_inv_rec(Sys& s, T* A, int lda, int o, int sz, T* W
   T* Aoo = A + o + (long long)o * lda;
   if (sz <= nb) {
     GEV_COUNT(s);
-    k_potrf_diag<T><<<1, 256, diag_smem<T>(), s.stream>>>(sz, Aoo, lda, (T*)s.dinv, nb, s.status, o);
-    copy2d<T>(s, sz, sz, (T*)s.dinv, nb, Aoo, lda);
+    k_potrf_diag<T><<<1, PD_NT, diag_smem<T>(), s.stream>>>(sz, Aoo, lda, 0, Aoo, lda, s.status, o);
     return;
   }
   int n1 = (sz / 2 + nb - 1) / nb * nb;
