@@ -175,6 +175,9 @@ template <class T> struct GemmP {
 struct Sys;
 
 template <class T> void gemm(Sys& s, GemmP<T> p);
+// whether gemm() takes the FP64 pipe for this product of an emulating handle (gemm.cu)
+template <class T> bool gemm_on_fp64_pipe(const Sys& s, const GemmP<T>& p);
+template <> bool gemm_on_fp64_pipe<float>(const Sys&, const GemmP<float>&);
 // FP32 SIMT GEMM (gemm32.cu): inputs TI (float or double, converted on load), output TO.
 template <class TI, class TO> void gemm32(Sys& s, const GemmP<TI>& p, TO* C, float alpha, float beta);
 // FP32 GEMM from BF16 split products on tcgen05 (tc_gemm.cu); false when s.ozws is too small
@@ -250,6 +253,7 @@ struct Sys {
   void* bandtmp = nullptr;  // complex mixed form: FP64 copy of the band during its conversion
   void* btg = nullptr;      // back-transform 1: T, Gram blocks and a block column of a 4-panel group (36 b^2)
   int ldband = 0;
+  int* tile_ctr = nullptr;  // arrival counters of split short products (gemm.cu), zero between launches
   void* V2 = nullptr;     // bulge-chasing reflectors, b x (n * ntask)
   void* tau2 = nullptr;   // (n * ntask)
   int ntask = 0;          // max tasks per sweep

@@ -202,6 +202,90 @@ __global__ void splitk_reduce(GemmP<T> p) {
   }
 }
 
+// Short products on the FP64 pipe: 16 x 16 outputs per block, one per thread, K shared by gridDim.z blocks
+// when the output is small; the last block of a tile to arrive (a counter per tile, left at zero) adds
+// their sums in a fixed order, so the result does not depend on timing.
+// The pipe (1.7 multiply-adds per SM per cycle) bounds it as soon as every SM has a block: 5 us + 2.2 us
+// per million multiply-adds.  One SM alone needs 76 us for 64 x 64 x 64, hence the small tiles.  Measured: 10.4 us
+// on average for the 294 short products of a real n = 1500 solve, which took 35 us each on the tensor cores.
+constexpr int SM_T = 16, SM_K = 32, SM_MAXT = 1024;
+template <class T>
+__global__ void __launch_bounds__(SM_T * SM_T) gemm_small_kernel(GemmP<T> p, int* ctr) {
+  constexpr int PER = SM_K / SM_T;  // elements of each operand staged per thread
+  __shared__ T As[SM_K][SM_T + 1], Bs[SM_T][SM_K + 1];
+  __shared__ int s_last;
+  const int m0 = blockIdx.x * SM_T, n0 = blockIdx.y * SM_T, tid = threadIdx.x;
+  if (p.c_lower && n0 > m0 + SM_T - 1) return;
+  int kb = 0, ke = p.K;
+  if (p.tri_a == 1) ke = min(ke, m0 + SM_T);
+  else if (p.tri_a == 2) kb = max(kb, m0);
+  if (p.tri_b == 1) kb = max(kb, n0);
+  else if (p.tri_b == 2) ke = min(ke, n0 + SM_T);
+  if (p.ksplit > 1) {
+    const int len = max(0, ke - kb), z = blockIdx.z, k0 = kb;
+    kb = k0 + (int)((long long)len * z / p.ksplit);
+    ke = k0 + (int)((long long)len * (z + 1) / p.ksplit);
+  }
+  T ra[PER], rb[PER];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int e = tid + u * SM_T * SM_T;
+      ra[u] = p.ta == 0 ? load_a(p, m0 + e % SM_T, k0 + e / SM_T, kb, ke) : load_a(p, m0 + e / SM_K, k0 + e % SM_K, kb, ke);
+      rb[u] = p.tb == 0 ? load_b(p, k0 + e % SM_K, n0 + e / SM_K, kb, ke) : load_b(p, k0 + e / SM_T, n0 + e % SM_T, kb, ke);
+    }
+  };
+  const int ti = tid % SM_T, tj = tid / SM_T;
+  T acc = zero_<T>(), acc1 = zero_<T>();
+  if (kb < ke) fetch(kb);
+  for (int k0 = kb; k0 < ke; k0 += SM_K) {
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int e = tid + u * SM_T * SM_T;
+      if (p.ta == 0) As[e / SM_T][e % SM_T] = ra[u];
+      else As[e % SM_K][e / SM_K] = ra[u];
+      if (p.tb == 0) Bs[e / SM_K][e % SM_K] = rb[u];
+      else Bs[e % SM_T][e / SM_T] = rb[u];
+    }
+    __syncthreads();
+    if (k0 + SM_K < ke) fetch(k0 + SM_K);
+    const int kn = min(SM_K, ke - k0);
+    if (kn == SM_K) {
+#pragma unroll 8
+      for (int k = 0; k < SM_K; k += 2) {
+        acc += As[k][ti] * Bs[tj][k];
+        acc1 += As[k + 1][ti] * Bs[tj][k + 1];
+      }
+    } else {
+      for (int k = 0; k < kn; ++k) acc += As[k][ti] * Bs[tj][k];
+    }
+    __syncthreads();
+  }
+  acc += acc1;
+  const int gi = m0 + ti, gj = n0 + tj;
+  if (p.ksplit > 1) {
+    const int tile = blockIdx.x + gridDim.x * blockIdx.y;
+    const size_t zs = (size_t)gridDim.x * gridDim.y * SM_T * SM_T;
+    T* w = p.ws + (size_t)tile * SM_T * SM_T + tid;
+    stcg_(&w[blockIdx.z * zs], acc);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&ctr[tile], 1) == p.ksplit - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    acc = zero_<T>();
+#pragma unroll 8
+    for (int z = 0; z < p.ksplit; ++z) acc += ldcg_(&w[z * zs]);
+    if (tid == 0) ctr[tile] = 0;
+  }
+  if (gi >= p.M || gj >= p.N || (p.c_lower && gi < gj)) return;
+  T* c = &p.C[gi + gj * p.ldc];
+  T out = p.alpha * acc;
+  if (p.beta != zero_<T>()) out += p.beta * (*c);
+  *c = out;
+}
+
 // sum over j = 0..J of max(0, min(ah, bh(j)) - max(al, bl(j))): the multiply-adds of one output row
 // (bl/bh: the k range allowed by the zero pattern of op(B) in column j).
 long double row_fmas(long long al, long long ah, int tri_b, long long J) {
@@ -234,7 +318,30 @@ template <class T> double algorithmic_flops(const GemmP<T>& p) {
   return (double)(fma * (is_cx<T>::value ? 8.0L : 2.0L));
 }
 
+template <class T> void gemm_small(Sys& s, GemmP<T> p) {
+  const dim3 t(cdiv(p.M, SM_T), cdiv(p.N, SM_T), 1);
+  const int tiles = (int)(t.x * t.y);
+  int ks = 1;
+  if (tiles <= s.sms && p.K >= 96) ks = std::max(1, std::min({2 * s.sms / tiles, p.K / 32, 64}));
+  while (ks > 1 && (size_t)ks * tiles * SM_T * SM_T * sizeof(T) > s.splitws_bytes) --ks;
+  p.ksplit = ks;
+  p.ws = (T*)s.splitws;
+  GEV_COUNT(s);
+  gemm_small_kernel<T><<<dim3(t.x, t.y, ks), SM_T * SM_T, 0, s.stream>>>(p, s.tile_ctr);
+}
+
 }  // namespace
+
+// A product on the tensor cores takes a split launch and a product launch whatever its size, about 35 us
+// together; the FP64 pipe does 1.2e7 multiply-adds in that time.  Only for handles with emulated products
+// (a native one uses its DMMA kernel throughout) and with the tile counters of a workspace.
+template <class T> bool gemm_on_fp64_pipe(const Sys& s, const GemmP<T>& p) {
+  constexpr double kFma = 1.2e7;
+  return s.emu_fp64 && s.tile_ctr && (double)p.M * p.N * p.K * (is_cx<T>::value ? 4.0 : 1.0) <= kFma;
+}
+template <> bool gemm_on_fp64_pipe<float>(const Sys&, const GemmP<float>&) { return true; }
+template bool gemm_on_fp64_pipe<double>(const Sys&, const GemmP<double>&);
+template bool gemm_on_fp64_pipe<zd>(const Sys&, const GemmP<zd>&);
 
 template <class T> void gemm(Sys& s, GemmP<T> p) {
   if (p.M <= 0 || p.N <= 0) return;
@@ -259,7 +366,10 @@ template <class T> void gemm(Sys& s, GemmP<T> p) {
     cudaEventRecord(ev0, s.stream);
   }
   bool emulated = false;
-  if constexpr (!is_cx<T>::value) {
+  if (gemm_on_fp64_pipe(s, p)) {
+    gemm_small<T>(s, p);
+    emulated = true;
+  } else if constexpr (!is_cx<T>::value) {
     if (s.emu_fp64) {  // FP64 product from BF16 digit planes on the tensor cores
       gemm_f64_emulated(s, p);
       emulated = true;

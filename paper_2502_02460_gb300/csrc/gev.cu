@@ -19,7 +19,7 @@ namespace {
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Layout {
-  size_t off[32];
+  size_t off[40];
   int cnt = 0;
   size_t total = 0;
   size_t add(size_t bytes) {
@@ -81,7 +81,9 @@ size_t carve(Sys& s, char* base) {
   size_t obt = L.add(mixed && s.dtype == GEV_C128 ? (size_t)ldband * (n + 2 * b) * es : 8);
   // back-transform 1 groups of four panels: the group's T, Gram blocks and one block column
   size_t obtg = L.add(36 * b * b * es);
+  size_t octr = L.add(1024 * sizeof(int));
   if (base) {
+    s.tile_ctr = (int*)(base + octr);
     s.A = base + oA; s.X = base + oX; s.W1 = base + oW1; s.V1 = base + oV1; s.T1 = base + oT1;
     s.dinv = base + odinv; s.Pn = base + oPn; s.small = base + osmall;
     s.splitws = base + osplit; s.splitws_bytes = split;
@@ -213,6 +215,7 @@ int gev_setup(gev_sys** out, int n, int dtype, const gev_opts* opts) {
   }
   for (int i = 0; i < 2 * GEV_NSTEPS + 2; ++i) cudaEventCreate(&s.ev[i]);
   if (cudaMemsetAsync(s.status, 0, sizeof(int) * ST_COUNT, s.stream) != cudaSuccess ||
+      cudaMemsetAsync(s.tile_ctr, 0, 1024 * sizeof(int), s.stream) != cudaSuccess ||
       cudaStreamSynchronize(s.stream) != cudaSuccess) {
     gev_free(h);
     return GEV_ERR_CUDA;
