@@ -42,16 +42,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 __device__ __forceinline__ zf warp_sum(zf v) { return make_zf(warp_sum(v.x), warp_sum(v.y)); }
 
-// progress flags between blocks: release store and acquire load at GPU scope
-__device__ __forceinline__ void st_release(int* p, int v) {
-  asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
-}
-__device__ __forceinline__ int ld_acquire(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
 // Bounded acquire-wait of one warp until *flag >= target; false on timeout / abort.
 __device__ __forceinline__ bool warp_wait_ge(const int* flag, int target, int* status, int* abort_flag, int site) {
   int good = 1;
@@ -75,38 +65,6 @@ __device__ __forceinline__ bool warp_wait_ge(const int* flag, int target, int* s
 
 __device__ __forceinline__ void bar_sync_n(int id, int n) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive_n(int id, int n) { asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(n) : "memory"); }
-
-// 1 / sqrt and the Householder scalars of alpha = x_0 and xn = sum_{i>0} |x_i|^2 (not both trivial):
-// with s = sign(Re alpha), r = 1 / ||x||:  beta = -s ||x||,  tau = 1 - alpha / beta = 1 + s r alpha,
-// scale = 1 / (alpha - beta): one reciprocal square root and one division, no other long FP64 chain
-__device__ __forceinline__ void house(double alpha, double xn, double& tau, double& beta, double& scale) {
-  const double q = alpha * alpha + xn, r = rsqrt(q), nrm = q * r;
-  beta = alpha >= 0.0 ? -nrm : nrm;
-  tau = 1.0 + fabs(alpha) * r;
-  scale = 1.0 / (alpha - beta);
-}
-__device__ __forceinline__ void house(float alpha, float xn, float& tau, float& beta, float& scale) {
-  const float nrm = sqrtf(alpha * alpha + xn);
-  beta = alpha >= 0.f ? -nrm : nrm;
-  tau = (beta - alpha) / beta;
-  scale = 1.f / (alpha - beta);
-}
-__device__ __forceinline__ void house(zd alpha, double xn, zd& tau, zd& beta, zd& scale) {
-  const double q = abs2_(alpha) + xn, r = rsqrt(q), nrm = q * r;
-  const double s = alpha.x >= 0.0 ? 1.0 : -1.0;
-  const zd d = make_zd(alpha.x + s * nrm, alpha.y);
-  const double g = 1.0 / abs2_(d);
-  beta = make_zd(-s * nrm, 0.0);
-  tau = make_zd(1.0 + fabs(alpha.x) * r, s * r * alpha.y);
-  scale = make_zd(g * d.x, -g * d.y);
-}
-__device__ __forceinline__ void house(zf alpha, float xn, zf& tau, zf& beta, zf& scale) {
-  const float nrm = sqrtf(abs2_(alpha) + xn), s = alpha.x >= 0.f ? 1.f : -1.f;
-  const zf bt = make_zf(-s * nrm, 0.f);
-  beta = bt;
-  tau = div_(bt - alpha, bt);
-  scale = div_(make_zf(1.f, 0.f), alpha - bt);
-}
 
 // Band -> tridiagonal by bulge chasing (one sweep per block at a time).  Task t of sweep s
 // annihilates the column below the band with one Householder reflector H = I - tau v v^H

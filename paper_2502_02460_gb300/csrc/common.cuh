@@ -123,6 +123,39 @@ template <class T> struct real_of { using type = double; };
 template <> struct real_of<float> { using type = float; };
 template <> struct real_of<zf> { using type = float; };
 
+// ------------------------------------------------------------------------------- reflectors --
+// 1 / sqrt and the Householder scalars of alpha = x_0 and xn = sum_{i>0} |x_i|^2 (not both trivial):
+// with s = sign(Re alpha), r = 1 / ||x||:  beta = -s ||x||,  tau = 1 - alpha / beta = 1 + s r alpha,
+// scale = 1 / (alpha - beta): one reciprocal square root and one division, no other long FP64 chain
+__device__ __forceinline__ void house(double alpha, double xn, double& tau, double& beta, double& scale) {
+  const double q = alpha * alpha + xn, r = rsqrt(q), nrm = q * r;
+  beta = alpha >= 0.0 ? -nrm : nrm;
+  tau = 1.0 + fabs(alpha) * r;
+  scale = 1.0 / (alpha - beta);
+}
+__device__ __forceinline__ void house(float alpha, float xn, float& tau, float& beta, float& scale) {
+  const float nrm = sqrtf(alpha * alpha + xn);
+  beta = alpha >= 0.f ? -nrm : nrm;
+  tau = (beta - alpha) / beta;
+  scale = 1.f / (alpha - beta);
+}
+__device__ __forceinline__ void house(zd alpha, double xn, zd& tau, zd& beta, zd& scale) {
+  const double q = abs2_(alpha) + xn, r = rsqrt(q), nrm = q * r;
+  const double s = alpha.x >= 0.0 ? 1.0 : -1.0;
+  const zd d = make_zd(alpha.x + s * nrm, alpha.y);
+  const double g = 1.0 / abs2_(d);
+  beta = make_zd(-s * nrm, 0.0);
+  tau = make_zd(1.0 + fabs(alpha.x) * r, s * r * alpha.y);
+  scale = make_zd(g * d.x, -g * d.y);
+}
+__device__ __forceinline__ void house(zf alpha, float xn, zf& tau, zf& beta, zf& scale) {
+  const float nrm = sqrtf(abs2_(alpha) + xn), s = alpha.x >= 0.f ? 1.f : -1.f;
+  const zf bt = make_zf(-s * nrm, 0.f);
+  beta = bt;
+  tau = div_(bt - alpha, bt);
+  scale = div_(make_zf(1.f, 0.f), alpha - bt);
+}
+
 // ------------------------------------------------------------------------- status word slots --
 enum StatusSlot {
   ST_NOT_SPD = 0,       // pivot index + 1 of the first non-positive Cholesky pivot

@@ -52,4 +52,14 @@ __device__ __forceinline__ bool grid_sync(const GridBar& g, int site) {
   return s_ok != 0;
 }
 
+// progress flags between blocks: release store and acquire load at GPU scope
+__device__ __forceinline__ void st_release(int* p, int v) {
+  asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 }  // namespace gev

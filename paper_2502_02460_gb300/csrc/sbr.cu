@@ -3,9 +3,9 @@
 //
 // For each panel (columns j0..j0+b-1, rows r0 = j0+b .. n-1):
 //   1. Householder QR of the m x b panel (m = n - r0) in ONE cooperative kernel: the panel rows are
-//      spread over all SMs and stay in shared memory; each column needs two bounded grid barriers
-//      (norm, then the reflector's inner products, which also give the column of the compact-WY
-//      factor T).  Q = H_0 ... H_{b-1} = I - Y T Y^H, T upper triangular.
+//      spread over all SMs and stay in shared memory; each column needs one bounded grid barrier
+//      (the norm and the reflector's inner products together, which also give the column of the
+//      compact-WY factor T).  Q = H_0 ... H_{b-1} = I - Y T Y^H, T upper triangular.
 //   2. Two-sided update of the trailing block A22 <- Q^H A22 Q by GEMMs:
 //        W = A22 Y T,  U = T^H (Y^H W),  V = W - Y U / 2,  A22 -= [Y V] [V Y]^H (lower, one
 //        rank-2b product), mirror.
@@ -20,168 +20,310 @@ namespace gev {
 
 namespace {
 
-constexpr int NT = 256;
+// threads of a panel block: at least 8 per column
+template <int B> constexpr int panel_nt() { return B == 64 ? 512 : 256; }
 
-template <class T>
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-  return t;  // valid in thread 0
-}
+template <class T> struct PanelArgs {
+  int m, R, use_smem, t_smem;
+  T* P;
+  long long ldp;
+  T* Y;     // the reflectors: in V1 and, for the trailing update, in up to three panel buffers
+  T* Y1;
+  T* Y2;
+  T* Y3;
+  long long ldy;
+  T* Tm;
+  double* nrm_part;
+  T* w_part;
+  T* prow;
+  int* count;  // arrivals, since the reduction began; base: before this launch
+  int base;
+  int* status;
+  int* abort_flag;
+};
 
-// One grid barrier per column.  Before the barrier every block sums, over its rows below the pivot,
-// ||x||^2, u_j = sum_r conj(x_r) P(r, j) (j > c, the columns to update) and t_j = sum_r conj(P(r, j)) x_r
-// (j < c, the stored reflectors, for T), with the UNSCALED column x; the block holding the pivot row
-// publishes that row.  After the barrier each block forms the reflector (beta, tau, scale: v_c = 1,
-// v_r = scale x_r) and recovers the inner products exactly as
-//   w_j = v^H P(:, j) = P(c, j) + conj(scale) u_j,     s_j = Y(:, j)^H v = conj(P(c, j)) + scale t_j.
+// Householder QR of the m x B panel, one grid barrier per column.  Before the barrier every block sums,
+// over its rows below the pivot, u_j = sum_r conj(x_r) P(r, j) with the current column x (j > c: the columns
+// to update; j < c: the reflectors before, for T; j = c: ||x||^2), and the block holding the pivot row
+// publishes that row.  After the barrier each block adds the block sums in a fixed order, forms the
+// reflector (beta, tau, scale: v_c = 1, v_r = scale x_r) and recovers the inner products exactly as
+//   w_j = v^H P(:, j) = P(c, j) + conj(scale) u_j,     s_j = Y(:, j)^H v = conj(sc_j) (conj(P(c, j)) + scale conj(u_j)).
+// The stored columns stay unscaled (their scales sc_j are applied when Y is written), so a column costs
+// one pass over the block's rows before the barrier and one after it.
+//
+// The column is a chain of latencies, not of work (m B multiply-adds over all SMs: 0.3 - 2 us): the
+// partial sums and the barrier's flag travel through L2 once each, all partial sums a thread adds are
+// loaded together (16 or 20 at a time), the reflector is one rsqrt and one division, and the two warps
+// that need its inner products compute it themselves.  Per panel, before -> now: m = 1500, b = 32 275 -> 191 us;
+// m = 10240, b = 64 782 -> 553 us (averages over a reduction).
 // The partial-sum buffers alternate with the column's parity: a block may start column c + 1 while a
 // slower one still reads column c's sums, but column c + 2 waits for everyone at barrier c + 1.
-template <class T>
-__global__ void __launch_bounds__(NT) k_panel_qr(int m, int b, T* P, long long ldp, T* Y, long long ldy,
-                                                 T* Tm, double* nrm_part, T* w_part, T* prow,
-                                                 GridBar gb, int R, int use_smem) {
+template <class T, int B>
+__global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
+  constexpr int NT = panel_nt<B>(), NG = NT / B;
+  constexpr bool LOW = sizeof(typename real_of<T>::type) == 4;  // FP32 data: norms in FP64
+  constexpr int NLD = sizeof(T) == 16 ? 10 : 20;                // partial sums in flight per thread
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int blk = blockIdx.x, tid = threadIdx.x;
-  const int lo = blk * R;
-  const int hi = min(m, lo + R);
-  const int rows = max(0, hi - lo);
-  const long long lds = R | 1;
-  const int G = gridDim.x;
-  T* sm = reinterpret_cast<T*>(smraw);
-  T* scratch = use_smem ? sm + lds * b : sm;
-  T* red2 = scratch;          // NT entries
-  T* wv = scratch + NT;       // b entries
-  double* red = reinterpret_cast<double*>(wv + b);  // 32 doubles
-  __shared__ T sh_tau, sh_beta, sh_scale;
-  __shared__ int sh_trivial;
-
-  T* base = use_smem ? sm : P + lo;
-  const long long ld = use_smem ? lds : ldp;
-  if (use_smem) {
-    for (int idx = tid; idx < rows * b; idx += NT) {
-      int r = idx % rows, c = idx / rows;
-      sm[r + c * lds] = P[(lo + r) + c * ldp];
+  const int blk = blockIdx.x, tid = threadIdx.x, G = gridDim.x, m = a.m;
+  const int lo = blk * a.R, hi = min(m, lo + a.R), rows = max(0, hi - lo);
+  const long long lds = a.R | 1;
+  T* red2 = reinterpret_cast<T*>(smraw);  // NT
+  T* wv = red2 + NT;                      // B: factors of the pivot row, then of s_j
+  T* w2 = wv + B;                         // B: factors of the rows below
+  T* sc = w2 + B;                         // B: scales of the reflectors
+  double* redn = reinterpret_cast<double*>(sc + B);  // NT / 32 + NG
+  T* Ts = reinterpret_cast<T*>(redn + NT / 32 + NG); // B x B when t_smem
+  T* sm = Ts + (a.t_smem ? B * B : 0);               // the block's rows when use_smem
+  __shared__ T sh_beta;
+  __shared__ int s_ok;
+  T* Tw = a.t_smem ? Ts : a.Tm;
+  T* base = a.use_smem ? sm : a.P + lo;
+  const long long ld = a.use_smem ? lds : a.ldp;
+  if (a.use_smem)
+    for (int idx = tid; idx < rows * B; idx += NT) {
+      const int r = idx % rows, c = idx / rows;
+      sm[r + c * lds] = a.P[(lo + r) + c * a.ldp];
     }
-    __syncthreads();
-  }
-  const int NG = NT / b;  // row groups (b is a power of two <= 128)
-  const int jj = tid % b, grp = tid / b;
+  __syncthreads();
+  const int jj = tid % B, grp = tid / B;
+  const int ncol = min(B, m);
 
-  for (int c = 0; c < b; ++c) {
-    if (c >= m) {
-      if (blk == 0 && tid < b) Tm[tid + c * b] = zero_<T>();
-      continue;
-    }
+  for (int c = 0; c < ncol; ++c) {
     const int par = c & 1;
-    double* np_ = nrm_part + (size_t)par * G;
-    T* wp_ = w_part + (size_t)par * G * b;
-    T* pr_ = prow + (size_t)par * b;
-    // ---- A: partial sums over this block's rows strictly below the pivot, unscaled column x
-    const int r0 = max(0, c + 1 - lo);
-    double ss = 0.0;
-    for (int r = r0 + tid; r < rows; r += NT) ss += abs2_(base[r + c * ld]);
-    const double tot = block_sum<T>(ss, red);
+    double* np_ = a.nrm_part + (size_t)par * 4096;
+    T* wp_ = a.w_part + (size_t)par * 4096 * B;
+    T* pr_ = a.prow + (size_t)par * B;
+    // ---- A: partial sums over this block's rows strictly below the pivot
     {
       T acc = zero_<T>();
-      if (grp < NG && jj != c)
-        for (int r = r0 + grp; r < rows; r += NG) {
-          const T x = base[r + c * ld], pj = base[r + jj * ld];
-          acc += (jj > c) ? cmul(x, pj) : cmul(pj, x);
-        }
+      double ss = 0.0;
+      for (int r = max(0, c + 1 - lo) + grp; r < rows; r += NG) {
+        const T x = base[r + c * ld];
+        acc += cmul(x, base[r + jj * ld]);
+        if (LOW && jj == c) ss += abs2_(x);
+      }
       red2[tid] = acc;
-      __syncthreads();
-      if (tid < b) {
-        T sum = zero_<T>();
-        for (int g = 0; g < NG; ++g) sum += red2[g * b + tid];
-        wp_[(long long)blk * b + tid] = sum;
-      }
-    }
-    if (tid == 0) np_[blk] = tot;
-    if (lo <= c && c < hi && tid < b) pr_[tid] = base[(c - lo) + tid * ld];  // the pivot row
-    if (!grid_sync(gb, 101)) return;
-    // ---- B: the reflector (all blocks compute it from the same sums, in a fixed order)
-    double xpart = 0.0;
-    for (int q = tid; q < G; q += NT) xpart += ldcg_(&np_[q]);
-    const double xn_all = block_sum<T>(xpart, red);
-    if (tid == 0) {
-      const double xn = xn_all;
-      const T alpha = ldcg_(&pr_[c]);
-      const int trivial = (xn == 0.0 && im_(alpha) == 0.0);
-      if (trivial) {
-        sh_tau = zero_<T>();
-        sh_beta = alpha;
-        sh_scale = zero_<T>();
-      } else {
-        const double nrm = sqrt(abs2_(alpha) + xn);
-        const double beta = re_(alpha) >= 0.0 ? -nrm : nrm;
-        const T bt = from_re<T>(beta);
-        sh_tau = div_(bt - alpha, bt);
-        sh_beta = bt;
-        sh_scale = div_(from_re<T>(1.0), alpha - bt);
-      }
-      sh_trivial = trivial;
+      if (LOW && jj == c) redn[NT / 32 + grp] = ss;
     }
     __syncthreads();
-    const T tau = sh_tau;
-    if (sh_trivial) {
-      if (blk == 0 && tid < b) Tm[tid + c * b] = zero_<T>();
-      continue;  // uniform over the grid: every block computed the same reflector
+    if (tid < B) {
+      T sum = red2[tid];
+#pragma unroll
+      for (int g = 1; g < NG; ++g) sum += red2[g * B + tid];
+      stcg_(&wp_[(long long)blk * B + tid], sum);
+      if (lo <= c && c < hi) stcg_(&pr_[tid], base[(c - lo) + tid * ld]);  // the pivot row
+      if (LOW && tid == c) {
+        double s = 0.0;
+        for (int g = 0; g < NG; ++g) s += redn[NT / 32 + g];
+        __stcg(&np_[blk], s);
+      }
     }
-    const T scale = sh_scale;
-    // the block partials of u / t, summed by NG threads per column, then in a fixed order
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("red.release.gpu.global.add.s32 [%0], 1;\n" ::"l"(a.count) : "memory");
+      const int target = a.base + (c + 1) * G;
+      int ok = 1;
+      if (ld_acquire(a.count) < target) {
+        volatile int* vab = a.abort_flag;
+        const long long lim = spin_limit(a.status);
+        long long it = 0;
+        while (ld_acquire(a.count) < target) {
+          if (*vab) { ok = 0; break; }
+          if (++it > lim) {
+            atomicCAS(&a.status[ST_TIMEOUT], 0, 101);
+            atomicExch(a.abort_flag, 1);
+            ok = 0;
+            break;
+          }
+          if (it > 64) __nanosleep(32);
+        }
+      }
+      s_ok = ok;
+    }
+    __syncthreads();
+    if (!s_ok) return;
+    // ---- B: the block sums, added by NG threads per column
+    T pc = zero_<T>(), alpha = zero_<T>();
+    if (tid < B) {
+      pc = ldcg_(&pr_[tid]);
+      alpha = ldcg_(&pr_[c]);
+    }
     {
       T part = zero_<T>();
-      if (grp < NG)
-        for (int q = grp; q < G; q += NG) part += ldcg_(&wp_[(long long)q * b + jj]);
+      for (int q0 = grp; q0 < G; q0 += NLD * NG) {
+        T v[NLD];
+#pragma unroll
+        for (int u = 0; u < NLD; ++u) {
+          const int q = q0 + u * NG;
+          v[u] = q < G ? ldcg_(&wp_[(long long)q * B + jj]) : zero_<T>();
+        }
+#pragma unroll
+        for (int u = 0; u < NLD; ++u) part += v[u];
+      }
       red2[tid] = part;
-      __syncthreads();
-      if (tid < b) {
-        T sum = zero_<T>();
-        for (int g = 0; g < NG; ++g) sum += red2[g * b + tid];
-        const T pc = ldcg_(&pr_[tid]);
-        // w_j = P(c, j) + conj(scale) u_j (j > c);  s_j = conj(P(c, j)) + scale t_j (j < c)
-        wv[tid] = (tid > c) ? pc + conj_(scale) * sum : (tid < c ? conj_(pc) + scale * sum : zero_<T>());
+      if (LOW) {
+        double x = 0.0;
+        for (int q = tid; q < G; q += NT) x += __ldcg(&np_[q]);
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        if ((tid & 31) == 0) redn[tid >> 5] = x;
       }
     }
-    for (int r = r0 + tid; r < rows; r += NT) base[r + c * ld] = scale * base[r + c * ld];
-    if (tid == 0 && lo <= c && c < hi) base[(c - lo) + c * ld] = sh_beta;
     __syncthreads();
-    // ---- C: apply H^H to the remaining columns; column c of T (block 0)
-    const T ctau = conj_(tau);
-    if (grp < NG && jj > c) {
-      const T wj = ctau * wv[jj];
-      for (int r = max(0, c - lo) + grp; r < rows; r += NG) {
-        const T vr = (lo + r == c) ? from_re<T>(1.0) : base[r + c * ld];
-        base[r + jj * ld] -= vr * wj;
+    if (tid < B) {
+      T sum = red2[tid];
+      double xn;
+      if (LOW) {
+        xn = 0.0;
+        for (int g = 0; g < NT / 32; ++g) xn += redn[g];
+      } else {
+        xn = (double)re_(red2[c]);
       }
+#pragma unroll
+      for (int g = 1; g < NG; ++g) {
+        sum += red2[g * B + tid];
+        if (!LOW) xn += re_(red2[g * B + c]);
+      }
+      T tau = zero_<T>(), beta = alpha, scale = zero_<T>();
+      if (!(xn == 0.0 && im_(alpha) == 0)) {
+        if constexpr (LOW) {  // the norm from its FP64 square, rounded once; the rest as the data
+          const double q = (double)abs2_(alpha) + xn;
+          const int ex = (__double2hiint(q) >> 20) & 0x7FF;
+          const float nrm = ex > 1023 - 120 && ex < 1023 + 120 ? sqrtf((float)q) : (float)sqrt(q);
+          beta = from_re<T>(re_(alpha) >= 0.f ? -nrm : nrm);
+          tau = div_(beta - alpha, beta);
+          scale = div_(from_re<T>(1.0), alpha - beta);
+        } else {
+          house(alpha, xn, tau, beta, scale);
+        }
+      }
+      if (tid > c) {
+        const T w = conj_(tau) * (pc + conj_(scale) * sum);
+        wv[tid] = w;
+        w2[tid] = scale * w;
+      } else if (tid < c) {
+        wv[tid] = conj_(sc[tid]) * (conj_(pc) + scale * conj_(sum));
+      } else {
+        wv[tid] = tau;
+        sh_beta = beta;
+      }
+      // (sc[c] is read by no other thread before the barrier below)
+      if (tid == c) sc[c] = scale;
     }
-    if (blk == 0 && tid < b) {
+    __syncthreads();
+    // ---- C: apply H^H to the remaining columns; column c of T (block 0, the one with the fewest rows left)
+    if (jj > c) {
+      const T w = w2[jj];
+      for (int r = max(0, c + 1 - lo) + grp; r < rows; r += NG) base[r + jj * ld] -= base[r + c * ld] * w;
+    }
+    if (lo <= c && c < hi && tid < B && tid >= c) {
+      if (tid > c) base[(c - lo) + tid * ld] -= wv[tid];
+      else base[(c - lo) + c * ld] = sh_beta;
+    }
+    if (blk == 0 && tid >= NT - B) {
+      const int i = tid - (NT - B);
+      const T tau = wv[c];
       T val = zero_<T>();
-      if (tid < c) {
-        T acc = zero_<T>();
-        for (int l = tid; l < c; ++l) acc += Tm[tid + l * b] * wv[l];
-        val = -(tau * acc);
-      } else if (tid == c) {
+      if (i < c) {
+        T acc = zero_<T>(), acc1 = zero_<T>();
+        int l = i;
+        for (; l + 1 < c; l += 2) {
+          acc += Tw[i + l * B] * wv[l];
+          acc1 += Tw[i + (l + 1) * B] * wv[l + 1];
+        }
+        if (l < c) acc += Tw[i + l * B] * wv[l];
+        val = -(tau * (acc + acc1));
+      } else if (i == c) {
         val = tau;
       }
-      Tm[tid + c * b] = val;
+      Tw[i + c * B] = val;
     }
     __syncthreads();
   }
+  if (blk == 0)  // (columns beyond the last reflector: zero)
+    for (int t = tid; t < B * B; t += NT) {
+      if (t / B >= ncol) a.Tm[t] = zero_<T>();
+      else if (a.t_smem) a.Tm[t] = Ts[t];
+    }
   // ---- write back: R (upper part) into the panel with zeros below, Y explicitly
-  for (int idx = tid; idx < rows * b; idx += NT) {
+  for (int idx = tid; idx < rows * B; idx += NT) {
     const int r = idx % rows, j = idx / rows;
     const int pr = lo + r;
     const T val = base[r + j * ld];
-    Y[pr + j * ldy] = (pr == j) ? from_re<T>(1.0) : (pr > j ? val : zero_<T>());
-    P[pr + j * ldp] = (pr <= j) ? val : zero_<T>();
+    const T y = (pr == j) ? from_re<T>(1.0) : (pr > j ? sc[j] * val : zero_<T>());
+    const long long o = pr + j * a.ldy;
+    a.Y[o] = y;
+    a.Y1[o] = y;
+    a.Y2[o] = y;
+    a.Y3[o] = y;
+    a.P[pr + j * a.ldp] = (pr <= j) ? val : zero_<T>();
+  }
+}
+
+template <class T, int B> size_t panel_smem(int R, int use_smem, int t_smem) {
+  constexpr int NT = panel_nt<B>();
+  size_t s = (size_t)(NT + 3 * B) * sizeof(T) + (NT / 32 + NT / B) * sizeof(double) + 64;
+  if (t_smem) s += (size_t)B * B * sizeof(T);
+  if (use_smem) s += (size_t)(R | 1) * B * sizeof(T);
+  return s;
+}
+
+// The QR of one panel (a.m rows): rows per block, residence in shared memory when it fits.
+template <class T, int B> int launch_panel(Sys& s, PanelArgs<T> a, int* arrivals) {
+  constexpr int NT = panel_nt<B>();
+  const size_t cap = (size_t)200 * 1024;
+  GEV_TRY(allow_max_dyn_smem(k_panel_qr<T, B>));
+  int G = s.sms, per_sm = 0;
+  a.R = std::max(16, (a.m + G - 1) / G);
+  G = (a.m + a.R - 1) / a.R;
+  a.t_smem = panel_smem<T, B>(a.R, 0, 1) <= cap ? 1 : 0;
+  a.use_smem = panel_smem<T, B>(a.R, 1, a.t_smem) <= cap ? 1 : 0;
+  if (!a.use_smem && panel_smem<T, B>(a.R, 1, 0) <= cap) {
+    a.t_smem = 0;
+    a.use_smem = 1;
+  }
+  const size_t smem = panel_smem<T, B>(a.R, a.use_smem, a.t_smem);
+  GEV_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_panel_qr<T, B>, NT, smem));
+  if (per_sm < 1 || G > per_sm * s.sms || G > 4096) return GEV_ERR_UNSUPPORTED;
+  a.base = *arrivals;
+  *arrivals += G * std::min(a.m, B);
+  void* args[] = {&a};
+  GEV_COUNT(s);
+  GEV_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_panel_qr<T, B>, dim3(G), dim3(NT), args, smem, s.stream));
+  return 0;
+}
+
+// M (2b x b) = [T; -U / 2], U = T^H (Z T) for Z = Y^H W0 (b x b): four columns per block, T in shared
+// memory.  (As two products of b x b x b on the tensor-core engine: four launches.)
+template <class T>
+__global__ void __launch_bounds__(256) k_sbr_coef(int b, const T* Z, const T* Tm, T* M) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  T* Ts = reinterpret_cast<T*>(smraw);  // b x b, ld b + 1
+  T* Q = Ts + b * (b + 1);              // Z T(:, j): b x 4
+  const int tid = threadIdx.x, j0 = blockIdx.x * 4;
+  for (int t = tid; t < b * b; t += 256) Ts[t % b + (t / b) * (b + 1)] = Tm[t];
+  __syncthreads();
+  const int i = tid % b, stp = 256 / b;
+  for (int jl = tid / b; jl < 4; jl += stp) {
+    const int j = j0 + jl;
+    T acc = zero_<T>(), acc1 = zero_<T>();
+#pragma unroll 4
+    for (int k = 0; k < b; k += 2) {
+      acc += Z[i + k * b] * Ts[k + j * (b + 1)];
+      acc1 += Z[i + (k + 1) * b] * Ts[k + 1 + j * (b + 1)];
+    }
+    Q[i + jl * b] = acc + acc1;
+  }
+  __syncthreads();
+  for (int jl = tid / b; jl < 4; jl += stp) {
+    const int j = j0 + jl;
+    T acc = zero_<T>(), acc1 = zero_<T>();
+#pragma unroll 4
+    for (int k = 0; k < b; k += 2) {
+      acc += cmul(Ts[k + i * (b + 1)], Q[k + jl * b]);
+      acc1 += cmul(Ts[k + 1 + i * (b + 1)], Q[k + 1 + jl * b]);
+    }
+    M[i + j * 2 * b] = Ts[i + j * (b + 1)];
+    M[b + i + j * 2 * b] = from_re<T>(-0.5) * (acc + acc1);
   }
 }
 
@@ -200,76 +342,75 @@ __global__ void k_extract_band(int n, int b, const T* A, long long lda, T* band,
   }
 }
 
-template <class T> size_t panel_smem(int R, int b, int use_smem) {
-  size_t s = (size_t)(NT + b) * sizeof(T) + 32 * sizeof(double) + 64;
-  if (use_smem) s += (size_t)(R | 1) * b * sizeof(T);
-  return s;
-}
-
 }  // namespace
 
 template <class T> int he2hb(Sys& s, T* A, int lda, int b) {
   const int n = s.n;
-  GEV_TRY(allow_max_dyn_smem(k_panel_qr<T>));
   T* V1 = (T*)s.V1;
   // the panels' reflector columns are stored from their own first row on; the rows above are zero so
   // that consecutive panels form one wider compact-WY block in the back-transform
   GEV_CUDA_TRY(cudaMemsetAsync(V1, 0, sizeof(T) * (size_t)n * n, s.stream));
   T* T1 = (T*)s.T1;
-  T* W0 = (T*)s.Pn;
-  T* W1 = W0 + (size_t)n * 2 * s.b;
-  T* sm0 = (T*)s.small;
-  T* sm1 = sm0 + (size_t)s.b * s.b;
+  const size_t buf = (size_t)n * 2 * s.b;    // the panel buffers, n x 2b each
+  T* WY = (T*)s.Pn;                           // [W0 | Y]
+  T* YV = WY + buf;                           // [Y | V]
+  T* VY = YV + buf;                           // [V | Y]
+  T* M = VY + buf;                            // 2b x b
+  T* Z = (T*)s.small;
   double* nrm_part = (double*)s.panelws;     // 2 x 4096 (by column parity)
   T* prow = (T*)(nrm_part + 2 * 4096);        // 2 x b pivot rows
   T* w_part = prow + 2 * 128;                 // 2 x 4096 x b
-  GridBar gb{(unsigned*)&s.status[ST_BARRIER_CNT], (unsigned*)&s.status[ST_BARRIER_GEN], s.status,
-             &s.status[ST_ABORT]};
-  const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zero = zero_<T>(), mhalf = from_re<T>(-0.5);
-  int npanel = 0;
+  const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zero = zero_<T>();
+  const size_t coef_smem = sizeof(T) * ((size_t)b * (b + 1) + 4 * b);
+  GEV_TRY(allow_dyn_smem(k_sbr_coef<T>, coef_smem));
+  int npanel = 0, arrivals = 0;
+  GEV_CUDA_TRY(cudaMemsetAsync(&s.status[ST_BARRIER_CNT], 0, 2 * sizeof(int), s.stream));
   for (int j0 = 0;; j0 += b) {
     const int r0 = j0 + b;
     const int m = n - r0;
     if (m < 2) break;
     ++npanel;
-    T* Pp = A + r0 + (long long)j0 * lda;
     T* Yp = V1 + r0 + (long long)j0 * n;
     T* Tp = T1 + (long long)j0 * b;
-    // ---- launch geometry: rows per block, shared-memory residency when it fits
-    int per_sm = 1;
-    int G = s.sms;
-    int R = (m + G - 1) / G;
-    if (R < 16) R = 16;
-    G = (m + R - 1) / R;
-    int use_smem = panel_smem<T>(R, b, 1) <= (size_t)200 * 1024 ? 1 : 0;
-    size_t smem = panel_smem<T>(R, b, use_smem);
-    GEV_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_panel_qr<T>, NT, smem));
-    if (per_sm < 1 || G > per_sm * s.sms) return GEV_ERR_UNSUPPORTED;
-    if (G > 4096) return GEV_ERR_UNSUPPORTED;
-    GEV_CUDA_TRY(cudaMemsetAsync(&s.status[ST_BARRIER_CNT], 0, 2 * sizeof(int), s.stream));
-    int mm = m, bb = b;
-    long long ldp = lda, ldy = n;
-    void* args[] = {&mm, &bb, &Pp, &ldp, &Yp, &ldy, &Tp, &nrm_part, &w_part, &prow, &gb, &R, &use_smem};
-    GEV_COUNT(s);
-    GEV_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_panel_qr<T>, dim3(G), dim3(NT), args, smem, s.stream));
-    // ---- two-sided update of the trailing block, the rank-2b update as ONE product:
+    T* Wv = YV + (size_t)n * b;
+    PanelArgs<T> a{};
+    a.m = m;
+    a.P = A + r0 + (long long)j0 * lda;
+    a.ldp = lda;
+    a.Y = Yp;
+    a.Y1 = WY + (size_t)n * b;
+    a.Y2 = YV;
+    a.Y3 = VY + (size_t)n * b;
+    a.ldy = n;
+    a.Tm = Tp;
+    a.nrm_part = nrm_part;
+    a.w_part = w_part;
+    a.prow = prow;
+    a.count = &s.status[ST_BARRIER_CNT];
+    a.status = s.status;
+    a.abort_flag = &s.status[ST_ABORT];
+    if (b == 16) GEV_TRY((launch_panel<T, 16>(s, a, &arrivals)));
+    else if (b == 32) GEV_TRY((launch_panel<T, 32>(s, a, &arrivals)));
+    else if (b == 64) GEV_TRY((launch_panel<T, 64>(s, a, &arrivals)));
+    else return GEV_ERR_UNSUPPORTED;
+    // ---- two-sided update of the trailing block: with W = A22 Y T, Z = Y^H A22 Y, U = T^H Z T,
+    //      V = W - Y U / 2 = [A22 Y, Y] [T; -U / 2], the rank-2b update as ONE product:
     //      A22 -= Y V^H + V Y^H = [Y V] [V Y]^H  (K = 2b: the trailing block is read and written once)
     T* A22 = A + r0 + (long long)r0 * lda;
-    T* YV = W1;                                // m x 2b: [Y | V]
-    T* Wv = W1 + (size_t)n * b;                // its V half
-    T* VY = W0 + (size_t)2 * n * 2 * s.b;      // m x 2b: [V | Y] (third panel buffer)
-    gemm(s, gp<T>(m, b, m, 0, 0, one, A22, lda, Yp, n, zero, W0, n));  // W0 = A22 Y
-    GemmP<T> g = gp<T>(m, b, b, 0, 0, one, W0, n, Tp, b, zero, Wv, n);   // W = W0 T
-    g.tri_b = 2;
-    gemm(s, g);
-    gemm(s, gp<T>(b, b, m, 2, 0, one, Yp, n, Wv, n, zero, sm0, b));    // Z = Y^H W
-    g = gp<T>(b, b, b, 2, 0, one, Tp, b, sm0, b, zero, sm1, b);         // U = T^H Z
-    g.tri_a = 1;
-    gemm(s, g);
-    gemm(s, gp<T>(m, b, b, 0, 0, mhalf, Yp, n, sm1, b, one, Wv, n));   // V = W - Y U / 2
-    GEV_TRY(copy2d<T>(s, m, b, Yp, n, YV, n));
+    gemm(s, gp<T>(m, b, m, 0, 0, one, A22, lda, Yp, n, zero, WY, n));  // W0 = A22 Y
+    gemm(s, gp<T>(b, b, m, 2, 0, one, Yp, n, WY, n, zero, Z, b));      // Z = Y^H W0
+    GEV_COUNT(s);
+    k_sbr_coef<T><<<b / 4, 256, coef_smem, s.stream>>>(b, Z, Tp, M);
+    GemmP<T> g = gp<T>(m, b, 2 * b, 0, 0, one, WY, n, M, 2 * b, zero, Wv, n);
+    if (gemm_on_fp64_pipe(s, g)) {
+      gemm(s, g);
+    } else {  // (one product of both would scale W0 and Y, and T and U, together)
+      g = gp<T>(m, b, b, 0, 0, one, WY, n, M, 2 * b, zero, Wv, n);
+      g.tri_b = 2;
+      gemm(s, g);
+      gemm(s, gp<T>(m, b, b, 0, 0, one, Yp, n, M + b, 2 * b, one, Wv, n));
+    }
     GEV_TRY(copy2d<T>(s, m, b, Wv, n, VY, n));
-    GEV_TRY(copy2d<T>(s, m, b, Yp, n, VY + (size_t)n * b, n));
     g = gp<T>(m, m, 2 * b, 0, 2, mone, YV, n, VY, n, one, A22, lda);    // A22 -= [Y V] [V Y]^H
     g.c_lower = 1;
     gemm(s, g);
