@@ -715,6 +715,13 @@ size_t gemm_f64_emulated_scratch(int M, int N, int K) { return oz_layout(M, N, K
 
 namespace {
 
+// K range of an exponent block: short enough for about six blocks per SM (a block is a chain of loads: with one
+// block per 32 vectors the pass over a 1500 x 32 operand took 40 us), at most 512, at least 64
+int exp_slab(const Sys& s, int nblk, int K) {
+  const int want = (int)cdiv(6 * s.sms, nblk);
+  return std::min(512, std::max(64, (int)(cdiv(cdiv(K, want), 64) * 64)));
+}
+
 // Exponents and digit planes of both operands.  K <= 128 (the thin products of the panels): one launch
 // that holds whole vectors in registers; else an exponent pass and a split pass, each over both operands.
 // (For a 1500 x 32 x 32 product the former two exponent and two split launches with their two memsets
@@ -738,12 +745,11 @@ void split_both(Sys& s, int M, int N, int K, const Opnd& a, const Opnd& b, int f
     else k_split_short<8><<<nb, 128, 0, s.stream>>>(q, K, KT);
     return;
   }
-  constexpr int SLAB = 512;
-  const int slabs = K <= 2 * SLAB ? 1 : (int)cdiv(K, SLAB);
-  if (slabs > 1) cudaMemsetAsync(E, 0x80, (size_t)((unsigned char*)(F + NT * ON) - (unsigned char*)E), s.stream);
   q.nblk0 = (int)cdiv(M, 32);
+  const int nblk = q.nblk0 + (int)cdiv(N, 32), slab = exp_slab(s, nblk, K), slabs = (int)cdiv(K, slab);
+  if (slabs > 1) cudaMemsetAsync(E, 0x80, (size_t)((unsigned char*)(F + NT * ON) - (unsigned char*)E), s.stream);
   GEV_COUNT(s);
-  k_vec_exp<<<dim3(q.nblk0 + cdiv(N, 32), slabs), 256, 0, s.stream>>>(q, K, slabs == 1 ? K : SLAB, slabs);
+  k_vec_exp<<<dim3(nblk, slabs), 256, 0, s.stream>>>(q, K, slab, slabs);
   q.nblk0 = (int)cdiv(ga * KT, 8);
   GEV_COUNT(s);
   k_split<<<q.nblk0 + cdiv(gb * KT, 8), 256, 0, s.stream>>>(q, K, KT);
@@ -917,11 +923,11 @@ bool gemm_f64_bdiag(Sys& s, int M, int N, int K, const BdOp& a, int bm, int bk, 
     GEV_COUNT(s);
     k_fill_exp<<<cdiv(L.Np, 256), 256, 0, s.stream>>>((int)L.Np, 1, F);
   } else if (Ke > 0) {
-    const int slabs = (int)cdiv(Ke, 512);
-    if (slabs > 1) cudaMemsetAsync(F, 0x80, L.Np * sizeof(int), s.stream);
     q.nblk0 = (int)cdiv(N, 32);
+    const int slab = exp_slab(s, q.nblk0, Ke), slabs = (int)cdiv(Ke, slab);
+    if (slabs > 1) cudaMemsetAsync(F, 0x80, L.Np * sizeof(int), s.stream);
     GEV_COUNT(s);
-    k_vec_exp<<<dim3(q.nblk0, slabs), 256, 0, s.stream>>>(q, Ke, slabs == 1 ? Ke : 512, slabs);
+    k_vec_exp<<<dim3(q.nblk0, slabs), 256, 0, s.stream>>>(q, Ke, slab, slabs);
   }
   if (Ke > 0) {
     q.nblk0 = (int)cdiv((long long)L.NT * (ON / 8) * L.KT, 8);
