@@ -218,8 +218,8 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
         if (m == 1 || (m == 0 ? t > 0 : len2 > 0)) {
 #pragma unroll 8
           for (int j = 0; j < TERMS; j += 2) {
-            acc += a[(j0 + j) * st] * x[j0 + j];
-            acc2 += a[(j0 + j + 1) * st] * x[j0 + j + 1];
+            mac(acc, a[(j0 + j) * st], x[j0 + j]);
+            mac(acc2, a[(j0 + j + 1) * st], x[j0 + j + 1]);
           }
         }
         part[tid] = acc + acc2;
@@ -272,10 +272,15 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
           constexpr int NW = NTH - 64;
           for (int idx = tid - 64; idx < B * B; idx += NW) {
             const int i = idx & (B - 1), q = idx / B;
-            if (t > 0 && i < len && (q > 0 || i > 0))
-              stcg_(&band[(B + i - q) + (long long)(p - B + q) * ldb],
-                    q == 0 ? zero_<T>() : Ls[i + q * LD] - v[i] * w[q]);
-            if (q > 0 && len2 > 0) Es[i + q * LD] -= mulc(z[i], v[q]);
+            if (t > 0 && i < len && (q > 0 || i > 0)) {
+              T val = zero_<T>();
+              if (q > 0) {
+                val = Ls[i + q * LD];
+                nmac(val, v[i], w[q]);
+              }
+              stcg_(&band[(B + i - q) + (long long)(p - B + q) * ldb], val);
+            }
+            if (q > 0 && len2 > 0) nmacc(Es[i + q * LD], z[i], v[q]);
           }
           const long long rid = (long long)s * ntask + t;
           for (int i = tid - 64; i < B; i += NW) V2[rid * B + i] = v[i];
@@ -288,9 +293,12 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
           const int c = idx / B, e = idx & (B - 1);
           const bool first = e < B - 1 - c;
           const int i = first ? c + 1 + e : e + 1, j = first ? c : B - 1 - c;
-          if (e < B - 1 && i < len && j < len)
-            stcg_(&band[(i - j) + (long long)(p + j) * ldb],
-                  Ds[i + j * LD] - (mulc(y[i], v[j]) + mulc(v[i], y[j])));
+          if (e < B - 1 && i < len && j < len) {
+            T val = Ds[i + j * LD];
+            nmacc(val, y[i], v[j]);
+            nmacc(val, v[i], y[j]);
+            stcg_(&band[(i - j) + (long long)(p + j) * ldb], val);
+          }
         }
         for (int i = tid - 32; i < len; i += NL)
           stcg_(&band[(long long)(p + i) * ldb],
@@ -461,12 +469,12 @@ __global__ void __launch_bounds__(8 * BTL_COLS) k_bt_level(int n, int k, int L, 
         T acc0 = zero_<T>(), acc1 = zero_<T>();
 #pragma unroll
         for (int i = 0; i <= NR; ++i) {
-          if (i & 1) acc1 += cmul(vq[8 * i], z[i]);
-          else acc0 += cmul(vq[8 * i], z[i]);
+          if (i & 1) cmac(acc1, vq[8 * i], z[i]);
+          else cmac(acc0, vq[8 * i], z[i]);
         }
         const T w = ts[8 * a + u] * sum8(acc0 + acc1);
 #pragma unroll
-        for (int i = 0; i <= NR; ++i) z[i] -= vq[8 * i] * w;
+        for (int i = 0; i <= NR; ++i) nmac(z[i], vq[8 * i], w);
       }
       if (8 * (a + NR) < left) y[8 * (a + NR)] = z[NR];
       if (a > 0) {

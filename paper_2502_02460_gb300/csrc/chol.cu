@@ -73,17 +73,6 @@ __device__ void inv_lower_blocked(int jb, const T* L, T* X, T* tmp) {
   }
 }
 
-// 1 / d for a positive d: the hardware's 20-bit reciprocal and two Newton-Raphson steps (y += y (1 - d y)),
-// within an ulp of the quotient; outside the exponents where the steps are safe, the division
-__device__ __forceinline__ double recip(double d) {
-  const int e = (__double2hiint(d) >> 20) & 0x7FF;
-  if (e < 24 || e > 2020) return 1.0 / d;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(d));
-  y = fma(y, fma(-d, y, 1.0), y);
-  return fma(y, fma(-d, y, 1.0), y);
-}
-
 // Factor the jb x jb diagonal block (lower) and invert the factor, blocked by SB, on 16 warps.  Step kb:
 //   1. warps 0 - 7 factor and invert the SB x SB diagonal block, one entry (i, j), j <= i, per thread:
 //      before pivot j the thread holds a_ij of the trailing matrix, after it x_ij of the inverse of the
@@ -153,7 +142,8 @@ __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long ld
           const T li = s_rinv[p & 1] * s_col[p & 1][i];
           const bool fac = j > p;
           const T m = fac ? conj_(s_col[p & 1][j]) : s_row[p & 1][j];
-          const T cur = (fac ? a : x) - li * m;
+          T cur = fac ? a : x;
+          nmac(cur, li, m);
           if (fac) a = cur;
           else x = cur;
         }
@@ -186,8 +176,8 @@ __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long ld
         T acc = zero_<T>(), acc1 = zero_<T>();
 #pragma unroll
         for (int p = 0; p < SB; p += 2) {
-          acc += mulc(L[i + (pc + p) * LDS], L[j + (pc + p) * LDS]);
-          acc1 += mulc(L[i + (pc + p + 1) * LDS], L[j + (pc + p + 1) * LDS]);
+          macc(acc, L[i + (pc + p) * LDS], L[j + (pc + p) * LDS]);
+          macc(acc1, L[i + (pc + p + 1) * LDS], L[j + (pc + p + 1) * LDS]);
         }
         L[i + j * LDS] -= acc + acc1;
       }
@@ -198,10 +188,10 @@ __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long ld
           T acc = zero_<T>(), acc1 = zero_<T>();
           int k = c;
           for (; k + 1 < kb; k += 2) {
-            acc += L[(kb + q) + k * LDS] * X[k + c * LDS];
-            acc1 += L[(kb + q) + (k + 1) * LDS] * X[(k + 1) + c * LDS];
+            mac(acc, L[(kb + q) + k * LDS], X[k + c * LDS]);
+            mac(acc1, L[(kb + q) + (k + 1) * LDS], X[(k + 1) + c * LDS]);
           }
-          if (k < kb) acc += L[(kb + q) + k * LDS] * X[k + c * LDS];
+          if (k < kb) mac(acc, L[(kb + q) + k * LDS], X[k + c * LDS]);
           S[t] = acc + acc1;
         }
       }
@@ -217,14 +207,14 @@ __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long ld
       o[u] = zero_<T>();
       if (t < nr * SB) {
         const int i = r0 + t % nr, p = t / nr;
-        for (int q = 0; q <= p; ++q) o[u] += mulc(L[i + (kb + q) * LDS], X[(kb + p) + (kb + q) * LDS]);
+        for (int q = 0; q <= p; ++q) macc(o[u], L[i + (kb + q) * LDS], X[(kb + p) + (kb + q) * LDS]);
       }
     }
     for (int t = tid; t < SB * kb; t += PD_NT) {
       const int q = t % SB, c = t / SB;
       if (q < bs) {
         T acc = zero_<T>();
-        for (int l = 0; l <= q; ++l) acc += X[(kb + q) + (kb + l) * LDS] * S[l + c * SB];
+        for (int l = 0; l <= q; ++l) mac(acc, X[(kb + q) + (kb + l) * LDS], S[l + c * SB]);
         X[(kb + q) + c * LDS] = -acc;
       }
     }
@@ -244,8 +234,8 @@ __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long ld
         T acc = zero_<T>(), acc1 = zero_<T>();
 #pragma unroll
         for (int p = 0; p < SB; p += 2) {
-          acc += mulc(L[(r0 + i) + (kb + p) * LDS], L[(r0 + j) + (kb + p) * LDS]);
-          acc1 += mulc(L[(r0 + i) + (kb + p + 1) * LDS], L[(r0 + j) + (kb + p + 1) * LDS]);
+          macc(acc, L[(r0 + i) + (kb + p) * LDS], L[(r0 + j) + (kb + p) * LDS]);
+          macc(acc1, L[(r0 + i) + (kb + p + 1) * LDS], L[(r0 + j) + (kb + p + 1) * LDS]);
         }
         L[(r0 + i) + (r0 + j) * LDS] -= acc + acc1;
       }

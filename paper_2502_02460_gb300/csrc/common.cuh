@@ -123,6 +123,53 @@ template <class T> struct real_of { using type = double; };
 template <> struct real_of<float> { using type = float; };
 template <> struct real_of<zf> { using type = float; };
 
+// --------------------------------------------------------------- FP64-pipe arithmetic (device) --
+// 1 / d: the hardware's 20-bit reciprocal and two Newton-Raphson steps (y += y (1 - d y)),
+// within an ulp of the quotient (about half a division's FP64 instructions); outside the exponents where the
+// steps are safe, zero and the non-finite ones included, the division
+__device__ __forceinline__ double recip(double d) {
+  const int e = (__double2hiint(d) >> 20) & 0x7FF;
+  if (e < 24 || e > 2020) return 1.0 / d;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(d));
+  y = fma(y, fma(-d, y, 1.0), y);
+  return fma(y, fma(-d, y, 1.0), y);
+}
+
+// acc += a b, conj(a) b, a conj(b), and the subtractions: two multiply-adds per component of complex data
+// (written with the operators they are a product, a multiply-add and an addition, and an FP64 instruction
+// occupies the pipe for the same time whichever it is)
+__device__ __forceinline__ void mac(float& c, float a, float b) { c += a * b; }
+__device__ __forceinline__ void mac(double& c, double a, double b) { c += a * b; }
+__device__ __forceinline__ void nmac(float& c, float a, float b) { c -= a * b; }
+__device__ __forceinline__ void nmac(double& c, double a, double b) { c -= a * b; }
+__device__ __forceinline__ void cmac(float& c, float a, float b) { c += a * b; }
+__device__ __forceinline__ void cmac(double& c, double a, double b) { c += a * b; }
+__device__ __forceinline__ void macc(float& c, float a, float b) { c += a * b; }
+__device__ __forceinline__ void macc(double& c, double a, double b) { c += a * b; }
+__device__ __forceinline__ void nmacc(float& c, float a, float b) { c -= a * b; }
+__device__ __forceinline__ void nmacc(double& c, double a, double b) { c -= a * b; }
+template <class Z> __device__ __forceinline__ void mac(Z& c, Z a, Z b) {
+  c.x = fma(-a.y, b.y, fma(a.x, b.x, c.x));
+  c.y = fma(a.y, b.x, fma(a.x, b.y, c.y));
+}
+template <class Z> __device__ __forceinline__ void nmac(Z& c, Z a, Z b) {
+  c.x = fma(a.y, b.y, fma(-a.x, b.x, c.x));
+  c.y = fma(-a.y, b.x, fma(-a.x, b.y, c.y));
+}
+template <class Z> __device__ __forceinline__ void cmac(Z& c, Z a, Z b) {
+  c.x = fma(a.y, b.y, fma(a.x, b.x, c.x));
+  c.y = fma(-a.y, b.x, fma(a.x, b.y, c.y));
+}
+template <class Z> __device__ __forceinline__ void macc(Z& c, Z a, Z b) {
+  c.x = fma(a.y, b.y, fma(a.x, b.x, c.x));
+  c.y = fma(a.y, b.x, fma(-a.x, b.y, c.y));
+}
+template <class Z> __device__ __forceinline__ void nmacc(Z& c, Z a, Z b) {
+  c.x = fma(-a.y, b.y, fma(-a.x, b.x, c.x));
+  c.y = fma(-a.y, b.x, fma(a.x, b.y, c.y));
+}
+
 // ------------------------------------------------------------------------------- reflectors --
 // 1 / sqrt and the Householder scalars of alpha = x_0 and xn = sum_{i>0} |x_i|^2 (not both trivial):
 // with s = sign(Re alpha), r = 1 / ||x||:  beta = -s ||x||,  tau = 1 - alpha / beta = 1 + s r alpha,
@@ -131,7 +178,7 @@ __device__ __forceinline__ void house(double alpha, double xn, double& tau, doub
   const double q = alpha * alpha + xn, r = rsqrt(q), nrm = q * r;
   beta = alpha >= 0.0 ? -nrm : nrm;
   tau = 1.0 + fabs(alpha) * r;
-  scale = 1.0 / (alpha - beta);
+  scale = recip(alpha - beta);
 }
 __device__ __forceinline__ void house(float alpha, float xn, float& tau, float& beta, float& scale) {
   const float nrm = sqrtf(alpha * alpha + xn);
@@ -143,7 +190,7 @@ __device__ __forceinline__ void house(zd alpha, double xn, zd& tau, zd& beta, zd
   const double q = abs2_(alpha) + xn, r = rsqrt(q), nrm = q * r;
   const double s = alpha.x >= 0.0 ? 1.0 : -1.0;
   const zd d = make_zd(alpha.x + s * nrm, alpha.y);
-  const double g = 1.0 / abs2_(d);
+  const double g = recip(abs2_(d));
   beta = make_zd(-s * nrm, 0.0);
   tau = make_zd(1.0 + fabs(alpha.x) * r, s * r * alpha.y);
   scale = make_zd(g * d.x, -g * d.y);

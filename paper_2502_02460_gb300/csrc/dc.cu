@@ -500,7 +500,7 @@ __device__ void eval_secular(int K, int j, int o, const double* delta, const dou
   for (int i = lane; i < K; i += 32) {
     const double di = (delta[i] - dO) - mu;
     const double zi = z[i];
-    const double t = zi / di;
+    const double t = zi * recip(di);
     if (i <= j) { a += zi * t; b += t * t; }
     else { c += zi * t; e += t * t; }
   }
@@ -686,7 +686,7 @@ __global__ void k_vectors(Node* nodes, DcArrays A, double* U, long long ldu) {
   double* col = U + (long long)(a + j) * ldu;  // rows 0 .. K-1 of column a + j
   double ss = 0.0;
   for (int i = threadIdx.x; i < K; i += blockDim.x) {
-    const double v = A.zp[a + i] / ((delta[i] - dO) - mu);
+    const double v = A.zp[a + i] * recip((delta[i] - dO) - mu);
     col[A.nd_g[a + i]] = v;
     ss += v * v;
   }

@@ -253,11 +253,11 @@ __global__ void __launch_bounds__(SM_T * SM_T) gemm_small_kernel(GemmP<T> p, int
     if (kn == SM_K) {
 #pragma unroll 8
       for (int k = 0; k < SM_K; k += 2) {
-        acc += As[k][ti] * Bs[tj][k];
-        acc1 += As[k + 1][ti] * Bs[tj][k + 1];
+        mac(acc, As[k][ti], Bs[tj][k]);
+        mac(acc1, As[k + 1][ti], Bs[tj][k + 1]);
       }
     } else {
-      for (int k = 0; k < kn; ++k) acc += As[k][ti] * Bs[tj][k];
+      for (int k = 0; k < kn; ++k) mac(acc, As[k][ti], Bs[tj][k]);
     }
     __syncthreads();
   }

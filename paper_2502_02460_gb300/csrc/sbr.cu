@@ -12,6 +12,7 @@
 // Y is kept explicitly (unit diagonal, zeros above) in the handle's V1 at the panel's position and
 // T in T1, for the back-transform  Y_out = Q1 Z = Q_0 (Q_1 (... Q_last Z)).
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "coop.cuh"
@@ -20,8 +21,9 @@ namespace gev {
 
 namespace {
 
-// threads of a panel block: at least 8 per column
-template <int B> constexpr int panel_nt() { return B == 64 ? 512 : 256; }
+// threads of a panel block: four (b = 16: eight) per column.  All four schedulers have a warp then, and the sums
+// over a column's threads, a chain of FP64 additions in one warp, stay short.
+template <int B> constexpr int panel_nt() { return B == 64 ? 256 : 128; }
 
 template <class T> struct PanelArgs {
   int m, R, use_smem, t_smem;
@@ -53,16 +55,16 @@ template <class T> struct PanelArgs {
 //
 // The column is a chain of latencies, not of work (m B multiply-adds over all SMs: 0.3 - 2 us): the
 // partial sums and the barrier's flag travel through L2 once each, all partial sums a thread adds are
-// loaded together (16 or 20 at a time), the reflector is one rsqrt and one division, and the two warps
-// that need its inner products compute it themselves.  Per panel, before -> now: m = 1500, b = 32 275 -> 191 us;
-// m = 10240, b = 64 782 -> 553 us (averages over a reduction).
+// loaded together (20 or 40 at a time), the reflector is one rsqrt and one division, and the two warps
+// that need its inner products compute it themselves.  Per panel, averages over a reduction: n = 1500, b = 32
+// 275 us at first, about 170 now; n = 10240, b = 64 782, about 520 now; complex n = 509, b = 32 440, about 220 now.
 // The partial-sum buffers alternate with the column's parity: a block may start column c + 1 while a
 // slower one still reads column c's sums, but column c + 2 waits for everyone at barrier c + 1.
 template <class T, int B>
 __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
   constexpr int NT = panel_nt<B>(), NG = NT / B;
   constexpr bool LOW = sizeof(typename real_of<T>::type) == 4;  // FP32 data: norms in FP64
-  constexpr int NLD = sizeof(T) == 16 ? 10 : 20;                // partial sums in flight per thread
+  constexpr int NLD = sizeof(T) == 16 ? 20 : 40;                // partial sums in flight per thread
   extern __shared__ __align__(16) unsigned char smraw[];
   const int blk = blockIdx.x, tid = threadIdx.x, G = gridDim.x, m = a.m;
   const int lo = blk * a.R, hi = min(m, lo + a.R), rows = max(0, hi - lo);
@@ -99,7 +101,7 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
       double ss = 0.0;
       for (int r = max(0, c + 1 - lo) + grp; r < rows; r += NG) {
         const T x = base[r + c * ld];
-        acc += cmul(x, base[r + jj * ld]);
+        cmac(acc, x, base[r + jj * ld]);
         if (LOW && jj == c) ss += abs2_(x);
       }
       red2[tid] = acc;
@@ -181,8 +183,9 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
 #pragma unroll
       for (int g = 1; g < NG; ++g) {
         sum += red2[g * B + tid];
-        if (!LOW) xn += re_(red2[g * B + c]);
+        if (!LOW && B > 32) xn += re_(red2[g * B + c]);
       }
+      if (!LOW && B <= 32) xn = __shfl_sync(B == 32 ? 0xffffffffu : 0xffffu, (double)re_(sum), c);
       T tau = zero_<T>(), beta = alpha, scale = zero_<T>();
       if (!(xn == 0.0 && im_(alpha) == 0)) {
         if constexpr (LOW) {  // the norm from its FP64 square, rounded once; the rest as the data
@@ -213,7 +216,7 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
     // ---- C: apply H^H to the remaining columns; column c of T (block 0, the one with the fewest rows left)
     if (jj > c) {
       const T w = w2[jj];
-      for (int r = max(0, c + 1 - lo) + grp; r < rows; r += NG) base[r + jj * ld] -= base[r + c * ld] * w;
+      for (int r = max(0, c + 1 - lo) + grp; r < rows; r += NG) nmac(base[r + jj * ld], base[r + c * ld], w);
     }
     if (lo <= c && c < hi && tid < B && tid >= c) {
       if (tid > c) base[(c - lo) + tid * ld] -= wv[tid];
@@ -227,10 +230,10 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
         T acc = zero_<T>(), acc1 = zero_<T>();
         int l = i;
         for (; l + 1 < c; l += 2) {
-          acc += Tw[i + l * B] * wv[l];
-          acc1 += Tw[i + (l + 1) * B] * wv[l + 1];
+          mac(acc, Tw[i + l * B], wv[l]);
+          mac(acc1, Tw[i + (l + 1) * B], wv[l + 1]);
         }
-        if (l < c) acc += Tw[i + l * B] * wv[l];
+        if (l < c) mac(acc, Tw[i + l * B], wv[l]);
         val = -(tau * (acc + acc1));
       } else if (i == c) {
         val = tau;
@@ -272,8 +275,11 @@ template <class T, int B> int launch_panel(Sys& s, PanelArgs<T> a, int* arrivals
   constexpr int NT = panel_nt<B>();
   const size_t cap = (size_t)200 * 1024;
   GEV_TRY(allow_max_dyn_smem(k_panel_qr<T, B>));
-  int G = s.sms, per_sm = 0;
-  a.R = std::max(16, (a.m + G - 1) / G);
+  // Blocks: a column costs a block 2 R / 4 b / 32 multiply-adds of FP64 pipe time for its R = m / G rows (twice
+  // that for complex data against additions) and G / 4 b / 32 additions for the G partial sums: least at G^2 = 2 m
+  // (4 m).
+  int G = std::min(s.sms, (int)std::ceil(std::sqrt((is_cx<T>::value ? 4.0 : 2.0) * a.m))), per_sm = 0;
+  a.R = std::max(8, (a.m + G - 1) / G);
   G = (a.m + a.R - 1) / a.R;
   a.t_smem = panel_smem<T, B>(a.R, 0, 1) <= cap ? 1 : 0;
   a.use_smem = panel_smem<T, B>(a.R, 1, a.t_smem) <= cap ? 1 : 0;
@@ -292,38 +298,33 @@ template <class T, int B> int launch_panel(Sys& s, PanelArgs<T> a, int* arrivals
   return 0;
 }
 
-// M (2b x b) = [T; -U / 2], U = T^H (Z T) for Z = Y^H W0 (b x b): four columns per block, T in shared
-// memory.  (As two products of b x b x b on the tensor-core engine: four launches.)
+// M (2b x b) = [T; -U / 2], U = T^H (Z T) for Z = Y^H W0 (b x b): one column per block of 4 b threads (four to
+// an output, each a quarter of the sum), T in shared memory.  (As two products of b x b x b on the tensor-core
+// engine: four launches.  With four columns per block it took 17 us for b = 32 and 29 us for b = 64.)
 template <class T>
 __global__ void __launch_bounds__(256) k_sbr_coef(int b, const T* Z, const T* Tm, T* M) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* Ts = reinterpret_cast<T*>(smraw);  // b x b, ld b + 1
-  T* Q = Ts + b * (b + 1);              // Z T(:, j): b x 4
-  const int tid = threadIdx.x, j0 = blockIdx.x * 4;
-  for (int t = tid; t < b * b; t += 256) Ts[t % b + (t / b) * (b + 1)] = Tm[t];
+  T* red = Ts + b * (b + 1);            // 4 x b
+  T* Q = red + 4 * b;                   // Z T(:, j)
+  const int tid = threadIdx.x, j = blockIdx.x, i = tid % b, h = tid / b, kq = b / 4;
+  for (int t = tid; t < b * b; t += 4 * b) Ts[t % b + (t / b) * (b + 1)] = Tm[t];
   __syncthreads();
-  const int i = tid % b, stp = 256 / b;
-  for (int jl = tid / b; jl < 4; jl += stp) {
-    const int j = j0 + jl;
-    T acc = zero_<T>(), acc1 = zero_<T>();
+  T acc = zero_<T>();
 #pragma unroll 4
-    for (int k = 0; k < b; k += 2) {
-      acc += Z[i + k * b] * Ts[k + j * (b + 1)];
-      acc1 += Z[i + (k + 1) * b] * Ts[k + 1 + j * (b + 1)];
-    }
-    Q[i + jl * b] = acc + acc1;
-  }
+  for (int k = h * kq; k < (h + 1) * kq; ++k) mac(acc, Z[i + k * b], Ts[k + j * (b + 1)]);
+  red[tid] = acc;
   __syncthreads();
-  for (int jl = tid / b; jl < 4; jl += stp) {
-    const int j = j0 + jl;
-    T acc = zero_<T>(), acc1 = zero_<T>();
+  if (h == 0) Q[i] = (red[i] + red[b + i]) + (red[2 * b + i] + red[3 * b + i]);
+  __syncthreads();
+  acc = zero_<T>();
 #pragma unroll 4
-    for (int k = 0; k < b; k += 2) {
-      acc += cmul(Ts[k + i * (b + 1)], Q[k + jl * b]);
-      acc1 += cmul(Ts[k + 1 + i * (b + 1)], Q[k + 1 + jl * b]);
-    }
+  for (int k = h * kq; k < (h + 1) * kq; ++k) cmac(acc, Ts[k + i * (b + 1)], Q[k]);
+  red[tid] = acc;
+  __syncthreads();
+  if (h == 0) {
     M[i + j * 2 * b] = Ts[i + j * (b + 1)];
-    M[b + i + j * 2 * b] = from_re<T>(-0.5) * (acc + acc1);
+    M[b + i + j * 2 * b] = from_re<T>(-0.5) * ((red[i] + red[b + i]) + (red[2 * b + i] + red[3 * b + i]));
   }
 }
 
@@ -361,7 +362,7 @@ template <class T> int he2hb(Sys& s, T* A, int lda, int b) {
   T* prow = (T*)(nrm_part + 2 * 4096);        // 2 x b pivot rows
   T* w_part = prow + 2 * 128;                 // 2 x 4096 x b
   const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zero = zero_<T>();
-  const size_t coef_smem = sizeof(T) * ((size_t)b * (b + 1) + 4 * b);
+  const size_t coef_smem = sizeof(T) * ((size_t)b * (b + 1) + 5 * b);
   GEV_TRY(allow_dyn_smem(k_sbr_coef<T>, coef_smem));
   int npanel = 0, arrivals = 0;
   GEV_CUDA_TRY(cudaMemsetAsync(&s.status[ST_BARRIER_CNT], 0, 2 * sizeof(int), s.stream));
@@ -400,7 +401,7 @@ template <class T> int he2hb(Sys& s, T* A, int lda, int b) {
     gemm(s, gp<T>(m, b, m, 0, 0, one, A22, lda, Yp, n, zero, WY, n));  // W0 = A22 Y
     gemm(s, gp<T>(b, b, m, 2, 0, one, Yp, n, WY, n, zero, Z, b));      // Z = Y^H W0
     GEV_COUNT(s);
-    k_sbr_coef<T><<<b / 4, 256, coef_smem, s.stream>>>(b, Z, Tp, M);
+    k_sbr_coef<T><<<b, 4 * b, coef_smem, s.stream>>>(b, Z, Tp, M);
     GemmP<T> g = gp<T>(m, b, 2 * b, 0, 0, one, WY, n, M, 2 * b, zero, Wv, n);
     if (gemm_on_fp64_pipe(s, g)) {
       gemm(s, g);
