@@ -16,14 +16,14 @@
 //   2^24, so the FP32 tensor-memory accumulator holds them exactly.  After each chunk the six exact
 //   sums are added, as integers in units of 2^-49, to one 64-bit integer accumulator per output
 //   (exact; integer operations are cheap on GB300 while FP64 additions are not).  The diagonals
-//   d = 8, 9 share one FP32 accumulator over all of K; its roundings stay near 2^-51 of the scale.
+//   d = 8, 9 have an FP32 accumulator each over all of K; its roundings stay near 2^-51 of the scale.
 //
 // Data flow: a split pass writes the 8 digit planes of op(A) and op(B) to global memory in the
 // order the MMAs consume them (one 16-deep k-slice of a 128-row A tile = 8 planes x 4 KB,
 // contiguous; of a 64-column B tile = 8 x 2 KB), so the GEMM kernel moves them with plain bulk
 // asynchronous copies into a 4-stage shared-memory ring.  Warp roles: warp 16 issues the copies,
-// warp 17 issues the 36 MMAs per slice (tcgen05, accumulators in TMEM: 6 exact diagonals + 1
-// shared, 64 columns each), warps 0-15 (one TMEM lane per output row, a quarter of its 64 columns
+// warp 17 issues the MMAs (tcgen05, accumulators in TMEM: 8 diagonals of 64 columns, all of it), warps
+// 0-15 (one TMEM lane per output row, a quarter of its 64 columns
 // each) drain the exact accumulators at every chunk end and write C.  The kernel is persistent for
 // short K, and its epilogue uses integer arithmetic only (see to_fp64): together they took the
 // 8192 x 8192 x 128 update from 1.97 to 0.90 ms, back-transform 2 at n = 10240, k = 2560 from 365 to
@@ -55,8 +55,7 @@ constexpr int SMEM_OZ = NSTAGE * STAGE + 1024;
 constexpr int NEPI_W = 16;                 // epilogue warps: TMEM lanes 32 (w % 4), columns 16 (w / 4)
 constexpr int HC = ON / 4;                  // output columns per epilogue thread
 constexpr int NTH = 32 * (NEPI_W + 2);      // + copy warp 16 + MMA warp 17
-constexpr int TMEM_COLS_OZ = 512;
-constexpr int SHARED_SLOT = DEXACT - 1;    // TMEM slot of d = 8, 9; exact d at slot d - 2
+constexpr int TMEM_COLS_OZ = 512;          // diagonal d at columns (d - 2) ON
 constexpr int GROUP_M = 16;                // raster: 16 row tiles share their B slices in L2
 constexpr int EXP_BAD = 1 << 20;           // exponent marking a non-finite entry
 constexpr int EXP_ZERO = -4000;            // exponent of an all-zero vector
@@ -526,9 +525,10 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
       }
     }
   } else if (warp == NEPI_W + 1) {
-    // ---- MMA warp: 36 digit-pair products per 16-deep slice
+    // ---- MMA warp: the 36 digit-pair products of a 16-deep slice in 13 MMAs of up to 256 columns (an MMA of
+    // 64 columns took about 75 cycles for its 32 of tensor work, also with A kept in the collector buffer; 36 of
+    // them per slice ran 8192^3 in 41.9 ms, these 13 in 24.0 ms, 0.87 of the BF16 peak)
     if (lane == 0) {
-      const uint32_t id = idesc_bf16(OM, ON);
       int sg = 0, cg = 0;  // slices and chunks, over all items
       for (int it = blockIdx.x; it < items && !*err; it += gridDim.x) {
         const OzItem w = oz_item(p, it);
@@ -546,23 +546,30 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
           }
           *consumed = sg + 1;
           fence_after();
-          const uint32_t a0 = su32(smem + slot * STAGE), b0 = a0 + A_STAGE;
-#pragma unroll
-          for (int pa = 1; pa <= NSLICE; ++pa) {
-#pragma unroll
-            for (int qb = 1; qb + pa <= DMAX; ++qb) {
-              const int d = pa + qb;
-              int col, en;
-              if (d <= DEXACT) {  // the first pair of diagonal d (pa = 1) restarts it at a chunk start
-                col = (d - 2) * ON;
-                en = (chunk_start && pa == 1) ? 0 : 1;
-              } else {  // the shared slot starts with the item's first MMA of d = 8 (pa = 1, qb = 7)
-                col = SHARED_SLOT * ON;
-                en = (s == 0 && pa == 1 && qb == DEXACT) ? 0 : 1;
-              }
-              mma_bf16(tmem + col, sdesc16(a0 + (pa - 1) * A_TILE), sdesc16(b0 + (qb - 1) * B_TILE), id, en);
-            }
-          }
+          const uint32_t a0 = su32(smem + slot * STAGE);
+          const uint64_t ad = sdesc16(a0), bd = sdesc16(a0 + A_STAGE);
+          // plane pa of A against planes qb .. qb + w - 1 of B in one MMA (64 w columns): the planes are
+          // adjacent in shared memory and their diagonals d = pa + qb .. in tensor memory.  pa = 1 touches
+          // every diagonal first: it restarts the exact ones (d <= 7) at a chunk start and the last two at
+          // the item's start.
+          auto mma = [&](int pa, int qb, int w, int en) {
+            mma_bf16(tmem + (pa + qb - 2) * ON, ad + ((pa - 1) * A_TILE >> 4), bd + ((qb - 1) * B_TILE >> 4),
+                     idesc_bf16(OM, w * ON), en);
+          };
+          const int en = chunk_start ? 0 : 1;
+          mma(1, 1, 4, en);
+          mma(1, 5, 2, en);
+          mma(1, 7, 2, s > 0 ? 1 : 0);
+          mma(2, 1, 4, 1);
+          mma(2, 5, 3, 1);
+          mma(3, 1, 3, 1);
+          mma(3, 4, 3, 1);
+          mma(4, 1, 3, 1);
+          mma(4, 4, 2, 1);
+          mma(5, 1, 4, 1);
+          mma(6, 1, 3, 1);
+          mma(7, 1, 2, 1);
+          mma(8, 1, 1, 1);
           commit(su32(&empty[slot]));
           if ((s % CHUNK) == CHUNK - 1 || s == w.nst - 1) {
             commit(su32(cfull));
@@ -599,11 +606,14 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
         }
         fence_after();
         if (c == nchunk - 1) {
-          uint32_t r[16];
-          tmem_ld16(lane_base + (uint32_t)(SHARED_SLOT * ON), r);
-          tmem_wait_ld();
 #pragma unroll
-          for (int q = 0; q < HC; ++q) sh[q] = __uint_as_float(r[q]);
+          for (int d = DEXACT + 1; d <= DMAX; ++d) {
+            uint32_t r[16];
+            tmem_ld16(lane_base + (uint32_t)((d - 2) * ON), r);
+            tmem_wait_ld();
+#pragma unroll
+            for (int q = 0; q < HC; ++q) sh[q] += __uint_as_float(r[q]);
+          }
         }
 #pragma unroll
         for (int d = 2; d <= DEXACT; ++d) {
@@ -652,7 +662,8 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
             // an Inf / NaN entry reached this output
             if (any && (Ei >= EXP_BAD || fj[u] >= EXP_BAD)) v = __longlong_as_double(0x7FF8000000000000ll);
             if (p.ksplit == 1) {
-              if (p.amode == -1) v = -v;
+              // (a sign bit: negation is an FP64 instruction here)
+              if (p.amode == -1) v = __longlong_as_double(__double_as_longlong(v) ^ (long long)(1ull << 63));
               else if (p.amode == 0) v = p.alpha * v;
               if (p.bmode == 1) v += cin[u];
               else if (p.bmode == 2) v = fma(p.beta, cin[u], v);
