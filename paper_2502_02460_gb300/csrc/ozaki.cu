@@ -7,14 +7,14 @@
 //   row i of op(A) is scaled by 2^-(E_i+1), column j of op(B) by 2^-(F_j+1) (E, F: the smallest
 //   exponents with |x| < 2^E over the row / column), so every scaled entry lies in (-1/2, 1/2);
 //   X = x 2^(55-E) truncated to an integer (|X| < 2^55) is written in balanced radix 2^7,
-//   X = sum_{p=1..8} a_p 2^(56-7p) with integer digits |a_p| <= 64 (integer arithmetic only), and
-//   a_p 2^-7p is stored as BF16, exactly.
+//   X = sum_{p=1..8} a_p 2^(56-7p) with integer digits |a_p| <= 64 (integer arithmetic only), stored as
+//   BF16, exactly.
 //
-//   A B = 2^(E_i+F_j+2) sum_{p,q} (a_p 2^-7p)(b_q 2^-7q); pairs with p + q >= 10 (each below 2^-58
-//   of the scale) are dropped.  For d = p + q <= 7 the products of diagonal d are integers times
-//   2^-7d of magnitude <= 2^12; summed over a K chunk of 512 with at most 6 pairs they stay below
+//   A B = 2^(E_i+F_j+2) sum_{p,q} a_p b_q 2^-7(p+q); pairs with p + q >= 10 (each below 2^-58
+//   of the scale) are dropped.  For d = p + q <= 7 the products of diagonal d are integers of
+//   magnitude <= 2^12; summed over a K chunk of 512 with at most 6 pairs they stay below
 //   2^24, so the FP32 tensor-memory accumulator holds them exactly.  After each chunk the six exact
-//   sums are added, as integers in units of 2^-49, to one 64-bit integer accumulator per output
+//   sums are added, in units of 2^-49, to one 64-bit integer accumulator per output
 //   (exact; integer operations are cheap on GB300 while FP64 additions are not).  The diagonals
 //   d = 8, 9 have an FP32 accumulator each over all of K; its roundings stay near 2^-51 of the scale.
 //
@@ -155,9 +155,9 @@ __global__ void __launch_bounds__(256) k_vec_exp(Opnd2 q, int K, int slab, int s
 
 __device__ __forceinline__ int clamp_exp(int e) { return e < -1100 ? EXP_ZERO : e; }
 
-// the balanced radix-2^7 digits of x 2^(55-E) (|x| < 2^E), as floats a_p 2^-7p.  X + sum_p 2^6 2^(56-7p)
+// the balanced radix-2^7 digits a_p of x 2^(55-E) (|x| < 2^E), as floats.  X + sum_p 2^6 2^(56-7p)
 // has the digits a_p + 64 in its plain 7-bit fields (the top one may reach 128), so a digit is a shift, a
-// mask that also sets the exponent of 1.5 2^23, and one exact FMA: no carries and no integer conversion.
+// mask that also sets the exponent of 1.5 2^23, and one exact subtraction: no carries, no integer conversion.
 __device__ __forceinline__ void digits(double x, int E, float out[NSLICE]) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const int be = (int)((bits >> 52) & 0x7FF);
@@ -178,8 +178,7 @@ __device__ __forceinline__ void digits(double x, int E, float out[NSLICE]) {
 #pragma unroll
   for (int p = 1; p <= NSLICE; ++p) {
     const uint32_t f = (uint32_t)(Y >> (56 - 7 * p)) & (p == 1 ? 0xFFu : 0x7Fu);
-    const float sc = __int_as_float((127 - 7 * p) << 23);  // 2^-7p
-    out[p - 1] = fmaf(__int_as_float(0x4B400000 | f), sc, -(12582912.0f + 64.0f) * sc);  // exact
+    out[p - 1] = __int_as_float(0x4B400000 | f) - (12582912.0f + 64.0f);  // exact
   }
 }
 
@@ -460,6 +459,41 @@ __device__ __forceinline__ double to_fp64(long long acc, float sh, int e) {
   return __longlong_as_double((long long)(b | (neg ? 1ull << 63 : 0ull)));
 }
 
+// The same where neither zero, NaN, overflow nor subnormal results can occur (|e| < 1000): sh is split into
+// 32-bit integer and fraction by FP32 conversions, and the 96 bits are normalised as three words with funnel
+// shifts.  About half the instructions; with the other per-output work thinned out too, a 6144 x 6144 x 128 update
+// went from 515 to 330 us (splits included; its MMAs are about 160).
+__device__ __forceinline__ double to_fp64_fast(long long acc, float sh, int e, uint32_t flip) {
+  const float x = sh * 562949953421312.0f;  // 2^49: |x| < 2^31
+  const int xi = __float2int_rd(x);
+  uint32_t l = __float2uint_rz((x - __int2float_rn(xi)) * 4294967296.0f);  // the fraction, [0, 1)
+  acc += xi;
+  const uint32_t neg = (uint32_t)((int)(acc >> 32) >> 31);  // all ones for a negative sum: two's complement
+  const unsigned long long mag = ((unsigned long long)acc ^ (((unsigned long long)neg << 32) | neg)) + (l == 0 ? neg & 1u : 0u);
+  l = (l ^ neg) + (neg & 1u);
+  uint32_t h = (uint32_t)(mag >> 32), m = (uint32_t)mag;
+  int ex = 63 - 49 + e + 1022;
+  if (h == 0) {
+    h = m;
+    m = l;
+    l = 0;
+    ex -= 32;
+    if (h == 0) {
+      h = m;
+      m = 0;
+      ex -= 32;
+      if (h == 0) return 0.0;
+    }
+  }
+  const int lz = __clz((int)h);
+  h = __funnelshift_l(m, h, lz);
+  m = __funnelshift_l(l, m, lz);
+  const uint32_t t = (m & 0x7FFu) | ((l << lz) != 0u ? 1u : 0u), up = (t + 0x3FFu + ((m >> 11) & 1u)) >> 11;
+  const uint32_t w0 = __funnelshift_r(m, h, 11), r0 = w0 + up;
+  const uint32_t w1 = (h >> 11) + (r0 < w0 ? 1u : 0u) + ((uint32_t)(ex - lz) << 20);
+  return __hiloint2double((int)(w1 | ((neg ^ flip) & 0x80000000u)), (int)r0);
+}
+
 // Persistent: a CTA per SM walks over the work items.  The copy warp runs ahead into the next item's
 // slices while the epilogue works, and the epilogue first drains all sums of an item into registers and
 // releases the tensor memory, so the conversion to FP64, the loads of C and the stores overlap the next
@@ -611,24 +645,26 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
             uint32_t r[16];
             tmem_ld16(lane_base + (uint32_t)((d - 2) * ON), r);
             tmem_wait_ld();
+            const float sc = __int_as_float((127 - 7 * d) << 23);  // 2^-7d
 #pragma unroll
-            for (int q = 0; q < HC; ++q) sh[q] += __uint_as_float(r[q]);
+            for (int q = 0; q < HC; ++q) sh[q] = fmaf(__uint_as_float(r[q]), sc, sh[q]);
           }
         }
+        // the sums of diagonal d are integers below (d - 1) 512 2^12: two neighbouring diagonals make one 32-bit
+        // integer (2^7 S_d + S_{d+1} < 2^31), and a wide multiply-add puts it in units of 2^-49
 #pragma unroll
-        for (int d = 2; d <= DEXACT; ++d) {
-          // the sums are integers times 2^-7d below 2^24: exact as 32-bit integers, one wide
-          // multiply-add each into units of 2^-49
+        for (int d = 2; d <= DEXACT; d += 2) {
           uint32_t r[16];
+          int t[HC];
           tmem_ld16(lane_base + (uint32_t)((d - 2) * ON), r);
           tmem_wait_ld();
-          const float up = __int_as_float((127 + 7 * d) << 23);  // 2^7d
-          const int f = 1 << (d == 2 ? 30 : 49 - 7 * d);
 #pragma unroll
-          for (int q = 0; q < HC; ++q) {
-            const long long t = (long long)__float2int_rn(__uint_as_float(r[q]) * up) * f;
-            acc[q] += d == 2 ? t << 5 : t;
-          }
+          for (int q = 0; q < HC; ++q) t[q] = __float2int_rn(__uint_as_float(r[q])) << 7;
+          tmem_ld16(lane_base + (uint32_t)((d - 1) * ON), r);
+          tmem_wait_ld();
+#pragma unroll
+          for (int q = 0; q < HC; ++q)
+            acc[q] += (long long)(t[q] + __float2int_rn(__uint_as_float(r[q]))) * (1 << (49 - 7 * (d + 1)));
         }
         fence_before();
         __syncwarp();
@@ -641,6 +677,33 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
       const int cmax = p.c_lower ? min(p.N, (gi >> rs) + 1) : p.N;  // columns [0, cmax) of this row are wanted
       double* crow = p.ksplit > 1 ? p.ws + (long long)w.z * p.M * p.N + gi : p.C + gi;
       const long long ld = p.ksplit > 1 ? p.M : p.ldc;
+      // Every exponent of the warp's rows and columns in the middle of the range, alpha = +-1, beta = 0 or 1 (or
+      // partial sums): the short conversion, with nothing else in its loop (one FP64 addition per output when C
+      // is added; a choice among multiplications and additions is evaluated in full otherwise).
+      {
+        const int gq = w.n0 + col0 + (lane & (HC - 1));
+        const int fl = (any && gq < p.N) ? p.F[gq] : 0;
+        const bool mid = any && (!row_ok || (Ei > -400 && Ei < 400)) && fl > -400 && fl < 400;
+        if (__all_sync(0xffffffffu, mid) && (p.ksplit > 1 || (p.amode != 0 && p.bmode != 2))) {
+          const uint32_t flip = (p.ksplit == 1 && p.amode == -1) ? 0xFFFFFFFFu : 0u;
+          const int nc = row_ok ? min(HC, cmax - (w.n0 + col0)) : 0;  // outputs of this thread
+          double* cp = crow + (long long)(w.n0 + col0) * ld;
+#pragma unroll
+          for (int h = 0; h < HC; h += 8) {
+            double cin[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) cin[u] = (read_c && h + u < nc) ? cp[(h + u) * ld] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              const int fj = __shfl_sync(0xffffffffu, fl, h + u);
+              double v = to_fp64_fast(acc[h + u], sh[h + u], Ei + fj + 2, flip);
+              if (read_c) v += cin[u];
+              if (h + u < nc) cp[(h + u) * ld] = v;
+            }
+          }
+          continue;
+        }
+      }
       if (row_ok) {
 #pragma unroll
         for (int h = 0; h < HC; h += 4) {
