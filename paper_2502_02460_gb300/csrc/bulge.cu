@@ -84,17 +84,18 @@ __device__ __forceinline__ void bar_arrive_n(int id, int n) { asm volatile("bar.
 //    warps equally: on GB300 the FP64 pipe, about 1.6 FMA per SM per cycle, bounds this kernel), their
 //    sums as a second, the three updates as a third.  Column 0 of the updated E, the next
 //    reflector's x, is E(:,0) - z (v_0 = 1): it comes out of the second phase, so warp 0 computes the
-//    next reflector (reduction, rsqrt, division: a long latency chain) while the other warps
-//    update, publishes it as soon as the stores of this task are done (a named barrier that the other
-//    warps only arrive at), and they wait for the next task's blocks and load them meanwhile.
+//    next reflector (reduction, rsqrt, reciprocal: a long latency chain) while the other warps
+//    update, wait for the next task's blocks and load them.  A warp of its own publishes the progress as
+//    soon as the stores of this task are done (a barrier that the others only arrive at): the release waits
+//    about 1000 cycles for the stores, in the middle of the chain when warp 0 issued it.
 //    Warp 1 finishes y (its inner product with v) while the rest update L and E.
 //  * Four barriers per task; D and E travel through registers, so that no wait holds the others up.
-// Measured (to_tridiag; one barrier-separated product after another and a lag of three tasks before):
-// real FP64 n = 10240, b = 64 447 -> 203 ms, n = 1500 37.1 -> 16.1 ms; complex FP64 n = 509 29.7 -> 13.2 ms;
-// FP32 n = 6144 82.9 -> 40.9 ms.
+// Measured (to_tridiag; one barrier-separated product after another, a lag of three tasks and the release in
+// warp 0 at first): real FP64 n = 10240, b = 64 447 -> 190 ms (bound by the FP64 pipe: 14000 of a task's 16000
+// cycles), n = 1500, b = 32 37.1 -> 12.2 ms; complex FP64 n = 509 29.7 -> 9.4 ms; FP32 n = 6144 82.9 -> 40 ms.
 // All arithmetic is in the data's own precision (FP32 for the mixed form).
 template <class T, int B, int NTH>
-__global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T* tau2, int ntask, int* progress,
+__global__ void __launch_bounds__(NTH + 32) k_bulge(int n, T* band, int ldb, T* V2, T* tau2, int ntask, int* progress,
                                                int* status, int* abort_flag, int stall) {
   using R = typename real_of<T>::type;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -117,6 +118,24 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
   if (tid == 0) bad = 0;
   __syncthreads();
 
+  // The publisher (the last warp): waits for the stores of a task (barrier 1, where the others only arrive) and
+  // releases the sweep's progress.  Barrier 3, in the middle of a task, keeps the others from completing barrier 1
+  // twice before it has left it once.
+  if (warp == NTH / 32) {
+    for (int s = blockIdx.x; s <= n - 3; s += gridDim.x)
+      for (int t = 0;; ++t) {
+        const int pn = s + 1 + t * B + B;
+        const bool more = pn < n && min(B, n - pn) > 1;
+        bar_sync_n(3, NTH + 32);
+        if (bad) return;
+        bar_sync_n(1, NTH + 32);
+        if (bad) return;
+        if (lane == 0) st_release(&progress[s], more ? t + 2 : INT_MAX);
+        if (!more) break;
+      }
+    return;
+  }
+
   // warp 0: the reflector of the B entries x (zero beyond len) -> v, conj(v) is formed with the loads
   auto reflect = [&](const T* x, T* v, int slot) {
     T xv[(B + 31) / 32];
@@ -130,7 +149,7 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
     s2 = warp_sum(s2);
     const T alpha = x[0];
     T tau = zero_<T>(), beta = alpha, scale = zero_<T>();
-    if (!(s2 == (R)0 && im_(alpha) == 0)) house(alpha, s2, tau, beta, scale);
+    if (!(is_zero(s2) && im_(alpha) == 0)) house(alpha, s2, tau, beta, scale);
 #pragma unroll
     for (int u = 0; u < (B + 31) / 32; ++u) {
       const int i = lane + 32 * u;
@@ -205,8 +224,11 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
         __syncwarp();
         for (int i = lane; i < B; i += 32) vc[i] = conj_(v[i]);
       }
-      __syncthreads();
-      if (bad) return;  // (uniform: set before the barrier, never cleared)
+      bar_sync_n(0, NTH);
+      if (bad) {  // (uniform: set before the barrier, never cleared)
+        bar_arrive_n(3, NTH + 32);
+        return;
+      }
       const T tau = sh_tau[cur];
       // ---- partial sums of w = v^H L, y = D v, z = E v: P threads per output
       {
@@ -224,7 +246,7 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
         }
         part[tid] = acc + acc2;
       }
-      __syncthreads();
+      bar_sync_n(0, NTH);
       for (int o = tid; o < O3; o += NTH) {
         T acc = part[o];
 #pragma unroll
@@ -238,15 +260,15 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
           xn_[i] = Es[i] - zz;
         }
       }
-      __syncthreads();
+      bar_sync_n(3, NTH + 32);
       if (warp == 0) {
         // ---- the next reflector, published once this task's stores are done
         if (more) {
           const T beta = reflect(xn_, vn, cur ^ 1);
           if (lane == 0) stcg_(&band[B + (long long)p * ldb], beta);
         }
-        bar_sync_n(1, NTH);
-        if (more && lane == 0) st_release(&progress[s], t + 2);
+        __syncwarp();
+        if (more) bar_arrive_n(1, NTH + 32);
       } else {
         if (warp == 1) {
           // y <- tau y - c v, c = |tau|^2 Re(v^H y) / 2
@@ -304,8 +326,8 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
           stcg_(&band[(long long)(p + i) * ldb],
                 from_re<T>(re_(Ds[i + i * LD]) - (R)2 * (R)re_(mulc(y[i], v[i]))));
         __syncwarp();
-        bar_arrive_n(1, NTH);
         if (more) {
+          bar_arrive_n(1, NTH + 32);
           fetch(t + 1);
           bar_sync_n(2, NL);  // every warp has left D, E and L: the next task may overwrite them
         }
@@ -324,6 +346,8 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
                 stcg_(&band[(B - q) + (long long)(p + q) * ldb], q == 0 ? xn_[0] : Es[q * LD]);
           }
         }
+        __syncwarp();
+        bar_arrive_n(1, NTH + 32);
         break;
       }
       T* tmp = Ls;
@@ -331,9 +355,8 @@ __global__ void __launch_bounds__(NTH) k_bulge(int n, T* band, int ldb, T* V2, T
       Es = tmp;
       cur ^= 1;
     }
-    __syncthreads();
+    bar_sync_n(0, NTH);
     if (bad) return;
-    if (tid == 0) st_release(&progress[s], INT_MAX);
   }
 }
 
@@ -690,7 +713,7 @@ template <class T, int B> int launch_bulge(Sys& s, int n, T* band, int ldb) {
   const size_t smem = bulge_smem<T>(B);
   GEV_TRY(allow_max_dyn_smem(k_bulge<T, B, NTH>));
   int per_sm = 0;
-  GEV_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bulge<T, B, NTH>, NTH, smem));
+  GEV_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bulge<T, B, NTH>, NTH + 32, smem));
   if (per_sm < 1) return GEV_ERR_UNSUPPORTED;
   // Sweep s+1 trails sweep s by a little over two tasks and a sweep runs (n - s) / b tasks, so at most
   // about n / (2b) sweeps are in flight: more blocks would only hold SMs (in a spin wait) that other
@@ -708,7 +731,7 @@ template <class T, int B> int launch_bulge(Sys& s, int n, T* band, int ldb) {
   int* ab = &s.status[ST_ABORT];
   void* args[] = {&nn, &band, &lb, &V2, &tau2, &nt, &prog, &st, &ab, &stall};
   GEV_COUNT(s);
-  GEV_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_bulge<T, B, NTH>, dim3(G), dim3(NTH), args, smem, s.stream));
+  GEV_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_bulge<T, B, NTH>, dim3(G), dim3(NTH + 32), args, smem, s.stream));
   return 0;
 }
 

@@ -124,7 +124,7 @@ template <> struct real_of<float> { using type = float; };
 template <> struct real_of<zf> { using type = float; };
 
 // --------------------------------------------------------------- FP64-pipe arithmetic (device) --
-// 1 / d: the hardware's 20-bit reciprocal and two Newton-Raphson steps (y += y (1 - d y)),
+// 1 / d: the hardware's 20-bit reciprocal and one third-order step (y += y (e + e^2), e = 1 - d y),
 // within an ulp of the quotient (about half a division's FP64 instructions); outside the exponents where the
 // steps are safe, zero and the non-finite ones included, the division
 __device__ __forceinline__ double recip(double d) {
@@ -132,9 +132,21 @@ __device__ __forceinline__ double recip(double d) {
   if (e < 24 || e > 2020) return 1.0 / d;
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(d));
-  y = fma(y, fma(-d, y, 1.0), y);
-  return fma(y, fma(-d, y, 1.0), y);
+  const double r = fma(-d, y, 1.0);
+  return fma(y, fma(r, r, r), y);
 }
+// 1 / sqrt(q), q > 0, the same way: y += y e (1/2 + 3/8 e), e = 1 - q y^2
+__device__ __forceinline__ double recip_sqrt(double q) {
+  const int e = (__double2hiint(q) >> 20) & 0x7FF;
+  if (e < 24 || e > 2020) return rsqrt(q);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(q));
+  const double r = fma(-(q * y), y, 1.0);
+  return fma(fma(0.375, r, 0.5), r * y, y);
+}
+// v == 0 without an FP64 comparison
+__device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) << 1) == 0; }
+__device__ __forceinline__ bool is_zero(float v) { return v == 0.f; }
 
 // acc += a b, conj(a) b, a conj(b), and the subtractions: two multiply-adds per component of complex data
 // (written with the operators they are a product, a multiply-add and an addition, and an FP64 instruction
@@ -171,14 +183,16 @@ template <class Z> __device__ __forceinline__ void nmacc(Z& c, Z a, Z b) {
 }
 
 // ------------------------------------------------------------------------------- reflectors --
-// 1 / sqrt and the Householder scalars of alpha = x_0 and xn = sum_{i>0} |x_i|^2 (not both trivial):
+// The Householder scalars of alpha = x_0 and xn = sum_{i>0} |x_i|^2 (not both trivial):
 // with s = sign(Re alpha), r = 1 / ||x||:  beta = -s ||x||,  tau = 1 - alpha / beta = 1 + s r alpha,
-// scale = 1 / (alpha - beta): one reciprocal square root and one division, no other long FP64 chain
+// scale = 1 / (alpha - beta) (real data: s r / tau): one reciprocal square root and one reciprocal, no other long
+// FP64 chain
 __device__ __forceinline__ void house(double alpha, double xn, double& tau, double& beta, double& scale) {
-  const double q = alpha * alpha + xn, r = rsqrt(q), nrm = q * r;
-  beta = alpha >= 0.0 ? -nrm : nrm;
-  tau = 1.0 + fabs(alpha) * r;
-  scale = recip(alpha - beta);
+  const double q = fma(alpha, alpha, xn), r = recip_sqrt(q);
+  const double sr = copysign(r, alpha);
+  tau = fma(fabs(alpha), r, 1.0);
+  beta = -(q * sr);
+  scale = sr * recip(tau);
 }
 __device__ __forceinline__ void house(float alpha, float xn, float& tau, float& beta, float& scale) {
   const float nrm = sqrtf(alpha * alpha + xn);
@@ -187,7 +201,7 @@ __device__ __forceinline__ void house(float alpha, float xn, float& tau, float& 
   scale = 1.f / (alpha - beta);
 }
 __device__ __forceinline__ void house(zd alpha, double xn, zd& tau, zd& beta, zd& scale) {
-  const double q = abs2_(alpha) + xn, r = rsqrt(q), nrm = q * r;
+  const double q = abs2_(alpha) + xn, r = recip_sqrt(q), nrm = q * r;
   const double s = alpha.x >= 0.0 ? 1.0 : -1.0;
   const zd d = make_zd(alpha.x + s * nrm, alpha.y);
   const double g = recip(abs2_(d));

@@ -57,7 +57,7 @@ template <class T> struct PanelArgs {
 // partial sums and the barrier's flag travel through L2 once each, all partial sums a thread adds are
 // loaded together (20 or 40 at a time), the reflector is one rsqrt and one division, and the two warps
 // that need its inner products compute it themselves.  Per panel, averages over a reduction: n = 1500, b = 32
-// 275 us at first, about 170 now; n = 10240, b = 64 782, about 520 now; complex n = 509, b = 32 440, about 220 now.
+// 275 us at first, 168 now; n = 10240, b = 64 782 -> 537; complex n = 509, b = 32 440 -> 270.
 // The partial-sum buffers alternate with the column's parity: a block may start column c + 1 while a
 // slower one still reads column c's sums, but column c + 2 waits for everyone at barrier c + 1.
 template <class T, int B>
@@ -300,7 +300,7 @@ template <class T, int B> int launch_panel(Sys& s, PanelArgs<T> a, int* arrivals
 
 // M (2b x b) = [T; -U / 2], U = T^H (Z T) for Z = Y^H W0 (b x b): one column per block of 4 b threads (four to
 // an output, each a quarter of the sum), T in shared memory.  (As two products of b x b x b on the tensor-core
-// engine: four launches.  With four columns per block it took 17 us for b = 32 and 29 us for b = 64.)
+// engine: four launches.  Four columns per block took 17 us for b = 32 and 29 us for b = 64, one 5.9 and 9.3 us.)
 template <class T>
 __global__ void __launch_bounds__(256) k_sbr_coef(int b, const T* Z, const T* Tm, T* M) {
   extern __shared__ __align__(16) unsigned char smraw[];
