@@ -4,7 +4,7 @@
 //  * Tearing (Cuppen): at every split m (between rows m-1 and m) with rho = e[m-1]:
 //      T = diag(T1 - |rho| e_last e_last^T, T2 - |rho| e_1 e_1^T) + |rho| u u^T,
 //      u = e_{m-1} + sign(rho) e_m.
-//  * Leaves (<= 32 rows): implicit QL with shifts, one block per leaf.
+//  * Leaves (<= 16 rows): implicit QL with shifts, one block per leaf.
 //  * Merge of two solved children T1' = Q1 D1 Q1^T, T2' = Q2 D2 Q2^T:
 //      T' = Q (D + r zz^T) Q^T,  z = [last row of Q1, sign(rho) first row of Q2] / sqrt(2),
 //      r = 2|rho|.  The poles (children eigenvalues, each list sorted) are merged by rank;
@@ -29,7 +29,10 @@ namespace gev {
 
 namespace {
 
-constexpr int LEAF = 32;
+constexpr int LEAF = 32;        // rows a leaf kernel holds
+// rows of a leaf, at most: the QL chain of 32 rows took 1.0 ms whatever the order, one of 16 rows a quarter, and the
+// merge level more costs about 0.15 ms
+constexpr int LEAF_ROWS = 16;
 constexpr double EPS = 2.220446049250313e-16;
 
 struct Node {
@@ -517,8 +520,9 @@ __device__ void eval_secular(int K, int j, int o, const double* delta, const dou
   f = 1.0 + r * (psi + phi);
 }
 
-// One warp per root (blockDim 256: 8 roots per block); lane 0 writes the result.
-__global__ void __launch_bounds__(256) k_secular(Node* nodes, DcArrays A, int* status) {
+// One warp per root, four to a block (one per scheduler: a warp's FP64 instructions do not wait for another's while
+// there are fewer roots than SMs hold); lane 0 writes the result.
+__global__ void __launch_bounds__(128) k_secular(Node* nodes, DcArrays A, int* status) {
   const Node nd = nodes[blockIdx.y];
   const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const bool lead = (threadIdx.x & 31) == 0;
@@ -827,7 +831,7 @@ int stedc(Sys& s, const double* d, const double* e, int k, double* w, double* Z,
   GEV_CUDA_TRY(cudaMemsetAsync(Qa, 0, sizeof(double) * (size_t)n * n, st));
   GEV_CUDA_TRY(cudaMemsetAsync(Qb, 0, sizeof(double) * (size_t)n * n, st));
   int nleaf = 1;
-  while ((n + nleaf - 1) / nleaf > LEAF) nleaf *= 2;
+  while ((n + nleaf - 1) / nleaf > LEAF_ROWS) nleaf *= 2;
   const unsigned eb = cdiv(n, 256) < 1024u ? cdiv(n, 256) : 1024u;
   GEV_CUDA_TRY(cudaMemsetAsync(&s.status[ST_DEFLATED], 0, sizeof(int), st));
   GEV_COUNT(s);
@@ -851,7 +855,7 @@ int stedc(Sys& s, const double* d, const double* e, int k, double* w, double* Z,
     k_merge_prep<<<nnodes, PREP_NTH, 0, st>>>(n, nleaf, span, A.nodes, e, w, Qa, ldq, A);
     GEV_TRY(last_error());
     GEV_COUNT(s);
-    k_secular<<<dim3(cdiv(smax, 8), nnodes), 256, 0, st>>>(A.nodes, A, s.status);
+    k_secular<<<dim3(cdiv(smax, 4), nnodes), 128, 0, st>>>(A.nodes, A, s.status);
     GEV_COUNT(s);
     k_zprime<<<dim3(cdiv(smax, 8), nnodes), 256, 0, st>>>(A.nodes, A);
     const int kcut = top ? k : 0x7fffffff;
