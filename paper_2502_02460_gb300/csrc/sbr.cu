@@ -89,6 +89,25 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
   __syncthreads();
   const int jj = tid % B, grp = tid / B;
   const int ncol = min(B, m);
+  // column c of T from the inner products in wv: T(0:c, c) = -tau T(0:c, 0:c) s, T(c, c) = tau; B threads
+  auto t_column = [&](int c) {
+    const int i = tid - (NT - B);
+    const T tau = wv[c];
+    T val = zero_<T>();
+    if (i < c) {
+      T acc = zero_<T>(), acc1 = zero_<T>();
+      int l = i;
+      for (; l + 1 < c; l += 2) {
+        mac(acc, Tw[i + l * B], wv[l]);
+        mac(acc1, Tw[i + (l + 1) * B], wv[l + 1]);
+      }
+      if (l < c) mac(acc, Tw[i + l * B], wv[l]);
+      val = -(tau * (acc + acc1));
+    } else if (i == c) {
+      val = tau;
+    }
+    Tw[i + c * B] = val;
+  };
 
   for (int c = 0; c < ncol; ++c) {
     const int par = c & 1;
@@ -121,6 +140,8 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
       }
     }
     __syncthreads();
+    // column c - 1 of T, while the others arrive (its inner products are in wv until the barrier)
+    if (blk == 0 && c > 0 && tid >= NT - B) t_column(c - 1);
     if (tid == 0) {
       asm volatile("red.release.gpu.global.add.s32 [%0], 1;\n" ::"l"(a.count) : "memory");
       const int target = a.base + (c + 1) * G;
@@ -213,7 +234,7 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
       if (tid == c) sc[c] = scale;
     }
     __syncthreads();
-    // ---- C: apply H^H to the remaining columns; column c of T (block 0, the one with the fewest rows left)
+    // ---- C: apply H^H to the remaining columns
     if (jj > c) {
       const T w = w2[jj];
       for (int r = max(0, c + 1 - lo) + grp; r < rows; r += NG) nmac(base[r + jj * ld], base[r + c * ld], w);
@@ -222,26 +243,10 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
       if (tid > c) base[(c - lo) + tid * ld] -= wv[tid];
       else base[(c - lo) + c * ld] = sh_beta;
     }
-    if (blk == 0 && tid >= NT - B) {
-      const int i = tid - (NT - B);
-      const T tau = wv[c];
-      T val = zero_<T>();
-      if (i < c) {
-        T acc = zero_<T>(), acc1 = zero_<T>();
-        int l = i;
-        for (; l + 1 < c; l += 2) {
-          mac(acc, Tw[i + l * B], wv[l]);
-          mac(acc1, Tw[i + (l + 1) * B], wv[l + 1]);
-        }
-        if (l < c) mac(acc, Tw[i + l * B], wv[l]);
-        val = -(tau * (acc + acc1));
-      } else if (i == c) {
-        val = tau;
-      }
-      Tw[i + c * B] = val;
-    }
     __syncthreads();
   }
+  if (blk == 0 && tid >= NT - B) t_column(ncol - 1);
+  __syncthreads();
   if (blk == 0)  // (columns beyond the last reflector: zero)
     for (int t = tid; t < B * B; t += NT) {
       if (t / B >= ncol) a.Tm[t] = zero_<T>();
