@@ -791,8 +791,7 @@ template <class T> int bt_levels_wy(Sys& s, int n, int k, int b, T* Y, int ldy) 
   const int ngroups = (n - 3) / b + 1;
   const int nlevels = ngroups + s.ntask;
   T* P = (T*)s.W1;  // (nblk b) x k products V^H Y (W1 is free during the back-transform)
-  T* Wb = (T*)s.Q;  // the W_j blocks of LCHUNK consecutive levels (Q is free once the divide and conquer is done)
-  constexpr int LCHUNK = 16;
+  T* Wb = (T*)s.Q;  // the W_j blocks of several consecutive levels (Q is free once the divide and conquer is done)
   size_t need = 0;
   int max_nblk = 0;
   for (int L = 0; L < nlevels; ++L) {
@@ -808,8 +807,10 @@ template <class T> int bt_levels_wy(Sys& s, int n, int k, int b, T* Y, int ldy) 
       need = std::max(need, gemm_f64_bdiag_scratch(rows, k, lb.nblk * b, 2 * b, b, cx));
     }
   }
-  if (need > s.ozws_bytes || (size_t)max_nblk * b * k * sizeof(T) > (size_t)n * n * sizeof(T) ||
-      (size_t)LCHUNK * max_nblk * 2 * b * b * sizeof(T) > (size_t)n * n * sizeof(double))
+  // levels whose W_j are formed in one launch: as many as the buffer holds
+  const size_t per_level = (size_t)std::max(max_nblk, 1) * 2 * b * b * sizeof(T);
+  const int LCHUNK = (int)std::min<size_t>(16, (size_t)n * n * sizeof(double) / per_level);
+  if (need > s.ozws_bytes || (size_t)max_nblk * b * k * sizeof(T) > (size_t)n * n * sizeof(T) || LCHUNK < 1)
     return GEV_ERR_UNSUPPORTED;
   const size_t smem = sizeof(T) * ((size_t)(2 * b + 1) * b + (size_t)b * (b + 1) + b) + 64;
   GEV_TRY(allow_dyn_smem(k_wy_level<T>, smem));

@@ -31,12 +31,13 @@ namespace gev {
 
 namespace {
 
-// band width of the k x k Rayleigh-Ritz solve: the caller's choice, else the library default (64; at
-// k = 4096 it measured faster than 32 and 16: the narrower band's cheaper bulge-chasing tasks do not pay
-// for the extra back-transform levels and thinner products)
-int rr_band(int want, int) {
+// band width of the k x k Rayleigh-Ritz solve (all k pairs): the caller's choice, else the width that measured
+// fastest for whole solves of that order (ms at b = 16 / 32 / 64: real 1000 33 / 32 / 38, 2048 - / 76 / 85, 4096
+// - / 233 / 222; complex 1024 64 / 66 / 137, 2048 - / 162 / 278)
+int rr_band(int want, int k, bool cx) {
   if (want == 16 || want == 32 || want == 64) return want;
-  return 0;
+  if (cx) return k <= 1024 ? 16 : 32;
+  return k < 4096 ? 32 : 64;
 }
 
 __device__ __forceinline__ double wsum(double v) {
@@ -376,10 +377,10 @@ int solve_mixed(Sys& s, const double* H, int ldh, const double* S, int lds, int 
     o.prec = GEV_PLAIN;
     o.timing = 0;
     o.workspace_limit = 0;
-    o.band_b = rr_band(s.opts.rr_band_b, k);
+    o.band_b = rr_band(s.opts.rr_band_b, k, false);
     o.fp64_emulation = s.emu_fp64;  // the Ritz pencil's products use the same FP64 engine
     o.check = 0;
-    o.one_stage = (s.opts.rr_one_stage == 1 || (s.opts.rr_one_stage == 0 && k >= 2048)) ? 1 : 2;
+    o.one_stage = s.opts.rr_one_stage == 1 ? 1 : 2;
     o.debug_stall = 0;
     gev_sys* h = nullptr;
     const int rc = gev_setup(&h, k, GEV_F64, &o);
@@ -601,10 +602,10 @@ int solve_mixed_cx(Sys& s, const zd* H, int ldh, const zd* S, int lds, int k, do
     o.prec = GEV_PLAIN;
     o.timing = 0;
     o.workspace_limit = 0;
-    o.band_b = rr_band(s.opts.rr_band_b, k);
+    o.band_b = rr_band(s.opts.rr_band_b, k, true);
     o.fp64_emulation = s.emu_fp64;
     o.check = 0;
-    o.one_stage = (s.opts.rr_one_stage == 1 || (s.opts.rr_one_stage == 0 && k >= 2048)) ? 1 : 2;
+    o.one_stage = s.opts.rr_one_stage == 1 ? 1 : 2;
     o.debug_stall = 0;
     gev_sys* h = nullptr;
     const int rc = gev_setup(&h, k, GEV_C128, &o);
