@@ -1,5 +1,5 @@
-"""Autotuner of the band width b of the two-stage tridiagonalisation (which is also the panel width of
-the one-stage route; each timed solve takes the route ``gev_opts.one_stage = 0`` picks automatically).
+"""Autotuner of the band width b of the two-stage tridiagonalisation, which ``gev_opts.one_stage = 0`` takes
+(b is also the panel width of the one-stage route).
 
 The full -> band step gains from a wide band (its products have inner dimension b), the bulge chasing
 and back-transform 2 lose from it (a band -> tridiagonal task costs ~6 b^2 flops on a 3n-task
