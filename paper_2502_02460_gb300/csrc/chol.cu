@@ -77,8 +77,8 @@ __device__ void inv_lower_blocked(int jb, const T* L, T* X, T* tmp) {
 //   1. warps 0 - 7 factor and invert the SB x SB diagonal block, one entry (i, j), j <= i, per thread:
 //      before pivot j the thread holds a_ij of the trailing matrix, after it x_ij of the inverse of the
 //      unit lower factor (a = L^ D L^^H, no square root in the chain of pivots).  Pivot p costs a thread one
-//      scaled row factor l_ip = a_ip / d_p and one multiply-add, a barrier and, in the one warp that owns
-//      the next pivot, its reciprocal; column p of a and row p of x travel through shared memory.  Meanwhile
+//      multiply-add, a barrier and, in the one warp that owns the next column, the pivot's reciprocal and the
+//      column's l_ip = a_ip / d_p; columns p of a and l and row p of x travel through shared memory.  Meanwhile
 //      warps 8 - 15 finish the trailing update of the step before (beyond this diagonal block) and form
 //      S = L(kb.., 0:kb) X(0:kb, 0:kb) for this block row of the inverse;
 //   2. all: L21 = A21 X11^H with the inverted diagonal block, and X(kb.., 0:kb) = -X11 S;
@@ -86,9 +86,15 @@ __device__ void inv_lower_blocked(int jb, const T* L, T* X, T* tmp) {
 // FP64 bounds it: 2 jb^3 / 6 multiply-adds at 1.7 per cycle on one SM are 28 us for 64 real rows (113 us
 // complex).  One warp gets a quarter of that rate at most (a warp instruction occupies its scheduler's FP64
 // unit for about 75 cycles), so a pivot chain in one warp's registers took 36 us for each 16 rows: 150 us for the
-// block, 70 us now.
+// block, 57 us now.
 // L goes to A (when wanted) and X = L^{-1} to Xout, both with zeros above the diagonal.  A non-positive
 // pivot records its index (first one, atomicCAS) and stops; nothing is written then.
+// d > 0 (and no NaN), on the bits: an FP64 comparison costs as much as a multiplication
+__device__ __forceinline__ bool positive(double d) {
+  const long long b = __double_as_longlong(d);
+  return b > 0 && b <= 0x7FF0000000000000ll;
+}
+
 constexpr int PD_NT = 512, PD_G = 256;  // threads in all, threads of the diagonal block's group
 template <class T>
 __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long lda, int want_l, T* Xout, long long ldx,
@@ -98,8 +104,8 @@ __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long ld
   T* X = L + NBMAX * LDS;
   T* S = X + NBMAX * LDS;  // SB x kb
   __shared__ int fail;
-  __shared__ T s_col[2][SB], s_row[2][SB];
-  __shared__ double s_rinv[2], s_d[SB], s_rs[SB];
+  __shared__ T s_col[2][SB], s_l[2][SB], s_row[2][SB];
+  __shared__ double s_d[SB], s_rs[SB];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) fail = 0;
   for (int t = tid; t < jb * jb; t += PD_NT) {
@@ -115,23 +121,23 @@ __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long ld
       const bool live = i < bs && j <= i;
       T a = live ? L[(kb + i) + (kb + j) * LDS] : zero_<T>();
       T x = from_re<T>(i == j ? 1.0 : 0.0);
-      // what pivot q needs: column q of a, row q of x, 1 / d_q
+      // what pivot q needs: column q of a and of l = a / d_q, row q of x
       auto publish = [&](int q) {
-        if (j == q && i >= q) s_col[q & 1][i] = a;
         if (i == q && j <= q) s_row[q & 1][j] = x;
-        if (warp == q / 2) {  // (uniform) the warp that holds (q, q)
+        if (warp == q / 2) {  // (uniform) the warp that holds column q
           const double dq = re_(shfl_(a, (q & 1) * SB + q));
-          const double ri = dq > 0.0 ? recip(dq) : 0.0;
-          if (lane == 0) {
-            s_rinv[q & 1] = ri;
-            s_d[q] = dq;
+          const double ri = positive(dq) ? recip(dq) : 0.0;
+          if (j == q && i >= q) {
+            s_col[q & 1][i] = a;
+            s_l[q & 1][i] = ri * a;
           }
+          if (lane == 0) s_d[q] = dq;
         }
       };
       publish(0);
       for (int p = 0; p < bs; ++p) {
         asm volatile("bar.sync 1, %0;\n" ::"n"(PD_G) : "memory");
-        if (!(s_d[p] > 0.0)) {
+        if (!positive(s_d[p])) {
           if (tid == 0) {
             fail = 1;
             atomicCAS(&status[ST_NOT_SPD], 0, j0 + kb + p + 1);
@@ -139,7 +145,7 @@ __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long ld
           break;  // uniform over the group
         }
         if (live && i > p) {
-          const T li = s_rinv[p & 1] * s_col[p & 1][i];
+          const T li = s_l[p & 1][i];
           const bool fac = j > p;
           const T m = fac ? conj_(s_col[p & 1][j]) : s_row[p & 1][j];
           T cur = fac ? a : x;
@@ -150,10 +156,10 @@ __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long ld
         if (p + 1 < bs) publish(p + 1);
       }
       asm volatile("bar.sync 1, %0;\n" ::"n"(PD_G) : "memory");
-      if (tid < bs) s_rs[tid] = s_d[tid] > 0.0 ? rsqrt(s_d[tid]) : 0.0;
+      if (tid < bs) s_rs[tid] = positive(s_d[tid]) ? recip_sqrt(s_d[tid]) : 0.0;
       asm volatile("bar.sync 1, %0;\n" ::"n"(PD_G) : "memory");
       if (live) {  // L = L^ D^{1/2} with l^_ij = a_ij / d_j, X = D^{-1/2} x
-        L[(kb + i) + (kb + j) * LDS] = i == j ? from_re<T>(sqrt(s_d[i])) : s_rs[j] * a;
+        L[(kb + i) + (kb + j) * LDS] = s_rs[j] * (i == j ? from_re<T>(s_d[i]) : a);
         X[(kb + i) + (kb + j) * LDS] = s_rs[i] * x;
       }
     } else if (kb > 0) {
