@@ -60,7 +60,11 @@ template <class T> struct PanelArgs {
 // 275 us at first, 168 now; n = 10240, b = 64 782 -> 537; complex n = 509, b = 32 440 -> 270.
 // The partial-sum buffers alternate with the column's parity: a block may start column c + 1 while a
 // slower one still reads column c's sums, but column c + 2 waits for everyone at barrier c + 1.
-template <class T, int B>
+//
+// CL > 0: the whole panel in one cluster of CL blocks.  A block then sends its sums (and the pivot row) to every block's
+// shared memory, and the grid barrier becomes the cluster's: no release through L2 (about 1000 cycles), no polls, no
+// partial sums from L2, CL of them instead of the grid's 50 to 150.
+template <class T, int B, int CL>
 __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
   constexpr int NT = panel_nt<B>(), NG = NT / B;
   constexpr bool LOW = sizeof(typename real_of<T>::type) == 4;  // FP32 data: norms in FP64
@@ -75,7 +79,10 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
   T* sc = w2 + B;                         // B: scales of the reflectors
   double* redn = reinterpret_cast<double*>(sc + B);  // NT / 32 + NG
   T* Ts = reinterpret_cast<T*>(redn + NT / 32 + NG); // B x B when t_smem
-  T* sm = Ts + (a.t_smem ? B * B : 0);               // the block's rows when use_smem
+  T* cw = Ts + (a.t_smem ? B * B : 0);               // cluster: 2 x CL x B sums, 2 x B pivot row, 2 x CL norms
+  T* cp = cw + 2 * CL * B;
+  double* cn = reinterpret_cast<double*>(cp + (CL ? 2 * B : 0));
+  T* sm = reinterpret_cast<T*>(cn + 2 * CL);         // the block's rows when use_smem
   __shared__ T sh_beta;
   __shared__ int s_ok;
   T* Tw = a.t_smem ? Ts : a.Tm;
@@ -127,53 +134,81 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
       if (LOW && jj == c) redn[NT / 32 + grp] = ss;
     }
     __syncthreads();
-    if (tid < B) {
-      T sum = red2[tid];
+    if constexpr (CL > 0) {
+      // group g sends to the blocks g, g + NG, ..
+      T sum = red2[jj];
 #pragma unroll
-      for (int g = 1; g < NG; ++g) sum += red2[g * B + tid];
-      stcg_(&wp_[(long long)blk * B + tid], sum);
-      if (lo <= c && c < hi) stcg_(&pr_[tid], base[(c - lo) + tid * ld]);  // the pivot row
-      if (LOW && tid == c) {
-        double s = 0.0;
-        for (int g = 0; g < NG; ++g) s += redn[NT / 32 + g];
-        __stcg(&np_[blk], s);
+      for (int g = 1; g < NG; ++g) sum += red2[g * B + jj];
+      const bool piv = lo <= c && c < hi;
+      const T pv = piv ? base[(c - lo) + jj * ld] : zero_<T>();
+      double nn = 0.0;
+      if (LOW && jj == c)
+        for (int g = 0; g < NG; ++g) nn += redn[NT / 32 + g];
+      for (int q = grp; q < CL; q += NG) {
+        st_peer(peer_addr(smem_u32(&cw[(par * CL + blk) * B + jj]), q), sum);
+        if (piv) st_peer(peer_addr(smem_u32(&cp[par * B + jj]), q), pv);
+        if (LOW && jj == c) st_peer(peer_addr(smem_u32(&cn[par * CL + blk]), q), nn);
       }
-    }
-    __syncthreads();
-    // column c - 1 of T, while the others arrive (its inner products are in wv until the barrier)
-    if (blk == 0 && c > 0 && tid >= NT - B) t_column(c - 1);
-    if (tid == 0) {
-      asm volatile("red.release.gpu.global.add.s32 [%0], 1;\n" ::"l"(a.count) : "memory");
-      const int target = a.base + (c + 1) * G;
-      int ok = 1;
-      if (ld_acquire(a.count) < target) {
-        volatile int* vab = a.abort_flag;
-        const long long lim = spin_limit(a.status);
-        long long it = 0;
-        while (ld_acquire(a.count) < target) {
-          if (*vab) { ok = 0; break; }
-          if (++it > lim) {
-            atomicCAS(&a.status[ST_TIMEOUT], 0, 101);
-            atomicExch(a.abort_flag, 1);
-            ok = 0;
-            break;
-          }
-          if (it > 64) __nanosleep(32);
+      __syncwarp();
+      asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+      // column c - 1 of T, while the others arrive
+      if (blk == 0 && c > 0 && tid >= NT - B) t_column(c - 1);
+      __syncwarp();
+      asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    } else {
+      if (tid < B) {
+        T sum = red2[tid];
+#pragma unroll
+        for (int g = 1; g < NG; ++g) sum += red2[g * B + tid];
+        stcg_(&wp_[(long long)blk * B + tid], sum);
+        if (lo <= c && c < hi) stcg_(&pr_[tid], base[(c - lo) + tid * ld]);  // the pivot row
+        if (LOW && tid == c) {
+          double s = 0.0;
+          for (int g = 0; g < NG; ++g) s += redn[NT / 32 + g];
+          __stcg(&np_[blk], s);
         }
       }
-      s_ok = ok;
+      __syncthreads();
+      // column c - 1 of T, while the others arrive (its inner products are in wv until the barrier)
+      if (blk == 0 && c > 0 && tid >= NT - B) t_column(c - 1);
+      if (tid == 0) {
+        asm volatile("red.release.gpu.global.add.s32 [%0], 1;\n" ::"l"(a.count) : "memory");
+        const int target = a.base + (c + 1) * G;
+        int ok = 1;
+        if (ld_acquire(a.count) < target) {
+          volatile int* vab = a.abort_flag;
+          const long long lim = spin_limit(a.status);
+          long long it = 0;
+          while (ld_acquire(a.count) < target) {
+            if (*vab) { ok = 0; break; }
+            if (++it > lim) {
+              atomicCAS(&a.status[ST_TIMEOUT], 0, 101);
+              atomicExch(a.abort_flag, 1);
+              ok = 0;
+              break;
+            }
+            if (it > 64) __nanosleep(32);
+          }
+        }
+        s_ok = ok;
+      }
+      __syncthreads();
+      if (!s_ok) return;
     }
-    __syncthreads();
-    if (!s_ok) return;
     // ---- B: the block sums, added by NG threads per column
     T pc = zero_<T>(), alpha = zero_<T>();
     if (tid < B) {
-      pc = ldcg_(&pr_[tid]);
-      alpha = ldcg_(&pr_[c]);
+      pc = CL ? cp[par * B + tid] : ldcg_(&pr_[tid]);
+      alpha = CL ? cp[par * B + c] : ldcg_(&pr_[c]);
     }
     {
       T part = zero_<T>();
-      for (int q0 = grp; q0 < G; q0 += NLD * NG) {
+      if constexpr (CL > 0) {
+#pragma unroll
+        for (int q = 0; q < CL; q += NG)
+          if (q + grp < CL) part += cw[(par * CL + q + grp) * B + jj];
+      }
+      for (int q0 = grp; CL == 0 && q0 < G; q0 += NLD * NG) {
         T v[NLD];
 #pragma unroll
         for (int u = 0; u < NLD; ++u) {
@@ -186,7 +221,7 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
       red2[tid] = part;
       if (LOW) {
         double x = 0.0;
-        for (int q = tid; q < G; q += NT) x += __ldcg(&np_[q]);
+        for (int q = tid; q < G; q += NT) x += CL ? cn[par * CL + q] : __ldcg(&np_[q]);
         for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
         if ((tid & 31) == 0) redn[tid >> 5] = x;
       }
@@ -267,39 +302,80 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
   }
 }
 
-template <class T, int B> size_t panel_smem(int R, int use_smem, int t_smem) {
+template <class T, int B, int CL> size_t panel_smem(int R, int use_smem, int t_smem) {
   constexpr int NT = panel_nt<B>();
   size_t s = (size_t)(NT + 3 * B) * sizeof(T) + (NT / 32 + NT / B) * sizeof(double) + 64;
   if (t_smem) s += (size_t)B * B * sizeof(T);
+  if (CL) s += (size_t)(2 * CL * B + 2 * B) * sizeof(T) + 2 * CL * sizeof(double);
   if (use_smem) s += (size_t)(R | 1) * B * sizeof(T);
   return s;
+}
+
+constexpr int PANEL_CL = 16;  // blocks of the one-cluster form (beyond the portable 8: asked for and checked)
+
+// Whether a panel of m rows goes to one cluster: its 16 SMs' FP64 pipe time for a column grows with m, the grid's
+// barrier does not.  full->band of the two forms (ms, grid / best limit): real n = 256, b = 32 1.38 / 1.02, 1500
+// 11.3 / 10.2 (limit 1000 to 2000), 3000 28.0 / 26.9 (1000 - 1500; 28.8 for all panels); b = 16 n = 2000 21.4 / 18.9 (from
+// 2000); b = 64 n = 3000 29.4 / 26.2 (2000); complex b = 16 n = 2000 40.1 / 39.5 (1000), b = 32 31.1 / 30.7 (500); FP32
+// n = 3000 22.9 / 22.2 (1000).
+template <class T, int B> bool panel_in_cluster(int m) {
+  const int lim = B == 16 ? 2400 : (B == 32 ? 1400 : 2000);
+  return m < (is_cx<T>::value ? lim / 3 : lim);
 }
 
 // The QR of one panel (a.m rows): rows per block, residence in shared memory when it fits.
 template <class T, int B> int launch_panel(Sys& s, PanelArgs<T> a, int* arrivals) {
   constexpr int NT = panel_nt<B>();
   const size_t cap = (size_t)200 * 1024;
-  GEV_TRY(allow_max_dyn_smem(k_panel_qr<T, B>));
+  if (panel_in_cluster<T, B>(a.m)) {
+    const auto kern = k_panel_qr<T, B, PANEL_CL>;
+    a.R = (a.m + PANEL_CL - 1) / PANEL_CL;
+    a.t_smem = a.use_smem = 1;
+    const size_t smem = panel_smem<T, B, PANEL_CL>(a.R, 1, 1);
+    if (smem <= cap) {
+      GEV_TRY(allow_max_dyn_smem(kern));
+      GEV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = PANEL_CL;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(PANEL_CL);
+      cfg.blockDim = dim3(NT);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = s.stream;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      int fit = 0;
+      if (cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) == cudaSuccess && fit >= 1) {
+        GEV_COUNT(s);
+        GEV_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a));
+        return 0;
+      }
+      cudaGetLastError();  // no cluster of this size here: the grid form
+    }
+  }
+  GEV_TRY(allow_max_dyn_smem(k_panel_qr<T, B, 0>));
   // Blocks: a column costs a block 2 R / 4 b / 32 multiply-adds of FP64 pipe time for its R = m / G rows (twice
   // that for complex data against additions) and G / 4 b / 32 additions for the G partial sums: least at G^2 = 2 m
   // (4 m).
   int G = std::min(s.sms, (int)std::ceil(std::sqrt((is_cx<T>::value ? 4.0 : 2.0) * a.m))), per_sm = 0;
   a.R = std::max(8, (a.m + G - 1) / G);
   G = (a.m + a.R - 1) / a.R;
-  a.t_smem = panel_smem<T, B>(a.R, 0, 1) <= cap ? 1 : 0;
-  a.use_smem = panel_smem<T, B>(a.R, 1, a.t_smem) <= cap ? 1 : 0;
-  if (!a.use_smem && panel_smem<T, B>(a.R, 1, 0) <= cap) {
+  a.t_smem = panel_smem<T, B, 0>(a.R, 0, 1) <= cap ? 1 : 0;
+  a.use_smem = panel_smem<T, B, 0>(a.R, 1, a.t_smem) <= cap ? 1 : 0;
+  if (!a.use_smem && panel_smem<T, B, 0>(a.R, 1, 0) <= cap) {
     a.t_smem = 0;
     a.use_smem = 1;
   }
-  const size_t smem = panel_smem<T, B>(a.R, a.use_smem, a.t_smem);
-  GEV_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_panel_qr<T, B>, NT, smem));
+  const size_t smem = panel_smem<T, B, 0>(a.R, a.use_smem, a.t_smem);
+  GEV_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_panel_qr<T, B, 0>, NT, smem));
   if (per_sm < 1 || G > per_sm * s.sms || G > 4096) return GEV_ERR_UNSUPPORTED;
   a.base = *arrivals;
   *arrivals += G * std::min(a.m, B);
   void* args[] = {&a};
   GEV_COUNT(s);
-  GEV_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_panel_qr<T, B>, dim3(G), dim3(NT), args, smem, s.stream));
+  GEV_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_panel_qr<T, B, 0>, dim3(G), dim3(NT), args, smem, s.stream));
   return 0;
 }
 
