@@ -870,15 +870,23 @@ void emulate(Sys& s, int M, int N, int K, Opnd a, size_t a_kstep, Opnd b, size_t
     p.MT = MT; p.NT = NT; p.KT = KT;
     p.alpha = alpha; p.beta = (k0 == 0) ? beta : 1.0;
     p.C = C; p.ldc = ldc; p.Ap = Ap; p.Bp = Bp; p.E = E; p.F = F; p.status = s.status;
-    // split K when the output has too few tiles to fill the GPU; a share is at least 8 slices (about 7 us
-    // of MMAs, of the order of the launch that sums the shares)
+    // split K when the output has too few tiles to fill the GPU in whole rounds; a share is at least 8 slices.  The cost
+    // in slices (0.6 us): rounds of items, each with its first copies, drain and epilogue, and the pass that sums the
+    // shares (launch, and their bytes at 5 TB/s).
     long long tiles = (long long)MT * NT;
     if (c_lower) tiles = (tiles + MT) / 2;
     int ks = 1;
-    if (2 * tiles <= s.sms && KT >= 16) {
-      ks = (int)std::min<long long>(s.sms / tiles, KT / 8);
-      ks = std::min(ks, 64);
-      while (ks > 1 && (size_t)ks * M * N * sizeof(double) > s.splitws_bytes) --ks;
+    if (tiles < 2 * s.sms && KT >= 16) {
+      const double item = 14.0, sum0 = 8.0, sum1 = (double)M * N * sizeof(double) / 3e6;
+      double best = cdiv(tiles, s.sms) * (KT + item);
+      for (int c = 2; c <= std::min(64, KT / 8); ++c) {
+        if ((size_t)c * M * N * sizeof(double) > s.splitws_bytes) break;
+        const double cost = cdiv(tiles * c, s.sms) * ((double)KT / c + item) + sum0 + sum1 * c;
+        if (cost < 0.97 * best) {
+          best = cost;
+          ks = c;
+        }
+      }
     }
     p.ksplit = ks;
     p.ws = ks > 1 ? static_cast<double*>(s.splitws) : nullptr;
