@@ -200,17 +200,15 @@ __device__ __forceinline__ void store_pair(double x0, double x1, int E, unsigned
 // Digit planes of both operands in one launch.  A warp takes 8 vectors x 16 elements (one slice of one
 // 8-row group): lane = 4 (row) + pair, so that every plane receives two contiguous 128-byte rows of core
 // matrices and global memory is read in 64-byte runs whichever index is contiguous.
-__global__ void __launch_bounds__(256) k_split(Opnd2 q, int K, int KT) {
-  const int w = blockIdx.x < q.nblk0 ? 0 : 1;
-  const long long blk = blockIdx.x - (w ? q.nblk0 : 0);
+__device__ __forceinline__ void split_tile(const Opnd2& q, int w, long long u, int K, int KT) {
   const Opnd o = q.o[w];
   const int R = q.R[w], TR = q.TR[w], lane = threadIdx.x & 31;
-  const long long RG = (long long)q.RT[w] * (TR / 8), u = blk * 8 + (threadIdx.x >> 5);
+  const long long RG = (long long)q.RT[w] * (TR / 8);
   if (u >= RG * KT) return;
   long long rg, kt;
   if (q.fast[w]) { rg = u % RG; kt = u / RG; } else { kt = u % KT; rg = u / KT; }
   const long long r = rg * 8 + (lane >> 2);
-  const int Er = (r < R) ? clamp_exp(q.E[w][r]) : EXP_ZERO;
+  const int Er = (r < R) ? (q.E[w] ? clamp_exp(q.E[w][r]) : 1) : EXP_ZERO;  // (no exponents: every entry below 2)
   double x[4];
 #pragma unroll
   for (int h = 0; h < 4; ++h) {
@@ -222,6 +220,10 @@ __global__ void __launch_bounds__(256) k_split(Opnd2 q, int K, int KT) {
 #pragma unroll
   for (int h = 0; h < 2; ++h)
     store_pair(x[2 * h], x[2 * h + 1], Er, base + toff16((int)(r % TR), h * 8 + (lane & 3) * 2), tile_bytes);
+}
+__global__ void __launch_bounds__(256) k_split(Opnd2 q, int K, int KT) {
+  const int w = blockIdx.x < q.nblk0 ? 0 : 1;
+  split_tile(q, w, (long long)(blockIdx.x - (w ? q.nblk0 : 0)) * 8 + (threadIdx.x >> 5), K, KT);
 }
 
 // The same for K <= 16 NS in one pass: the warp holds its 8 vectors entirely, so the exponents come out
@@ -309,10 +311,8 @@ __device__ __forceinline__ double bd_at(const BdOp& o, long long i, long long kk
 // Row exponents and digit planes of a block-diagonal op(A) in the compact layout: row tile mt holds
 // only the slices of its K range (bd_range).  One warp per row of the padded MT x 128 rows; lane l
 // takes 8 consecutive columns of the range and writes 16 bytes to each plane.
-__global__ void k_split_bd(int M, BdOp o, int bm, int bk, int MT, int* E, unsigned char* out) {
-  const long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+__device__ __forceinline__ void split_bd_row(long long i, int M, const BdOp& o, int bm, int bk, int* E, unsigned char* out) {
   const int lane = threadIdx.x & 31;
-  if (i >= (long long)MT * OM) return;  // uniform per warp
   const int mt = (int)(i / OM);
   int f = 0, c = 0;
   bd_range(bm, bk, mt, &f, &c);
@@ -342,6 +342,36 @@ __global__ void k_split_bd(int M, BdOp o, int bm, int bk, int MT, int* E, unsign
   }
 }
 
+__global__ void __launch_bounds__(256) k_split_bd(int M, BdOp o, int bm, int bk, int MT, int* E, unsigned char* out) {
+  const long long i = (blockIdx.x * 256ll + threadIdx.x) >> 5;
+  if (i < (long long)MT * OM) split_bd_row(i, M, o, bm, bk, E, out);  // uniform per warp
+}
+
+// What the two products of a back-transform-2 level read, in one launch: the planes of both block-diagonal
+// operands and of the level's rows of Y.
+struct BdSide {
+  BdOp o;
+  int M, bm, bk, MT, nblk;  // nblk: grid blocks
+  int* E;
+  unsigned char* out;
+};
+__global__ void __launch_bounds__(256) k_level_prep(BdSide a1, BdSide a2, Opnd2 y, int K, int KT) {
+  int blk = blockIdx.x;
+  const int warp = threadIdx.x >> 5;
+  if (blk < a1.nblk) {
+    const long long i = blk * 8ll + warp;
+    if (i < (long long)a1.MT * OM) split_bd_row(i, a1.M, a1.o, a1.bm, a1.bk, a1.E, a1.out);
+    return;
+  }
+  blk -= a1.nblk;
+  if (blk < a2.nblk) {
+    const long long i = blk * 8ll + warp;
+    if (i < (long long)a2.MT * OM) split_bd_row(i, a2.M, a2.o, a2.bm, a2.bk, a2.E, a2.out);
+    return;
+  }
+  split_tile(y, 0, (blk - a2.nblk) * 8ll + warp, K, KT);
+}
+
 struct OzP {
   int M, N, K, koff, c_lower, tri_a, tri_b, cx;  // cx: complex product in the real embedding
   int MT, NT, KT, ksplit;
@@ -352,7 +382,7 @@ struct OzP {
   const unsigned char* Ap;
   const unsigned char* Bp;
   const int* E;
-  const int* F;
+  const int* F;  // null: 1 for every column (entries below 2)
   int* status;
   // block-diagonal op(A) (0: off): block j has rows [j bd_bm, (j+1) bd_bm) and its non-zero columns
   // [j bd_bk, (j+1) bd_bk); the A planes then hold, per row tile, only that tile's K range (compact)
@@ -682,7 +712,7 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
       // is added; a choice among multiplications and additions is evaluated in full otherwise).
       {
         const int gq = w.n0 + col0 + (lane & (HC - 1));
-        const int fl = (any && gq < p.N) ? p.F[gq] : 0;
+        const int fl = (any && gq < p.N) ? (p.F ? p.F[gq] : 1) : 0;
         const bool mid = any && (!row_ok || (Ei > -400 && Ei < 400)) && fl > -400 && fl < 400;
         if (__all_sync(0xffffffffu, mid) && (p.ksplit > 1 || (p.amode != 0 && p.bmode != 2))) {
           const uint32_t flip = (p.ksplit == 1 && p.amode == -1) ? 0xFFFFFFFFu : 0u;
@@ -713,7 +743,7 @@ __global__ void __launch_bounds__(NTH, 1) ozaki_kernel(OzP p) {
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             const int gj = w.n0 + col0 + h + u;
-            fj[u] = (any && gj < cmax) ? p.F[gj] : EXP_ZERO;
+            fj[u] = (any && gj < cmax) ? (p.F ? p.F[gj] : 1) : EXP_ZERO;
             cin[u] = (read_c && gj < cmax) ? crow[gj * ld] : 0.0;
           }
 #pragma unroll
@@ -964,18 +994,32 @@ BdLayout bd_layout(int Me, int N, int Ke, int bme, int bke) {
   return L;
 }
 
+// the product launch of a block-diagonal product (embedded units; blocks bme x bke)
+void launch_bdiag(Sys& s, const BdLayout& L, int Me, int N, int Ke, int rs, int bme, int bke, const int* E, const int* F,
+                  const unsigned char* Ap, const unsigned char* Bp, double alpha, double beta, void* C, long long ldc) {
+  OzP p{};
+  p.M = Me; p.N = N; p.K = Ke; p.koff = 0; p.c_lower = 0;
+  p.tri_a = 0; p.tri_b = 0; p.cx = rs;
+  p.MT = L.MT; p.NT = L.NT; p.KT = L.KT; p.ksplit = 1;
+  p.alpha = alpha; p.beta = beta;
+  p.C = static_cast<double*>(C);
+  p.ldc = ldc << rs;
+  p.ws = nullptr;
+  p.Ap = Ap; p.Bp = Bp; p.E = E; p.F = F; p.status = s.status;
+  p.bd_bm = bme;
+  p.bd_bk = bke;
+  p.amode = alpha_mode(alpha);
+  p.bmode = beta_mode(beta);
+  GEV_COUNT(s);
+  ozaki_kernel<<<std::min<long long>((long long)L.MT * L.NT, s.sms), NTH, SMEM_OZ, s.stream>>>(p);
+}
+
 }  // namespace
 
 size_t gemm_f64_bdiag_scratch(int M, int N, int K, int bm, int bk, int cx) {
   const int e = cx ? 2 : 1;
   return bd_layout(e * M, N, e * K, e * bm, e * bk).total;
 }
-
-namespace {
-__global__ void k_fill_exp(int n, int v, int* E) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) E[i] = v;
-}
-}  // namespace
 
 bool gemm_f64_bdiag(Sys& s, int M, int N, int K, const BdOp& a, int bm, int bk, const void* B, long long ldb,
                     double alpha, double beta, void* C, long long ldc, bool b_below_two) {
@@ -997,14 +1041,11 @@ bool gemm_f64_bdiag(Sys& s, int M, int N, int K, const BdOp& a, int bm, int bk, 
   Opnd2 q{};
   q.o[0] = b;
   q.R[0] = N;
-  q.E[0] = F;
+  q.E[0] = b_below_two ? nullptr : F;  // every entry of B below 2 in magnitude: exponent 1, no pass over B
   q.TR[0] = ON;
   q.RT[0] = L.NT;
   q.out[0] = Bp;
-  if (b_below_two) {  // every entry of B below 2 in magnitude: the column exponents are 1, no pass over B
-    GEV_COUNT(s);
-    k_fill_exp<<<cdiv(L.Np, 256), 256, 0, s.stream>>>((int)L.Np, 1, F);
-  } else if (Ke > 0) {
+  if (!b_below_two && Ke > 0) {
     q.nblk0 = (int)cdiv(N, 32);
     const int slab = exp_slab(s, q.nblk0, Ke), slabs = (int)cdiv(Ke, slab);
     if (slabs > 1) cudaMemsetAsync(F, 0x80, L.Np * sizeof(int), s.stream);
@@ -1016,21 +1057,46 @@ bool gemm_f64_bdiag(Sys& s, int M, int N, int K, const BdOp& a, int bm, int bk, 
     GEV_COUNT(s);
     k_split<<<q.nblk0, 256, 0, s.stream>>>(q, Ke, L.KT);
   }
-  OzP p{};
-  p.M = Me; p.N = N; p.K = Ke; p.koff = 0; p.c_lower = 0;
-  p.tri_a = 0; p.tri_b = 0; p.cx = rs;
-  p.MT = L.MT; p.NT = L.NT; p.KT = L.KT; p.ksplit = 1;
-  p.alpha = alpha; p.beta = beta;
-  p.C = static_cast<double*>(C);
-  p.ldc = ldc << rs;
-  p.ws = nullptr;
-  p.Ap = Ap; p.Bp = Bp; p.E = E; p.F = F; p.status = s.status;
-  p.bd_bm = bme;
-  p.bd_bk = bke;
-  p.amode = alpha_mode(alpha);
-  p.bmode = beta_mode(beta);
+  launch_bdiag(s, L, Me, N, Ke, rs, bme, bke, E, q.E[0], Ap, Bp, alpha, beta, C, ldc);
+  return true;
+}
+
+// One level of back-transform 2 on columns whose entries stay below 2 in magnitude:
+//   P (M1 x N) = op(A1) Y,  Y -= op(A2) P,   Y: rows x N, blocks b x 2b of A1 and 2b x b of A2 (complex units).
+// Four launches: the planes of A1, A2 and Y, the first product, the planes of P, the second product.  (Two exponent
+// fills, two launches for the A sides and two for the B sides before: 137 us a level at n = 4096, b = 32, k = 1229.)
+// False, with nothing launched, when s.ozws is too small.
+bool gemm_f64_bdiag_level(Sys& s, int M1, int rows, int N, const BdOp& a1, const BdOp& a2, int b, void* Y, long long ldy,
+                          void* P, long long ldp) {
+  if (M1 <= 0 || rows <= 0 || N <= 0) return true;
+  const int rs = a1.cx ? 1 : 0, be = b << rs;
+  const int Me = M1 << rs, Re = rows << rs;
+  const BdLayout L1 = bd_layout(Me, N, Re, be, 2 * be), L2 = bd_layout(Re, N, Me, 2 * be, be);
+  const size_t e2 = rup(L1.Mp * sizeof(int), 256), p1 = e2 + rup(L2.Mp * sizeof(int), 256);
+  const size_t p2 = p1 + (size_t)L1.MT * L1.acount * A_STAGE, bp = p2 + (size_t)L2.MT * L2.acount * A_STAGE;
+  if (!s.ozws || bp + (size_t)L1.NT * std::max(L1.KT, L2.KT) * B_STAGE > s.ozws_bytes) return false;
+  if (allow_dyn_smem(ozaki_kernel, SMEM_OZ) != 0) return false;
+  unsigned char* base = static_cast<unsigned char*>(s.ozws);
+  int* E1 = reinterpret_cast<int*>(base);
+  int* E2 = reinterpret_cast<int*>(base + e2);
+  unsigned char* Bp = base + bp;
+  const BdSide s1{a1, Me, be, 2 * be, L1.MT, (int)cdiv((long long)L1.MT * OM, 8), E1, base + p1};
+  const BdSide s2{a2, Re, 2 * be, be, L2.MT, (int)cdiv((long long)L2.MT * OM, 8), E2, base + p2};
+  Opnd2 q{};
+  q.o[0] = Opnd{Y, ldy, 1, 0, a1.cx ? 2 : 0, 0, 0};  // column j, element k
+  q.R[0] = N;
+  q.TR[0] = ON;
+  q.RT[0] = L1.NT;
+  q.out[0] = Bp;
   GEV_COUNT(s);
-  ozaki_kernel<<<std::min<long long>((long long)L.MT * L.NT, s.sms), NTH, SMEM_OZ, s.stream>>>(p);
+  k_level_prep<<<s1.nblk + s2.nblk + cdiv((long long)L1.NT * (ON / 8) * L1.KT, 8), 256, 0, s.stream>>>(s1, s2, q, Re, L1.KT);
+  launch_bdiag(s, L1, Me, N, Re, rs, be, 2 * be, E1, nullptr, base + p1, Bp, 1.0, 0.0, P, ldp);
+  q.o[0].X = P;
+  q.o[0].sr = ldp;
+  q.nblk0 = (int)cdiv((long long)L2.NT * (ON / 8) * L2.KT, 8);
+  GEV_COUNT(s);
+  k_split<<<q.nblk0, 256, 0, s.stream>>>(q, Me, L2.KT);
+  launch_bdiag(s, L2, Re, N, Me, rs, 2 * be, be, E2, nullptr, base + p2, Bp, -1.0, 1.0, Y, ldy);
   return true;
 }
 
