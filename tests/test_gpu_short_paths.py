@@ -1,10 +1,16 @@
-"""The paths taken by short work, at the sizes where they can go wrong.
+"""Paths chosen by size (short work, ragged edges, limits of a dispatch), at the sizes where they can go wrong.
 
 * Divide and conquer: batched merge products (nodes up to 384 rows) and the parallel deflation scan with
   its rotation runs, on tridiagonals that deflate in every way (equal leaves, glued Wilkinson blocks, zero
   couplings).  Bound: the method is backward stable, 64 n eps ||T||_1 as for the other FP64 steps.
 * Back-transform 2 reflector by reflector (16 columns per block, 8 lanes per column), at ragged windows and
   column counts, against the eigen-equation of the reduced matrix with the same bound.
+* Its tensor-core form with prepared levels (orders with n k b >= 3e7), ragged levels and columns: same bound.
+* Panels on both sides of the one-cluster limit: full -> band -> tridiagonal keeps trace and Frobenius norm to
+  64 n eps of the latter.
+* Emulated products whose K is shared by whole rounds of the SMs, and rows and columns whose exponents lie
+  outside the middle of the range (the general output conversion): |err| <= K s_i t_j 2^-51 with the powers of two
+  s_i, t_j above the largest entry of a row and a column (the scheme's normwise bound).
 """
 import numpy as np
 import pytest
@@ -81,3 +87,72 @@ def test_two_stage_back(dev, n, k, b, cx, emu):
         w = w.cpu().numpy()[:k]
     assert np.max(np.abs(A @ Y - Y * w)) <= 64 * n * EPS * norm
     assert np.max(np.abs(Y.conj().T @ Y - np.eye(k))) <= 64 * n * EPS
+
+
+@pytest.mark.parametrize("n,k,b,cx", [(1037, 1000, 32, False), (901, 901, 64, False), (611, 600, 32, True), (703, 703, 16, True)])
+def test_solve_with_prepared_levels(dev, n, k, b, cx):
+    import torch
+
+    from paper_2502_02460_gb300 import gev
+
+    g = torch.Generator(device=dev)
+    g.manual_seed(n)
+    dt = torch.complex128 if cx else torch.float64
+    H = torch.randn((n, n), generator=g, device=dev, dtype=dt)
+    H = H + H.mH
+    norm = float(H.abs().sum(dim=0).max())
+    with gev.Solver(n, complex_=cx, device=dev, band_b=b) as s:
+        w, C = s.solve(H, torch.eye(n, device=dev, dtype=dt), k)
+    assert float((H @ C - C * w).abs().max()) <= 64 * n * EPS * norm
+    assert float((C.mH @ C - torch.eye(k, device=dev, dtype=dt)).abs().max()) <= 64 * n * EPS
+
+
+@pytest.mark.parametrize("n,b,cx", [(23, 16, False), (1440, 32, False), (2075, 64, False), (2430, 16, False), (505, 32, True),
+                                    (830, 16, True), (740, 64, True)])
+def test_to_tridiagonal_keeps_norms(dev, n, b, cx):
+    import torch
+
+    from paper_2502_02460_gb300 import gev
+
+    g = torch.Generator(device=dev)
+    g.manual_seed(n)
+    A = torch.randn((n, n), generator=g, device=dev, dtype=torch.complex128 if cx else torch.float64)
+    A = (A + A.mH).contiguous()
+    trace, fro2 = float(A.diagonal().real.sum()), float((A.abs() ** 2).sum())
+    with gev.Solver(n, complex_=cx, device=dev, band_b=b) as s:
+        s.he2hb(gev.cm(A))
+        d, e = s.hb2st()
+    assert abs(float(d.sum()) - trace) <= 64 * n * EPS * fro2**0.5
+    assert abs(float((d * d).sum() + 2 * (e * e).sum()) - fro2) <= 64 * n * EPS * fro2
+
+
+@pytest.mark.parametrize("M,N,K,spread", [(9800, 64, 1000, 0), (130, 70, 5000, 0), (19500, 64, 300, 0), (300, 200, 77, 900),
+                                          (260, 130, 700, 500)])
+def test_emulated_product_shares_and_ranges(dev, M, N, K, spread):
+    import ctypes
+
+    import torch
+
+    from paper_2502_02460_gb300 import gev
+
+    L = gev.lib()
+    L.gev_gemm_f64_scratch_bytes.restype = ctypes.c_size_t
+    g = torch.Generator(device=dev)
+    g.manual_seed(M + K)
+    A = torch.randn((K, M), generator=g, device=dev, dtype=torch.float64)  # column-major M x K
+    B = torch.randn((K, N), generator=g, device=dev, dtype=torch.float64)  # column-major N x K (op(B) = B^T)
+    ea = torch.randint(-spread, spread + 1, (M,), generator=g, device=dev).to(torch.float64) // 2
+    ref = A.T @ B
+    A, B = A * torch.exp2(ea)[None, :], B * torch.exp2(-ea[:1]) if spread else B
+    ref = (ref * torch.exp2(ea)[:, None] * torch.exp2(-ea[:1])) if spread else ref
+    C = torch.empty((N, M), device=dev, dtype=torch.float64)
+    nb = L.gev_gemm_f64_scratch_bytes(M, N, K)
+    W = torch.empty(nb, dtype=torch.uint8, device=dev)
+    st = torch.zeros(16, dtype=torch.int32, device=dev)
+    p, d = (lambda t: ctypes.c_void_p(t.data_ptr())), ctypes.c_double
+    stream = ctypes.c_void_p(torch.cuda.current_stream(dev).cuda_stream)
+    rc = L.gev_gemm_f64(M, N, K, 0, 1, d(1.0), p(A), M, p(B), N, d(0.0), p(C), M, 1, stream, p(st), p(W), ctypes.c_size_t(nb))
+    assert rc == 0
+    s = torch.exp2(torch.floor(torch.log2(A.abs().amax(dim=0))) + 1)
+    t = torch.exp2(torch.floor(torch.log2(B.abs().amax(dim=0))) + 1)
+    assert bool(((C.T - ref).abs() <= K * s[:, None] * t[None, :] * 2.0**-51).all())
