@@ -25,6 +25,56 @@ namespace {
 // over a column's threads, a chain of FP64 additions in one warp, stay short.
 template <int B> constexpr int panel_nt() { return B == 64 ? 256 : 128; }
 
+// The sum of N <= 63 FP64 values in integer arithmetic: each is taken to 57 bits below the largest exponent and added
+// as a 64-bit integer, the total is rounded once.  An FP64 addition occupies a scheduler's pipe for 64 to 72 cycles, the
+// dozen integer instructions here for about 24.  The error is below N 2^-56 of the largest value (N 2^-53 of the partial
+// sums for additions), and the result does not depend on the order.  Exponents near either end: additions.
+template <int N> __device__ __forceinline__ double sum_block(const double (&v)[N]) {
+  static_assert(N < 64, "57 bits and the sum's carry fit 63");
+  int emax = 0;
+#pragma unroll
+  for (int u = 0; u < N; ++u) emax = max(emax, (__double2hiint(v[u]) >> 20) & 0x7FF);
+  if (emax < 100 || emax > 2000) {
+    double t = 0.0;
+#pragma unroll
+    for (int u = 0; u < N; ++u) t += v[u];
+    return t;
+  }
+  long long acc = 0;
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    const long long b = __double_as_longlong(v[u]);
+    const int sh = emax - ((int)(b >> 52) & 0x7FF);
+    const long long m = ((b & 0xFFFFFFFFFFFFFll) | (1ll << 52)) << 4;
+    const long long x = sh > 62 ? 0 : m >> sh;
+    acc += b < 0 ? -x : x;
+  }
+  if (acc == 0) return 0.0;
+  unsigned long long mag = acc < 0 ? 0ull - (unsigned long long)acc : (unsigned long long)acc;
+  const int lz = __clzll((long long)mag);
+  mag <<= lz;
+  const unsigned lo = (unsigned)mag & 0x7FFu;
+  unsigned long long r = mag >> 11;
+  r += (lo > 0x400u || (lo == 0x400u && (r & 1))) ? 1 : 0;
+  r += (unsigned long long)(emax + 6 - lz) << 52;  // (the mantissa's leading bit adds one to the exponent)
+  return __longlong_as_double((long long)(r | (acc < 0 ? 1ull << 63 : 0ull)));
+}
+template <int N> __device__ __forceinline__ zd sum_block(const zd (&v)[N]) {
+  double a[N], b[N];
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    a[u] = v[u].x;
+    b[u] = v[u].y;
+  }
+  return make_zd(sum_block(a), sum_block(b));
+}
+template <int N> __device__ __forceinline__ float sum_block(const float (&v)[N]) {
+  float t = 0.f;
+#pragma unroll
+  for (int u = 0; u < N; ++u) t += v[u];
+  return t;
+}
+
 template <class T> struct PanelArgs {
   int m, R, use_smem, t_smem;
   T* P;
@@ -57,7 +107,7 @@ template <class T> struct PanelArgs {
 // partial sums and the barrier's flag travel through L2 once each, all partial sums a thread adds are
 // loaded together (20 or 40 at a time), the reflector is one rsqrt and one division, and the two warps
 // that need its inner products compute it themselves.  Per panel, averages over a reduction: n = 1500, b = 32
-// 275 us at first, 168 now; n = 10240, b = 64 782 -> 537; complex n = 509, b = 32 440 -> 270.
+// 275 us at first, 168 now; n = 10240, b = 64 782 -> 480; complex n = 509, b = 32 440 -> 270.
 // The partial-sum buffers alternate with the column's parity: a block may start column c + 1 while a
 // slower one still reads column c's sums, but column c + 2 waits for everyone at barrier c + 1.
 //
@@ -215,8 +265,7 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
           const int q = q0 + u * NG;
           v[u] = q < G ? ldcg_(&wp_[(long long)q * B + jj]) : zero_<T>();
         }
-#pragma unroll
-        for (int u = 0; u < NLD; ++u) part += v[u];
+        part += sum_block(v);
       }
       red2[tid] = part;
       if (LOW) {
@@ -357,9 +406,9 @@ template <class T, int B> int launch_panel(Sys& s, PanelArgs<T> a, int* arrivals
   }
   GEV_TRY(allow_max_dyn_smem(k_panel_qr<T, B, 0>));
   // Blocks: a column costs a block 2 R / 4 b / 32 multiply-adds of FP64 pipe time for its R = m / G rows (twice
-  // that for complex data against additions) and G / 4 b / 32 additions for the G partial sums: least at G^2 = 2 m
-  // (4 m).
-  int G = std::min(s.sms, (int)std::ceil(std::sqrt((is_cx<T>::value ? 4.0 : 2.0) * a.m))), per_sm = 0;
+  // that for complex data against additions) and G / 4 b / 32 sums of a third of that time for the G partial sums: least
+  // at G^2 = 6 m (12 m).
+  int G = std::min(s.sms, (int)std::ceil(std::sqrt((is_cx<T>::value ? 12.0 : 6.0) * a.m))), per_sm = 0;
   a.R = std::max(8, (a.m + G - 1) / G);
   G = (a.m + a.R - 1) / a.R;
   a.t_smem = panel_smem<T, B, 0>(a.R, 0, 1) <= cap ? 1 : 0;
