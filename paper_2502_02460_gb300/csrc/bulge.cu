@@ -886,10 +886,11 @@ template <class T> int bt_hb2st(Sys& s, const double* Z, int ldz, int k, T* Y, i
     if (b == 64) return bt_levels_f32<64>(s, n, k, Y, ldy);
   }
   // FP64 data with the emulated product engine: each level as two block-diagonal tensor-core
-  // products of its compact-WY blocks, unless the level is short.  A level costs about 86 us in that form
-  // (six launches) + 0.26 ps n k b, and 12 us + 2.8 ps n k b reflector by reflector on the FP64 pipe
-  // (complex: four times the work in both): equal at n k b = 3e7.
-  constexpr double kBtNative = 3e7;
+  // products of its compact-WY blocks, unless the level is short: four launches against one.  Back-transform 2, ms, tensor
+  // cores / reflector by reflector, at n k b (complex: 4 n k b): real b = 32 16M 4.0 / 2.9, 24M 6.1 / 5.5, 30M 6.1 / 6.5,
+  // 38M 6.2 / 7.6; b = 16 12M 11.7 / 7.5, 24M 12.6 / 13.5; b = 64 19M 2.6 / 2.2, 32M 2.6 / 2.8; complex b = 16 20M 6.6 / 5.5,
+  // 41M 7.0 / 9.4; b = 32 20M 4.2 / 3.5, 41M 4.3 / 4.6.
+  constexpr double kBtNative = 2.6e7;
   if constexpr (std::is_same<T, double>::value || std::is_same<T, zd>::value) {
     const double fma = (double)n * k * b * (is_cx<T>::value ? 4 : 1);  // of a level, on the FP64 pipe
     if (s.emu_fp64 && fma >= kBtNative) {

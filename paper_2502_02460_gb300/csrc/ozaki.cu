@@ -25,9 +25,8 @@
 // warp 17 issues the MMAs (tcgen05, accumulators in TMEM: 8 diagonals of 64 columns, all of it), warps
 // 0-15 (one TMEM lane per output row, a quarter of its 64 columns
 // each) drain the exact accumulators at every chunk end and write C.  The kernel is persistent for
-// short K, and its epilogue uses integer arithmetic only (see to_fp64): together they took the
-// 8192 x 8192 x 128 update from 1.97 to 0.90 ms, back-transform 2 at n = 10240, k = 2560 from 365 to
-// 167 ms.  Every mbarrier wait is bounded; on expiry the kernel records ST_TIMEOUT, waits (bounded) for
+// short K, and its epilogue uses integer arithmetic only (see to_fp64).  8192^3 takes 24 ms (40 at first),
+// 6144 x 6144 x 128 0.33 ms (1.16), back-transform 2 at n = 10240, k = 2560 137 ms (365).  Every mbarrier wait is bounded; on expiry the kernel records ST_TIMEOUT, waits (bounded) for
 // its copies and MMAs in flight, frees TMEM and returns.
 #include <cuda_bf16.h>
 

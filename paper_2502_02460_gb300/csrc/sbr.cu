@@ -107,7 +107,7 @@ template <class T> struct PanelArgs {
 // partial sums and the barrier's flag travel through L2 once each, all partial sums a thread adds are
 // loaded together (20 or 40 at a time), the reflector is one rsqrt and one division, and the two warps
 // that need its inner products compute it themselves.  Per panel, averages over a reduction: n = 1500, b = 32
-// 275 us at first, 168 now; n = 10240, b = 64 782 -> 480; complex n = 509, b = 32 440 -> 270.
+// 275 us at first, 127 now (in a cluster); n = 10240, b = 64 782 -> 410; complex n = 509, b = 32 440 -> 270 (grid form).
 // The partial-sum buffers alternate with the column's parity: a block may start column c + 1 while a
 // slower one still reads column c's sums, but column c + 2 waits for everyone at barrier c + 1.
 //
