@@ -425,6 +425,8 @@ template <class T> int mult(Sys& s, const T* X, int ldx, const T* Y, int ldy, in
   const int n = s.n;
   GemmP<T> g = gp<T>(n, k, n, 2, 0, from_re<T>(1.0), X, ldx, Y, ldy, zero_<T>(), C, ldc);
   g.tri_a = 2;
+  // (a caller's C may be its Y: the digit planes are made before C is written)
+  g.alias = C < Y + (size_t)ldy * k && Y < C + (size_t)ldc * k ? 1 : 0;
   gemm(s, g);
   return last_error();
 }

@@ -264,6 +264,7 @@ template <class T> struct GemmP {
   int ksplit;  // set by the launcher
   T* ws;       // split-K partials (launcher-owned)
   int lowp;    // 1: FP64 operands, products and sums in FP32 (mixed form); 0: native precision
+  int alias;   // 1: C may be an operand's memory: the engine must have read both before it writes
 };
 
 struct Sys;

@@ -818,6 +818,9 @@ int stedc(Sys& s, const double* d, const double* e, int k, double* w, double* Z,
   A.colmap = (int*)take(ni4); A.colmap2 = (int*)take(ni4); A.dwork = (double*)take(nd8);
   A.nodes = (Node*)take(sizeof(Node) * (size_t)(n / 2 + 2));
   if ((size_t)(p - (char*)s.dcws) > s.dcws_bytes) return GEV_ERR_OOM;
+  // every list entry is a valid index from the start: where the input holds NaN, ranks collide and entries stay
+  // unwritten
+  GEV_CUDA_TRY(cudaMemsetAsync(s.dcws, 0, (size_t)(p - (char*)s.dcws), st));
 
   double* Qa = s.Q;
   double* Qb = s.Q2;

@@ -156,3 +156,21 @@ def test_emulated_product_shares_and_ranges(dev, M, N, K, spread):
     s = torch.exp2(torch.floor(torch.log2(A.abs().amax(dim=0))) + 1)
     t = torch.exp2(torch.floor(torch.log2(B.abs().amax(dim=0))) + 1)
     assert bool(((C.T - ref).abs() <= K * s[:, None] * t[None, :] * 2.0**-51).all())
+
+
+def test_mult_in_place(dev):
+    """C = X^T Y into Y's own memory, at a size of the short products."""
+    import torch
+
+    from paper_2502_02460_gb300 import gev
+
+    n, k = 100, 40
+    g = torch.Generator(device=dev)
+    g.manual_seed(1)
+    X = torch.randn((n, n), generator=g, device=dev, dtype=torch.float64).tril()
+    Y = torch.randn((n, k), generator=g, device=dev, dtype=torch.float64)
+    Xb, Yb = gev.cm(X), gev.cm(Y)
+    with gev.Solver(n, device=dev) as s:
+        p = gev._ptr
+        assert gev.lib().gev_step_mult(s.h, p(Xb), n, p(Yb), n, k, p(Yb), n) == 0
+    assert float((Yb.T - X.T @ Y).abs().max()) <= 1e-13 * n * float((X.T @ Y).abs().max())
