@@ -9,11 +9,12 @@
 //      T' = Q (D + r zz^T) Q^T,  z = [last row of Q1, sign(rho) first row of Q2] / sqrt(2),
 //      r = 2|rho|.  The poles (children eigenvalues, each list sorted) are merged by rank;
 //      deflation (|r z_i| <= tol, or two poles so close that a Givens rotation zeroing one
-//      z-component leaves an off-diagonal <= tol) is one sequential scan; the K remaining roots of
-//      the secular equation 1 + r sum z_i^2/(delta_i - lambda) = 0 are found one per thread in
+//      z-component leaves an off-diagonal <= tol) is tested in parallel, one by one only behind a
+//      rotation; the K remaining roots of
+//      the secular equation 1 + r sum z_i^2/(delta_i - lambda) = 0 are found one per warp in
 //      coordinates shifted to the nearest pole, by a bracketed two-pole rational iteration; z is
 //      recomputed from the roots (Gu-Eisenstat) so the eigenvectors u_j = z_i/(delta_i - lambda_j)
-//      are numerically orthogonal; the new eigenvectors Q u_j come from two GEMMs that use the
+//      are numerically orthogonal; the new eigenvectors Q u_j come from two products that use the
 //      block structure (columns that live in the top child only, in both, in the bottom only).
 //  * Columns are never physically sorted: colmap[a + p] gives the physical column of the p-th
 //    smallest eigenvalue of the node starting at a.  At the top merge only the k lowest
