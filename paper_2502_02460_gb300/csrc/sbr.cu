@@ -113,7 +113,8 @@ template <class T> struct PanelArgs {
 //
 // CL > 0: the whole panel in one cluster of CL blocks.  A block then sends its sums (and the pivot row) to every block's
 // shared memory, and the grid barrier becomes the cluster's: no release through L2 (about 1000 cycles), no polls, no
-// partial sums from L2, CL of them instead of the grid's 50 to 150.
+// partial sums from L2, CL of them instead of the grid's 50 to 150.  A block's shared memory may only be written once it
+// is known to run, so one cluster barrier stands before the first column; its arrivals overlap the load of the rows.
 template <class T, int B, int CL>
 __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
   constexpr int NT = panel_nt<B>(), NG = NT / B;
@@ -123,6 +124,7 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
   const int blk = blockIdx.x, tid = threadIdx.x, G = gridDim.x, m = a.m;
   const int lo = blk * a.R, hi = min(m, lo + a.R), rows = max(0, hi - lo);
   const long long lds = a.R | 1;
+  if constexpr (CL > 0) asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
   T* red2 = reinterpret_cast<T*>(smraw);  // NT
   T* wv = red2 + NT;                      // B: factors of the pivot row, then of s_j
   T* w2 = wv + B;                         // B: factors of the rows below
@@ -144,6 +146,7 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
       sm[r + c * lds] = a.P[(lo + r) + c * a.ldp];
     }
   __syncthreads();
+  if constexpr (CL > 0) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");  // every block has started
   const int jj = tid % B, grp = tid / B;
   const int ncol = min(B, m);
   // column c of T from the inner products in wv: T(0:c, c) = -tau T(0:c, 0:c) s, T(c, c) = tau; B threads
