@@ -62,7 +62,7 @@ int gev_step_stedc(gev_sys* s, const double* d, const double* e, int k, double* 
    dtype. */
 int gev_step_back(gev_sys* s, const double* Z, int ldz, int k, void* Y, int ldy);
 
-/* Step 7 (Mult.): C = X^H Y, X lower triangular (n x n), Y n x k. */
+/* Step 7 (Mult.): C = X^H Y, X lower triangular (n x n), Y n x k.  C may share memory with Y or X. */
 int gev_step_mult(gev_sys* s, const void* X, int ldx, const void* Y, int ldy, int k, void* C,
                   int ldc);
 

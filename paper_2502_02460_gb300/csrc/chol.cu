@@ -423,11 +423,14 @@ template <class T> int hegst(Sys& s, const T* H, int ldh, const T* X, int ldx, T
 
 template <class T> int mult(Sys& s, const T* X, int ldx, const T* Y, int ldy, int k, T* C, int ldc) {
   const int n = s.n;
-  GemmP<T> g = gp<T>(n, k, n, 2, 0, from_re<T>(1.0), X, ldx, Y, ldy, zero_<T>(), C, ldc);
+  // a caller's C may lie in the memory of its Y or X: the product then goes through the handle's scratch, whatever the engine
+  const bool over = overlap(C, ldc, n, k, Y, ldy, n, k) || overlap<T>(C, ldc, n, k, X, ldx, n, n);
+  T* out = over ? (T*)s.W1 : C;
+  const int ldo = over ? n : ldc;
+  GemmP<T> g = gp<T>(n, k, n, 2, 0, from_re<T>(1.0), X, ldx, Y, ldy, zero_<T>(), out, ldo);
   g.tri_a = 2;
-  // (a caller's C may be its Y: the digit planes are made before C is written)
-  g.alias = C < Y + (size_t)ldy * k && Y < C + (size_t)ldc * k ? 1 : 0;
   gemm(s, g);
+  if (over) GEV_TRY(copy2d<T>(s, n, k, out, ldo, C, ldc));
   return last_error();
 }
 

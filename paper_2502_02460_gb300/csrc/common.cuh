@@ -264,11 +264,19 @@ template <class T> struct GemmP {
   int ksplit;  // set by the launcher
   T* ws;       // split-K partials (launcher-owned)
   int lowp;    // 1: FP64 operands, products and sums in FP32 (mixed form); 0: native precision
-  int alias;   // 1: C may be an operand's memory: the engine must have read both before it writes
 };
 
 struct Sys;
 
+// whether two column-major matrices share memory (their address ranges, gaps between columns included)
+template <class T>
+bool overlap(const T* a, long long lda, int arows, int acols, const T* b, long long ldb, int brows, int bcols) {
+  const uintptr_t a0 = (uintptr_t)a, b0 = (uintptr_t)b;
+  const uintptr_t a1 = (uintptr_t)(a + (acols - 1) * lda + arows), b1 = (uintptr_t)(b + (bcols - 1) * ldb + brows);
+  return a0 < b1 && b0 < a1;
+}
+
+// C must not share memory with an operand: blocks write their outputs while others still read
 template <class T> void gemm(Sys& s, GemmP<T> p);
 // whether gemm() takes the FP64 pipe for this product of an emulating handle (gemm.cu)
 template <class T> bool gemm_on_fp64_pipe(const Sys& s, const GemmP<T>& p);

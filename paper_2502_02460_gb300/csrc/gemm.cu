@@ -337,7 +337,7 @@ template <class T> void gemm_small(Sys& s, GemmP<T> p) {
 // (a native one uses its DMMA kernel throughout) and with the tile counters of a workspace.
 template <class T> bool gemm_on_fp64_pipe(const Sys& s, const GemmP<T>& p) {
   constexpr double kFma = 1.2e7;
-  return s.emu_fp64 && s.tile_ctr && !p.alias && (double)p.M * p.N * p.K * (is_cx<T>::value ? 4.0 : 1.0) <= kFma;
+  return s.emu_fp64 && s.tile_ctr && (double)p.M * p.N * p.K * (is_cx<T>::value ? 4.0 : 1.0) <= kFma;
 }
 template <> bool gemm_on_fp64_pipe<float>(const Sys&, const GemmP<float>&) { return true; }
 template bool gemm_on_fp64_pipe<double>(const Sys&, const GemmP<double>&);

@@ -174,3 +174,34 @@ def test_mult_in_place(dev):
         p = gev._ptr
         assert gev.lib().gev_step_mult(s.h, p(Xb), n, p(Yb), n, k, p(Yb), n) == 0
     assert float((Yb.T - X.T @ Y).abs().max()) <= 1e-13 * n * float((X.T @ Y).abs().max())
+
+
+@pytest.mark.parametrize("emu", [0, 1])
+@pytest.mark.parametrize("cx", [False, True])
+@pytest.mark.parametrize("over", ["Y", "X", "Y shifted", "X shifted"])
+@pytest.mark.parametrize("n,k", [(100, 40), (100, 100), (300, 200)])
+def test_mult_over_an_operand(dev, n, k, over, cx, emu):
+    """C = X^H Y into memory that holds Y or X (also from its middle on), with either engine, below and above the size of the
+    short products (1.2e7 multiply-adds).  Bound: the emulated products' n s t (2^-52.6 + 2^-53 + n 2^-62.2) with
+    s <= 2 max |X|, t <= 2 max |Y|, twice that for complex data's double inner dimension and sqrt(2) for its two parts."""
+    import torch
+
+    from paper_2502_02460_gb300 import gev
+
+    g = torch.Generator(device=dev)
+    g.manual_seed(n + k)
+    dt = torch.complex128 if cx else torch.float64
+    X = torch.randn((n, n), generator=g, device=dev, dtype=dt).tril()
+    Y = torch.randn((n, k), generator=g, device=dev, dtype=dt)
+    ref = X.mH @ Y
+    mem = torch.zeros(2 * n * n + n * k + 7, dtype=dt, device=dev)  # X, then Y, then room behind it
+    Xb, Yb = mem[: n * n].view(n, n), mem[n * n: n * n + n * k].view(k, n)
+    Xb.copy_(X.T)
+    Yb.copy_(Y.T)
+    o = {"Y": n * n, "X": 0, "Y shifted": n * n + n + 7, "X shifted": n + 7}[over]
+    Cb = mem[o: o + n * k].view(k, n)
+    with gev.Solver(n, complex_=cx, device=dev, fp64_emulation=emu) as s:
+        p = gev._ptr
+        assert gev.lib().gev_step_mult(s.h, p(Xb), n, p(Yb), n, k, p(Cb), n) == 0
+    bound = 16 * n * 2.0**-51 * float(X.abs().max()) * float(Y.abs().max())
+    assert float((Cb.T - ref).abs().max()) <= bound
