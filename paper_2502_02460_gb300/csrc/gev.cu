@@ -19,7 +19,7 @@ namespace {
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Layout {
-  size_t off[40];
+  size_t off[32];
   int cnt = 0;
   size_t total = 0;
   size_t add(size_t bytes) {
@@ -81,9 +81,7 @@ size_t carve(Sys& s, char* base) {
   size_t obt = L.add(mixed && s.dtype == GEV_C128 ? (size_t)ldband * (n + 2 * b) * es : 8);
   // back-transform 1 groups of four panels: the group's T, Gram blocks and one block column
   size_t obtg = L.add(36 * b * b * es);
-  size_t octr = L.add(1024 * sizeof(int));
   if (base) {
-    s.tile_ctr = (int*)(base + octr);
     s.A = base + oA; s.X = base + oX; s.W1 = base + oW1; s.V1 = base + oV1; s.T1 = base + oT1;
     s.dinv = base + odinv; s.Pn = base + oPn; s.small = base + osmall;
     s.splitws = base + osplit; s.splitws_bytes = split;
@@ -91,7 +89,9 @@ size_t carve(Sys& s, char* base) {
     s.V2 = base + oV2; s.tau2 = base + otau2; s.ntask = (int)ntask; s.phase = base + ophase;
     s.d = (double*)(base + od); s.e = (double*)(base + oe); s.w = (double*)(base + ow);
     s.Q = (double*)(base + oQ); s.q_bytes = qbytes; s.Q2 = (double*)(base + oQ2);
-    s.dcws = base + odc; s.dcws_bytes = dcws;
+    // (the divide and conquer's arrays take 160 n bytes of its 512 n + 1 MB; the tile counters stand at its end)
+    s.dcws = base + odc; s.dcws_bytes = dcws - 1024 * sizeof(int);
+    s.tile_ctr = (int*)(base + odc + s.dcws_bytes);
     s.Yk = base + oYk;
     s.Zk = (double*)(base + oZk);
     s.prog = (int*)(base + oprog);
