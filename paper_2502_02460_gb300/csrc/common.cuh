@@ -362,7 +362,9 @@ struct Sys {
   int* tile_ctr = nullptr;  // arrival counters of split short products (gemm.cu), zero between launches
   void* V2 = nullptr;     // bulge-chasing reflectors, b x (n * ntask)
   void* tau2 = nullptr;   // (n * ntask)
-  int ntask = 0;          // max tasks per sweep
+  int ntask = 0;          // max tasks per sweep at the band width in use
+  void* tau2_ws = nullptr;  // the workspace's room for tau2: n * ntask_ws, the tasks at the handle's band width
+  int ntask_ws = 0;
   void* phase = nullptr;  // complex: diagonal phases folded into back-transform 2 (n)
   double* d = nullptr;    // tridiagonal diagonal (n)
   double* e = nullptr;    // off-diagonal (n)

@@ -86,7 +86,7 @@ size_t carve(Sys& s, char* base) {
     s.dinv = base + odinv; s.Pn = base + oPn; s.small = base + osmall;
     s.splitws = base + osplit; s.splitws_bytes = split;
     s.band = base + oband; s.ldband = ldband;
-    s.V2 = base + oV2; s.tau2 = base + otau2; s.ntask = (int)ntask; s.phase = base + ophase;
+    s.V2 = base + oV2; s.tau2 = s.tau2_ws = base + otau2; s.ntask = s.ntask_ws = (int)ntask; s.phase = base + ophase;
     s.d = (double*)(base + od); s.e = (double*)(base + oe); s.w = (double*)(base + ow);
     s.Q = (double*)(base + oQ); s.q_bytes = qbytes; s.Q2 = (double*)(base + oQ2);
     // (the divide and conquer's arrays take 160 n bytes of its 512 n + 1 MB; the tile counters stand at its end)

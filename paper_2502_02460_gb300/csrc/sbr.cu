@@ -497,6 +497,11 @@ template <class T> int he2hb(Sys& s, T* A, int lda, int b) {
   const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zero = zero_<T>();
   const size_t coef_smem = sizeof(T) * ((size_t)b * (b + 1) + 5 * b);
   GEV_TRY(allow_dyn_smem(k_sbr_coef<T>, coef_smem));
+  // tasks of a sweep of the chase that follows.  V2 holds b n ntask entries for every b up to the handle's width; the
+  // scalars of a narrower band outgrow their own room and go to Zk, which only complete solves (at the handle's width) use
+  s.ntask = (n + b - 1) / b + 2;
+  s.tau2 = s.ntask <= s.ntask_ws ? s.tau2_ws : (void*)s.Zk;
+  if (s.ntask > s.ntask_ws && sizeof(T) * (size_t)s.ntask > sizeof(double) * (size_t)n) return GEV_ERR_UNSUPPORTED;
   int npanel = 0, arrivals = 0;
   GEV_CUDA_TRY(cudaMemsetAsync(&s.status[ST_BARRIER_CNT], 0, 2 * sizeof(int), s.stream));
   for (int j0 = 0;; j0 += b) {

@@ -205,3 +205,24 @@ def test_mult_over_an_operand(dev, n, k, over, cx, emu):
         assert gev.lib().gev_step_mult(s.h, p(Xb), n, p(Yb), n, k, p(Cb), n) == 0
     bound = 16 * n * 2.0**-51 * float(X.abs().max()) * float(Y.abs().max())
     assert float((Cb.T - ref).abs().max()) <= bound
+
+
+@pytest.mark.parametrize("cx", [False, True])
+@pytest.mark.parametrize("n,k,width,b", [(300, 90, 64, 16), (300, 90, 64, 32), (37, 37, 32, 16), (1100, 700, 64, 16)])
+def test_band_narrower_than_the_handles(dev, n, k, width, b, cx):
+    """Reduction by steps with a narrower band than the handle's: its sweeps have more tasks.  Bound as above."""
+    from paper_2502_02460_gb300 import gev
+
+    rng = np.random.default_rng(n + b)
+    A = rng.standard_normal((n, n)) + (1j * rng.standard_normal((n, n)) if cx else 0)
+    A = A + A.conj().T
+    norm = np.abs(A).sum(axis=0).max()
+    with gev.Solver(n, complex_=cx, device=dev, band_b=width) as s:
+        for bb in (b, width, b):  # the handle's own width in between
+            assert s.he2hb(gev.cm_from_numpy(A, dev), bb) == bb
+            d, e = s.hb2st()
+            w, Z, _ = s.stedc(d, e, k)
+            Y = gev.numpy_from_cm(s.back(Z, k))
+            w = w.cpu().numpy()[:k]
+            assert np.max(np.abs(A @ Y - Y * w)) <= 64 * n * EPS * norm
+            assert np.max(np.abs(Y.conj().T @ Y - np.eye(k))) <= 64 * n * EPS
