@@ -74,7 +74,10 @@ typedef struct {
   int device;            /* CUDA device ordinal */
   void* cuda_stream;     /* cudaStream_t on that device (NULL = legacy default stream) */
   int prec;              /* gev_precision */
-  int band_b;            /* band width of the full->band step (0 = automatic; rounded up to 16, 32 or 64) */
+  int band_b;            /* band width of the full->band step (0 = automatic; rounded up to 16, 32 or 64).
+                            -16, -32, -64: solves use that width, and the workspace of a plain-form handle
+                            also holds the steps' bands to 32 (real data from n = 2048 on: 64), unless
+                            workspace_limit leaves no room for them */
   int panel_nb;          /* block size of Cholesky / inversion (0 = automatic) */
   double refine_tol;     /* mixed form: target residual (0 = 1e-11) */
   int refine_max_iter;   /* mixed form: refinement iteration cap (0 = 4) */

@@ -34,8 +34,8 @@ int gev_step_trtri(gev_sys* s, void* A, int lda);
 int gev_step_hegst(gev_sys* s, const void* H, int ldh, const void* X, int ldx, void* A, int lda);
 
 /* Step 4a (full -> band, two-stage tridiagonalisation stage 1): A (full Hermitian, both
-   triangles, overwritten) = Q1 B Q1^H with B of lower band width b (16, 32 or 64, at most the
-   width the handle was set up for; 0 = handle default).  The compact-WY blocks of Q1 and the band B stay in the handle for steps 4b
+   triangles, overwritten) = Q1 B Q1^H with B of lower band width b (16, 32 or 64, at most what
+   the handle was set up for; 0 = handle default).  The compact-WY blocks of Q1 and the band B stay in the handle for steps 4b
    and 6.  *b_used (host, optional) receives b. */
 int gev_step_he2hb(gev_sys* s, void* A, int lda, int b, int* b_used);
 

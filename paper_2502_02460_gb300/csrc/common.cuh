@@ -340,6 +340,7 @@ struct Sys {
   cudaStream_t stream = nullptr;
   int nb = 64;      // Cholesky / inversion block
   int b = 64;       // band width of the full -> band step
+  int b_cap = 64;   // widest one the workspace holds (steps)
   int sms = 152;
 
   // workspace (device)

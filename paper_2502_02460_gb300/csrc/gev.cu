@@ -38,9 +38,18 @@ int pick_band(int n, int want) {
   return p;
 }
 
+// The default width and the widest one the workspace holds.  band_b <= -16: a tuning table, not a user, chose the width of
+// solves, so that steps may ask for wider bands.
+void set_band(Sys& s) {
+  const int want = s.opts.band_b;
+  s.b = s.b_cap = pick_band(s.n, want <= -16 ? -want : want);
+  if (want <= -16 && s.opts.prec == GEV_PLAIN)
+    s.b_cap = std::max(s.b, s.dtype == GEV_F64 && s.n >= 2048 ? 64 : 32);
+}
+
 // Carve the workspace.  With base == nullptr only the size is computed.
 size_t carve(Sys& s, char* base) {
-  const size_t n = (size_t)s.n, es = s.es(), b = (size_t)s.b, nb = (size_t)s.nb;
+  const size_t n = (size_t)s.n, es = s.es(), b = (size_t)s.b_cap, nb = (size_t)s.nb;
   Layout L;
   size_t oA = L.add(n * n * es), oX = L.add(n * n * es), oW1 = L.add(n * n * es),
          oV1 = L.add(n * n * es), oT1 = L.add(b * (n + b) * es), odinv = L.add(nb * (n + nb) * es),
@@ -48,10 +57,10 @@ size_t carve(Sys& s, char* base) {
   size_t split = 4 * n * 2 * b * es;
   if (split < ((size_t)16 << 20)) split = (size_t)16 << 20;
   size_t osplit = L.add(split);
-  const int ldband = 3 * s.b + 2;
-  const size_t ntask = (n + b - 1) / b + 2;
+  const int ldband = 3 * s.b_cap + 2;
+  const size_t ntask = (n + s.b - 1) / s.b + 2;  // of solves, at the default width
   size_t oband = L.add((size_t)ldband * (n + 2 * b) * es);
-  size_t oV2 = L.add(b * n * ntask * es), otau2 = L.add(n * ntask * es), ophase = L.add(n * 16);
+  size_t oV2 = L.add(b * n * ((n + b - 1) / b + 2) * es), otau2 = L.add(n * ntask * es), ophase = L.add(n * 16);
   size_t od = L.add(n * 8), oe = L.add(n * 8), ow = L.add(n * 8);
   const size_t ntl = (n + 63) / 64;
   const size_t qbytes = std::max(n * n * 8, ntl * ntl * 64 * es);
@@ -133,7 +142,7 @@ int init_sys(Sys& s, int n, int dtype, const gev_opts* opts) {
   s.stream = (cudaStream_t)s.opts.cuda_stream;
   s.nb = 64;
   if (s.opts.panel_nb > 0 && s.opts.panel_nb < 64) s.nb = (s.opts.panel_nb + 7) / 8 * 8;
-  s.b = pick_band(n, s.opts.band_b);
+  set_band(s);
   s.emu_fp64 = s.opts.fp64_emulation < 0 ? 1 : (s.opts.fp64_emulation ? 1 : 0);
   s.fp32_tc = 0;
   if (s.opts.prec == GEV_MIXED) {
@@ -197,6 +206,10 @@ int gev_setup(gev_sys** out, int n, int dtype, const gev_opts* opts) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s.opts.device);
   if (sms > 0) s.sms = sms;
   size_t bytes = carve(s, nullptr);
+  if (s.opts.workspace_limit && bytes > s.opts.workspace_limit) {  // without the room for wider bands
+    s.b_cap = s.b;
+    bytes = carve(s, nullptr);
+  }
   if (s.opts.workspace_limit && bytes > s.opts.workspace_limit) {
     delete h;
     return GEV_ERR_OOM;
@@ -428,7 +441,7 @@ int gev_step_he2hb(gev_sys* h, void* A, int lda, int b, int* b_used) {
   if (lda < s.n) return -3;
   if (b != 0 && (b < 16 || b > 64)) return -4;
   int bb = b ? pick_band(s.n, b) : s.b;
-  if (bb > s.b) return GEV_ERR_UNSUPPORTED;  // workspace sized for the handle's band width
+  if (bb > s.b_cap) return GEV_ERR_UNSUPPORTED;  // the workspace holds no wider band
   int r = s.dtype == GEV_C128 ? he2hb<zd>(s, (zd*)A, lda, bb) : he2hb<double>(s, (double*)A, lda, bb);
   if (r) return r;
   GEV_CUDA_TRY(cudaStreamSynchronize(s.stream));

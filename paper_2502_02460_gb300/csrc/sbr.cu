@@ -485,7 +485,7 @@ template <class T> int he2hb(Sys& s, T* A, int lda, int b) {
   // that consecutive panels form one wider compact-WY block in the back-transform
   GEV_CUDA_TRY(cudaMemsetAsync(V1, 0, sizeof(T) * (size_t)n * n, s.stream));
   T* T1 = (T*)s.T1;
-  const size_t buf = (size_t)n * 2 * s.b;    // the panel buffers, n x 2b each
+  const size_t buf = (size_t)n * 2 * b;      // the panel buffers, n x 2b each
   T* WY = (T*)s.Pn;                           // [W0 | Y]
   T* YV = WY + buf;                           // [Y | V]
   T* VY = YV + buf;                           // [V | Y]
@@ -497,8 +497,8 @@ template <class T> int he2hb(Sys& s, T* A, int lda, int b) {
   const T one = from_re<T>(1.0), mone = from_re<T>(-1.0), zero = zero_<T>();
   const size_t coef_smem = sizeof(T) * ((size_t)b * (b + 1) + 5 * b);
   GEV_TRY(allow_dyn_smem(k_sbr_coef<T>, coef_smem));
-  // tasks of a sweep of the chase that follows.  V2 holds b n ntask entries for every b up to the handle's width; the
-  // scalars of a narrower band outgrow their own room and go to Zk, which only complete solves (at the handle's width) use
+  // tasks of a sweep of the chase that follows.  V2 holds b n ntask entries for every b the handle accepts; the
+  // scalars of a band narrower than its default outgrow their own room and go to Zk, which only complete solves (at the default width) use
   s.ntask = (n + b - 1) / b + 2;
   s.tau2 = s.ntask <= s.ntask_ws ? s.tau2_ws : (void*)s.Zk;
   if (s.ntask > s.ntask_ws && sizeof(T) * (size_t)s.ntask > sizeof(double) * (size_t)n) return GEV_ERR_UNSUPPORTED;

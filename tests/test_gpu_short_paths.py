@@ -226,3 +226,49 @@ def test_band_narrower_than_the_handles(dev, n, k, width, b, cx):
             w = w.cpu().numpy()[:k]
             assert np.max(np.abs(A @ Y - Y * w)) <= 64 * n * EPS * norm
             assert np.max(np.abs(Y.conj().T @ Y - np.eye(k))) <= 64 * n * EPS
+
+
+@pytest.mark.parametrize("n,b,cx", [(300, 32, False), (300, 32, True), (2100, 64, False), (2100, 16, False)])
+def test_band_wider_than_the_tables_choice(dev, n, b, cx):
+    """A handle whose width came from the table still reduces by steps to the bands that were its default.  Bound as above."""
+    import torch
+
+    from paper_2502_02460_gb300 import gev
+
+    g = torch.Generator(device=dev)
+    g.manual_seed(n + b)
+    A = torch.randn((n, n), generator=g, device=dev, dtype=torch.complex128 if cx else torch.float64)
+    A = A + A.mH
+    norm, k = float(A.abs().sum(dim=0).max()), n // 7
+    with gev.Solver(n, complex_=cx, device=dev) as s:
+        own = s.band_b
+        for bb in (b, own, b):
+            assert s.he2hb(gev.cm(A), bb) == bb
+            d, e = s.hb2st()
+            w, Z, _ = s.stedc(d, e, k)
+            Y = gev.logical(s.back(Z, k))
+            assert float((A @ Y - Y * w[:k]).abs().max()) <= 64 * n * EPS * norm
+            assert float((Y.mH @ Y - torch.eye(k, device=dev, dtype=A.dtype)).abs().max()) <= 64 * n * EPS
+
+
+def test_band_limits_of_a_handle(dev):
+    """An explicit width refuses wider bands; a limit at the explicit width's bytes still sets up a default handle."""
+    import ctypes
+
+    import torch
+
+    from paper_2502_02460_gb300 import gev
+
+    with gev.Solver(300, device=dev, band_b=16) as s:
+        with pytest.raises(gev.GevError) as err:
+            s.he2hb(torch.zeros((300, 300), dtype=torch.float64, device=dev), 32)
+        assert err.value.code == 7
+    for n, former in ((300, 32), (2100, 64)):
+        o = gev.Opts()
+        gev.lib().gev_default_opts(ctypes.byref(o))
+        o.band_b = former
+        limit = gev.lib().gev_workspace_bytes(n, gev.GEV_F64, ctypes.byref(o))
+        with gev.Solver(n, device=dev, workspace_limit=limit) as s:
+            A = torch.eye(n, dtype=torch.float64, device=dev)
+            w, _ = s.solve_cm(2.0 * A, A, 3)
+            assert float((w - 2.0).abs().max()) <= 64 * n * EPS

@@ -38,3 +38,13 @@ def nbytes(L, n, dtype, prec, band_b):
     (4096, 1, 1, 64, 5363512064)])
 def test_workspace_does_not_grow(L, n, dtype, prec, band_b, most):
     assert nbytes(L, n, dtype, prec, band_b) <= most
+
+
+@pytest.mark.parametrize("n,dtype,prec,default,widest", [(300, 0, 0, 16, 32), (1500, 0, 0, 32, 32), (2100, 0, 0, 32, 64),
+                                                         (300, 1, 0, 16, 32), (2100, 1, 0, 32, 32), (2100, 0, 1, 32, 32)])
+def test_room_for_wider_bands(L, n, dtype, prec, default, widest):
+    """A width chosen by the table (negative band_b) leaves room for the bands that steps may ask for."""
+    own, wide, auto = (nbytes(L, n, dtype, prec, b) for b in (default, widest, -default))
+    assert auto >= wide >= own
+    assert auto == own or widest > default
+    assert nbytes(L, n, dtype, prec, -1) == nbytes(L, n, dtype, prec, 0)
