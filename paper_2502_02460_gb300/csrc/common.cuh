@@ -194,6 +194,8 @@ __device__ __forceinline__ void house(double alpha, double xn, double& tau, doub
   beta = -(q * sr);
   scale = sr * recip(tau);
 }
+// the norm of an FP32 column from its FP64 square: the root in FP64 too, rounded once
+__device__ __forceinline__ float norm_low(double q) { return (float)sqrt(q); }
 __device__ __forceinline__ void house(float alpha, float xn, float& tau, float& beta, float& scale) {
   const float nrm = sqrtf(alpha * alpha + xn);
   beta = alpha >= 0.f ? -nrm : nrm;

@@ -296,10 +296,8 @@ __global__ void __launch_bounds__(panel_nt<B>()) k_panel_qr(PanelArgs<T> a) {
       if (!LOW && B <= 32) xn = __shfl_sync(B == 32 ? 0xffffffffu : 0xffffu, (double)re_(sum), c);
       T tau = zero_<T>(), beta = alpha, scale = zero_<T>();
       if (!(xn == 0.0 && im_(alpha) == 0)) {
-        if constexpr (LOW) {  // the norm from its FP64 square, rounded once; the rest as the data
-          const double q = (double)abs2_(alpha) + xn;
-          const int ex = (__double2hiint(q) >> 20) & 0x7FF;
-          const float nrm = ex > 1023 - 120 && ex < 1023 + 120 ? sqrtf((float)q) : (float)sqrt(q);
+        if constexpr (LOW) {  // the norm in FP64; the rest as the data
+          const float nrm = norm_low((double)abs2_(alpha) + xn);
           beta = from_re<T>(re_(alpha) >= 0.f ? -nrm : nrm);
           tau = div_(beta - alpha, beta);
           scale = div_(from_re<T>(1.0), alpha - beta);
