@@ -124,9 +124,10 @@ template <> struct real_of<float> { using type = float; };
 template <> struct real_of<zf> { using type = float; };
 
 // --------------------------------------------------------------- FP64-pipe arithmetic (device) --
-// 1 / d: the hardware's 20-bit reciprocal and one third-order step (y += y (e + e^2), e = 1 - d y),
-// within an ulp of the quotient (about half a division's FP64 instructions); outside the exponents where the
-// steps are safe, zero and the non-finite ones included, the division
+// 1 / d: the hardware's 20-bit reciprocal y and one step of the third-order hyperpower iteration (the geometric series
+// 1 / d = y (1 + e + e^2 + ..), e = 1 - d y, cut after e^2; M. Altman, Pacific J. Math. 10, 1960, for inverses): the cut
+// is below e^3 < 2^-55, so that the last rounding decides: within an ulp of the quotient, with about half a division's
+// FP64 instructions.  Outside the exponents where the steps are safe, zero and the non-finite ones included, the division.
 __device__ __forceinline__ double recip(double d) {
   const int e = (__double2hiint(d) >> 20) & 0x7FF;
   if (e < 24 || e > 2020) return 1.0 / d;
@@ -135,7 +136,9 @@ __device__ __forceinline__ double recip(double d) {
   const double r = fma(-d, y, 1.0);
   return fma(y, fma(r, r, r), y);
 }
-// 1 / sqrt(q), q > 0, the same way: y += y e (1/2 + 3/8 e), e = 1 - q y^2
+// 1 / sqrt(q), q > 0, the same way with the binomial series of (1 - e)^(-1/2), e = 1 - q y^2, cut after e^2 (Householder's
+// iteration of order three; A. S. Householder, The Numerical Treatment of a Single Nonlinear Equation, 1970).  Two roundings,
+// of q y (it enters by half) and of the result, and the cut: within 1.75 ulp.
 __device__ __forceinline__ double recip_sqrt(double q) {
   const int e = (__double2hiint(q) >> 20) & 0x7FF;
   if (e < 24 || e > 2020) return rsqrt(q);

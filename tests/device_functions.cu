@@ -21,4 +21,29 @@ int t_norm_low(int n, const double* q, float* out) {
   return map(n, [=] __device__(int i) { out[i] = norm_low(q[i]); });
 }
 
+int t_recip(int n, const double* x, double* out) {
+  return map(n, [=] __device__(int i) { out[i] = recip(x[i]); });
+}
+int t_divide(int n, const double* x, double* out) {
+  return map(n, [=] __device__(int i) { out[i] = 1.0 / x[i]; });
+}
+int t_recip_sqrt(int n, const double* x, double* out) {
+  return map(n, [=] __device__(int i) { out[i] = recip_sqrt(x[i]); });
+}
+int t_rsqrt(int n, const double* x, double* out) {
+  return map(n, [=] __device__(int i) { out[i] = rsqrt(x[i]); });
+}
+// out: n x 3, tau, beta, scale
+int t_house(int n, const double* alpha, const double* xn, double* out) {
+  return map(n, [=] __device__(int i) { house(alpha[i], xn[i], out[3 * i], out[3 * i + 1], out[3 * i + 2]); });
+}
+int t_house_cx(int n, const double* alpha, const double* xn, double* out) {
+  return map(n, [=] __device__(int i) {
+    zd tau, beta, scale;
+    house(make_zd(alpha[2 * i], alpha[2 * i + 1]), xn[i], tau, beta, scale);
+    double* o = out + 6 * i;
+    o[0] = tau.x; o[1] = tau.y; o[2] = beta.x; o[3] = beta.y; o[4] = scale.x; o[5] = scale.y;
+  });
+}
+
 }
