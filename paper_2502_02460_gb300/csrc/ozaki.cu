@@ -34,6 +34,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "int_sums.cuh"
 #include "tcgen05.cuh"
 
 namespace gev {
@@ -445,82 +446,6 @@ __device__ __forceinline__ OzItem oz_item(const OzP& p, int it) {
   w.s_lo = s_lo;
   w.nst = s_hi - s_lo;
   return w;
-}
-
-
-// (acc 2^-49 + sh) 2^e rounded once to FP64, in integer arithmetic: GB300 runs about 1.7 FP64 operations
-// (conversions included) per SM per cycle, and at eight of them per output the epilogue of a 128 x 64
-// tile took about 19 us.  sh (|sh| < 2^-18) joins acc in units of 2^-81 (acc:lo, 96 bits); the magnitude is
-// normalised with a count of leading zeros and rounded to nearest even.
-__device__ __forceinline__ double to_fp64(long long acc, float sh, int e) {
-  const uint32_t sb = __float_as_uint(sh);
-  const int se = (int)((sb >> 23) & 0xFF);
-  const unsigned long long sm = (sb & 0x7FFFFFu) | 0x800000u;
-  const int sft = se - 150 + 81;  // sh 2^81 = sm 2^sft (a zero or denormal sh has sft < -24)
-  long long si = sft >= 0 ? (long long)(sm << sft) : (sft > -25 ? (long long)(sm >> -sft) : 0);
-  if (sb >> 31) si = -si;
-  acc += si >> 32;
-  uint32_t lo = (uint32_t)si;
-  const bool neg = acc < 0;
-  unsigned long long m = (unsigned long long)acc;
-  if (neg) {  // two's complement of the 96 bits
-    lo = 0u - lo;
-    m = ~m + (lo == 0 ? 1ull : 0ull);
-  }
-  int ex = 63 - 49 + e;  // exponent of bit 63 of m
-  if ((m >> 32) == 0) {
-    m = (m << 32) | lo;
-    lo = 0;
-    ex -= 32;
-  }
-  if (m == 0) return 0.0;
-  const int lz = __clzll((long long)m);
-  const unsigned long long low = ((unsigned long long)lo) << lz;  // lz < 32 whenever lo != 0
-  m = (m << lz) | (low >> 32);
-  ex -= lz;
-  const uint32_t rem = ((uint32_t)m & 0x7FFu) | ((uint32_t)low != 0u ? 1u : 0u);
-  unsigned long long mant = m >> 11;  // 2^52 <= mant < 2^53
-  mant += (rem > 0x400u || (rem == 0x400u && (mant & 1))) ? 1ull : 0ull;
-  // (a carry to 2^53 moves the exponent up by itself: the fields add, up to infinity)
-  unsigned long long b = mant + ((unsigned long long)(ex + 1022) << 52);
-  if (ex > 1023) b = 0x7FF0000000000000ull;
-  else if (ex < -1022) b = ex < -1076 ? 0ull : (mant + (1ull << (-1023 - ex))) >> (-1022 - ex);  // subnormal
-  return __longlong_as_double((long long)(b | (neg ? 1ull << 63 : 0ull)));
-}
-
-// The same where neither zero, NaN, overflow nor subnormal results can occur (|e| < 1000): sh is split into
-// 32-bit integer and fraction by FP32 conversions, and the 96 bits are normalised as three words with funnel
-// shifts.  About half the instructions; with the other per-output work thinned out too, a 6144 x 6144 x 128 update
-// went from 515 to 330 us (splits included; its MMAs are about 160).
-__device__ __forceinline__ double to_fp64_fast(long long acc, float sh, int e, uint32_t flip) {
-  const float x = sh * 562949953421312.0f;  // 2^49: |x| < 2^31
-  const int xi = __float2int_rd(x);
-  uint32_t l = __float2uint_rz((x - __int2float_rn(xi)) * 4294967296.0f);  // the fraction, [0, 1)
-  acc += xi;
-  const uint32_t neg = (uint32_t)((int)(acc >> 32) >> 31);  // all ones for a negative sum: two's complement
-  const unsigned long long mag = ((unsigned long long)acc ^ (((unsigned long long)neg << 32) | neg)) + (l == 0 ? neg & 1u : 0u);
-  l = (l ^ neg) + (neg & 1u);
-  uint32_t h = (uint32_t)(mag >> 32), m = (uint32_t)mag;
-  int ex = 63 - 49 + e + 1022;
-  if (h == 0) {
-    h = m;
-    m = l;
-    l = 0;
-    ex -= 32;
-    if (h == 0) {
-      h = m;
-      m = 0;
-      ex -= 32;
-      if (h == 0) return 0.0;
-    }
-  }
-  const int lz = __clz((int)h);
-  h = __funnelshift_l(m, h, lz);
-  m = __funnelshift_l(l, m, lz);
-  const uint32_t t = (m & 0x7FFu) | ((l << lz) != 0u ? 1u : 0u), up = (t + 0x3FFu + ((m >> 11) & 1u)) >> 11;
-  const uint32_t w0 = __funnelshift_r(m, h, 11), r0 = w0 + up;
-  const uint32_t w1 = (h >> 11) + (r0 < w0 ? 1u : 0u) + ((uint32_t)(ex - lz) << 20);
-  return __hiloint2double((int)(w1 | ((neg ^ flip) & 0x80000000u)), (int)r0);
 }
 
 // Persistent: a CTA per SM walks over the work items.  The copy warp runs ahead into the next item's

@@ -16,6 +16,7 @@
 
 #include "common.cuh"
 #include "coop.cuh"
+#include "int_sums.cuh"
 
 namespace gev {
 
@@ -24,56 +25,6 @@ namespace {
 // threads of a panel block: four (b = 16: eight) per column.  All four schedulers have a warp then, and the sums
 // over a column's threads, a chain of FP64 additions in one warp, stay short.
 template <int B> constexpr int panel_nt() { return B == 64 ? 256 : 128; }
-
-// The sum of N <= 63 FP64 values in integer arithmetic: each is taken to 57 bits below the largest exponent and added
-// as a 64-bit integer, the total is rounded once.  An FP64 addition occupies a scheduler's pipe for 64 to 72 cycles, the
-// dozen integer instructions here for about 24.  The error is below N 2^-56 of the largest value (N 2^-53 of the partial
-// sums for additions), and the result does not depend on the order.  Exponents near either end: additions.
-template <int N> __device__ __forceinline__ double sum_block(const double (&v)[N]) {
-  static_assert(N < 64, "57 bits and the sum's carry fit 63");
-  int emax = 0;
-#pragma unroll
-  for (int u = 0; u < N; ++u) emax = max(emax, (__double2hiint(v[u]) >> 20) & 0x7FF);
-  if (emax < 100 || emax > 2000) {
-    double t = 0.0;
-#pragma unroll
-    for (int u = 0; u < N; ++u) t += v[u];
-    return t;
-  }
-  long long acc = 0;
-#pragma unroll
-  for (int u = 0; u < N; ++u) {
-    const long long b = __double_as_longlong(v[u]);
-    const int sh = emax - ((int)(b >> 52) & 0x7FF);
-    const long long m = ((b & 0xFFFFFFFFFFFFFll) | (1ll << 52)) << 4;
-    const long long x = sh > 62 ? 0 : m >> sh;
-    acc += b < 0 ? -x : x;
-  }
-  if (acc == 0) return 0.0;
-  unsigned long long mag = acc < 0 ? 0ull - (unsigned long long)acc : (unsigned long long)acc;
-  const int lz = __clzll((long long)mag);
-  mag <<= lz;
-  const unsigned lo = (unsigned)mag & 0x7FFu;
-  unsigned long long r = mag >> 11;
-  r += (lo > 0x400u || (lo == 0x400u && (r & 1))) ? 1 : 0;
-  r += (unsigned long long)(emax + 6 - lz) << 52;  // (the mantissa's leading bit adds one to the exponent)
-  return __longlong_as_double((long long)(r | (acc < 0 ? 1ull << 63 : 0ull)));
-}
-template <int N> __device__ __forceinline__ zd sum_block(const zd (&v)[N]) {
-  double a[N], b[N];
-#pragma unroll
-  for (int u = 0; u < N; ++u) {
-    a[u] = v[u].x;
-    b[u] = v[u].y;
-  }
-  return make_zd(sum_block(a), sum_block(b));
-}
-template <int N> __device__ __forceinline__ float sum_block(const float (&v)[N]) {
-  float t = 0.f;
-#pragma unroll
-  for (int u = 0; u < N; ++u) t += v[u];
-  return t;
-}
 
 template <class T> struct PanelArgs {
   int m, R, use_smem, t_smem;

@@ -1,5 +1,6 @@
 // The scalar device functions of csrc, element by element over arrays, for tests/test_gpu_device_functions.py.
 #include "common.cuh"
+#include "int_sums.cuh"
 
 using namespace gev;
 
@@ -7,6 +8,11 @@ namespace {
 
 template <class F> __global__ void k_map(int n, F f) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) f(i);
+}
+template <int N> __device__ double row_sum(const double* v) {
+  double a[N];
+  for (int u = 0; u < N; ++u) a[u] = v[u];
+  return sum_block(a);
 }
 template <class F> int map(int n, F f) {
   k_map<<<(n + 255) / 256, 256>>>(n, f);
@@ -44,6 +50,20 @@ int t_house_cx(int n, const double* alpha, const double* xn, double* out) {
     double* o = out + 6 * i;
     o[0] = tau.x; o[1] = tau.y; o[2] = beta.x; o[3] = beta.y; o[4] = scale.x; o[5] = scale.y;
   });
+}
+
+// v: n x 20 or n x 40
+int t_sum_block_20(int n, const double* v, double* out) {
+  return map(n, [=] __device__(int i) { out[i] = row_sum<20>(v + 20 * i); });
+}
+int t_sum_block_40(int n, const double* v, double* out) {
+  return map(n, [=] __device__(int i) { out[i] = row_sum<40>(v + 40 * i); });
+}
+int t_to_fp64(int n, const long long* acc, const float* sh, const int* e, double* out) {
+  return map(n, [=] __device__(int i) { out[i] = to_fp64(acc[i], sh[i], e[i]); });
+}
+int t_to_fp64_fast(int n, const long long* acc, const float* sh, const int* e, double* out) {
+  return map(n, [=] __device__(int i) { out[i] = to_fp64_fast(acc[i], sh[i], e[i], i & 1 ? 0xFFFFFFFFu : 0u); });
 }
 
 }

@@ -1,4 +1,4 @@
-"""Scalar device functions of csrc (common.cuh) against their definitions, element by element.
+"""Scalar device functions of csrc (common.cuh, int_sums.cuh) against their definitions, element by element.
 
 * norm_low, the norm of an FP32 panel column: the FP64 root rounded once to FP32, so it equals numpy's float32(sqrt(q))
   in every bit (IEEE 754 gives both operations one result).
@@ -11,10 +11,16 @@
   r = 1 / sqrt(q) by half.  Real: beta = q r 3.25 u; tau = 1 + |alpha| r, at most 2, 4.25 u absolute; scale = s r / tau 6.7 u.
   Complex: beta 4.25 u; tau 8.2 u absolute; scale = conj(d) / |d|^2 with d = alpha - beta to 5.25 u, |d|^2 to 12.5 u:
   scale (alpha - beta) within 26.5 u of 1.
+* sum_block against exact sums: each of the N values is cut to 57 bits below the largest exponent, less than 2^-56 of the
+  largest value, and the total is rounded once; where the largest exponent is near either end it is the plain sum, in every bit.
+* to_fp64, (acc 2^-49 + sh) 2^e with sh cut to units of 2^-81, against the exact value rounded once to nearest even, in every
+  bit, from subnormal results to overflow; to_fp64_fast, for the middle of the range, to half an ulp and the rounding of
+  sh's fraction, in units of 2^-49: 2^-25 in FP32 and 2^-32 of its integer form.
 """
 import ctypes
 import os
 import subprocess
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -137,3 +143,86 @@ def test_house_complex(fns):
     # scale (alpha - beta) = 1
     dx, dy = x + s * nrm, y
     assert np.max(np.hypot(o[:, 4] * dx - o[:, 5] * dy - 1, o[:, 4] * dy + o[:, 5] * dx)) <= 27 * u
+
+
+@pytest.mark.parametrize("N", [20, 40])
+def test_sum_block(fns, N):
+    rng = np.random.default_rng(N)
+    n = 4000
+    v = rng.standard_normal((n, N)) * 2.0 ** rng.integers(-30, 30, (n, N)) * 2.0 ** rng.integers(-900, 900, (n, 1))
+    v[:500] *= 2.0 ** rng.integers(-60, 1, (500, N))   # far apart
+    v[500:1000, 1:N:2] = -v[500:1000, 0:N:2]           # cancels exactly
+    v[1000:1200, :] = 0.0
+    v[1200:1400, 3:] = 0.0
+    v[1400:1800] = np.sign(v[1400:1800]) * np.repeat(rng.uniform(1.0, 2.0, (400, 1)), N, 1)  # equal magnitudes
+    v[1800:1900] = 1.9999999999999998                  # the largest carry
+    base = np.ldexp(rng.uniform(1.0, 2.0, (800, N)), rng.integers(-20, 0, (800, N)))
+    base[:, 0] = 1.5
+    for q, biased in enumerate([0, 1, 99, 100, 101, 2000, 2001, 2040]):  # exponents at the limits
+        v[2000 + 100 * q:2100 + 100 * q] = np.ldexp(base[100 * q:100 * q + 100], biased - 1023)
+    v[2900, 0], v[2901, 1], v[2902, 2] = np.inf, np.nan, -np.inf
+    f = getattr(fns, f"t_sum_block_{N}")
+    out = call(f, [v], np.float64, (n,))
+    top = ((v.view(np.int64) >> 52) & 0x7FF).max(axis=1)
+    mid = (top >= 100) & (top <= 2000)
+    with np.errstate(all="ignore"):
+        plain = np.zeros(n)
+        for u in range(N):
+            plain = plain + v[:, u]
+    assert np.array_equal(out[~mid], plain[~mid], equal_nan=True) and mid.sum() > 3000 and (~mid).sum() > 500
+    for i in np.flatnonzero(mid):
+        exact = sum(map(Fraction, v[i]))
+        bound = N * Fraction(2) ** -56 * Fraction(np.abs(v[i]).max()) + Fraction(np.spacing(abs(out[i]))) / 2
+        assert abs(Fraction(out[i]) - exact) <= bound
+    assert np.array_equal(call(f, [v[mid][:, ::-1]], np.float64, (int(mid.sum()),)), out[mid])  # any order
+
+
+def _accumulators(n, seed):
+    """(acc, sh) as the product kernel forms them: |acc| < 2^62, |sh| < 2^-18; ties and carries of every width among them."""
+    rng = np.random.default_rng(seed)
+    acc = rng.integers(-(1 << 62), 1 << 62, n) >> rng.integers(0, 62, n)
+    sh = (rng.uniform(-1.0, 1.0, n) * 2.0 ** -rng.integers(18, 90, n)).astype(np.float32)
+    sh[::5] = 0.0
+    k = rng.integers(1, 10, n)
+    tie = np.arange(n) % 5 == 0  # acc = odd or even mantissa and exactly half a unit, or all ones
+    acc[tie] = (((rng.integers(1 << 52, 1 << 53, n) << 1) + 1) << (k - 1) >> rng.integers(0, 2, n))[tie]
+    acc[7::50] = (1 << 62) - 1
+    acc[8::50] = -(1 << 53) + 1
+    acc[9::50] = 0
+    acc[10::50], sh[10::50] = 0, 0.0
+    return rng, acc, sh
+
+
+def _shifted(total, k):
+    """total 2^k rounded once to FP64 (CPython's integer division and conversion round to nearest even)."""
+    try:
+        return float(total << k) if k >= 0 else total / (1 << -k)
+    except OverflowError:
+        return np.inf if total > 0 else -np.inf
+
+
+def test_to_fp64_rounds_once(fns):
+    n = 60000
+    rng, acc, sh = _accumulators(n, 11)
+    e = np.concatenate([rng.integers(-1140, 1140, n // 3), rng.integers(-1090, -1010, n // 3), rng.integers(-20, 20, n // 3)])
+    e = e.astype(np.int32)
+    out = call(fns.t_to_fp64, [acc, sh, e], np.float64, (n,))
+    want = np.empty(n)
+    for i in range(n):
+        low = Fraction(float(sh[i])) * 2**81
+        si = abs(low).__floor__() * (1 if low >= 0 else -1)
+        want[i] = _shifted((int(acc[i]) << 32) + si, int(e[i]) - 81)
+    assert np.array_equal(out, want)
+    sub = (np.abs(want) < 2.0**-1022) & (want != 0)
+    assert sub.sum() > 3000 and np.isinf(want).sum() > 300
+
+
+def test_to_fp64_fast(fns):
+    n = 40000
+    rng, acc, sh = _accumulators(n, 12)
+    e = rng.integers(-800, 801, n).astype(np.int32)
+    out = call(fns.t_to_fp64_fast, [acc, sh, e], np.float64, (n,))
+    for i in range(n):
+        scale = Fraction(2) ** int(e[i])
+        exact = (Fraction(int(acc[i]), 1 << 49) + Fraction(float(sh[i]))) * scale * (-1 if i & 1 else 1)
+        assert abs(Fraction(out[i]) - exact) <= Fraction(np.spacing(abs(out[i]))) / 2 + scale * (Fraction(2) ** -74 + Fraction(2) ** -81)

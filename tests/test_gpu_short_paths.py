@@ -272,3 +272,50 @@ def test_band_limits_of_a_handle(dev):
             A = torch.eye(n, dtype=torch.float64, device=dev)
             w, _ = s.solve_cm(2.0 * A, A, 3)
             assert float((w - 2.0).abs().max()) <= 64 * n * EPS
+
+
+@pytest.mark.parametrize("M,N,K", [(130, 70, 40), (300, 65, 200)])
+def test_emulated_product_at_the_ends_of_the_range(dev, M, N, K):
+    """Rows scaled by powers of two so that outputs are subnormal, vanish or overflow.  The digits do not depend on the scale, so
+    an output is that of the unscaled rows with another exponent, both rounded to nearest: within one unit in the last place
+    (2^-1074 at least), infinite where that is.  General alpha and beta: the two further roundings, in every bit."""
+    import ctypes
+
+    import torch
+
+    from paper_2502_02460_gb300 import gev
+
+    L = gev.lib()
+    L.gev_gemm_f64_scratch_bytes.restype = ctypes.c_size_t
+    rng = np.random.default_rng(M)
+    A0, B0 = rng.standard_normal((K, M)), rng.standard_normal((N, K))  # column-major op(A) = A0^T, op(B) = B0^T
+    ea = rng.integers(-640, -560, M)                      # with 2^-440: subnormal and vanishing outputs
+    up = np.arange(M) % 3 == 1
+    ea[up] = rng.integers(715, 735, up.sum())             # with 2^300: finite and infinite outputs
+    C0 = rng.standard_normal((N, M))
+    nb = L.gev_gemm_f64_scratch_bytes(M, N, K)
+    W = torch.empty(nb, dtype=torch.uint8, device=dev)
+    st = torch.zeros(16, dtype=torch.int32, device=dev)
+    p, d = (lambda t: ctypes.c_void_p(t.data_ptr())), ctypes.c_double
+    stream = ctypes.c_void_p(torch.cuda.current_stream(dev).cuda_stream)
+
+    def product(A, B, alpha, beta, C):
+        A, B, C = (torch.from_numpy(np.ascontiguousarray(x)).to(dev) for x in (A, B, C))
+        rc = L.gev_gemm_f64(M, N, K, 1, 0, d(alpha), p(A), K, p(B), K, d(beta), p(C), M, 1, stream, p(st), p(W),
+                            ctypes.c_size_t(nb))
+        assert rc == 0
+        return C.cpu().numpy()
+
+    A = np.ldexp(A0.T, ea[:, None])
+    base = product(A0.T, B0, 1.0, 0.0, C0)
+    low = product(A, np.ldexp(B0, -440), 1.0, 0.0, C0)
+    high = product(A, np.ldexp(B0, 300), 1.0, 0.0, C0)
+    with np.errstate(over="ignore", under="ignore"):
+        want_low, want_high = np.ldexp(base, (ea - 440)[None, :]), np.ldexp(base, (ea + 300)[None, :])
+    for got, want in ((low, want_low), (high, want_high)):
+        fin = np.isfinite(want)
+        assert np.array_equal(got[~fin], want[~fin]) and np.all(np.isfinite(got[fin]))
+        assert np.all(np.abs(got[fin] - want[fin]) <= np.spacing(np.abs(want[fin])))
+    assert np.any((low != 0) & (np.abs(low) < 2.0**-1022)) and np.any(low == 0)
+    assert np.any(np.isinf(high)) and np.any(np.isfinite(high[:, up]))
+    assert np.array_equal(product(A, np.ldexp(B0, -440), 1.5, 0.5, C0), 1.5 * low + 0.5 * C0)
