@@ -111,11 +111,17 @@ typedef struct {
                             back-transform, in FP64 (plain form) or FP32 (real mixed form; the complex
                             mixed form returns GEV_ERR_UNSUPPORTED); panel width = the band width.
                             2: two-stage (full -> band, bulge chasing, two back-transforms).
-                            0 = automatic (default): two-stage, which measured faster on GB300 at every
-                            order (the one-stage form's matrix-vector products are bound by the FP64
-                            pipe, the two-stage route's products run on the tensor cores) */
+                            0 = automatic (default): two-stage with emulated products, where it measured
+                            faster on GB300 at every order (the one-stage form's matrix-vector products are
+                            bound by the FP64 pipe, the two-stage route's products run on the tensor cores).
+                            Its vectors carry a few more rounding errors: real n = 4096 and complex
+                            n = 2048 lie 1.25 to 1.7 times further from the exact ones, both near
+                            0.1 eps ||A|| / gap; one_stage = 1 keeps the other route.  With native products
+                            (fp64_emulation = 0) one-stage from n = 2048 on for k >= n/2, and up to 8192
+                            for fewer pairs (real data from 2560), where that measured faster */
   int rr_one_stage;      /* mixed form, the FP64 Rayleigh-Ritz solve of the refinement (all k pairs of
-                            a k x k pencil): 1 = one-stage, 2 = two-stage, 0 = automatic (two-stage) */
+                            a k x k pencil): 1 = one-stage, 2 = two-stage, 0 = automatic (two-stage; with
+                            native products one-stage for k >= 2048) */
 } gev_opts;
 
 typedef struct {

@@ -482,11 +482,18 @@ template <class T> int hb2st(Sys& s, double* d, double* e);
 int stedc(Sys& s, const double* d, const double* e, int k, double* w, double* Z, int ldz, int* deflated);
 template <class T> int back(Sys& s, const double* Z, int ldz, int k, T* Y, int ldy);
 template <class T> int bt_he2hb(Sys& s, T* Y, int ldy, int k);
-// the route of a plain-form solve (gev_opts.one_stage: 1 one-stage, 2 or 0 (automatic) two-stage).  Two-stage
-// measured faster at every order and number of pairs (ms, the better band width of 32 and 64 against one-stage):
-// real n = 1500, k = n / 4 44 / 69; 2048, k = n / 4 68 / 99, k = n 76 / 100; 4096 172 / 244, 222 / 254; 8192
-// 600 / 905, 807 / 979; complex 2048 144 / 210, 162 / 215; 4096 400 / 681.
-inline bool one_stage_for(int opt) { return opt == 1; }
+// The route of a plain-form solve of order n for k pairs (gev_opts.one_stage: 1 one-stage, 2 two-stage, 0 automatic).
+// Emulated products: two-stage, which measured faster at every order and number of pairs (ms, the better band width of 32
+// and 64 against one-stage): real n = 1500, k = n / 4 44 / 69; 2048, k = n / 4 68 / 99, k = n 76 / 100; 4096 172 / 244,
+// 222 / 254; 8192 600 / 905, 807 / 979; complex 2048 144 / 210, 162 / 215; 4096 400 / 681.
+// Native products run on the FP64 pipe, where the second back-transform's 2 n^2 k operations tell: real 2048, k = n / 4
+// 159 / 165, n / 2 172 / 173, n 198 / 190; 3000 312 / 307, 351 / 332, 452 / 382; 4096 566 / 538, 672 / 607, 890 / 726; 8192, k =
+// n / 4 3057 / 2772, n 5606 / 4276; complex 2048 535 / 459, 583 / 485, 678 / 537; 4096 2011 / 1775, 2372 / 2001, 3132 / 2435.
+inline bool one_stage_for(const Sys& s, int n, int k) {
+  if (s.opts.one_stage == 1) return true;
+  if (s.opts.one_stage == 2 || s.emu_fp64 || n < 2048) return false;
+  return 2 * (long long)k >= n || (n <= 8192 && (s.dtype == GEV_C128 || n >= 2560));
+}
 // one-stage Householder tridiagonalisation into s.d / s.e, and Y = Q Z for it (td1.cu)
 template <class T> int he2td(Sys& s, T* A, int lda);
 template <class T> int back_td(Sys& s, const double* Z, int ldz, int k, T* Y, int ldy);

@@ -568,7 +568,7 @@ template <class T> int solve_t(Sys& s, const T* H, int ldh, const T* S, int lds,
   GEV_TRY(hegst<T>(s, H, ldh, X, n, A, n));
   s.have_factor = true;
   s.factor_kind = 0;
-  const bool one = one_stage_for(s.opts.one_stage);
+  const bool one = one_stage_for(s, n, k);
   // steps 4a / 4b: two-stage tridiagonalisation (or the one-stage reduction, timed as "to_tridiag")
   mark(GEV_STEP_TO_BAND);
   if (!one) GEV_TRY(he2hb<T>(s, A, n, s.b));

@@ -33,11 +33,20 @@ namespace {
 
 // band width of the k x k Rayleigh-Ritz solve (all k pairs): the caller's choice, else the width that measured
 // fastest for whole solves of that order (ms at b = 16 / 32 / 64: real 1000 33 / 32 / 38, 2048 - / 76 / 85, 4096
-// - / 233 / 222; complex 1024 64 / 66 / 137, 2048 - / 162 / 278)
-int rr_band(int want, int k, bool cx) {
+// - / 233 / 222; complex 1024 64 / 66 / 137, 2048 - / 162 / 278).  With native products, mixed solves of n = 2 k at b = 16 /
+// 32 / 64: real k = 1024 256 / 235 / 234, 2048 1106 / 1051 / 1041; complex 1024 1137 / 1066 / 1068, 2048 4822 / 4646 / 4638.
+int rr_band(const Sys& s, int k) {
+  const int want = s.opts.rr_band_b;
   if (want == 16 || want == 32 || want == 64) return want;
-  if (cx) return k <= 1024 ? 16 : 32;
+  if (!s.emu_fp64) return 64;
+  if (s.dtype == GEV_C128) return k <= 1024 ? 16 : 32;
   return k < 4096 ? 32 : 64;
+}
+// and its route: native products take one stage from k = 2048 on (mixed solves of n = 2 k, two / one: real k = 1024 234 / 236,
+// 2048 1041 / 1034, 4096 6566 / 6420; complex 1024 1068 / 1022, 2048 4638 / 4511; emulated products: one_stage_for)
+int rr_route(const Sys& s, int k) {
+  if (s.opts.rr_one_stage == 1) return 1;
+  return s.opts.rr_one_stage != 2 && !s.emu_fp64 && k >= 2048 ? 1 : 2;
 }
 
 __device__ __forceinline__ double wsum(double v) {
@@ -377,10 +386,10 @@ int solve_mixed(Sys& s, const double* H, int ldh, const double* S, int lds, int 
     o.prec = GEV_PLAIN;
     o.timing = 0;
     o.workspace_limit = 0;
-    o.band_b = rr_band(s.opts.rr_band_b, k, false);
+    o.band_b = rr_band(s, k);
     o.fp64_emulation = s.emu_fp64;  // the Ritz pencil's products use the same FP64 engine
     o.check = 0;
-    o.one_stage = s.opts.rr_one_stage == 1 ? 1 : 2;
+    o.one_stage = rr_route(s, k);
     o.debug_stall = 0;
     gev_sys* h = nullptr;
     const int rc = gev_setup(&h, k, GEV_F64, &o);
@@ -602,10 +611,10 @@ int solve_mixed_cx(Sys& s, const zd* H, int ldh, const zd* S, int lds, int k, do
     o.prec = GEV_PLAIN;
     o.timing = 0;
     o.workspace_limit = 0;
-    o.band_b = rr_band(s.opts.rr_band_b, k, true);
+    o.band_b = rr_band(s, k);
     o.fp64_emulation = s.emu_fp64;
     o.check = 0;
-    o.one_stage = s.opts.rr_one_stage == 1 ? 1 : 2;
+    o.one_stage = rr_route(s, k);
     o.debug_stall = 0;
     gev_sys* h = nullptr;
     const int rc = gev_setup(&h, k, GEV_C128, &o);

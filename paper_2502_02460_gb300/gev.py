@@ -176,7 +176,7 @@ class Solver:
         if band_b == 0:  # the autotuner's table (tune.py) for this dtype, precision and order
             from . import tune
 
-            band_b = tune.pick_band(n, complex_, mixed)
+            band_b = tune.pick_band(n, complex_, mixed, native=fp64_emulation == 0)
             o.band_b = -band_b  # (the width of solves; steps may use wider bands)
         self.band_b = band_b
         o.panel_nb = panel_nb

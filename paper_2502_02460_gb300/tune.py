@@ -42,9 +42,16 @@ def load(path: str = TABLE) -> dict:
     return _table
 
 
-def pick_band(n: int, complex_: bool, mixed: bool, table: dict | None = None) -> int:
+def pick_band(n: int, complex_: bool, mixed: bool, table: dict | None = None, native: bool = False) -> int:
     """The tuned band width for a problem of order n (0 when the table has no entry: the library's
-    default)."""
+    default).
+
+    ``native``: FP64 products on the FP64 pipe, which the table's emulated ones say nothing about: a plain solve then
+    gains from a band of 32 over 16 at every order (ms at 16 / 32 / 64, k = n/4: real 512 43 / 31 / 29, 900 76 / 57 /
+    56, 1800 174 / 138 / 138; complex 512 148 / 103 / 96, 1000 274 / 207 / 210, 1800 580 / 459 / 469), and real data from
+    order 2048 on from 64 (4096 in two stages 620 at 32, 566 at 64)."""
+    if native and not mixed:
+        return 64 if n >= 2048 and not complex_ else 32
     t = (table if table is not None else load()).get("entries", {}).get(key(complex_, mixed), {})
     if not t:
         return 0

@@ -157,3 +157,26 @@ def test_one_stage_mixed_matches_oracle(dev, n, k, cluster):
     compare_to_oracle(p, w, C, k, resid_bound=1e-11)
     assert rep["refine_resid"] <= 1e-11
     assert rep["ms"]["to_band"] < 0.5 and rep["ms"]["back_band"] < 0.5
+
+
+@pytest.mark.parametrize("emu,n,k,cx,one", [(0, 2047, 2047, False, False), (0, 2100, 1050, False, True),
+                                            (0, 2100, 1049, False, False), (0, 2560, 40, False, True), (0, 2048, 40, True, True),
+                                            (1, 2100, 2100, False, False), (1, 2560, 40, False, False)])
+def test_automatic_route(dev, emu, n, k, cx, one):
+    """The route of a default handle, from the step times (the one-stage reduction has no full -> band step), and its results
+    against torch's eigenvalues: the method is backward stable, 64 n eps ||H||_1."""
+    import torch
+
+    g = gv()
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(n + k)
+    H = torch.randn((n, n), generator=gen, device=dev, dtype=torch.complex128 if cx else torch.float64)
+    H = H + H.mH
+    S = torch.eye(n, device=dev, dtype=H.dtype)
+    with g.Solver(n, complex_=cx, device=dev, fp64_emulation=emu, timing=1) as s:
+        w, C = s.solve(H, S, k)
+        ms = s.last_report["ms"]
+    assert (ms["to_band"] < 0.02 * ms["to_tridiag"]) == one
+    bound = 64 * n * 2.0**-52 * float(H.abs().sum(dim=0).max())
+    assert float((w - torch.linalg.eigvalsh(H)[:k]).abs().max()) <= bound
+    assert float((H @ C - C * w).abs().max()) <= bound

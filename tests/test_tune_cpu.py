@@ -34,3 +34,13 @@ def test_committed_table_is_well_formed():
             assert min(times, key=times.get) == ent["b"], (form, order)
             cx, mixed = form.startswith("c128"), form.endswith("mixed")
             assert tune.pick_band(int(order), cx, mixed, table) == ent["b"]
+
+
+def test_native_products_keep_the_wider_bands():
+    """The table holds times with emulated products; with native ones 16 columns are slower at every order."""
+    for n in (100, 512, 1024, 2047):
+        assert tune.pick_band(n, False, False, native=True) == 32
+    assert tune.pick_band(2048, False, False, native=True) == tune.pick_band(20000, False, False, native=True) == 64
+    for n in (100, 1500, 4096, 20000):
+        assert tune.pick_band(n, True, False, native=True) == 32
+        assert tune.pick_band(n, True, True, native=True) == tune.pick_band(n, True, True)
