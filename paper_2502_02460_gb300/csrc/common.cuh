@@ -469,6 +469,8 @@ inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) /
 // Returns 0 or GEV_ERR_CUDA (the failing call is reported on stderr).
 int set_dyn_smem(const void* func, int bytes);
 template <class F> int allow_max_dyn_smem(F* func) { return set_dyn_smem((const void*)func, -1); }
+int set_wide_cluster(const void* func);
+template <class F> int allow_wide_cluster(F* func) { return set_wide_cluster((const void*)func); }  // more than 8 blocks
 template <class F> int allow_dyn_smem(F* func, size_t bytes) { return set_dyn_smem((const void*)func, (int)bytes); }
 
 // ---------------------------------------------------------------------------- step launchers --

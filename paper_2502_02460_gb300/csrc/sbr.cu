@@ -335,7 +335,7 @@ template <class T, int B> int launch_panel(Sys& s, PanelArgs<T> a, int* arrivals
     const size_t smem = panel_smem<T, B, PANEL_CL>(a.R, 1, 1);
     if (smem <= cap) {
       GEV_TRY(allow_max_dyn_smem(kern));
-      GEV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      GEV_TRY(allow_wide_cluster(kern));
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
       at[0].val.clusterDim.x = PANEL_CL;

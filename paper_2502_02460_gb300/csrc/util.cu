@@ -3,6 +3,7 @@
 // and the per-column phase normalisation of the eigenvectors.
 #include <map>
 #include <mutex>
+#include <set>
 #include <utility>
 
 #include "common.cuh"
@@ -28,6 +29,18 @@ int set_dyn_smem(const void* func, int bytes) {
   }
   GEV_CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, want));
   done[key] = want;
+  return 0;
+}
+
+int set_wide_cluster(const void* func) {
+  static std::mutex mu;
+  static std::set<std::pair<const void*, int>> done;  // (kernel, device)
+  int dev = 0;
+  GEV_CUDA_TRY(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(mu);
+  if (done.count({func, dev})) return 0;
+  GEV_CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  done.insert({func, dev});
   return 0;
 }
 
