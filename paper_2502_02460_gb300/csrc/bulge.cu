@@ -787,7 +787,6 @@ template <class T, int B> int bt_levels(Sys& s, int n, int k, T* Y, int ldy) {
 // launching anything, when the handle's scratch cannot hold a level's product.
 template <class T> int bt_levels_wy(Sys& s, int n, int k, int b, T* Y, int ldy) {
   constexpr int cx = is_cx<T>::value ? 1 : 0;
-  constexpr bool f32 = std::is_same<T, float>::value;
   const int ngroups = (n - 3) / b + 1;
   const int nlevels = ngroups + s.ntask;
   T* P = (T*)s.W1;  // (nblk b) x k products V^H Y (W1 is free during the back-transform)
@@ -799,13 +798,8 @@ template <class T> int bt_levels_wy(Sys& s, int n, int k, int b, T* Y, int ldy) 
     if (lb.nblk == 0) continue;
     max_nblk = std::max(max_nblk, lb.nblk);
     const int rows = std::min(lb.nblk * 2 * b, n - lb.w00);
-    if constexpr (f32) {
-      need = std::max(need, gemm_f32_bdiag_scratch(lb.nblk * b, k, rows, b, 2 * b));
-      need = std::max(need, gemm_f32_bdiag_scratch(rows, k, lb.nblk * b, 2 * b, b));
-    } else {
-      need = std::max(need, gemm_f64_bdiag_scratch(lb.nblk * b, k, rows, b, 2 * b, cx));
-      need = std::max(need, gemm_f64_bdiag_scratch(rows, k, lb.nblk * b, 2 * b, b, cx));
-    }
+    need = std::max(need, gemm_f64_bdiag_scratch(lb.nblk * b, k, rows, b, 2 * b, cx));
+    need = std::max(need, gemm_f64_bdiag_scratch(rows, k, lb.nblk * b, 2 * b, b, cx));
   }
   // levels whose W_j are formed in one launch: as many as the buffer holds
   const size_t per_level = (size_t)std::max(max_nblk, 1) * 2 * b * b * sizeof(T);
@@ -835,18 +829,13 @@ template <class T> int bt_levels_wy(Sys& s, int n, int k, int b, T* Y, int ldy) 
     T* Yl = Y + lb.w00;
     const int M1 = lb.nblk * b;
     BdOp a2{2, cx, b, n, s.ntask, lb.g_lo, L, ngroups, lb.nblk, lb.w00, nullptr, nullptr, Wl};
-    if constexpr (f32) {
-      if (!gemm_f32_bdiag(s, M1, k, rows, a1, b, 2 * b, Yl, ldy, 1.f, 0.f, P, M1)) return GEV_ERR_CUDA;
-      if (!gemm_f32_bdiag(s, rows, k, M1, a2, 2 * b, b, P, M1, -1.f, 1.f, Yl, ldy)) return GEV_ERR_CUDA;
-    } else {
-      // From orthonormal Z (s.z_unit), Y's columns stay unit vectors under the orthogonal transforms
-      // (|y_ij| <= 1), and |P_qj| = |v_q^H y_j| <= ||v_q|| <= sqrt(2) (a Householder vector with
-      // v(0) = 1): both below 2, so their scales need no pass over the data
-      const bool u = s.z_unit;
-      if (u && gemm_f64_bdiag_level(s, M1, rows, k, a1, a2, b, Yl, ldy, P, M1)) continue;
-      if (!gemm_f64_bdiag(s, M1, k, rows, a1, b, 2 * b, Yl, ldy, 1.0, 0.0, P, M1, u)) return GEV_ERR_CUDA;
-      if (!gemm_f64_bdiag(s, rows, k, M1, a2, 2 * b, b, P, M1, -1.0, 1.0, Yl, ldy, u)) return GEV_ERR_CUDA;
-    }
+    // From orthonormal Z (s.z_unit), Y's columns stay unit vectors under the orthogonal transforms
+    // (|y_ij| <= 1), and |P_qj| = |v_q^H y_j| <= ||v_q|| <= sqrt(2) (a Householder vector with
+    // v(0) = 1): both below 2, so their scales need no pass over the data
+    const bool u = s.z_unit;
+    if (u && gemm_f64_bdiag_level(s, M1, rows, k, a1, a2, b, Yl, ldy, P, M1)) continue;
+    if (!gemm_f64_bdiag(s, M1, k, rows, a1, b, 2 * b, Yl, ldy, 1.0, 0.0, P, M1, u)) return GEV_ERR_CUDA;
+    if (!gemm_f64_bdiag(s, rows, k, M1, a2, 2 * b, b, P, M1, -1.0, 1.0, Yl, ldy, u)) return GEV_ERR_CUDA;
   }
   return last_error();
 }
@@ -879,8 +868,8 @@ template <class T> int bt_hb2st(Sys& s, const double* Z, int ldz, int k, T* Y, i
   }
   if (n <= 2) return 0;
   if constexpr (std::is_same<T, float>::value) {
-    // (the block-diagonal BF16x6 form, bt_levels_wy<float>, measured slower than this register kernel
-    // at n = 16384: 747 ms against 556 ms, its split passes and short-K products being latency bound)
+    // (block-diagonal BF16x6 products on the tensor cores measured slower than this register kernel at n = 16384: 747 ms
+    // against 556 ms, their split passes and short-K products being latency bound)
     if (b == 16) return bt_levels_f32<16>(s, n, k, Y, ldy);
     if (b == 32) return bt_levels_f32<32>(s, n, k, Y, ldy);
     if (b == 64) return bt_levels_f32<64>(s, n, k, Y, ldy);

@@ -324,11 +324,6 @@ size_t gemm_f64_bdiag_scratch(int M, int N, int K, int bm, int bk, int cx);
 // both products of a back-transform-2 level, P = op(A1) Y and Y -= op(A2) P, for entries below 2 (ozaki.cu)
 bool gemm_f64_bdiag_level(Sys& s, int M1, int rows, int N, const BdOp& a1, const BdOp& a2, int b, void* Y, long long ldy,
                           void* P, long long ldp);
-// The same in FP32 from BF16x6 (or x3, s.fp32_tc) split products on the tensor cores (tc_gemm.cu);
-// real data only.
-bool gemm_f32_bdiag(Sys& s, int M, int N, int K, const BdOp& a, int bm, int bk, const float* B, long long ldb,
-                    float alpha, float beta, float* C, long long ldc);
-size_t gemm_f32_bdiag_scratch(int M, int N, int K, int bm, int bk);
 template <class T> GemmP<T> gp(int M, int N, int K, int ta, int tb, T alpha, const T* A, long long lda,
                                const T* B, long long ldb, T beta, T* C, long long ldc) {
   GemmP<T> p{};

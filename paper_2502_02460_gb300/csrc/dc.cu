@@ -43,7 +43,6 @@ struct Node {
   int ndefl;         // deflated count
   int nrot;          // Givens rotations applied
   int Kout;          // eigenvectors to form (roots with final position < kcut)
-  int Dout;          // deflated vectors with final position < kcut
   double r;          // 2|rho|
   double zn2;        // sum of squared non-deflated z
 };
@@ -476,7 +475,7 @@ __global__ void __launch_bounds__(PREP_NTH) k_merge_prep(int n, int nleaf, int s
       nd.a = a; nd.m = m; nd.c = c;
       nd.K = K; nd.K1 = K1; nd.K2 = K2; nd.K3 = K3; nd.ndefl = D; nd.nrot = R;
       nd.r = r; nd.zn2 = zn2;
-      nd.Kout = K; nd.Dout = D;
+      nd.Kout = K;
     }
   }
   // apply the rotations, in order, to the physical columns (rows a .. c-1)
@@ -636,7 +635,7 @@ __global__ void __launch_bounds__(256) k_zprime(Node* nodes, DcArrays A) {
 }
 
 // Final positions of roots and deflated entries within each node; eigenvalues in sorted order.
-__global__ void k_positions(Node* nodes, DcArrays A, int kcut, int* status) {
+__global__ void k_positions(Node* nodes, DcArrays A) {
   Node& nd = nodes[blockIdx.y];
   const int a = nd.a, K = nd.K, D = nd.ndefl;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < K + D; t += gridDim.x * blockDim.x) {
@@ -659,24 +658,20 @@ __global__ void k_positions(Node* nodes, DcArrays A, int kcut, int* status) {
   }
 }
 
-// The roots / deflated entries of the top merge whose position is below kcut are prefixes of their lists
-// (positions increase): Kout and Dout, by bisection.  The deflation count goes to the status words.
+// The roots of the top merge whose position is below kcut are a prefix of their list (positions increase): Kout, by
+// bisection.  The deflation count goes to the status words.
 __global__ void k_count_out(Node* nodes, DcArrays A, int kcut, int* status) {
   Node& nd = nodes[0];
-  if (threadIdx.x > 1) return;
-  const int* pos = (threadIdx.x ? A.pos_d : A.pos_r) + nd.a;
-  int lo = 0, hi = threadIdx.x ? nd.ndefl : nd.K;
+  if (threadIdx.x > 0) return;
+  const int* pos = A.pos_r + nd.a;
+  int lo = 0, hi = nd.K;
   while (lo < hi) {
     const int md = (lo + hi) >> 1;
     if (pos[md] < kcut) lo = md + 1;
     else hi = md;
   }
-  if (threadIdx.x) {
-    nd.Dout = lo;
-    status[ST_DEFLATED] = nd.ndefl;
-  } else {
-    nd.Kout = lo;
-  }
+  nd.Kout = lo;
+  status[ST_DEFLATED] = nd.ndefl;
 }
 
 // U (gather order rows x Kout, ld ldu) column j: u_i = z'_i/(delta_i - lambda_j), normalised.
@@ -709,8 +704,8 @@ __global__ void k_vectors(Node* nodes, DcArrays A, double* U, long long ldu) {
   for (int i = threadIdx.x; i < K; i += blockDim.x) col[i] *= inv;
 }
 
-// Qg[:, a + g] = Q[:, nd_col] (rows a .. c-1) in gather order; deflated columns (position < kcut)
-// go straight to Qout[:, a + K + u].
+// Qg[:, a + g] = Q[:, nd_col] (rows a .. c-1) in gather order; deflated columns go straight to
+// Qout[:, a + K + u].
 __global__ void k_gather(Node* nodes, DcArrays A, const double* Q, long long ldq, double* Qg,
                          double* Qout) {
   const Node nd = nodes[blockIdx.y];
@@ -723,7 +718,6 @@ __global__ void k_gather(Node* nodes, DcArrays A, const double* Q, long long ldq
       Qg[(a + i) + (long long)(a + g) * ldq] = Q[(a + i) + (long long)src * ldq];
   } else if (t < nd.K + nd.ndefl) {
     const int u = t - nd.K;
-    if (A.pos_d[a + u] >= 0x7fffffff) return;
     const int src = A.df_col[a + u];
     for (int i = threadIdx.x; i < nn; i += blockDim.x)
       Qout[(a + i) + (long long)(a + nd.K + u) * ldq] = Q[(a + i) + (long long)src * ldq];
@@ -864,7 +858,7 @@ int stedc(Sys& s, const double* d, const double* e, int k, double* w, double* Z,
     k_zprime<<<dim3(cdiv(smax, 8), nnodes), 256, 0, st>>>(A.nodes, A);
     const int kcut = top ? k : 0x7fffffff;
     GEV_COUNT(s);
-    k_positions<<<dim3(cdiv(smax, 256), nnodes), 256, 0, st>>>(A.nodes, A, kcut, s.status);
+    k_positions<<<dim3(cdiv(smax, 256), nnodes), 256, 0, st>>>(A.nodes, A);
     if (top) {
       GEV_COUNT(s);
       k_count_out<<<1, 32, 0, st>>>(A.nodes, A, kcut, s.status);
