@@ -621,7 +621,8 @@ def main():
         peak = mp.get("bf16_tflops_sustained", 1764.7)
         achieved = EMU_PAIRS * fp64_tf if fp64_tf else None
         roof_kernel = ("ozaki_kernel + k_split/k_vec_exp (FP64 products as 36 BF16 digit-pair tcgen05 MMAs, "
-                       "achieved = 36 x FP64 algorithmic flops / time of every FP64 product launch)")
+                       "achieved = 36 x FP64 algorithmic flops / time of every FP64 product launch, the short products "
+                       "that run on the FP64 pipe counted alike)")
         peak_source = f"{src} bf16_tflops_sustained"
     else:
         peak = mp.get("bf16_tflops_sustained", 1764.7) * FP64_NOMINAL_TF / BF16_NOMINAL_TF

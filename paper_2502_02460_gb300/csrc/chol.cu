@@ -73,6 +73,12 @@ __device__ void inv_lower_blocked(int jb, const T* L, T* X, T* tmp) {
   }
 }
 
+// d > 0 (and no NaN), on the bits: an FP64 comparison costs as much as a multiplication
+__device__ __forceinline__ bool positive(double d) {
+  const long long b = __double_as_longlong(d);
+  return b > 0 && b <= 0x7FF0000000000000ll;
+}
+
 // Factor the jb x jb diagonal block (lower) and invert the factor, blocked by SB, on 16 warps.  Step kb:
 //   1. warps 0 - 7 factor and invert the SB x SB diagonal block, one entry (i, j), j <= i, per thread:
 //      before pivot j the thread holds a_ij of the trailing matrix, after it x_ij of the inverse of the
@@ -87,14 +93,9 @@ __device__ void inv_lower_blocked(int jb, const T* L, T* X, T* tmp) {
 // complex).  One warp gets a quarter of that rate at most (a warp instruction occupies its scheduler's FP64
 // unit for about 75 cycles), so a pivot chain in one warp's registers took 36 us for each 16 rows: 150 us for the
 // block, 57 us now.
-// L goes to A (when wanted) and X = L^{-1} to Xout, both with zeros above the diagonal.  A non-positive
+// L goes to A (when wanted; its diagonal is d_j recip_sqrt(d_j), within 2.75 2^-53 of the root) and X = L^{-1} to
+// Xout, both with zeros above the diagonal.  A non-positive
 // pivot records its index (first one, atomicCAS) and stops; nothing is written then.
-// d > 0 (and no NaN), on the bits: an FP64 comparison costs as much as a multiplication
-__device__ __forceinline__ bool positive(double d) {
-  const long long b = __double_as_longlong(d);
-  return b > 0 && b <= 0x7FF0000000000000ll;
-}
-
 constexpr int PD_NT = 512, PD_G = 256;  // threads in all, threads of the diagonal block's group
 template <class T>
 __global__ void __launch_bounds__(PD_NT) k_potrf_diag(int jb, T* A, long long lda, int want_l, T* Xout, long long ldx,

@@ -2,10 +2,12 @@
 // full Hermitian A -> band B of width b, A = Q1 B Q1^H, and the matching back-transform Y = Q1 Z.
 //
 // For each panel (columns j0..j0+b-1, rows r0 = j0+b .. n-1):
-//   1. Householder QR of the m x b panel (m = n - r0) in ONE cooperative kernel: the panel rows are
-//      spread over all SMs and stay in shared memory; each column needs one bounded grid barrier
-//      (the norm and the reflector's inner products together, which also give the column of the
-//      compact-WY factor T).  Q = H_0 ... H_{b-1} = I - Y T Y^H, T upper triangular.
+//   1. Householder QR of the m x b panel (m = n - r0) in ONE kernel: the panel rows are spread over the
+//      blocks and stay in shared memory; each column needs one barrier (the norm and the reflector's
+//      inner products together, which also give the column of the compact-WY factor T).  Long panels: a
+//      cooperative grid over all SMs, whose barrier gives up after a bounded wait; short ones: one cluster
+//      of 16 blocks and its hardware barrier, which has no limit and needs none (all blocks of a cluster
+//      run, and none leaves before the last column).  Q = H_0 ... H_{b-1} = I - Y T Y^H, T upper triangular.
 //   2. Two-sided update of the trailing block A22 <- Q^H A22 Q by GEMMs:
 //        W = A22 Y T,  U = T^H (Y^H W),  V = W - Y U / 2,  A22 -= [Y V] [V Y]^H (lower, one
 //        rank-2b product), mirror.
@@ -56,7 +58,7 @@ template <class T> struct PanelArgs {
 //
 // The column is a chain of latencies, not of work (m B multiply-adds over all SMs: 0.3 - 2 us): the
 // partial sums and the barrier's flag travel through L2 once each, all partial sums a thread adds are
-// loaded together (20 or 40 at a time), the reflector is one rsqrt and one division, and the two warps
+// loaded together (20 or 40 at a time), the reflector is one reciprocal root and one reciprocal, and the two warps
 // that need its inner products compute it themselves.  Per panel, averages over a reduction: n = 1500, b = 32
 // 275 us at first, 127 now (in a cluster); n = 10240, b = 64 782 -> 410; complex n = 509, b = 32 440 -> 270 (grid form).
 // The partial-sum buffers alternate with the column's parity: a block may start column c + 1 while a
