@@ -115,8 +115,9 @@ typedef struct {
                             faster on GB300 at every order (the one-stage form's matrix-vector products are
                             bound by the FP64 pipe, the two-stage route's products run on the tensor cores).
                             Its vectors carry a few more rounding errors: real n = 4096 and complex
-                            n = 2048 lie 1.25 to 1.7 times further from the exact ones, both near
-                            0.1 eps ||A|| / gap; one_stage = 1 keeps the other route.  With native products
+                            n = 2048 lie 1.3 to 2 times further from the exact ones (both near
+                            0.1 eps ||A|| / gap), and are orthogonal to 6e-12 instead of 1.3e-12
+                            (real 4096); one_stage = 1 keeps the other route.  With native products
                             (fp64_emulation = 0) one-stage from n = 2048 on for k >= n/2, and up to 8192
                             for fewer pairs (real data from 2560), where that measured faster */
   int rr_one_stage;      /* mixed form, the FP64 Rayleigh-Ritz solve of the refinement (all k pairs of
